@@ -52,11 +52,11 @@ static Loc loc_of(const gi_exec* e, int t) {
   return l;
 }
 
-// Weights of the CUDA-core convolution kernel: float W[group][tap][in_slice][OS*4 co][4 ci],
-// a group being OS consecutive output slices; entries beyond Cin / Cout are zero.
-static void pack_conv_simt(const OpNode& op, int cin, int storage, int os, std::vector<uint8_t>* blob, LaunchRec* r) {
+// Weights of the CUDA-core convolution kernel: float W[group][tap][in_slice][32 co][4 ci],
+// a group being 8 consecutive output slices; entries beyond Cin / Cout are zero.
+static void pack_conv_simt(const OpNode& op, int cin, int storage, std::vector<uint8_t>* blob, LaunchRec* r) {
   const int taps = op.d.kh * op.d.kw, sin = slices(cin), sout = slices(op.d.cout);
-  const int groups = (sout + os - 1) / os, jn = os * 4;
+  const int groups = (sout + 7) / 8, jn = 32;
   const uint64_t nw = static_cast<uint64_t>(groups) * taps * sin * jn * 4;
   const uint64_t woff = blob_reserve(blob, nw * sizeof(float));
   const uint64_t boff = blob_reserve(blob, static_cast<uint64_t>(groups) * jn * sizeof(float));
@@ -509,10 +509,7 @@ gi_status lower(const gi_graph& g, gi_exec* e) {
             conv_kxk_tc_pack(op.weights.data(), op.bias.data(), din->c, op.d.cout, op.d.kh, &e->weight_blob, &r);
           } else {
             r.kernel = GI_KERNEL_CONV_SIMT;
-            const int sout = slices(op.d.cout);
-            const int os = sout >= 8 ? 8 : sout >= 4 ? 4 : sout >= 2 ? 2 : 1;
-            r.tc_nt = os;
-            pack_conv_simt(op, din->c, e->storage, os, &e->weight_blob, &r);
+            pack_conv_simt(op, din->c, e->storage, &e->weight_blob, &r);
           }
           info.bytes += taps * din->c * op.d.cout * eb;
           info.flops = 2 * taps * out_px * din->c * op.d.cout;

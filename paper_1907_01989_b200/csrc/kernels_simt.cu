@@ -176,57 +176,145 @@ struct ConvGeom {
   int kh, kw, sh, sw, dh, dw, pt, pl;
 };
 
-// One thread = one output pixel x OS output slices.  Weights W[group][tap][in_slice][OS*4][4]
-// are read with warp-uniform addresses (one broadcast L1 transaction per float4).
-template <typename T, int OS>
-__global__ void __launch_bounds__(128) conv_simt_kernel(const T* __restrict__ in, const float4* __restrict__ w,
-                                                        const float* __restrict__ bias, const T* __restrict__ res,
-                                                        T* __restrict__ out, ConvGeom g, Epilogue ep) {
+// Direct convolution on the CUDA cores: fp32 storage, and the shapes no tensor-core kernel runs in fp16 storage.
+//
+// A warp owns 32 output pixels x 32 output channels of the batch's flattened pixel axis, a lane 4 pixels x 8 channels.  The sum
+// runs over units of (tap, 4 input channels); a unit is 32 pixel-slices + 512 bytes of weights, one 16-byte cp.async of each per
+// lane into a ring of kConvStages units that belongs to the warp alone, so nothing waits for another warp.  Even and odd input
+// channels are summed in the two halves of packed fp32 pairs (fma.rn.f32x2: pixel-slice and weights are pairs as they lie).
+// The sum is split over `kw` warps of a CTA until the launch fills the chip - a layer of the last stage at batch 2 has 20 such
+// tiles of 240 units each - and the partial sums are added in warp order through shared memory, so results do not depend on
+// timing.  What bounds it: at small batch the chain of a launch (about 4 us), at large batch the shared-memory reads
+// (12 16-byte reads per 64 packed multiply-adds).  The kernel before it gave one pixel and up to 32 channels to a thread
+// that walked the whole sum by itself: 7x7 960 -> 160 at batch 2 took 225 us with one block per 32 channels (16 us now, each
+// with an event pair around it); MobileNetV2-224 in fp32 storage at batch 2 3849 -> 352 us.
+constexpr int kConvStages = 6;
+constexpr int kConvStageBytes = 1024;  // 32 pixel-slices (512 bytes in fp32 storage) and 32 channels x 4 weights
+constexpr int kConvWarpBytes = kConvStages * kConvStageBytes;
+constexpr int kConvMaxSplit = 16;
+
+__device__ __forceinline__ void cp_async_px(unsigned dst, const float* src, bool valid) {
+  const unsigned n = valid ? 16u : 0u;  // 0: nothing is read, zeros are written
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
+}
+__device__ __forceinline__ void cp_async_px(unsigned dst, const __half* src, bool valid) {
+  const unsigned n = valid ? 8u : 0u;
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
+}
+__device__ __forceinline__ void fma2(unsigned long long& acc, float a0, float a1, float b0, float b1) {
+  unsigned long long a, b;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(a) : "f"(a0), "f"(a1));
+  asm("mov.b64 %0, {%1, %2};" : "=l"(b) : "f"(b0), "f"(b1));
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
+}
+
+template <typename T>
+__global__ void __launch_bounds__(32 * kConvMaxSplit) conv_simt_kernel(const T* __restrict__ in, const float4* __restrict__ w,
+                                                                       const float* __restrict__ bias, const T* __restrict__ res,
+                                                                       T* __restrict__ out, ConvGeom g, Epilogue ep, int kw) {
+  extern __shared__ __align__(128) unsigned char conv_smem[];
   pdl_launch_dependents();
-  pdl_wait();
-  const int pix = blockIdx.x * 128 + threadIdx.x;
-  const int grp = blockIdx.y, b = blockIdx.z;
-  if (pix >= g.Pout) return;
-  constexpr int JN = OS * 4;
-  float acc[JN];
-#pragma unroll
-  for (int j = 0; j < JN; ++j) acc[j] = 0.f;
-  const bool real = pix < g.Ho * g.Wo;
-  if (real) {
-    const int oy = pix / g.Wo, ox = pix - oy * g.Wo;
-    const float4* wg = w + static_cast<size_t>(grp) * g.kh * g.kw * g.Sin * JN;
-    for (int ky = 0; ky < g.kh; ++ky) {
-      const int iy = oy * g.sh - g.pt + ky * g.dh;
-      if (iy < 0 || iy >= g.H) continue;
-      for (int kx = 0; kx < g.kw; ++kx) {
-        const int ix = ox * g.sw - g.pl + kx * g.dw;
-        if (ix < 0 || ix >= g.W) continue;
-        const float4* wt = wg + static_cast<size_t>(ky * g.kw + kx) * g.Sin * JN;
-        const T* ip = in + (static_cast<size_t>(b) * g.Pin + iy * g.W + ix) * 4;
-        for (int s = 0; s < g.Sin; ++s) {
-          const float4 x = Px<T>::load(ip + static_cast<size_t>(s) * g.B * g.Pin * 4);
-          const float4* ws = wt + s * JN;
-#pragma unroll
-          for (int j = 0; j < JN; ++j) {
-            const float4 wv = __ldg(ws + j);
-            acc[j] = fmaf(x.x, wv.x, acc[j]);
-            acc[j] = fmaf(x.y, wv.y, acc[j]);
-            acc[j] = fmaf(x.z, wv.z, acc[j]);
-            acc[j] = fmaf(x.w, wv.w, acc[j]);
-          }
-        }
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int part = warp % kw, tpc = (blockDim.x >> 5) / kw;
+  const long long m_total = static_cast<long long>(g.B) * g.Pout;
+  const long long m0 = (static_cast<long long>(blockIdx.x) * tpc + warp / kw) * 32;
+  const int grp = blockIdx.y, taps = g.kh * g.kw, units = taps * g.Sin;
+  const int u0 = static_cast<int>(static_cast<long long>(units) * part / kw), u1 = static_cast<int>(static_cast<long long>(units) * (part + 1) / kw);
+  unsigned char* ring = conv_smem + warp * kConvWarpBytes;
+  const unsigned ring_s = static_cast<unsigned>(__cvta_generic_to_shared(ring));
+
+  // this lane copies one pixel: m0 + lane
+  const long long m = m0 + lane;
+  const int b = m < m_total ? static_cast<int>(m / g.Pout) : 0;
+  const int rem = m < m_total ? static_cast<int>(m - static_cast<long long>(b) * g.Pout) : g.Pout;
+  const int oy = rem / g.Wo, ox = rem - oy * g.Wo;
+  const bool real = rem < g.Ho * g.Wo;
+  const int y0 = oy * g.sh - g.pt, x0 = ox * g.sw - g.pl;
+  const size_t slice_step = static_cast<size_t>(g.B) * g.Pin * 4;
+  const float4* wsrc = w + (static_cast<size_t>(grp) * units + u0) * 32 + lane;
+  int tap = u0 / g.Sin, s = u0 - tap * g.Sin;
+  bool ok = false;
+  const T* src = in;
+  auto at_tap = [&]() {
+    const int ky = tap / g.kw, kx = tap - ky * g.kw;
+    const int iy = y0 + ky * g.dh, ix = x0 + kx * g.dw;
+    ok = real && iy >= 0 && iy < g.H && ix >= 0 && ix < g.W;
+    src = in + (ok ? (static_cast<size_t>(b) * g.Pin + static_cast<size_t>(iy) * g.W + ix) * 4 : 0) + s * slice_step;
+  };
+  at_tap();
+  auto issue = [&](int u) {
+    if (u < u1) {
+      const unsigned dst = ring_s + ((u - u0) % kConvStages) * kConvStageBytes;
+      cp_async_px(dst + lane * 4 * static_cast<unsigned>(sizeof(T)), src, ok);
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 512 + lane * 16), "l"(wsrc) : "memory");
+      wsrc += 32;
+      src += slice_step;
+      if (++s == g.Sin) {
+        s = 0;
+        ++tap;
+        at_tap();
       }
     }
-  }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+
+  pdl_wait();
+  for (int i = 0; i < kConvStages - 1; ++i) issue(u0 + i);
+  const int pl = lane & 7, cl = lane >> 3;  // pixels pl + 8 i, channels cl + 4 j: lane cl holds component cl of every output slice
+  unsigned long long acc[4][8];
 #pragma unroll
-  for (int o = 0; o < OS; ++o) {
-    const int so = grp * OS + o;
-    if (so >= g.Sout) break;
-    const size_t idx = ((static_cast<size_t>(so) * g.B + b) * g.Pout + pix) * 4;
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 8; ++j) acc[i][j] = 0ull;
+  for (int u = u0; u < u1; ++u) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(kConvStages - 2) : "memory");
+    __syncwarp();
+    const unsigned char* st = ring + ((u - u0) % kConvStages) * kConvStageBytes;
+    float4 x[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) x[i] = Px<T>::load(reinterpret_cast<const T*>(st) + (pl + 8 * i) * 4);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const float4 wv = *reinterpret_cast<const float4*>(st + 512 + (cl + 4 * j) * 16);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        fma2(acc[i][j], x[i].x, x[i].y, wv.x, wv.y);
+        fma2(acc[i][j], x[i].z, x[i].w, wv.z, wv.w);
+      }
+    }
+    __syncwarp();
+    issue(u + kConvStages - 1);
+  }
+
+  // partial sums: [output slice][pixel] float4 in the warp's own ring, then summed over the parts in order
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncwarp();
+  float* part_sum = reinterpret_cast<float*>(ring);
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      float lo, hi;
+      asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(acc[i][j]));
+      part_sum[(j * 32 + pl + 8 * i) * 4 + cl] = lo + hi;
+    }
+  __syncthreads();
+  const float4* first = reinterpret_cast<const float4*>(conv_smem + (warp - part) * kConvWarpBytes);
+  for (int i = part * 32 + lane; i < 256; i += kw * 32) {
+    const int so = grp * 8 + (i >> 5);
+    const long long mo = m0 + (i & 31);
+    if (so >= g.Sout || mo >= m_total) continue;
+    const size_t idx = (static_cast<size_t>(so) * m_total + mo) * 4;
     float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (real) {
-      const float4 bv = *reinterpret_cast<const float4*>(bias + (grp * OS + o) * 4);
-      v = make_float4(acc[o * 4] + bv.x, acc[o * 4 + 1] + bv.y, acc[o * 4 + 2] + bv.z, acc[o * 4 + 3] + bv.w);
+    if (static_cast<int>(mo % g.Pout) < g.Ho * g.Wo) {  // the padding pixel of an odd plane holds zeros
+      v = *reinterpret_cast<const float4*>(bias + so * 4);
+      for (int k = 0; k < kw; ++k) {
+        const float4 q = first[k * (kConvWarpBytes / 16) + i];
+        v.x += q.x;
+        v.y += q.y;
+        v.z += q.z;
+        v.w += q.w;
+      }
       v = epilogue<T>(v, ep, res, idx);
     }
     Px<T>::store(out + idx, v);
@@ -506,28 +594,32 @@ int launch_unpack(const LaunchRec& r, const Ptrs& p, int storage, void* stream) 
 }
 
 template <typename T>
-static void conv_dispatch(const LaunchRec& r, const Ptrs& p, cudaStream_t st) {
+static int conv_dispatch(const LaunchRec& r, const Ptrs& p, cudaStream_t st) {
   const ConvGeom g = geom(r);
-  const int os = r.tc_nt;
-  const dim3 grid(blocks_for(g.Pout, 128), (g.Sout + os - 1) / os, r.B);
-  const T* in = static_cast<const T*>(p.in0);
-  const float4* w = static_cast<const float4*>(p.wts);
-  const float* b = static_cast<const float*>(p.bias);
-  const T* res = static_cast<const T*>(p.res);
-  T* out = static_cast<T*>(p.out);
-  switch (os) {
-    case 8: launch_pdl(conv_simt_kernel<T, 8>, grid, 128, 0, st, in, w, b, res, out, g, r.ep); break;
-    case 4: launch_pdl(conv_simt_kernel<T, 4>, grid, 128, 0, st, in, w, b, res, out, g, r.ep); break;
-    case 2: launch_pdl(conv_simt_kernel<T, 2>, grid, 128, 0, st, in, w, b, res, out, g, r.ep); break;
-    default: launch_pdl(conv_simt_kernel<T, 1>, grid, 128, 0, st, in, w, b, res, out, g, r.ep); break;
+  const long long tiles = (static_cast<long long>(g.B) * g.Pout + 31) / 32;
+  const int groups = (g.Sout + 7) / 8, units = g.kh * g.kw * g.Sin;
+  // split the sum until there are 16 warps per SM or a warp has 4 units left: 7x7 960 -> 160 at batch 2, 225 -> 16 us (event pair around one launch)
+  int kw = 1;
+  while (kw < kConvMaxSplit && tiles * groups * kw < 148 * 16 && units >= kw * 8) kw *= 2;
+  const int warps = kw > 8 ? kw : 8, tpc = warps / kw;
+  const size_t smem = static_cast<size_t>(warps) * kConvWarpBytes;
+  static bool attr_done_dev[kMaxDevices] = {};
+  bool& attr_done = attr_done_dev[current_device_slot()];
+  if (!attr_done) {
+    const cudaError_t e = cudaFuncSetAttribute(conv_simt_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kConvMaxSplit * kConvWarpBytes);
+    if (e != cudaSuccess) return static_cast<int>(e);
+    attr_done = true;
   }
+  const long long blocks = (tiles + tpc - 1) / tpc;
+  if (blocks > 2147483647LL || groups > 65535) return static_cast<int>(cudaErrorInvalidConfiguration);
+  return static_cast<int>(launch_pdl(conv_simt_kernel<T>, dim3(static_cast<unsigned>(blocks), groups), 32 * warps, smem, st,
+                                     static_cast<const T*>(p.in0), static_cast<const float4*>(p.wts), static_cast<const float*>(p.bias),
+                                     static_cast<const T*>(p.res), static_cast<T*>(p.out), g, r.ep, kw));
 }
 
 int launch_conv_simt(const LaunchRec& r, const Ptrs& p, int storage, void* stream) {
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (r.B > 65535) return static_cast<int>(cudaErrorInvalidConfiguration);
-  GI_BY_STORAGE(conv_dispatch<__half>(r, p, st), conv_dispatch<float>(r, p, st));
-  return static_cast<int>(cudaGetLastError());
+  return storage == GI_F16 ? conv_dispatch<__half>(r, p, st) : conv_dispatch<float>(r, p, st);
 }
 
 int launch_depthwise(const LaunchRec& r, const Ptrs& p, int storage, void* stream) {

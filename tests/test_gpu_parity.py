@@ -90,6 +90,18 @@ PW_CASES = [  # batch, hw, cin, cout, residual, act
 ]
 
 
+@pytest.mark.parametrize("storage", STORAGES)
+@pytest.mark.parametrize("case", [(2, 1, 1, 1280, 33, 1, 1),   # 4 stored pixels, the sum split over 16 warps, one channel in the last group
+                                  (1, 3, 11, 35, 32, 1, 1),    # 34 stored pixels: a tile of two pixels, a ragged input slice
+                                  (3, 5, 7, 5, 40, 3, 1),      # 18 units of (tap, slice): parts of different lengths
+                                  (1, 4, 4, 3, 8, 2, 2),       # fewer units than pipeline stages
+                                  (1, 40, 40, 96, 300, 1, 1),  # a part per warp of one tile only: no split
+                                  (2, 13, 9, 24, 7, 3, 3)])
+def test_direct_convolution_tiles_and_splits(storage, case):
+    """The CUDA-core convolution at the edges of its 32 x 32 tiles and of the split of its sum (every tensor, padding included)."""
+    check_all_tensors(wl.single_conv(*case), storage, api.GI_PW_SIMT)
+
+
 @pytest.mark.parametrize("case", PW_CASES)
 def test_pointwise_fp32(case):
     batch, hw, cin, cout, residual, act = case
