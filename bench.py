@@ -624,7 +624,8 @@ def main():
     ex.bind(dev)
     ops = ex.ops()
     # ops that run inside another op's kernel, or need no kernel at all, launch nothing
-    n_launch = sum(1 for o in ops if api.KERNEL_NAMES[o.kernel] != "none")
+    launches = ex.launches()  # what one step launches; ops() describes the operators one by one
+    n_launch = sum(1 for x in launches if api.KERNEL_NAMES[x.kernel] != "none")
     # every rank draws its own images: rank r holds images [r*B, (r+1)*B) of the global batch
     x_host = wl.make_input(spec, images=shard_images(rank, args.batch)).astype(np.float16)
     x_pin = torch.from_numpy(x_host).pin_memory()
@@ -756,7 +757,7 @@ def main():
             per_op += np.array(ex.run_timed([x_dev], [out_dev], stream))
         per_op /= reps
         fam = {}
-        for o, t in zip(ops, per_op):
+        for o, t in zip(launches, per_op):
             name = api.KERNEL_NAMES[o.kernel]
             if name == "none":  # nothing was launched for this op (it ran inside another op's kernel, or needs none)
                 continue
@@ -804,9 +805,10 @@ def main():
         if args.per_op:
             with open(args.per_op, "w") as fh:
                 fh.write("# op kernel in_shape out_shape bytes flops ms GB/s TFLOP/s frac_of_roofline\n")
-                for i, (o, t) in enumerate(zip(ops, per_op)):
-                    ti = ex.tensor(o.inputs[0]) if o.inputs[0] >= 0 else None
-                    to = ex.tensor(o.output) if o.output >= 0 else None
+                for i, (o, t) in enumerate(zip(launches, per_op)):
+                    ti = ex.tensor(ops[i].inputs[0]) if ops[i].inputs[0] >= 0 else None
+                    last = ops[i + max(o.n_ops, 1) - 1].output
+                    to = ex.tensor(last) if last >= 0 else None
                     roof = max(o.bytes / (peaks["hbm_gbs"] * 1e9), o.flops / (peaks["bf16_tflops_sustained"] * 1e12)) * 1e3
                     fh.write(f"{i} {api.KERNEL_NAMES[o.kernel]} "
                              f"{(ti.h, ti.w, ti.c) if ti else '-'} {(to.h, to.w, to.c) if to else '-'} {o.bytes} {o.flops} "
@@ -879,7 +881,7 @@ def main():
                     graph_ms = a.elapsed_time(b) / 100
             except Exception as exc:  # graph capture is an extra, never the headline
                 graph_ms = f"capture failed: {type(exc).__name__}"
-            b1_launches = sum(1 for o in ex1.ops() if api.KERNEL_NAMES[o.kernel] != "none")
+            b1_launches = sum(1 for x in ex1.launches() if api.KERNEL_NAMES[x.kernel] != "none")
 
         gc.enable()
         cpu = None

@@ -192,6 +192,19 @@ typedef struct gi_op_info {
   uint64_t flops;       /* algorithmic flops (2 per multiply-add) */
 } gi_op_info;
 
+/* What gi_run launches at an executed op.  gi_op_info describes the ops one by one, each with the kernel chosen for it
+ * alone; with GI_XOP_AUTO, GI_PW_AUTO, `fuse` set and fp16 storage, gi_run launches a depthwise 3x3 op with the ops
+ * around it as ONE kernel where that is faster: the tensors between them are then never stored (their place in the arena
+ * may hold anything), and results are those of the ops one after the other up to the order of fp32 sums.  Under
+ * GI_PLAN_NAIVE gi_op_info itself says so: its `kernel` is then that of the launch, and GI_KERNEL_NONE marks the ops inside
+ * one.  (GI_XOP_OFF keeps one kernel per op.) */
+typedef struct gi_launch_info {
+  int32_t kernel;       /* GI_KERNEL_*; GI_KERNEL_NONE: no launch here, another op's kernel runs this op */
+  int32_t n_ops;        /* executed ops up to the next launch (0 for GI_KERNEL_NONE) */
+  uint64_t bytes;       /* algorithmic bytes of the launch: its inputs, residual and outputs once, weights once */
+  uint64_t flops;
+} gi_launch_info;
+
 enum { GI_EXEC_PACK = 100, GI_EXEC_UNPACK = 101 };
 enum {
   GI_KERNEL_PACK = 1, GI_KERNEL_UNPACK = 2, GI_KERNEL_CONV_SIMT = 3, GI_KERNEL_POINTWISE_TC = 4,
@@ -202,7 +215,8 @@ enum {
   GI_KERNEL_CONV_TC = 14,             /* k x k convolution, any number of input channels, on the tensor cores */
   GI_KERNEL_INVERTED_RESIDUAL = 15,   /* this op (1x1 expansion) and the next two (depthwise 3x3, 1x1 projection) as one kernel */
   GI_KERNEL_POINTWISE_MM = 16,        /* 1x1 convolution, wide tiles for tensor-bound shapes */
-  GI_KERNEL_POINTWISE_CHAIN = 17      /* this op (1x1) and the next one (1x1) as one kernel; both outputs are stored */
+  GI_KERNEL_POINTWISE_CHAIN = 17,     /* this op (1x1) and the next one (1x1) as one kernel; both outputs are stored */
+  GI_KERNEL_BLOCK_MMA = 18            /* gi_exec_launch only: a depthwise 3x3 op with the ops around it as one kernel */
 };
 
 /* ---- graph construction (Section 3.1, "Initialization": the sub-graph given to the GPU backend) ---- */
@@ -251,6 +265,7 @@ GI_API gi_status gi_compile(const gi_graph* g, const gi_compile_options* opt, gi
 GI_API gi_status gi_exec_query(const gi_exec* e, gi_exec_info* info);
 GI_API gi_status gi_exec_tensor(const gi_exec* e, gi_tensor t, gi_tensor_info* info);
 GI_API gi_status gi_exec_op(const gi_exec* e, int32_t index, gi_op_info* info);
+GI_API gi_status gi_exec_launch(const gi_exec* e, int32_t index, gi_launch_info* info);
 
 /* Copy the packed weights (info.weight_bytes) into the caller's device buffer, asynchronously
  * on `stream` (a cudaStream_t, NULL for the default stream).  Must precede gi_run; the buffer

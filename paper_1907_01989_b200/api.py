@@ -30,7 +30,7 @@ GI_PW_AUTO, GI_PW_SIMT, GI_PW_TC_PAIR, GI_PW_TC_LANE, GI_PW_TC_WIDE, GI_PW_RULE 
 GI_XOP_AUTO, GI_XOP_OFF, GI_XOP_ON, GI_XOP_CHAIN = 0, 1, 2, 3
 GI_STATIC_ARENA_BYTES = 16 << 20
 KERNEL_NAMES = {1: "pack", 2: "unpack", 3: "conv_simt", 4: "pointwise_tc", 5: "depthwise", 6: "eltwise", 7: "pool",
-                8: "resize", 9: "conv3x3_tc", 10: "pointwise_ts", 11: "depthwise_pointwise", 12: "none", 13: "concat", 14: "conv_tc", 15: "inverted_residual", 16: "pointwise_mm", 17: "pointwise_chain"}
+                8: "resize", 9: "conv3x3_tc", 10: "pointwise_ts", 11: "depthwise_pointwise", 12: "none", 13: "concat", 14: "conv_tc", 15: "inverted_residual", 16: "pointwise_mm", 17: "pointwise_chain", 18: "block_mma"}
 
 _KIND = {wl.CONV2D: GI_OP_CONV2D, wl.DEPTHWISE: GI_OP_DEPTHWISE_CONV2D, wl.ADD: GI_OP_ADD,
          wl.ACTIVATION: GI_OP_ACTIVATION, wl.GLOBAL_AVG_POOL: GI_OP_GLOBAL_AVG_POOL,
@@ -69,8 +69,12 @@ class gi_op_info(C.Structure):
                 ("bytes", C.c_uint64), ("flops", C.c_uint64)]
 
 
+class gi_launch_info(C.Structure):
+    _fields_ = [("kernel", C.c_int32), ("n_ops", C.c_int32), ("bytes", C.c_uint64), ("flops", C.c_uint64)]
+
+
 EXPORTS = ["gi_graph_create", "gi_graph_input", "gi_add_op", "gi_graph_output", "gi_graph_destroy", "gi_compile",
-           "gi_exec_query", "gi_exec_tensor", "gi_exec_op", "gi_exec_bind", "gi_run", "gi_run_static", "gi_run_timed", "gi_device_status", "gi_selftest_bounded_wait", "gi_exec_destroy",
+           "gi_exec_query", "gi_exec_tensor", "gi_exec_op", "gi_exec_launch", "gi_exec_bind", "gi_run", "gi_run_static", "gi_run_timed", "gi_device_status", "gi_selftest_bounded_wait", "gi_exec_destroy",
            "gi_slice8_tensor_bytes", "gi_slice8_pointwise_blob_bytes", "gi_slice8_pointwise_pack", "gi_slice8_pointwise_run",
            "gi_status_str", "gi_last_error", "gi_tensor_bytes", "gi_f32_to_f16"]
 
@@ -103,6 +107,8 @@ def lib() -> C.CDLL:
     L.gi_exec_query.argtypes = [vp, C.POINTER(gi_exec_info)]
     L.gi_exec_tensor.argtypes = [vp, C.c_int32, C.POINTER(gi_tensor_info)]
     L.gi_exec_op.argtypes = [vp, C.c_int32, C.POINTER(gi_op_info)]
+    L.gi_exec_launch.argtypes = [vp, C.c_int32, C.POINTER(gi_launch_info)]
+    L.gi_exec_launch.restype = C.c_int32
     L.gi_exec_bind.argtypes = [vp, vp, C.c_size_t, vp]
     L.gi_run.argtypes = [vp, C.POINTER(vp), C.POINTER(vp), vp, C.c_size_t, vp]
     L.gi_run_static.argtypes = [vp, C.POINTER(vp), C.POINTER(vp), vp]
@@ -291,6 +297,15 @@ class Executable:
 
     def ops(self) -> List[gi_op_info]:
         return [self.op(i) for i in range(self.info.n_ops)]
+
+    def launch(self, i: int) -> gi_launch_info:
+        """What gi_run launches at executed op i (kernel "none": nothing, another launch covers it)."""
+        li = gi_launch_info()
+        _check(lib().gi_exec_launch(self._h, i, C.byref(li)), "gi_exec_launch")
+        return li
+
+    def launches(self) -> List[gi_launch_info]:
+        return [self.launch(i) for i in range(self.info.n_ops)]
 
     # -- device side -------------------------------------------------------------------
     def bind(self, device="cuda:0", stream=None) -> None:

@@ -1,0 +1,1232 @@
+// A depthwise 3x3 convolution with the convolutions around it as ONE kernel, for any plane size:
+//   1x1 expansion -> depthwise 3x3 -> 1x1 projection (+ residual)   an inverted-residual block
+//   3x3 stride-2 stem on a 3-channel NHWC image -> depthwise 3x3 -> 1x1   the first layers of the MobileNets
+//   depthwise 3x3 -> 1x1                                            a depthwise-separable pair
+// The tensors between the operators - up to six times as wide as the block's ends - never reach memory; they are rounded to
+// fp16 exactly where the separate kernels would have stored them.
+//
+// Why the warp-level matrix instruction.  All operators run on mma.sync.m16n8k16 (fp16 operands, fp32 sums), because its
+// register fragments chain: the depthwise result leaves the tensor core in the very registers in which the projection wants
+// its A operand, so of the two hidden tensors one is written to shared memory once (the 3x3 window has to gather from it)
+// and the other not at all.  Measured on one SM: one m16n8k16 per 2 cycles, 21 cycles of latency, one ldmatrix.x4 per 4
+// cycles.  tcgen05.mma has four times that rate, but its results come back through tensor memory and its A operand goes out
+// through shared memory, and a depthwise slice would occupy it for 47 cycles per instruction at N = 8.
+//
+// The depthwise operator as a matrix product.  A hidden pixel-slice is 4 channels (8 bytes); two neighbouring pixels are one
+// 16-byte row of an ldmatrix matrix.  Stride 1: an output PAIR (x, x+1) of one slice reads 4 input pixels x 4 channels = 16
+// values per window row, and produces 2 pixels x 4 channels = 8: one m16n8k16 per window row with the 3 taps in a banded
+// 16 x 8 operand.  Its 16 rows are 16 pairs, and a warp walks TR output rows down, so that the fragment of a hidden row serves
+// the three output rows around it in the very registers ldmatrix left it in (pairing vertical neighbours in the 16 rows needs
+// fewer loads, but every other fragment then has to be put together by register moves).  Stride 2: 16 output columns,
+// 4 channels x 2 output rows; 5 window rows = 5 instructions.  The N axis is ordered so that lane t of a quad holds channel t
+// of both outputs: packing the results of two slices gives half of the projection's A fragment with no shuffle.  Channels are
+// permuted to match when the weights are packed.
+//
+// Walk.  A unit is a tile of output pixels of one image (or whole small images); its CTA - or cluster of CTAs, each taking
+// every ks-th chunk of the hidden channels, their partial sums added in rank order through distributed shared memory - walks
+// the hidden channels in chunks of 16 or 32: the first operator of chunk c+1 into one of two hidden tiles while the depthwise
+// operator and the projection consume chunk c from the other; one barrier per chunk.  Weights arrive by cp.async, resident
+// when they fit, else through a ring of four chunks; they are requested before the previous kernel has finished.
+//
+// What bounds it.  Small launches: the chain of one unit (4.5 us for a pair, 6 to 10 us for a block at batch 1, against 4 us
+// for each of the two to four launches it replaces).  Large ones: nothing alone - on 56x56 24 -> 144 -> 24 at batch 256 a
+// chunk takes 1840 cycles of an SM for 800 of the matrix pipe, 770 of issue slots per scheduler and about 900 of shared
+// memory, with 16 warps to cover 21-cycle matrix and 30-cycle shared-memory latencies; 173 us against 194 us as three
+// kernels.  Measured on one B200, MobileNetV2: batch 1 225 -> 197 us, 21 images of 205 pixels 340 -> 288, batch 256 1413 ->
+// 1385; segmentation network batch 1 289 -> 246, batch 16 961 -> 874.
+#include <cuda_fp16.h>
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <cmath>
+#include <cstdlib>
+#include <cstring>
+#include <type_traits>
+
+#include "kernels.h"
+#include "pdl.cuh"
+#include "sm100_ptx.cuh"
+
+namespace gi {
+namespace {
+
+using namespace ptx;
+
+constexpr int kTableBytes = 1024;  // banded depthwise operands of 4 slices: [slice][16 lanes][3 window rows + pad] x 4 bytes
+constexpr int kBiasBytes = 64;     // 16 floats
+constexpr int kDwBiasBytes = 256;  // bias of 16 channels, each four times: the start value of a fragment of sums
+constexpr int kSubFixed = kBiasBytes + kTableBytes + kDwBiasBytes;
+constexpr int kRing = 4;
+constexpr int kSmemPerSm = 227 * 1024;
+
+// How the first operator is computed: none (the input is the hidden tensor), a 1x1 expansion from up to 16 / 24 / 32 / 160
+// channels, or the stem
+enum First { kNone = 0, kExp16 = 1, kExp24 = 2, kExp32 = 3, kExpWide = 4, kStem = 5 };
+
+// Bytes between the slices of a hidden tile: a constant, so that slices are immediate offsets.  32 modulo 128: the stores
+// of 4 pixels x 4 slices by half a warp meet 32 different banks.
+__host__ __device__ constexpr int slice_bytes(int first) { return first == kExpWide ? 18 * 128 + 32 : 36 * 128 + 32; }
+__host__ __device__ constexpr int tile_pixels(int first) { return slice_bytes(first) / 8 - 2; }
+// warps an SM holds: 128 registers a thread for 16 warps, 255 for 8 (96 sums per thread and more; tr: output rows a warp
+// walks down)
+__host__ __device__ constexpr int max_warps(int s, int np, int tr) { return (s == 1 ? tr : 1) * np >= 6 || tr == 4 ? 8 : 16; }
+// bytes of one 16-channel sub-block of packed weights: first operator's fragments and bias, banded depthwise operands and
+// bias, projection fragments
+__host__ __device__ constexpr int sub_bytes(int ke, int np) { return ke * 512 + kSubFixed + np * 512; }
+
+struct BlockParams {
+  const __half* in;
+  const __half* res;
+  __half* out;
+  const unsigned char* wts;
+  const float* bias;  // projection bias, 16 * NP floats
+  int B, H, W, Ho, Wo;                  // depthwise input and output planes
+  int in_px, in_img;                    // elements between pixels / images of the input
+  int o_px, res_img;                    // ... between pixels of the output, images of the residual (its pixels: 4)
+  long long in_sl, o_sl, o_img, res_sl; // elements between slices (and output images)
+  int sin, sout;      // input and output slices
+  int ke;             // 16-channel steps of a wide expansion's sum
+  int pad_t, pad_l;
+  int tw, nb, ni;     // output columns of a tile, bands of TR output rows, images of a unit
+  int tiles_x, tiles_y, units;
+  int rows, pitch, sub_px;  // hidden tile of one image: rows, pixels per row (even), rows * pitch
+  int n_list, mt;           // pixels the first operator computes, in groups of 16
+  int whole;                // a unit is whole images
+  int compact;              // the list holds image pixels only; the border of the hidden tile stays zero
+  int pw, ncols, ngroups;   // columns per band; columns and groups of 16 columns of a unit
+  int eg, en;               // groups of 16 list pixels for a warp with / without a column group
+  int nch, ks;              // chunks of hidden channels; CTAs sharing a unit
+  int resident;
+  unsigned x_pitch;
+  unsigned off_bias, off_tab, off_x, off_raw, off_hid, off_red;
+  unsigned x_bytes, tab_bytes;  // of one of the two input tiles / tables (narrow expansions; otherwise there is one)
+  unsigned mul_pitch, mul_w, mul_hw, mul_per, mul_tx;  // ceil(2^32 / d): division of a small number by d is one high multiplication
+  unsigned hi_e, hi_d;  // upper clamp of the hidden activations, two halves (6 or infinity)
+  int act_pre, act_post, has_res;
+  int res_x;            // the residual is the block's input: it is still in shared memory
+  int wide;             // both pixels of a pair are one aligned 16-byte store
+  int pad_px;           // an odd plane holds one more pixel: zero it
+  int Hi, Wi, spt, spl, raw_rows, raw_words;  // stem: image, its padding, the staged rows
+};
+
+__device__ __forceinline__ void cp_async16(unsigned dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+// 8 (4) bytes of which the first `bytes` are read and the others written as zeros
+__device__ __forceinline__ void cp_async8(unsigned dst, const void* src, unsigned bytes) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void cp_async4(unsigned dst, const void* src, unsigned bytes) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+__device__ __forceinline__ void ldsm4(unsigned addr, unsigned (&r)[4]) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void ldsm2(unsigned addr, unsigned& a, unsigned& b) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0, %1}, [%2];" : "=r"(a), "=r"(b) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void mma16816(float (&d)[4], const unsigned (&a)[4], unsigned b0, unsigned b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+// the same with the sum started from c0..c3 (a bias): saves copying it into the accumulators
+__device__ __forceinline__ void mma16816c(float (&d)[4], const unsigned (&a)[4], unsigned b0, unsigned b1, float c0, float c1, float c2,
+                                          float c3) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%10, %11, %12, %13};"
+      : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(c0), "f"(c1), "f"(c2), "f"(c3));
+}
+__device__ __forceinline__ void mma1688(float (&d)[4], unsigned a0, unsigned a1, unsigned b0) {
+  asm("mma.sync.aligned.m16n8k8.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5}, {%6}, {%0, %1, %2, %3};"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a0), "r"(a1), "r"(b0));
+}
+__device__ __forceinline__ uint4 lds128(unsigned addr) {
+  uint4 v;
+  asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ uint2 lds64(unsigned addr) {
+  uint2 v;
+  asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ unsigned lds32(unsigned addr) {
+  unsigned v;
+  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ void sts32(unsigned addr, unsigned a) { asm volatile("st.shared.u32 [%0], %1;" ::"r"(addr), "r"(a) : "memory"); }
+__device__ __forceinline__ void sts64(unsigned addr, unsigned a, unsigned b) {
+  asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(addr), "r"(a), "r"(b) : "memory");
+}
+__device__ __forceinline__ void sts128(unsigned addr, unsigned a, unsigned b, unsigned c, unsigned d) {
+  asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+}
+__device__ __forceinline__ float4 ld_cluster_f4(unsigned addr) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ unsigned min_f16x2(unsigned a, unsigned b) {
+  unsigned d;
+  asm("min.f16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
+  return d;
+}
+__device__ __forceinline__ unsigned prmt(unsigned a, unsigned sel) { return __byte_perm(a, 0u, sel); }
+
+__device__ __forceinline__ float act_f(float v, int act) {
+  if (act != GI_ACT_NONE) v = fmaxf(v, 0.0f);
+  if (act == GI_ACT_RELU6) v = fminf(v, 6.0f);
+  return v;
+}
+
+// Four consecutive channels (one pixel-slice) of the projection, bias included: activation, residual, activation, fp16.
+__device__ __forceinline__ uint2 finish4(const BlockParams& p, float v0, float v1, float v2, float v3, const uint2& r) {
+  if (p.act_pre != GI_ACT_NONE) {
+    v0 = act_f(v0, p.act_pre);
+    v1 = act_f(v1, p.act_pre);
+    v2 = act_f(v2, p.act_pre);
+    v3 = act_f(v3, p.act_pre);
+  }
+  if (p.has_res) {
+    const float2 r01 = __half22float2(*reinterpret_cast<const __half2*>(&r.x));
+    const float2 r23 = __half22float2(*reinterpret_cast<const __half2*>(&r.y));
+    v0 += r01.x;
+    v1 += r01.y;
+    v2 += r23.x;
+    v3 += r23.y;
+    if (p.act_post != GI_ACT_NONE) {
+      v0 = act_f(v0, p.act_post);
+      v1 = act_f(v1, p.act_post);
+      v2 = act_f(v2, p.act_post);
+      v3 = act_f(v3, p.act_post);
+    }
+  }
+  return make_uint2(pack_f16x2<false>(v0, v1), pack_f16x2<false>(v2, v3));
+}
+
+__host__ __device__ __forceinline__ int div_by(int i, unsigned mul) {
+#ifdef __CUDA_ARCH__
+  return static_cast<int>(__umulhi(static_cast<unsigned>(i), mul));
+#else
+  return static_cast<int>((static_cast<uint64_t>(i) * mul) >> 32);
+#endif
+}
+
+struct UnitPos {
+  int img0, y0, x0;  // first image, first output row / column
+};
+__host__ __device__ __forceinline__ UnitPos unit_pos(const BlockParams& p, int unit, int th_rows) {
+  UnitPos u;
+  if (p.whole || p.tiles_x * p.tiles_y == 1) {
+    u.img0 = unit * p.ni;
+    u.y0 = u.x0 = 0;
+  } else {
+    u.img0 = div_by(unit, p.mul_per);
+    const int r = unit - u.img0 * (p.tiles_x * p.tiles_y);
+    const int ty = p.tiles_x == 1 ? r : div_by(r, p.mul_tx);
+    u.y0 = ty * th_rows;
+    u.x0 = (r - ty * p.tiles_x) * p.tw;
+  }
+  return u;
+}
+
+// Where pixel `i` of the unit's list lies: `hid` is its pixel index in the hidden tile; (im, y, x) its place in the
+// depthwise input; `in` says whether that is inside the image.
+struct ListPx {
+  int hid, im, y, x;
+  bool in;
+};
+__host__ __device__ __forceinline__ ListPx list_pixel(const BlockParams& p, const UnitPos& u, int stride, int i) {
+  ListPx l;
+  if (p.compact) {
+    l.im = div_by(i, p.mul_hw);
+    const int rem = i - l.im * (p.H * p.W);
+    l.y = div_by(rem, p.mul_w);
+    l.x = rem - l.y * p.W;
+    const int r = l.y + p.pad_t, c = l.x + p.pad_l;
+    l.hid = (r < p.rows && c < p.pitch) ? l.im * p.sub_px + r * p.pitch + c : p.ni * p.sub_px;  // else: a pixel nothing reads
+    l.in = u.img0 + l.im < p.B;
+  } else {
+    const int q = div_by(i, p.mul_pitch);
+    const int c = i - q * p.pitch;
+    l.im = p.ni > 1 ? q / p.rows : 0;
+    l.y = u.y0 * stride - p.pad_t + (q - l.im * p.rows);
+    l.x = u.x0 * stride - p.pad_l + c;
+    l.hid = i;
+    l.in = static_cast<unsigned>(l.y) < static_cast<unsigned>(p.H) && static_cast<unsigned>(l.x) < static_cast<unsigned>(p.W) &&
+           u.img0 + l.im < p.B;
+  }
+  return l;
+}
+
+// Column `col` of the unit's column list -> image, band, position (pair or single column) within the band.
+__host__ __device__ __forceinline__ void column_pos(const BlockParams& p, int col, int& im, int& band, int& pos) {
+  const int q = col / p.pw;
+  pos = col - q * p.pw;
+  im = q / p.nb;
+  band = q - im * p.nb;
+}
+
+// A lane's output column relative to the unit, in one word (the kernel is short of registers): image (0xff: no column), first
+// row, x.
+__device__ __forceinline__ unsigned lane_col(const BlockParams& p, int stride, int tr, int col) {
+  int im, band, pos;
+  column_pos(p, col < p.ncols ? col : 0, im, band, pos);
+  return static_cast<unsigned>(col < p.ncols ? im : 0xff) << 24 | static_cast<unsigned>(band * tr) << 12 |
+         static_cast<unsigned>(stride == 1 ? 2 * pos : pos);
+}
+
+// Store one column's projection results, of 16-channel blocks j0 .. j0 + NJ - 1.  a[v][j][q][f]; HALF: which half of a fragment
+// the column is.  Stride 1: v = row (from v0), q = pixel of the pair; stride 2: v = row pair, q = row of it.
+template <int S, int HALF, int NV, int NJ>
+__device__ __forceinline__ void store_col(const BlockParams& p, const UnitPos& u, unsigned xres, unsigned col, int v0, int j0, int t,
+                                          const float (&a)[NV][NJ][2][2][4]) {
+  constexpr int H2 = HALF * 2;
+  const int img = u.img0 + static_cast<int>(col >> 24), x = u.x0 + static_cast<int>(col & 0xfffu);
+  const int y0 = u.y0 + static_cast<int>(col >> 12 & 0xfffu) + (S == 1 ? v0 : 2 * v0);
+  if (col >> 24 == 0xffu || img >= p.B || x >= p.Wo) return;
+  const int px0 = y0 * p.Wo + x, rows = p.Ho - y0;
+  const bool two = S == 1 && x + 1 < p.Wo;
+  const int o_row = p.Wo * p.o_px, r_row = p.Wo * 4;
+  constexpr int kRows = S == 1 ? NV : 2 * NV;
+#pragma unroll
+  for (int j = 0; j < NJ; ++j) {
+    const int slice = 4 * (j0 + j) + t;
+    if (slice >= p.sout) continue;
+    __half* dst = p.out + (slice * p.o_sl + img * p.o_img + static_cast<long long>(px0) * p.o_px);
+    uint2 r0[kRows], r1[kRows];  // the residual of all rows first: their latencies overlap
+    if (S == 1 && p.res_x) {
+      const unsigned i = (static_cast<unsigned>(img - u.img0) * p.rows + (y0 - u.y0) + p.pad_t) * p.pitch + (x - u.x0) + p.pad_l;
+      unsigned at = xres + i * p.x_pitch + slice * 8;
+#pragma unroll
+      for (int v = 0; v < kRows; ++v, at += p.pitch * p.x_pitch) {
+        r0[v] = lds64(at);
+        r1[v] = lds64(at + p.x_pitch);
+      }
+    } else if (p.has_res) {
+      const __half* rs = p.res + (slice * p.res_sl + static_cast<long long>(img) * p.res_img + static_cast<long long>(px0) * 4);
+#pragma unroll
+      for (int v = 0; v < kRows; ++v, rs += r_row) {
+        if (v >= rows) break;
+        if (S == 1 && p.wide) {
+          const uint4 rr = *reinterpret_cast<const uint4*>(rs);
+          r0[v] = make_uint2(rr.x, rr.y);
+          r1[v] = make_uint2(rr.z, rr.w);
+        } else {
+          r0[v] = *reinterpret_cast<const uint2*>(rs);
+          if (two) r1[v] = *reinterpret_cast<const uint2*>(rs + 4);
+        }
+      }
+    }
+#pragma unroll
+    for (int v = 0; v < kRows; ++v, dst += o_row) {
+      if (v >= rows) break;
+      if (S == 1) {
+        const uint2 o0 = finish4(p, a[v][j][0][0][H2], a[v][j][0][0][H2 + 1], a[v][j][0][1][H2], a[v][j][0][1][H2 + 1], r0[v]);
+        const uint2 o1 = finish4(p, a[v][j][1][0][H2], a[v][j][1][0][H2 + 1], a[v][j][1][1][H2], a[v][j][1][1][H2 + 1], r1[v]);
+        if (p.wide) {
+          *reinterpret_cast<uint4*>(dst) = make_uint4(o0.x, o0.y, o1.x, o1.y);
+        } else {
+          *reinterpret_cast<uint2*>(dst) = o0;
+          if (two) *reinterpret_cast<uint2*>(dst + p.o_px) = o1;
+          if (p.pad_px && v == rows - 1 && x + (two ? 1 : 0) == p.Wo - 1) *reinterpret_cast<uint2*>(dst + (two ? 8 : 4)) = make_uint2(0, 0);
+        }
+      } else {
+        const float(&f)[2][4] = a[v / 2][j][v & 1];
+        *reinterpret_cast<uint2*>(dst) = finish4(p, f[0][H2], f[0][H2 + 1], f[1][H2], f[1][H2 + 1], r0[v]);
+        if (p.pad_px && v == rows - 1 && x == p.Wo - 1) *reinterpret_cast<uint2*>(dst + 4) = make_uint2(0, 0);
+      }
+    }
+  }
+}
+
+// S: stride.  NP: 16-channel blocks of the output.  TR: output rows a warp walks down.  HC: 16-channel sub-blocks per chunk.
+template <int S, int FIRST, int NP, int TR, int HC>
+__global__ void __launch_bounds__(32 * max_warps(S, NP, TR), 1) block_mma_kernel(const BlockParams p) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  const unsigned smem = smem_u32(smem_raw);
+  const int tid = threadIdx.x, nthr = blockDim.x;
+  const int warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+  constexpr bool kHasFirst = FIRST != kNone, kWideExp = FIRST == kExpWide;
+  constexpr int SL = slice_bytes(FIRST);
+  constexpr int kHidBytes = HC * 4 * SL;
+  constexpr int NV = S == 1 ? TR : TR / 2;  // fragments of sums down a column: rows, or pairs of rows
+  const int ke = kWideExp ? p.ke : FIRST == kNone ? 0 : FIRST == kExp16 ? 1 : 2;
+  const int subb = ke * 512 + kSubFixed + NP * 512;
+  const int stage_bytes = HC * subb;
+  const int rank = p.ks > 1 ? static_cast<int>(cluster_ctarank()) : 0;
+  const int unit0 = blockIdx.x / p.ks, ustep = gridDim.x / p.ks;
+  const int nchl = (p.nch - rank + p.ks - 1) / p.ks;  // chunks of this CTA: rank, rank + ks, ...
+  const int th_rows = p.nb * TR;
+  const int my_units = unit0 < p.units ? (p.units - unit0 + ustep - 1) / ustep : 0;
+  const int total = nchl * my_units;
+
+  pdl_launch_dependents();
+
+  auto load_weights = [&](int run, int c) {
+    const unsigned dst = smem + (p.resident ? run : run & (kRing - 1)) * stage_bytes;
+    const unsigned char* src = p.wts + static_cast<size_t>(rank + c * p.ks) * stage_bytes;
+    for (int i = tid * 16; i < stage_bytes; i += nthr * 16) cp_async16(dst + i, src + i);
+  };
+  if (p.resident) {
+    for (int c = 0; c < nchl; ++c) load_weights(c, c);
+  } else {
+    load_weights(0, 0);
+    if (1 < total) load_weights(1, 1 % nchl);
+  }
+  // shared memory that must start at zero: borders of compact tiles, channels beyond the input's last slice
+  if (FIRST != kStem && (p.compact || (p.sin & 1))) {
+    for (unsigned i = p.off_x + tid * 16; i < p.off_red; i += nthr * 16) sts128(smem + i, 0u, 0u, 0u, 0u);
+  }
+  for (int i = tid; i < NP * 4; i += nthr) cp_async16(smem + p.off_bias + i * 16, reinterpret_cast<const float4*>(p.bias) + i);
+  __syncthreads();
+  pdl_wait();
+
+  const unsigned tab0 = smem + p.off_tab, xs0 = smem + p.off_x, raw = smem + p.off_raw, hid0 = smem + p.off_hid, red = smem + p.off_red;
+  constexpr bool kTwoX = kHasFirst && !kWideExp && FIRST != kStem;  // the next unit's input arrives during this one
+
+  // expansion: the unit's input tile, [list pixel][channel].  The table says what a list pixel's hidden value is clamped to
+  // (zero outside the image); for a wide expansion, whose list may leave out the border, also where it goes
+  auto load_x = [&](const UnitPos& u, int buf) {
+    const unsigned xs = xs0 + buf * p.x_bytes, tab = tab0 + buf * p.tab_bytes;
+    constexpr int kSlices = FIRST == kExp16 ? 4 : FIRST == kExp24 ? 6 : FIRST == kExp32 ? 8 : 0;
+    for (int i = tid; i < p.mt * 16; i += nthr) {
+      const bool listed = i < p.n_list;
+      const ListPx l = list_pixel(p, u, S, listed ? i : 0);
+      const bool in = listed && l.in;
+      if (listed) {
+        const __half* src = p.in;
+        if (in) src += static_cast<long long>(u.img0 + l.im) * p.in_img + static_cast<long long>(l.y * p.W + l.x) * p.in_px;
+        const unsigned n = in ? 8u : 0u;
+        const long long step = in ? p.in_sl : 0;
+        unsigned dst = xs + i * p.x_pitch;
+        if (kTwoX) {
+#pragma unroll
+          for (int s = 0; s < kSlices; ++s, src += step)
+            if (s < p.sin) cp_async8(dst + s * 8, src, n);
+        } else {
+          for (int s = 0; s < p.sin; ++s, src += step, dst += 8) cp_async8(dst, src, n);
+        }
+      }
+      if (kWideExp) sts64(tab + i * 8, static_cast<unsigned>(listed ? l.hid : p.ni * p.sub_px) * 8u, in ? p.hi_e : 0u);
+      else sts32(tab + i * 4, in ? p.hi_e : 0u);
+    }
+  };
+  // no first operator: a chunk of the input goes straight into a hidden tile (a ring of them)
+  auto load_hidden = [&](int run) {
+    const int k = run / nchl, c = run - k * nchl, chunk = rank + c * p.ks;
+    if (c == 0) {  // a thread's own pixels of the unit, kept for its other chunks
+      const UnitPos u = unit_pos(p, unit0 + k * ustep, th_rows);
+      for (int i = tid; i < p.n_list; i += nthr) {
+        const ListPx l = list_pixel(p, u, S, i);
+        sts32(tab0 + i * 4, static_cast<unsigned>(l.in ? (u.img0 + l.im) * p.in_img + (l.y * p.W + l.x) * p.in_px : -1));
+      }
+    }
+    unsigned dst = hid0 + (run & (kRing - 1)) * kHidBytes + tid * 8;
+    const int s0 = chunk * HC * 4, ns = p.sin - s0;  // slices beyond the last one are zeros: their weights are, too
+    for (int i = tid; i < p.n_list; i += nthr, dst += nthr * 8) {
+      const int at = static_cast<int>(lds32(tab0 + i * 4));
+      const __half* src = p.in + (at < 0 ? 0 : at) + s0 * p.in_sl;
+#pragma unroll
+      for (int s = 0; s < HC * 4; ++s, src += p.in_sl) cp_async8(dst + s * SL, s < ns ? src : p.in, s < ns && at >= 0 ? 8u : 0u);
+    }
+  };
+  // stem: the rows of the image under the unit's hidden tile, as 4-byte words from the aligned word that holds a row's first
+  // value; rows outside the image are zeros, columns outside it hold neighbours' values that build_x masks
+  const long long halves = static_cast<long long>(p.B) * p.Hi * p.Wi * 3;
+  auto load_raw = [&](const UnitPos& u) {
+    const int iy0 = 2 * (u.y0 - p.pad_t) - p.spt, ix0 = 2 * (u.x0 - p.pad_l) - p.spl;
+    for (int r = warp; r < p.raw_rows; r += nthr >> 5) {
+      const int iy = iy0 + r;
+      const bool row_in = static_cast<unsigned>(iy) < static_cast<unsigned>(p.Hi);
+      const long long first = ((static_cast<long long>(u.img0) * p.Hi + iy) * p.Wi + ix0) * 3;
+      const long long word0 = first >> 1;
+      for (int w = lane; w < p.raw_words; w += 32) {
+        const long long h = (word0 + w) * 2;
+        const unsigned n = !row_in || h < 0 || h >= halves ? 0u : h + 1 < halves ? 4u : 2u;
+        cp_async4(raw + (r * p.raw_words + w) * 4, n ? p.in + h : p.in, n);
+      }
+    }
+  };
+  // stem: [list pixel][10 ky + 3 kx + c], the 9 values of a window row from 5 words
+  auto build_x = [&](const UnitPos& u) {
+    const int iy0 = 2 * (u.y0 - p.pad_t) - p.spt, ix0 = 2 * (u.x0 - p.pad_l) - p.spl;
+    const unsigned par0 = static_cast<unsigned>(((static_cast<long long>(u.img0) * p.Hi + iy0) * p.Wi + ix0) & 1);
+    for (int i = tid; i < p.mt * 16; i += nthr) {
+      if (i >= p.n_list) {
+        sts32(tab0 + i * 4, 0u);
+        continue;
+      }
+      const int r = div_by(i, p.mul_pitch), c = i - r * p.pitch;
+      const int ix = ix0 + 2 * c;
+      sts32(tab0 + i * 4, static_cast<unsigned>(u.y0 - p.pad_t + r) < static_cast<unsigned>(p.H) &&
+                                 static_cast<unsigned>(u.x0 - p.pad_l + c) < static_cast<unsigned>(p.W)
+                             ? p.hi_e : 0u);
+      unsigned o[16];
+#pragma unroll
+      for (int ky = 0; ky < 3; ++ky) {
+        const unsigned at = raw + ((2 * r + ky) * p.raw_words + 3 * c) * 4;
+        unsigned w[5];
+#pragma unroll
+        for (int q = 0; q < 5; ++q) w[q] = lds32(at + q * 4);
+        const unsigned sh = ((par0 + (ky & 1) * p.Wi) & 1) * 16;  // an even number of rows further on the parity is the same
+#pragma unroll
+        for (int q = 0; q < 4; ++q) o[ky * 5 + q] = __funnelshift_r(w[q], w[q + 1], sh);
+        o[ky * 5 + 4] = (w[4] >> sh) & 0xffffu;
+        if (ix < 0 || ix + 2 >= p.Wi) {
+          if (static_cast<unsigned>(ix) >= static_cast<unsigned>(p.Wi)) {
+            o[ky * 5] = 0u;
+            o[ky * 5 + 1] &= 0xffff0000u;
+          }
+          if (static_cast<unsigned>(ix + 1) >= static_cast<unsigned>(p.Wi)) {
+            o[ky * 5 + 1] &= 0xffffu;
+            o[ky * 5 + 2] = 0u;
+          }
+          if (static_cast<unsigned>(ix + 2) >= static_cast<unsigned>(p.Wi)) o[ky * 5 + 3] = o[ky * 5 + 4] = 0u;
+        }
+      }
+      o[15] = 0u;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) sts128(xs0 + i * 80 + q * 16, o[q * 4], o[q * 4 + 1], o[q * 4 + 2], o[q * 4 + 3]);
+    }
+  };
+  if (my_units > 0) {
+    if (FIRST == kStem) {
+      load_raw(unit_pos(p, unit0, th_rows));
+    } else if (kHasFirst) {
+      load_x(unit_pos(p, unit0, th_rows), 0);
+    } else {
+      load_hidden(0);
+      cp_async_commit();
+      if (1 < total) load_hidden(1);
+    }
+  }
+  cp_async_commit();
+
+  // this lane's rows of the depthwise A operand, and which half of a banded weight word it takes
+  unsigned dw_base;
+  const unsigned row_b = p.pitch * 8;
+  {
+    int col = warp * 16 + (lane & 15);
+    if (col >= p.ncols) col = 0;
+    int im, band, pos;
+    column_pos(p, col, im, band, pos);
+    dw_base = static_cast<unsigned>(im * p.sub_px + band * TR * S * p.pitch) * 8u + pos * 16u + (lane >> 4) * 16u;
+  }
+  const unsigned col0 = lane_col(p, S, TR, warp * 16 + g), col1 = lane_col(p, S, TR, warp * 16 + g + 8);
+  const bool band_lane = (g >> 2) == (t & 1);
+  const unsigned sel_a = !band_lane ? 0x4444u : ((g >> 1) & 1) ? 0x1044u : 0x4410u;
+  const unsigned sel_b = !band_lane ? 0x4444u : ((g >> 1) & 1) ? 0x3244u : 0x4432u;
+  const bool odd = g & 1;
+  const unsigned sel_a0 = odd ? 0x4444u : sel_a, sel_b0 = odd ? 0x4444u : sel_b;  // window rows of the first output row only
+  const unsigned sel_a1 = odd ? sel_a : 0x4444u, sel_b1 = odd ? sel_b : 0x4444u;  // ... of the second only
+  const unsigned dw_entry = ((t >> 1) * 8 + g) * 16;
+  const bool has_group = warp < p.ngroups;
+  // this warp's groups of 16 list pixels
+  const int mt0 = has_group ? warp * p.eg : p.ngroups * p.eg + (warp - p.ngroups) * p.en;
+  const int mt1 = min(p.mt, mt0 + (has_group ? p.eg : p.en));
+
+  if (kHasFirst) cp_async_wait<0>();
+  else cp_async_wait<1>();
+  __syncthreads();
+  int run = 0;
+  for (int k = 0; k < my_units; ++k, run += nchl) {
+    const int unit = unit0 + k * ustep;
+    if (FIRST == kStem) {
+      cp_async_wait<0>();
+      __syncthreads();
+      build_x(unit_pos(p, unit, th_rows));
+    }
+
+    float acc[NV][NP][2][2][4];  // sums start at the bias (a cluster's: in its first CTA)
+#pragma unroll
+    for (int j = 0; j < NP; ++j) {
+      const uint4 q = rank ? make_uint4(0u, 0u, 0u, 0u) : lds128(smem + p.off_bias + (4 * j + t) * 16);
+#pragma unroll
+      for (int v = 0; v < NV; ++v)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          acc[v][j][i >> 1][0][(i & 1) * 2] = __uint_as_float(q.x);
+          acc[v][j][i >> 1][0][(i & 1) * 2 + 1] = __uint_as_float(q.y);
+          acc[v][j][i >> 1][1][(i & 1) * 2] = __uint_as_float(q.z);
+          acc[v][j][i >> 1][1][(i & 1) * 2 + 1] = __uint_as_float(q.w);
+        }
+    }
+    const unsigned xs = xs0 + (kTwoX ? (k & 1) * p.x_bytes : 0u), tab = tab0 + (kTwoX ? (k & 1) * p.tab_bytes : 0u);
+    const int steps = kHasFirst ? nchl + 1 : nchl;
+#pragma unroll 1
+    for (int it = 0; it < steps; ++it) {
+      if (kHasFirst && !kTwoX && it == 0) cp_async_wait<0>();
+      else cp_async_wait<1>();
+      __syncthreads();
+      if (kHasFirst) {
+        if (!p.resident && it < nchl && run + it + 2 < total) load_weights(run + it + 2, it + 2 >= nchl ? (it + 2) % nchl : it + 2);
+        if (k + 1 < my_units) {
+          if (FIRST == kStem && it == 0) load_raw(unit_pos(p, unit + ustep, th_rows));
+          if (kTwoX && it == 0) load_x(unit_pos(p, unit + ustep, th_rows), (k + 1) & 1);
+          if (kWideExp && it == nchl) load_x(unit_pos(p, unit + ustep, th_rows), 0);
+        }
+      } else if (run + it + 2 < total) {
+        if (!p.resident) load_weights(run + it + 2, (it + 2) % nchl);
+        load_hidden(run + it + 2);
+      }
+      cp_async_commit();
+
+      // ---- first operator of chunk `it`
+      if (kHasFirst && it < nchl && mt0 < mt1) {
+        const int r = run + it;
+        const unsigned ws = smem + (p.resident ? it : r & (kRing - 1)) * stage_bytes;
+        const unsigned hb = hid0 + (r & 1) * kHidBytes + t * SL;
+        if (!kWideExp) {
+          const uint4 b0 = lds128(ws + lane * 16);
+          const uint4 b1 = FIRST == kExp16 ? b0 : lds128(ws + 512 + lane * 16);
+          const uint4 q = lds128(ws + ke * 512 + t * 16);
+          const float be[4] = {__uint_as_float(q.x), __uint_as_float(q.y), __uint_as_float(q.z), __uint_as_float(q.w)};
+          constexpr unsigned XP = FIRST == kExp16 || FIRST == kExp24 ? 48 : 80;
+          unsigned xa = xs + (mt0 * 16 + (lane & 15)) * XP + (lane >> 4) * 16;
+          unsigned xh = xs + (mt0 * 16 + (lane & 15)) * XP + 32;  // kExp24: channels 16..23
+          unsigned at = hb + (mt0 * 16 + g) * 8, tb = tab + (mt0 * 16 + g) * 4;
+          auto some = [&](auto count) {  // `count` groups in flight
+            constexpr int N = decltype(count)::value;
+            unsigned a[N][4], a2[N][4], hi[N][2];
+            float c[N][2][4];
+#pragma unroll
+            for (int i = 0; i < N; ++i) {
+              ldsm4(xa + i * 16 * XP, a[i]);
+              if (FIRST == kExp24) ldsm2(xh + i * 16 * XP, a2[i][0], a2[i][1]);
+              if (FIRST == kExp32 || FIRST == kStem) ldsm4(xa + i * 16 * XP + 32, a2[i]);
+              hi[i][0] = lds32(tb + i * 64);
+              hi[i][1] = lds32(tb + i * 64 + 32);
+            }
+#pragma unroll
+            for (int i = 0; i < N; ++i) {
+              mma16816c(c[i][0], a[i], b0.x, b0.y, be[0], be[1], be[0], be[1]);
+              mma16816c(c[i][1], a[i], b0.z, b0.w, be[2], be[3], be[2], be[3]);
+              if (FIRST == kExp24) {
+                mma1688(c[i][0], a2[i][0], a2[i][1], b1.x);
+                mma1688(c[i][1], a2[i][0], a2[i][1], b1.z);
+              }
+              if (FIRST == kExp32 || FIRST == kStem) {
+                mma16816(c[i][0], a2[i], b1.x, b1.y);
+                mma16816(c[i][1], a2[i], b1.z, b1.w);
+              }
+            }
+#pragma unroll
+            for (int i = 0; i < N; ++i)
+#pragma unroll
+              for (int half = 0; half < 2; ++half)
+                sts64(at + i * 128 + half * 64, min_f16x2(pack_f16x2<true>(c[i][0][half * 2], c[i][0][half * 2 + 1]), hi[i][half]),
+                      min_f16x2(pack_f16x2<true>(c[i][1][half * 2], c[i][1][half * 2 + 1]), hi[i][half]));
+            xa += N * 16 * XP;
+            xh += N * 16 * XP;
+            at += N * 128;
+            tb += N * 64;
+          };
+          int n = mt1 - mt0;
+#pragma unroll 1
+          for (; n >= 2; n -= 2) some(std::integral_constant<int, 2>{});
+          if (n) some(std::integral_constant<int, 1>{});
+        } else {
+          float be[HC][4];
+#pragma unroll
+          for (int h = 0; h < HC; ++h) {
+            const uint4 q = lds128(ws + h * subb + ke * 512 + t * 16);
+            be[h][0] = __uint_as_float(q.x);
+            be[h][1] = __uint_as_float(q.y);
+            be[h][2] = __uint_as_float(q.z);
+            be[h][3] = __uint_as_float(q.w);
+          }
+#pragma unroll 1
+          for (int m0 = mt0; m0 < mt1; m0 += 2) {  // two groups at a time share the weight fragments
+            const bool second = m0 + 1 < mt1;
+            float c[2][HC][2][4];
+            unsigned xa = xs + (m0 * 16 + (lane & 15)) * p.x_pitch + (lane >> 4) * 16;
+            const unsigned xb = second ? 16 * p.x_pitch : 0u;
+            unsigned wk = ws + lane * 16;
+            auto step = [&](auto first) {
+              unsigned a[2][4];
+              ldsm4(xa, a[0]);
+              ldsm4(xa + xb, a[1]);
+#pragma unroll
+              for (int h = 0; h < HC; ++h) {
+                const uint4 b = lds128(wk + h * subb);
+#pragma unroll
+                for (int mm = 0; mm < 2; ++mm) {
+                  if (decltype(first)::value) {
+                    mma16816c(c[mm][h][0], a[mm], b.x, b.y, be[h][0], be[h][1], be[h][0], be[h][1]);
+                    mma16816c(c[mm][h][1], a[mm], b.z, b.w, be[h][2], be[h][3], be[h][2], be[h][3]);
+                  } else {
+                    mma16816(c[mm][h][0], a[mm], b.x, b.y);
+                    mma16816(c[mm][h][1], a[mm], b.z, b.w);
+                  }
+                }
+              }
+              xa += 32;
+              wk += 512;
+            };
+            step(std::true_type{});
+#pragma unroll 2
+            for (int kk = 1; kk < ke; ++kk) step(std::false_type{});
+#pragma unroll
+            for (int mm = 0; mm < 2; ++mm) {
+              if (mm == 1 && !second) break;
+#pragma unroll
+              for (int half = 0; half < 2; ++half) {
+                const uint2 e = lds64(tab + ((m0 + mm) * 16 + g + half * 8) * 8);
+                const unsigned at = hb + e.x;
+#pragma unroll
+                for (int h = 0; h < HC; ++h)
+                  sts64(at + h * 4 * SL, min_f16x2(pack_f16x2<true>(c[mm][h][0][half * 2], c[mm][h][0][half * 2 + 1]), e.y),
+                        min_f16x2(pack_f16x2<true>(c[mm][h][1][half * 2], c[mm][h][1][half * 2 + 1]), e.y));
+              }
+            }
+          }
+        }
+      }
+
+      // ---- depthwise and projection of the chunk before it (without a first operator: of chunk `it`)
+      const int dc = kHasFirst ? it - 1 : it;
+      if (dc >= 0 && has_group) {
+        const int r = run + dc;
+        const unsigned ws = smem + (p.resident ? dc : r & (kRing - 1)) * stage_bytes;
+        const unsigned hb = hid0 + (kHasFirst ? (r & 1) : (r & (kRing - 1))) * kHidBytes + dw_base;
+        constexpr int kRows = S == 1 ? TR + 2 : 2 * TR + 1;  // hidden rows under the column
+        unsigned rb[kRows];
+#pragma unroll
+        for (int i = 0; i < kRows; ++i) rb[i] = hb + i * row_b;
+#pragma unroll
+        for (int h = 0; h < HC; ++h) {
+          const unsigned wd = ws + h * subb + ke * 512 + kBiasBytes;
+          unsigned af[NV][2][4];
+#pragma unroll
+          for (int sp = 0; sp < 2; ++sp) {
+            float d[2][NV][4];
+#pragma unroll
+            for (int s2 = 0; s2 < 2; ++s2) {
+              const int sl = sp * 2 + s2;
+              const uint4 w = lds128(wd + sl * 256 + dw_entry);
+              const uint4 bq = lds128(wd + kTableBytes + sl * 64 + t * 16);
+              const float bd[4] = {__uint_as_float(bq.x), __uint_as_float(bq.y), __uint_as_float(bq.z), __uint_as_float(bq.w)};
+              if (S == 1) {
+                const unsigned b0[3] = {prmt(w.x, sel_a), prmt(w.y, sel_a), prmt(w.z, sel_a)};
+                const unsigned b1[3] = {prmt(w.x, sel_b), prmt(w.y, sel_b), prmt(w.z, sel_b)};
+#pragma unroll
+                for (int rr = 0; rr < kRows; ++rr) {
+                  unsigned a[4];
+                  ldsm4(rb[rr] + (h * 4 + sl) * SL, a);
+#pragma unroll
+                  for (int ky = 0; ky < 3; ++ky) {
+                    const int v = rr - ky;
+                    if (v < 0 || v >= TR) continue;
+                    if (ky == 0) mma16816c(d[s2][v], a, b0[ky], b1[ky], bd[0], bd[1], bd[2], bd[3]);
+                    else mma16816(d[s2][v], a, b0[ky], b1[ky]);
+                  }
+                }
+              } else {
+                const unsigned wm = odd ? w.x : w.z;
+                const unsigned b0[5] = {prmt(w.x, sel_a0), prmt(w.y, sel_a0), prmt(wm, sel_a), prmt(w.y, sel_a1), prmt(w.z, sel_a1)};
+                const unsigned b1[5] = {prmt(w.x, sel_b0), prmt(w.y, sel_b0), prmt(wm, sel_b), prmt(w.y, sel_b1), prmt(w.z, sel_b1)};
+#pragma unroll
+                for (int rr = 0; rr < kRows; ++rr) {
+                  unsigned a[4];
+                  ldsm4(rb[rr] + (h * 4 + sl) * SL, a);
+                  const int v = rr >> 2, q = rr & 3;
+                  if (v < NV && q == 0) mma16816c(d[s2][v < NV ? v : 0], a, b0[q], b1[q], bd[0], bd[1], bd[2], bd[3]);
+                  else if (v < NV) mma16816(d[s2][v < NV ? v : 0], a, b0[q], b1[q]);
+                  if (q == 0 && v > 0) mma16816(d[s2][v > 0 ? v - 1 : 0], a, b0[4], b1[4]);
+                }
+              }
+            }
+#pragma unroll
+            for (int v = 0; v < NV; ++v)
+#pragma unroll
+              for (int q = 0; q < 2; ++q) {
+                af[v][q][sp * 2] = min_f16x2(pack_f16x2<true>(d[0][v][q], d[1][v][q]), p.hi_d);
+                af[v][q][sp * 2 + 1] = min_f16x2(pack_f16x2<true>(d[0][v][2 + q], d[1][v][2 + q]), p.hi_d);
+              }
+          }
+          const unsigned wp = wd + kTableBytes + kDwBiasBytes + lane * 16;
+#pragma unroll
+          for (int j = 0; j < NP; ++j) {
+            const uint4 b = lds128(wp + j * 512);
+#pragma unroll
+            for (int v = 0; v < NV; ++v)
+#pragma unroll
+              for (int q = 0; q < 2; ++q) {
+                mma16816(acc[v][j][q][0], af[v][q], b.x, b.y);
+                mma16816(acc[v][j][q][1], af[v][q], b.z, b.w);
+              }
+          }
+        }
+      }
+    }
+
+    const UnitPos u = unit_pos(p, unit, th_rows);
+    if (p.ks == 1) {
+      if (has_group) {
+        store_col<S, 0, NV, NP>(p, u, xs, col0, 0, 0, t, acc);
+        store_col<S, 1, NV, NP>(p, u, xs, col1, 0, 0, t, acc);
+      }
+    } else {
+      // partial sums of the cluster's CTAs: every CTA leaves its own in shared memory and adds up its share of the tiles
+      // over the ranks, in rank order
+      if (has_group) {
+#pragma unroll
+        for (int v = 0; v < NV; ++v)
+#pragma unroll
+          for (int j = 0; j < NP; ++j) {
+            const unsigned at = red + ((warp * NV + v) * NP + j) * 2048 + lane * 16;
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+              sts128(at + i * 512, __float_as_uint(acc[v][j][i >> 1][i & 1][0]), __float_as_uint(acc[v][j][i >> 1][i & 1][1]),
+                     __float_as_uint(acc[v][j][i >> 1][i & 1][2]), __float_as_uint(acc[v][j][i >> 1][i & 1][3]));
+          }
+      }
+      cluster_sync();
+      const int tiles = p.ngroups * NV * NP;
+      for (int ti = warp * p.ks + rank; ti < tiles; ti += (nthr >> 5) * p.ks) {
+        float s[1][1][2][2][4];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) s[0][0][i >> 3][(i >> 2) & 1][i & 3] = 0.0f;
+        for (int r = 0; r < p.ks; ++r) {
+          const unsigned at = mapa_shared(red + ti * 2048 + lane * 16, r);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const float4 x = ld_cluster_f4(at + i * 512);
+            s[0][0][i >> 1][i & 1][0] += x.x;
+            s[0][0][i >> 1][i & 1][1] += x.y;
+            s[0][0][i >> 1][i & 1][2] += x.z;
+            s[0][0][i >> 1][i & 1][3] += x.w;
+          }
+        }
+        const int j = ti % NP, gv = ti / NP, gid = gv / NV, v = gv % NV;
+        store_col<S, 0, 1, 1>(p, u, xs, lane_col(p, S, TR, gid * 16 + g), v, j, t, s);
+        store_col<S, 1, 1, 1>(p, u, xs, lane_col(p, S, TR, gid * 16 + g + 8), v, j, t, s);
+      }
+      cluster_sync();  // nobody overwrites or leaves while a neighbour still reads
+    }
+  }
+  cp_async_wait<0>();
+}
+
+// ---------------------------------------------------------------- host side
+// Shared memory of one CTA under a configuration, and the offsets the kernel uses.
+struct Layout {
+  int rows, pitch, sub_px, n_list, mt, compact, pw, ncols, ngroups, nw, eg, en;
+  unsigned x_pitch, x_bytes, tab_bytes, off_bias, off_tab, off_x, off_raw, off_hid, off_red, bytes;
+  int stage_bytes, resident, nch, raw_rows, raw_words;
+};
+
+int ke_of(const LaunchRec& r, const BlockCfg& c) { return c.first == kNone ? 0 : c.first == kStem ? 2 : (r.C + 15) / 16; }
+
+// cost of a column group's depthwise and projection relative to a group of 16 list pixels; it only divides the list between
+// warps that have a column group and warps that have none
+double group_cost(const LaunchRec& r, const BlockCfg& c) {
+  const int nv = c.s == 1 ? c.tr : c.tr / 2;
+  const double d = 4.0 * (c.s == 1 ? 3 : 5) * nv + 4.0 * c.np * nv + 8.0;
+  return d / (2.0 * ke_of(r, c) + 3.0);
+}
+
+bool layout_of(const LaunchRec& r, const BlockCfg& c, Layout* l) {
+  const int th = c.nb * c.tr;
+  l->rows = c.s == 1 ? th + 2 : 2 * th + 1;
+  l->pitch = c.s == 1 ? c.tw + 2 : 2 * c.tw + 2;
+  l->sub_px = l->rows * l->pitch;
+  l->compact = c.whole && c.first == kExpWide;
+  l->n_list = l->compact ? c.ni * r.H * r.W : c.ni * l->sub_px;
+  l->mt = (l->n_list + 15) / 16;
+  if (c.ni * l->sub_px > tile_pixels(c.first) || l->mt * 16 > tile_pixels(c.first) + 2) return false;
+  l->pw = c.s == 1 ? c.tw / 2 : c.tw;
+  l->ncols = c.ni * c.nb * l->pw;
+  l->ngroups = (l->ncols + 15) / 16;
+  const int cap = max_warps(c.s, c.np, c.tr);
+  if (l->ngroups > cap) return false;
+  // warps without a column group still help with the first operator
+  l->nw = std::min(cap, std::max(l->ngroups, std::min(c.nw_min, c.first != kNone ? (l->mt + 1) / 2 : 4)));
+  {
+    const double gc = group_cost(r, c);
+    const double share = (l->mt + l->ngroups * gc) / l->nw;
+    int eg = static_cast<int>(share - gc + 0.5);
+    if (l->nw == l->ngroups) eg = (l->mt + l->nw - 1) / l->nw;
+    l->eg = std::max(0, std::min(eg, (l->mt + l->nw - 1) / l->nw));
+    const int rest = l->mt - l->eg * l->ngroups;
+    l->en = l->nw > l->ngroups ? std::max(0, (rest + l->nw - l->ngroups - 1) / (l->nw - l->ngroups)) : 0;
+    if (c.first == kNone) l->eg = l->en = 0;
+  }
+  const int ke = ke_of(r, c);
+  const int chid = c.first == kNone ? r.C : r.Cmid;
+  l->nch = (chid + 16 * c.hc - 1) / (16 * c.hc);
+  if (c.ks > l->nch) return false;
+  const int nchl = (l->nch + c.ks - 1) / c.ks;
+  l->stage_bytes = c.hc * sub_bytes(ke, c.np);
+  l->resident = nchl <= kRing || nchl * l->stage_bytes <= c.resident_kb * 1024;
+  const int nslot = l->resident ? nchl : kRing;
+  const int xw = ke * 2 - (c.first == kExp24 ? 1 : 0);  // 16-byte units of a list pixel; an odd number of them is free of conflicts
+  l->x_pitch = c.first == kNone ? 0u : c.first == kStem ? 80u : static_cast<unsigned>((xw % 2 ? xw : xw + 1) * 16);
+  l->raw_rows = l->raw_words = 0;
+  if (c.first == kStem) {
+    l->raw_rows = 2 * l->rows + 1;
+    l->raw_words = ((2 * l->pitch + 1) * 3 + 2) / 2 + 1;
+  }
+  const int two = c.first != kNone && c.first != kExpWide && c.first != kStem ? 2 : 1;
+  l->tab_bytes = static_cast<unsigned>(round_up_u64(l->mt * (c.first == kExpWide ? 128 : 64), 128));
+  l->x_bytes = static_cast<unsigned>(round_up_u64(l->mt * 16 * l->x_pitch, 128));
+  l->off_bias = static_cast<unsigned>(nslot * l->stage_bytes);
+  l->off_tab = static_cast<unsigned>(round_up_u64(l->off_bias + c.np * 64, 128));
+  l->off_x = l->off_tab + two * l->tab_bytes;
+  l->off_raw = l->off_x + two * l->x_bytes;
+  l->off_hid = static_cast<unsigned>(round_up_u64(l->off_raw + l->raw_rows * l->raw_words * 4 + (l->raw_rows ? 32 : 0), 128));
+  l->off_red = l->off_hid + (c.first == kNone ? kRing : 2) * c.hc * 4 * slice_bytes(c.first);
+  l->bytes = l->off_red + (c.ks > 1 ? l->ngroups * (c.s == 1 ? c.tr : c.tr / 2) * c.np * 2048 : 0);
+  return l->bytes <= kSmemPerSm - 1024;
+}
+
+// (two CTAs that together ask for exactly 227 KB do not share an SM: measured)
+int ctas_per_sm(const BlockCfg& c, const Layout& l) {
+  return std::max(1, std::min<int>((kSmemPerSm - 1024) / (static_cast<int>(l.bytes) + 1024), max_warps(c.s, c.np, c.tr) / l.nw));
+}
+
+// Clusters of `ks` CTAs that run at the same time with one CTA per SM: a cluster stays inside one of the chip's GPCs.  Found
+// from the jump of a launch's time at one cluster more (8: 15, 4: 33, 2: 73).
+int cluster_slots(int ks) { return ks == 8 ? 15 : ks == 4 ? 33 : ks == 2 ? 73 : 148; }
+
+// Estimated time of a launch, for choosing a configuration.  Two bounds, both in SM cycles: the chain of one CTA's units (its
+// chunks one after the other, `lat`), and the throughput of an SM's matrix and shared-memory pipes under all its CTAs'
+// units (`thr`).  The coefficients are a least-squares fit to 6100 measured launches (110 shapes of MobileNetV2 at batch 1 to
+// 256 and image sizes 128 to 513, about 50 configurations each; rms error 13 %; the configuration it picks takes 1.07 times
+// the best one's time in the geometric mean).
+double block_cost_us(const LaunchRec& r, const BlockCfg& c, const Layout& l) {
+  const bool expansion = c.first != kNone && c.first != kStem;
+  const int ke = ke_of(r, c), nv = c.s == 1 ? c.tr : c.tr / 2;
+  const int occ = ctas_per_sm(c, l), slots = cluster_slots(c.ks) * occ;
+  const double upc = (c.units + std::min(c.units, slots) - 1) / std::min(c.units, slots);  // units per CTA
+  const double per_sm = (std::min(c.units, slots) * c.ks + 147) / 148;
+  const double nchl = (l.nch + c.ks - 1) / c.ks, ew = std::max(l.eg, l.en), thr_n = l.nw * 32.0;
+  const double dw = (4.0 * (c.s == 1 ? 3 : 5) * nv + 4.0 * c.np * nv) * c.hc;
+  double lat = 236.8 + (nchl + 1) * (443 + 34.49 * ew * ke * c.hc + 6.063 * dw + 521.9 * c.hc);
+  if (c.first == kStem) lat += 2432 * l.n_list / thr_n;
+  if (c.first == kNone) lat += (nchl + 1) * 14.16 * l.n_list * 4 / thr_n;
+  if (c.ks == 1) lat += 695.4 * c.np * nv;
+  else lat += 3492 + 1735 * l.ngroups * c.np * nv / (c.ks * static_cast<double>(l.nw));
+  double thr = 317.1 + 130.4 * l.ngroups * c.np * nv + nchl * (3.538 * l.mt * ke * 2 * c.hc + 4.459 * l.ngroups * dw + 74.9 * l.ngroups * c.hc);
+  if (expansion) thr += 1.235 * l.n_list * slices(r.C);
+  if (c.first == kStem) thr += 3.48 * l.n_list;
+  const double a = upc * lat, b = upc * per_sm * thr;
+  return 2.904 + std::cbrt(a * a * a + b * b * b) / 1965.0;
+}
+
+template <int S, int FIRST, int NP, int TR, int HC>
+int launch_t(const BlockParams& p, int nw, unsigned smem, int grid, cudaStream_t stream) {
+  auto kern = block_mma_kernel<S, FIRST, NP, TR, HC>;
+  static bool attr_done_dev[kMaxDevices] = {};
+  bool& attr_done = attr_done_dev[current_device_slot()];
+  if (!attr_done) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemPerSm);
+    if (e != cudaSuccess) return static_cast<int>(e);
+    attr_done = true;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(nw * 32);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = p.ks;
+  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = p.ks > 1 ? 2 : 1;
+  return static_cast<int>(cudaLaunchKernelEx(&cfg, kern, p));
+}
+
+// rows per warp and sub-blocks per chunk follow from the channel counts (each_config)
+template <int S, int FIRST>
+int launch_np(const BlockCfg& c, const BlockParams& p, int nw, unsigned smem, int grid, cudaStream_t st) {
+  constexpr int HC = FIRST == kExpWide ? 2 : 1;
+  if constexpr (S == 2) {
+    if (c.np == 2) return launch_t<2, FIRST, 2, 2, HC>(p, nw, smem, grid, st);
+    if (c.np == 4) return launch_t<2, FIRST, 4, 2, HC>(p, nw, smem, grid, st);
+    if constexpr (FIRST == kExpWide) {
+      if (c.np == 6) return launch_t<2, FIRST, 6, 2, HC>(p, nw, smem, grid, st);
+      if (c.np == 10) return launch_t<2, FIRST, 10, 2, HC>(p, nw, smem, grid, st);
+    }
+  } else {
+    if (c.np == 2) return c.tr == 2 ? launch_t<1, FIRST, 2, 2, HC>(p, nw, smem, grid, st) : launch_t<1, FIRST, 2, 1, HC>(p, nw, smem, grid, st);
+    if (c.np == 4) return c.tr == 2 ? launch_t<1, FIRST, 4, 2, HC>(p, nw, smem, grid, st) : launch_t<1, FIRST, 4, 1, HC>(p, nw, smem, grid, st);
+    if constexpr (FIRST == kExpWide) {
+      if (c.np == 6) return launch_t<1, FIRST, 6, 1, HC>(p, nw, smem, grid, st);
+      if (c.np == 10) return launch_t<1, FIRST, 10, 1, HC>(p, nw, smem, grid, st);
+    } else {
+      if (c.np == 1) return c.tr == 4 ? launch_t<1, FIRST, 1, 4, HC>(p, nw, smem, grid, st) : launch_t<1, FIRST, 1, 2, HC>(p, nw, smem, grid, st);
+    }
+  }
+  return static_cast<int>(cudaErrorInvalidConfiguration);
+}
+
+template <int S>
+int launch_first(const BlockCfg& c, const BlockParams& p, int nw, unsigned smem, int grid, cudaStream_t st) {
+  switch (c.first) {
+    case kNone: return launch_np<S, kNone>(c, p, nw, smem, grid, st);
+    case kExp16: return launch_np<S, kExp16>(c, p, nw, smem, grid, st);
+    case kExp24: return launch_np<S, kExp24>(c, p, nw, smem, grid, st);
+    case kExp32: return launch_np<S, kExp32>(c, p, nw, smem, grid, st);
+    case kStem:
+      if constexpr (S == 1) return launch_np<1, kStem>(c, p, nw, smem, grid, st);
+      return static_cast<int>(cudaErrorInvalidConfiguration);
+    default: return launch_np<S, kExpWide>(c, p, nw, smem, grid, st);
+  }
+}
+
+unsigned magic(uint64_t d) { return static_cast<unsigned>(std::min<uint64_t>(0xffffffffull, (0xffffffffull + d) / d)); }
+
+// Calls f(configuration, layout) for every configuration that runs the block in `r`.
+template <class F>
+void each_config(const LaunchRec& r, int kind, F&& f) {
+  if (r.kh != 3 || r.kw != 3 || r.sh != r.sw || (r.sh != 1 && r.sh != 2) || r.dh != 1 || r.dw != 1) return;
+  if (r.pt < 0 || r.pt > 2 || r.pl < 0 || r.pl > 2 || r.W < 2 || r.H < 1) return;
+  if (kind == BLOCK_STEM && (r.sh != 1 || r.C != 3)) return;
+  if ((kind == BLOCK_STEM || kind == BLOCK_EXPANSION) && r.Cmid < 16) return;
+  BlockCfg c;
+  c.s = r.sh;
+  c.first = kind == BLOCK_STEM ? kStem : kind == BLOCK_PAIR ? kNone : r.C <= 16 ? kExp16 : r.C <= 24 ? kExp24 : r.C <= 32 ? kExp32 : kExpWide;
+  const int np_raw = (r.Co2 + 15) / 16;
+  if (c.first == kExpWide) {
+    c.np = np_raw <= 2 ? 2 : np_raw <= 4 ? 4 : np_raw <= 6 ? 6 : np_raw <= 10 ? 10 : 0;
+    if (r.C > 160) return;
+  } else {
+    c.np = np_raw == 1 && c.s == 1 ? 1 : np_raw <= 2 ? 2 : np_raw <= 4 ? 4 : 0;
+  }
+  if (c.np == 0) return;
+  const int64_t in_plane = kind == BLOCK_STEM ? static_cast<int64_t>(r.stem_h) * r.stem_w * 3 : static_cast<int64_t>(plane_pixels(r.H, r.W)) * 4;
+  if (r.B * in_plane * (kind == BLOCK_PAIR ? (r.C + 3) / 4 : 1) >= (1LL << 31)) return;  // offsets inside the input are 32-bit
+  if (static_cast<int64_t>(r.Ho) * r.Wo * std::max(4, r.Co2) >= (1LL << 31)) return;
+  c.hc = c.first == kExpWide ? 2 : 1;
+  const int wo_even = (r.Wo + 1) / 2 * 2;
+  const int tr_hi = c.s == 2 ? 2 : c.np == 1 ? 4 : c.np <= 4 ? 2 : 1, tr_lo = c.s == 2 ? 2 : c.np == 1 ? 2 : 1;
+  for (c.tr = tr_lo; c.tr <= tr_hi; c.tr *= 2)
+    for (int tx = 1; tx <= 32; ++tx) {
+      c.tw = ((wo_even + tx - 1) / tx + 1) / 2 * 2;
+      c.tiles_x = (r.Wo + c.tw - 1) / c.tw;
+      if (c.tiles_x != tx) continue;
+      for (c.nb = 1; c.nb <= 28; ++c.nb) {
+        const int th = c.nb * c.tr;
+        if (th - c.tr >= r.Ho) break;
+        c.tiles_y = (r.Ho + th - 1) / th;
+        c.whole = c.tiles_x == 1 && c.tiles_y == 1;
+        for (c.ni = 1; c.ni <= (c.whole && kind != BLOCK_STEM ? 8 : 1) && c.ni <= r.B; ++c.ni) {
+          const long long units = c.whole ? (r.B + c.ni - 1) / c.ni : static_cast<long long>(r.B) * c.tiles_x * c.tiles_y;
+          if (units > (1 << 28) || static_cast<uint64_t>(units) * c.tiles_x * c.tiles_y >= (1ull << 32)) continue;
+          c.units = static_cast<int>(units);
+          for (c.ks = 1; c.ks <= 8; c.ks *= 2) {
+            if (c.ks > 1 && units * c.ks > 148 * 2) break;  // a split pays only while SMs would be idle ...
+            for (c.nw_min = 8; c.nw_min <= max_warps(c.s, c.np, c.tr); c.nw_min += 8) {
+              for (int rk = 0; rk < 2; ++rk) {
+                c.resident_kb = rk ? 48 : 0;
+                Layout l;
+                if (!layout_of(r, c, &l) || (c.nw_min > 8 && l.nw <= 8)) break;  // nw_min 8 has given the same layout
+                if (rk && !l.resident) break;
+                // ... in one wave
+                if (c.ks == 1 || units <= cluster_slots(c.ks) * ctas_per_sm(c, l)) f(c, l);
+                if (l.resident) break;
+              }
+            }
+          }
+        }
+      }
+    }
+}
+
+uint16_t half_bits(float v) { return f32_to_f16_rne(v); }
+
+}  // namespace
+
+// Chooses tile, image and cluster split for the block in `r` (C -> Cmid -> Co2, or C -> Co2 for BLOCK_PAIR; stride r.sh, output
+// Ho x Wo).  False if no configuration runs it; `us` receives the estimate the choice was made by.
+bool block_mma_choose(const LaunchRec& r, int kind, BlockCfg* best, double* us) {
+  double best_cost = 0.0;
+  bool found = false;
+  each_config(r, kind, [&](const BlockCfg& c, const Layout& l) {
+    const double cost = block_cost_us(r, c, l);
+    if (found && cost >= best_cost) return;
+    found = true;
+    best_cost = cost;
+    *best = c;
+  });
+  if (us) *us = best_cost;
+  return found;
+}
+
+// Packs all weights of the block in sub-blocks of 16 hidden channels (layout: sub_bytes), biases in fp32.
+// we: [chid][cin], for the stem [chid][3][3][3], null for a pair; wd [9][chid], wp [cout][chid].
+void block_mma_pack(const float* we, const float* be, const float* wd, const float* bd, const float* wp, const float* bp, int cin,
+                    int chid, int cout, const BlockCfg& c, std::vector<uint8_t>* blob, LaunchRec* r) {
+  const int ke = c.first == kNone ? 0 : c.first == kStem ? 2 : (cin + 15) / 16, np = c.np;
+  const int nsub = (chid + 16 * c.hc - 1) / (16 * c.hc) * c.hc;
+  const size_t sb = sub_bytes(ke, np);
+  const uint64_t woff = round_up_u64(blob->size(), 256);
+  const uint64_t boff = round_up_u64(woff + nsub * sb, 256);
+  blob->resize(boff + static_cast<size_t>(np) * 16 * sizeof(float), 0);
+  auto hid_of = [](int sub, int f, int n) { return 16 * sub + 4 * (n >> 1) + 2 * f + (n & 1); };
+  // weight of hidden channel h at position k of the first operator's sum
+  auto first_weight = [&](int h, int k) -> float {
+    if (c.first == kStem) {
+      const int ky = k / 10, e = k % 10;
+      return ky < 3 && e < 9 ? we[(static_cast<size_t>(h) * 3 + ky) * 9 + e] : 0.0f;
+    }
+    return k < cin ? we[static_cast<size_t>(h) * cin + k] : 0.0f;
+  };
+  for (int sub = 0; sub < nsub; ++sub) {
+    uint8_t* base = blob->data() + woff + sub * sb;
+    uint16_t* e = reinterpret_cast<uint16_t*>(base);
+    for (int kk = 0; kk < ke; ++kk)
+      for (int lane = 0; lane < 32; ++lane)
+        for (int w = 0; w < 8; ++w) {  // halves of {frag 0: b0, b1; frag 1: b0, b1}
+          const int f = w >> 2, hi8 = (w >> 1) & 1, lo = w & 1;
+          const int n = lane >> 2, t = lane & 3;
+          const int k = kk * 16 + hi8 * 8 + 2 * t + lo, h = hid_of(sub, f, n);
+          if (h < chid) e[(kk * 32 + lane) * 8 + w] = half_bits(first_weight(h, k));
+        }
+    float* ebias = reinterpret_cast<float*>(base + ke * 512);
+    uint16_t* tabl = reinterpret_cast<uint16_t*>(base + ke * 512 + kBiasBytes);
+    float* dbias = reinterpret_cast<float*>(base + ke * 512 + kBiasBytes + kTableBytes);
+    for (int ch = 0; ch < 16; ++ch) {
+      const int h = sub * 16 + ch;
+      if (h >= chid) break;
+      if (c.first != kNone) ebias[ch] = be[h];
+      for (int i = 0; i < 4; ++i) dbias[ch * 4 + i] = bd[h];
+    }
+    for (int sl = 0; sl < 4; ++sl)
+      for (int jh = 0; jh < 2; ++jh)
+        for (int g = 0; g < 8; ++g) {
+          const int h = sub * 16 + sl * 4 + (g >> 1);
+          if (h >= chid) continue;
+          uint16_t* word = tabl + ((sl * 16 + jh * 8 + g) * 4) * 2;
+          for (int ky = 0; ky < 3; ++ky)
+            for (int b = 0; b < 2; ++b) {
+              // stride 1: input pixel j of the window row feeds output pixel q of the pair through tap j - q;
+              // stride 2: one output column, tap j
+              const int j = b * 2 + jh, q = c.s == 1 ? (g & 1) : 0, dx = j - q;
+              if (dx >= 0 && dx <= 2) word[ky * 2 + b] = half_bits(wd[static_cast<size_t>(ky * 3 + dx) * chid + h]);
+            }
+        }
+    uint16_t* q = reinterpret_cast<uint16_t*>(base + ke * 512 + kSubFixed);
+    for (int j = 0; j < np; ++j)
+      for (int lane = 0; lane < 32; ++lane)
+        for (int w = 0; w < 8; ++w) {
+          const int f = w >> 2, hi8 = (w >> 1) & 1, lo = w & 1;
+          const int n = lane >> 2, t = lane & 3;
+          const int h = sub * 16 + hi8 * 8 + lo * 4 + t, co = hid_of(j, f, n);
+          if (h < chid && co < cout) q[(j * 32 + lane) * 8 + w] = half_bits(wp[static_cast<size_t>(co) * chid + h]);
+        }
+  }
+  float* b = reinterpret_cast<float*>(blob->data() + boff);
+  for (int i = 0; i < cout; ++i) b[i] = bp[i];
+  r->wts = Loc{W_WEIGHTS, 0, woff};
+  r->bias = Loc{W_WEIGHTS, 0, boff};
+  r->wts_bytes = nsub * sb;
+}
+
+namespace {
+// Everything but the pointers.
+BlockParams params_of(const LaunchRec& r, const BlockCfg& c, const Layout& l) {
+  BlockParams p{};
+  p.B = r.B;
+  p.H = r.H;
+  p.W = r.W;
+  p.Ho = r.Ho;
+  p.Wo = r.Wo;
+  const int P = plane_pixels(r.H, r.W), Po = plane_pixels(r.Ho, r.Wo);
+  const bool nhwc_in = r.nhwc_in && c.first != kStem;
+  p.in_px = nhwc_in ? r.C : 4;
+  p.in_img = nhwc_in ? r.H * r.W * r.C : P * 4;
+  p.in_sl = nhwc_in ? 4 : static_cast<long long>(r.B) * P * 4;
+  p.o_px = r.nhwc_out ? r.Co2 : 4;
+  p.o_img = r.nhwc_out ? static_cast<long long>(r.Ho) * r.Wo * r.Co2 : Po * 4;
+  p.o_sl = r.nhwc_out ? 4 : static_cast<long long>(r.B) * Po * 4;
+  p.res_img = Po * 4;
+  p.res_sl = static_cast<long long>(r.B) * Po * 4;
+  p.sin = slices(r.C);
+  p.sout = slices(r.Co2);
+  p.ke = ke_of(r, c);
+  p.pad_t = r.pt;
+  p.pad_l = r.pl;
+  p.tw = c.tw;
+  p.nb = c.nb;
+  p.ni = c.ni;
+  p.tiles_x = c.tiles_x;
+  p.tiles_y = c.tiles_y;
+  p.units = c.units;
+  p.rows = l.rows;
+  p.pitch = l.pitch;
+  p.sub_px = l.sub_px;
+  p.n_list = l.n_list;
+  p.mt = l.mt;
+  p.whole = c.whole;
+  p.compact = l.compact;
+  p.pw = l.pw;
+  p.ncols = l.ncols;
+  p.ngroups = l.ngroups;
+  p.eg = l.eg;
+  p.en = l.en;
+  p.nch = l.nch;
+  p.ks = c.ks;
+  p.resident = l.resident;
+  p.x_pitch = l.x_pitch;
+  p.off_bias = l.off_bias;
+  p.x_bytes = l.x_bytes;
+  p.tab_bytes = l.tab_bytes;
+  p.off_tab = l.off_tab;
+  p.off_x = l.off_x;
+  p.off_raw = l.off_raw;
+  p.off_hid = l.off_hid;
+  p.off_red = l.off_red;
+  p.mul_pitch = magic(l.pitch);
+  p.mul_w = magic(r.W);
+  p.mul_hw = magic(static_cast<uint64_t>(r.H) * r.W);
+  p.mul_per = magic(static_cast<uint64_t>(c.tiles_x) * c.tiles_y);
+  p.mul_tx = magic(c.tiles_x);
+  p.hi_e = r.ep.act_pre == GI_ACT_RELU6 ? 0x46004600u : 0x7c007c00u;
+  const int dact = c.first != kNone ? r.ep_mid.act_pre : r.ep.act_pre;
+  p.hi_d = dact == GI_ACT_RELU6 ? 0x46004600u : 0x7c007c00u;
+  p.act_pre = r.ep2.act_pre;
+  p.act_post = r.ep2.act_post;
+  p.has_res = r.ep2.has_res;
+  p.wide = !r.nhwc_out && r.Wo % 2 == 0;
+  p.pad_px = !r.nhwc_out && (r.Ho * r.Wo) % 2;
+  p.Hi = r.stem_h;
+  p.Wi = r.stem_w;
+  p.spt = r.stem_pt;
+  p.spl = r.stem_pl;
+  p.raw_rows = l.raw_rows;
+  p.raw_words = l.raw_words;
+  return p;
+}
+}  // namespace
+
+int launch_block_mma(const LaunchRec& r, const Ptrs& ptr, void* stream) {
+  const BlockCfg& c = r.block;
+  Layout l;
+  if (!layout_of(r, c, &l)) return static_cast<int>(cudaErrorInvalidConfiguration);
+  BlockParams p = params_of(r, c, l);
+  p.in = static_cast<const __half*>(ptr.in0);
+  p.res = static_cast<const __half*>(ptr.res);
+  p.out = static_cast<__half*>(ptr.out);
+  p.wts = static_cast<const unsigned char*>(ptr.wts);
+  p.bias = static_cast<const float*>(ptr.bias);
+  p.res_x = p.has_res && ptr.res == ptr.in0 && !r.nhwc_in && c.s == 1 && c.first != kNone && c.first != kExpWide && c.first != kStem;
+  const long long slots = c.ks > 1 ? c.units : static_cast<long long>(device_sm_count()) * ctas_per_sm(c, l);
+  const int grid = static_cast<int>(std::min<long long>(c.units, std::max<long long>(1, slots))) * c.ks;
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  return c.s == 1 ? launch_first<1>(c, p, l.nw, l.bytes, grid, st) : launch_first<2>(c, p, l.nw, l.bytes, grid, st);
+}
+
+}  // namespace gi

@@ -441,6 +441,48 @@ gi_status plan_memory(gi_exec* e) {
   return GI_OK;
 }
 
+// With groups the tensors inside a group are never stored, and a group reads its input while it writes its output, which as
+// separate ops may share bytes.  So the offsets of the tensors that remain are planned again, by size, over the list of
+// launches; the arena the caller provides stays the planned one, which is larger: it had to hold the tensors in between.
+void plan_run(gi_exec* e) {
+  e->run_offset.clear();
+  if (e->groups.empty() || e->opt.planner == GI_PLAN_NAIVE) return;  // the naive plan shares no byte: it stands
+  std::vector<int> step(e->ops.size());
+  std::vector<char> inside(e->tensors.size(), 0);
+  for (size_t i = 0; i < e->ops.size(); ++i) step[i] = static_cast<int>(i);
+  for (const OpGroup& gr : e->groups)
+    for (int k = 0; k < gr.n; ++k) {
+      step[gr.first + k] = gr.first;
+      if (k + 1 < gr.n) inside[e->ops[gr.first + k].out] = 1;
+    }
+  const std::vector<TensorPlan> planned = e->plan;
+  for (size_t t = 0; t < e->plan.size(); ++t) {
+    e->plan[t].first = static_cast<int>(e->ops.size());
+    e->plan[t].last = -1;
+    if (inside[t] || planned[t].intermediate == 2) e->plan[t].intermediate = 0;
+  }
+  auto use = [&](int t, int at) {
+    while (t >= 0) {  // the tensor itself and, if it is placed inside another one, its holder
+      e->plan[t].first = std::min(e->plan[t].first, at);
+      e->plan[t].last = std::max(e->plan[t].last, at);
+      t = planned[t].view_of;
+    }
+  };
+  for (size_t i = 0; i < e->ops.size(); ++i)
+    for (int t : {e->ops[i].in0, e->ops[i].in1, e->ops[i].residual, e->ops[i].out}) use(t, step[i]);
+  const uint64_t total = plan_by_size(e);
+  if (total <= e->arena_bytes) {
+    e->run_offset.resize(e->plan.size(), 0);
+    for (size_t t = 0; t < e->plan.size(); ++t) e->run_offset[t] = e->plan[t].offset;
+    for (size_t t = 0; t < e->plan.size(); ++t)
+      if (planned[t].intermediate == 2)
+        e->run_offset[t] = e->run_offset[planned[t].view_of] + (planned[t].offset - planned[planned[t].view_of].offset);
+  } else {
+    e->groups.clear();
+  }
+  e->plan = planned;
+}
+
 }  // namespace gi
 
 using namespace gi;
@@ -503,7 +545,11 @@ gi_status gi_compile(const gi_graph* g, const gi_compile_options* opt, gi_exec**
       e->ops.push_back(p);
     }
     s = plan_memory(e);
-    if (s == GI_OK) s = lower(*g, e);
+    if (s == GI_OK) {
+      find_groups(*g, e);
+      plan_run(e);
+      s = lower(*g, e);
+    }
     if (s != GI_OK) {
       delete e;
       return s;
@@ -559,6 +605,20 @@ gi_status gi_exec_op(const gi_exec* e, int32_t index, gi_op_info* info) {
   if (!e || !info) return fail(GI_E_INVALID, "gi_exec_op: null argument");
   if (index < 0 || index >= static_cast<int>(e->op_info.size())) return fail(GI_E_INVALID, "gi_exec_op: index out of range");
   *info = e->op_info[index];
+  return GI_OK;
+}
+
+gi_status gi_exec_launch(const gi_exec* e, int32_t index, gi_launch_info* info) {
+  if (!e || !info) return fail(GI_E_INVALID, "gi_exec_launch: null argument");
+  if (index < 0 || index >= static_cast<int>(e->run_info.size())) return fail(GI_E_INVALID, "gi_exec_launch: index out of range");
+  std::memset(info, 0, sizeof *info);
+  const gi_op_info& r = e->run_info[index];
+  info->kernel = r.kernel;
+  info->n_ops = r.kernel == GI_KERNEL_NONE ? 0 : 1;
+  for (size_t i = index + 1; r.kernel != GI_KERNEL_NONE && i < e->run_info.size() && e->run_info[i].kernel == GI_KERNEL_NONE; ++i)
+    ++info->n_ops;
+  info->bytes = r.bytes;
+  info->flops = r.flops;
   return GI_OK;
 }
 

@@ -49,6 +49,19 @@ struct Epilogue {
   int act_post = GI_ACT_NONE;
 };
 
+// Configuration of the kernel that runs a depthwise convolution and the convolutions around it (block_mma.cu), chosen at
+// compile time.
+enum BlockKind { BLOCK_EXPANSION = 0, BLOCK_PAIR = 1, BLOCK_STEM = 2 };
+struct BlockCfg {
+  int s = 1, first = 0;         // stride of the depthwise operator; how the operator in front of it is computed
+  int np = 2, tr = 2, hc = 1;   // 16-channel output blocks, output rows per warp, 16-channel sub-blocks per chunk
+  int tw = 2, nb = 1, ni = 1;   // output columns of a tile, bands of `tr` rows, images per unit
+  int tiles_x = 1, tiles_y = 1, whole = 0, units = 1;
+  int ks = 1;                   // CTAs (a cluster) that share a unit's hidden channels
+  int nw_min = 8;               // warps of a CTA, if the first operator has work for them
+  int resident_kb = 0;          // weights of at most this size stay in shared memory
+};
+
 // Parameters of one kernel launch; pointers are resolved by gi_run from the Locs.
 struct LaunchRec {
   int kernel = 0;  // GI_KERNEL_*
@@ -88,6 +101,12 @@ struct LaunchRec {
   // two consecutive 1x1 convolutions as one kernel: `out` / `res` / `ep` / `wts` are the first one's (Cmid its output
   // channels), `out2` / `ep2` / `wts2` / Co2 the second one's; `bias` holds both bias vectors
   Loc out2;
+  // depthwise 3x3 and the convolutions around it as one kernel: `ep` is the first operator's epilogue, `ep_mid` the depthwise
+  // one's behind it, `ep2` the projection's; Cmid / Co2, stride, pads and (Ho, Wo) as above; (H, W) the depthwise input
+  BlockCfg block;
+  int nhwc_out = 0;  // it writes the caller's NHWC output itself
+  int lead = -1, dw_op = -1;  // executed ops: the convolution in front of the depthwise one (or -1), the depthwise one
+  int stem_h = 0, stem_w = 0, stem_pt = 0, stem_pl = 0;  // image and padding of a stem in front of the depthwise operator
 };
 
 struct FusedOp {
@@ -106,6 +125,13 @@ struct TensorPlan {
   int view_slice = 0;  // first slice of `view_of` that this tensor occupies
 };
 
+// Consecutive executed ops that gi_run launches as one kernel.
+struct OpGroup {
+  int first = 0, n = 0, kind = 0;
+  double us = 0.0;  // estimated time
+  LaunchRec rec;    // geometry and configuration
+};
+
 }  // namespace gi
 
 struct gi_exec {
@@ -114,7 +140,10 @@ struct gi_exec {
   std::vector<gi::TensorDesc> tensors;
   std::vector<gi::TensorPlan> plan;
   std::vector<gi::FusedOp> ops;       // executed ops in order
-  std::vector<gi_op_info> op_info;
+  std::vector<gi_op_info> op_info;    // the ops one by one (gi_exec_op)
+  std::vector<gi_op_info> run_info;   // kernel, bytes and flops of what gi_run launches at each op (gi_exec_launch)
+  std::vector<gi::OpGroup> groups;    // runs of ops that are launched as one kernel
+  std::vector<uint64_t> run_offset;   // arena offset per tensor when there are groups (empty: the plan's)
   std::vector<gi::LaunchRec> launches;
   std::vector<uint8_t> weight_blob;   // host staging copy of all packed weights
   int n_inputs = 0, n_outputs = 0, n_fused = 0;
@@ -138,8 +167,10 @@ uint16_t f32_to_f16_rne(float f);
 // compile-step pieces (gi_compile.cc)
 gi_status fuse_graph(const gi_graph& g, bool enable, std::vector<FusedOp>* out);
 gi_status plan_memory(gi_exec* e);
+void plan_run(gi_exec* e);  // arena offsets for the grouped ops; drops the groups if they do not fit the planned arena
 
 // weight packing + launch records (gi_lower.cc)
+void find_groups(const gi_graph& g, gi_exec* e);
 gi_status lower(const gi_graph& g, gi_exec* e);
 
 // run module (gi_run.cu)

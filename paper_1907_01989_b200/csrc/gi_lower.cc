@@ -1,6 +1,7 @@
 // Lowering: choose a kernel per executed op, pack its weights into the kernel's operand
 // layout (fp16 storage: weights rounded to fp16 once, biases stay fp32) and record the
 // launch geometry.  Host work only.
+#include <algorithm>
 #include <cstdlib>
 #include <cstring>
 
@@ -47,7 +48,7 @@ static Loc loc_of(const gi_exec* e, int t) {
     l.index = d.output_index;
   } else {
     l.where = W_ARENA;
-    l.offset = e->plan[t].offset;
+    l.offset = e->run_offset.empty() ? e->plan[t].offset : e->run_offset[t];
   }
   return l;
 }
@@ -172,6 +173,16 @@ static bool private_between(const gi_exec* e, int t, size_t i) {
          e->tensors[t].output_index < 0 && e->tensors[t].input_index < 0;
 }
 
+// The same, without a look at the memory plan's kind of tensor: only the next executed op reads it.
+static bool private_to_next(const gi_exec* e, int t, size_t i) {
+  if (t < 0 || e->plan[t].intermediate != 1) return false;
+  for (size_t j = 0; j < e->ops.size(); ++j) {
+    const FusedOp& o = e->ops[j];
+    if (j != i + 1 && (o.in0 == t || o.in1 == t || o.residual == t)) return false;
+  }
+  return true;
+}
+
 // Executed ops i, i + 1, i + 2 are the three convolutions of an inverted-residual block - 1x1 expansion, depthwise
 // 3x3, 1x1 projection (with or without the residual sum) - and the two tensors between them have no other reader, so
 // that one kernel may run all three and keep those tensors on chip.
@@ -238,7 +249,174 @@ static int nhwc_pack_feeding_only(const gi_exec* e, int t, size_t reader) {
   return pack;
 }
 
-gi_status lower(const gi_graph& g, gi_exec* e) {
+static bool clamps_at_zero(int act) { return act == GI_ACT_RELU || act == GI_ACT_RELU6; }
+
+// A run of executed ops that block_mma.cu may run as one kernel: `n` ops of which the first `lead` stand in front of the
+// depthwise one; the graph's input conversion before them and output conversion behind them included where the kernel reads /
+// writes the caller's NHWC tensor itself.
+struct BlockOps {
+  int n = 0, kind = 0;
+  int first = -1, dw = -1, pw = -1;  // executed ops: the convolution in front (or -1), the depthwise one, the 1x1 one
+  int pack = 0, unpack = 0;          // the run starts / ends with a layout conversion
+};
+
+// The run that starts at executed op `i`.  The tensors between its ops must have no other reader.  Where the tensors in
+// memory lie is settled afterwards (plan_run), so their places do not matter here.
+static BlockOps block_ops_at(const gi_graph& g, const gi_exec* e, size_t i) {
+  BlockOps b;
+  const size_t n_ops = e->ops.size();
+  size_t k = i;
+  if (e->ops[k].kind == GI_EXEC_PACK) {
+    if (!private_to_next(e, e->ops[k].out, k)) return BlockOps();
+    b.pack = 1;
+    ++k;
+  }
+  if (k >= n_ops) return BlockOps();
+  const FusedOp& a = e->ops[k];
+  b.kind = BLOCK_PAIR;
+  if (a.kind == GI_OP_CONV2D) {
+    const gi_op_desc& d = g.ops[a.graph_op].d;
+    const TensorDesc& in = e->tensors[a.in0];
+    const bool stem = b.pack && in.c == 3 && d.kh == 3 && d.kw == 3 && d.stride_h == 2 && d.stride_w == 2 && d.dilation_h == 1 &&
+                      d.dilation_w == 1 && d.pad_t <= 1 && d.pad_l <= 1;
+    if (!stem && !is_plain_pointwise(d)) return BlockOps();
+    if (a.residual >= 0 || a.act_post != GI_ACT_NONE || !clamps_at_zero(a.act_pre) || !private_to_next(e, a.out, k)) return BlockOps();
+    b.kind = stem ? BLOCK_STEM : BLOCK_EXPANSION;
+    b.first = static_cast<int>(k);
+    ++k;
+  }
+  if (b.pack && b.kind != BLOCK_STEM && e->tensors[e->ops[i].out].c % 4 != 0) return BlockOps();
+  if (k + 1 >= n_ops) return BlockOps();
+  const FusedOp& d = e->ops[k];
+  const FusedOp& c = e->ops[k + 1];
+  if (d.kind != GI_OP_DEPTHWISE_CONV2D || c.kind != GI_OP_CONV2D || !is_plain_pointwise(g.ops[c.graph_op].d)) return BlockOps();
+  if (d.residual >= 0 || d.act_post != GI_ACT_NONE || !clamps_at_zero(d.act_pre)) return BlockOps();
+  if (c.in0 != d.out || c.residual == d.out || !private_to_next(e, d.out, k)) return BlockOps();
+  if (b.first >= 0 && (d.in0 != a.out || c.residual == a.out)) return BlockOps();
+  if (b.pack && (b.first >= 0 ? a.in0 : d.in0) != e->ops[i].out) return BlockOps();
+  if (b.pack && c.residual == e->ops[i].out) return BlockOps();
+  b.dw = static_cast<int>(k);
+  b.pw = static_cast<int>(k + 1);
+  if (k + 2 < n_ops) {
+    const FusedOp& u = e->ops[k + 2];
+    if (u.kind == GI_EXEC_UNPACK && u.in0 == c.out && private_to_next(e, c.out, k + 1) && e->tensors[c.out].c % 4 == 0) b.unpack = 1;
+  }
+  b.n = b.pw - static_cast<int>(i) + 1 + b.unpack;
+  return b;
+}
+
+// Launch geometry of such a run.
+static LaunchRec block_rec(const gi_graph& g, const gi_exec* e, const BlockOps& b) {
+  const FusedOp& d = e->ops[b.dw];
+  const FusedOp& c = e->ops[b.pw];
+  const gi_op_desc& dd = g.ops[d.graph_op].d;
+  const TensorDesc &din = e->tensors[d.in0], &dmid = e->tensors[d.out], &dout = e->tensors[c.out];
+  LaunchRec r;
+  r.kernel = GI_KERNEL_BLOCK_MMA;
+  r.B = e->batch;
+  r.H = din.h;
+  r.W = din.w;
+  r.C = b.first >= 0 ? e->tensors[e->ops[b.first].in0].c : din.c;
+  r.Ho = dmid.h;
+  r.Wo = dmid.w;
+  r.Co = dmid.c;
+  r.Cmid = dmid.c;
+  r.Co2 = dout.c;
+  r.kh = dd.kh;
+  r.kw = dd.kw;
+  r.sh = dd.stride_h;
+  r.sw = dd.stride_w;
+  r.dh = dd.dilation_h;
+  r.dw = dd.dilation_w;
+  r.pt = dd.pad_t;
+  r.pl = dd.pad_l;
+  r.ep.act_pre = b.first >= 0 ? e->ops[b.first].act_pre : d.act_pre;
+  r.ep_mid.act_pre = d.act_pre;
+  r.ep2.act_pre = c.act_pre;
+  r.ep2.has_res = c.residual >= 0;
+  r.ep2.act_post = c.act_post;
+  r.nhwc_in = b.pack;
+  r.nhwc_out = b.unpack;
+  if (b.kind == BLOCK_STEM) {
+    const FusedOp& a = e->ops[b.first];
+    r.stem_h = e->tensors[a.in0].h;
+    r.stem_w = e->tensors[a.in0].w;
+    r.stem_pt = g.ops[a.graph_op].d.pad_t;
+    r.stem_pl = g.ops[a.graph_op].d.pad_l;
+  }
+  return r;
+}
+
+// Estimated time of the run's ops as launches of their own: 4 us each (what a launch adds to a chain of them) plus their bytes
+// at the rates the kernels reach inside MobileNetV2 - 6 TB/s, 3.2 for a stencil on planes without a straight-line form, 4 for
+// the stem - plus 4 ns per input channel of a 1x1 convolution (its chain of matrix instructions).  Against the measured
+// times of the network's ops at batch 1, 21 and 256 it is within 15 %.
+static double separate_us(const gi_exec* e, const OpGroup& gr) {
+  double us = 0.0;
+  auto bytes = [&](int t) {
+    return t < 0 ? 0.0 : 2.0 * e->batch * e->tensors[t].h * e->tensors[t].w * slices(e->tensors[t].c) * 4;
+  };
+  for (int i = gr.first; i < gr.first + gr.n; ++i) {
+    const FusedOp& o = e->ops[i];
+    const double b = bytes(o.in0) + bytes(o.out) + bytes(o.residual);
+    double rate = 6.0e6;  // bytes per us
+    if (o.kind == GI_EXEC_PACK) {
+      const TensorDesc& d = e->tensors[o.out];
+      // the stem reads an even image itself (conv3x3_tc_reads_nhwc)
+      if (gr.rec.lead >= 0 && gr.rec.stem_h > 0 && conv3x3_tc_reads_nhwc(d.c, d.h, d.w, 2, 1, gr.rec.stem_pt, gr.rec.stem_pl)) continue;
+    }
+    if (o.kind == GI_OP_CONV2D) {
+      if (gr.rec.stem_h > 0 && i == gr.rec.lead) rate = 4.0e6;
+      else us += 0.004 * e->tensors[o.in0].c;
+    }
+    if (o.kind == GI_OP_DEPTHWISE_CONV2D) {
+      const int w = e->tensors[o.out].w;
+      if (w != 112 && w != 56 && w != 28 && w != 14 && w != 7) rate = 3.2e6;
+    }
+    us += 4.0 + b / rate;
+  }
+  return us;
+}
+
+// Which runs of executed ops gi_run launches as one kernel each (e->groups): where the kernel's estimate is below that of the
+// ops' own kernels.  Not when the caller asked for one kernel per op or for a particular kernel.
+void find_groups(const gi_graph& g, gi_exec* e) {
+  e->groups.clear();
+  if (e->storage != GI_F16 || !e->opt.fuse || e->opt.cross_op != GI_XOP_AUTO || e->opt.pointwise != GI_PW_AUTO) return;
+  for (size_t i = 0; i < e->ops.size(); ++i) {
+    const BlockOps b = block_ops_at(g, e, i);
+    if (b.n == 0) continue;
+    OpGroup gr;
+    gr.first = static_cast<int>(i);
+    gr.n = b.n;
+    gr.rec = block_rec(g, e, b);
+    gr.rec.lead = b.first;
+    gr.rec.dw_op = b.dw;
+    double us = 0.0;
+    for (const OpGroup& o : e->groups)  // blocks of a network repeat: the same geometry, the same choice
+      if (o.kind == b.kind && o.rec.H == gr.rec.H && o.rec.W == gr.rec.W && o.rec.C == gr.rec.C && o.rec.Cmid == gr.rec.Cmid &&
+          o.rec.Co2 == gr.rec.Co2 && o.rec.sh == gr.rec.sh && o.rec.Ho == gr.rec.Ho && o.rec.Wo == gr.rec.Wo) {
+        gr.rec.block = o.rec.block;
+        us = o.us;
+      }
+    if (us == 0.0 && !block_mma_choose(gr.rec, b.kind, &gr.rec.block, &us)) continue;
+    if (us > separate_us(e, gr)) continue;
+    gr.kind = b.kind;
+    gr.us = us;
+    e->groups.push_back(gr);
+    i += b.n - 1;
+  }
+}
+
+static const OpGroup* group_of(const gi_exec* e, size_t i) {
+  for (const OpGroup& gr : e->groups)
+    if (static_cast<int>(i) >= gr.first && static_cast<int>(i) < gr.first + gr.n) return &gr;
+  return nullptr;
+}
+
+// One pass over the executed ops.  `grouped`: runs of ops in e->groups become one launch; otherwise every op is lowered by
+// itself.  `pack`: also pack the weights.
+static gi_status lower_pass(const gi_graph& g, gi_exec* e, bool grouped, bool pack) {
   const int eb = elem_bytes(e->storage);
   const uint64_t B = static_cast<uint64_t>(e->batch);
   int absorbed = 0;  // this many following ops run inside the kernel of an op already lowered
@@ -254,6 +432,33 @@ gi_status lower(const gi_graph& g, gi_exec* e) {
     info.output = f.out;
     info.act_pre = f.act_pre;
     info.act_post = f.act_post;
+    if (const OpGroup* gr = grouped ? group_of(e, i) : nullptr) {
+      if (static_cast<int>(i) == gr->first) {
+        r = gr->rec;
+        const int lead = r.lead;
+        const FusedOp& d = e->ops[r.dw_op];
+        const FusedOp& c = e->ops[r.dw_op + 1];
+        const int in = lead >= 0 ? e->ops[lead].in0 : d.in0;
+        r.in0 = r.nhwc_in ? Loc{W_INPUT, e->tensors[in].input_index, 0} : loc_of(e, in);
+        r.out = r.nhwc_out ? Loc{W_OUTPUT, e->ops[gr->first + gr->n - 1].io_index, 0} : loc_of(e, c.out);
+        r.res = loc_of(e, c.residual);
+        const OpNode &wd = g.ops[d.graph_op], &wp = g.ops[c.graph_op];
+        const OpNode* we = lead >= 0 ? &g.ops[e->ops[lead].graph_op] : nullptr;
+        block_mma_pack(we ? we->weights.data() : nullptr, we ? we->bias.data() : nullptr, wd.weights.data(), wd.bias.data(),
+                       wp.weights.data(), wp.bias.data(), r.C, r.Cmid, r.Co2, r.block, &e->weight_blob, &r);
+        const uint64_t px_in = B * e->tensors[in].h * e->tensors[in].w, px_hid = B * r.H * r.W, px_out = B * r.Ho * r.Wo;
+        const uint64_t taps = we ? static_cast<uint64_t>(we->d.kh) * we->d.kw : 0, cmid = r.Cmid, cin = r.C, cout = r.Co2;
+        info.bytes = (px_in * (r.nhwc_in ? cin : slices(r.C) * 4) + px_out * slices(r.Co2) * 4 * (r.ep2.has_res ? 2 : 1) +
+                      taps * cin * cmid + 9 * cmid + cmid * cout) * eb;
+        info.flops = 2 * taps * px_hid * cin * cmid + 18 * px_out * cmid + 2 * px_out * cmid * cout;
+      } else {
+        r.kernel = GI_KERNEL_NONE;
+      }
+      info.kernel = r.kernel;
+      e->launches.push_back(r);
+      e->op_info.push_back(info);
+      continue;
+    }
     r.B = e->batch;
     r.ep.act_pre = f.act_pre;
     r.ep.has_res = f.residual >= 0;
@@ -335,7 +540,7 @@ gi_status lower(const gi_graph& g, gi_exec* e) {
           }
           if (!r.dw_staged && e->batch > 65535)
             return fail(GI_E_UNSUPPORTED, "gi_compile: depthwise convolution: batch above 65535 with a shape only the plain kernel runs");
-          pack_depthwise(op, din->c, e->storage, &e->weight_blob, &r);
+          if (pack) pack_depthwise(op, din->c, e->storage, &e->weight_blob, &r);
           info.bytes += taps * din->c * eb;
           info.flops = 2 * taps * out_px * din->c;
           if (e->storage == GI_F16 && e->opt.cross_op == GI_XOP_ON && pointwise_follows(g, e, i) &&
@@ -348,7 +553,7 @@ gi_status lower(const gi_graph& g, gi_exec* e) {
             const OpNode& pw = g.ops[n.graph_op];
             const TensorDesc& d2 = e->tensors[n.out];
             r.kernel = GI_KERNEL_DEPTHWISE_POINTWISE;
-            depthwise_pointwise_pack(pw.weights.data(), pw.bias.data(), din->c, pw.d.cout, din->w, &e->weight_blob, &r);
+            if (pack) depthwise_pointwise_pack(pw.weights.data(), pw.bias.data(), din->c, pw.d.cout, din->w, &e->weight_blob, &r);
             r.Co2 = pw.d.cout;
             r.ep2.act_pre = n.act_pre;
             r.ep2.has_res = n.residual >= 0;
@@ -410,7 +615,7 @@ gi_status lower(const gi_graph& g, gi_exec* e) {
               r.ep2.act_post = fp.act_post;
               r.out = loc_of(e, fp.out);
               r.res = loc_of(e, fp.residual);
-              inverted_residual_pack(op.weights.data(), op.bias.data(), dwn.weights.data(), dwn.bias.data(), pwn.weights.data(),
+              if (pack) inverted_residual_pack(op.weights.data(), op.bias.data(), dwn.weights.data(), dwn.bias.data(), pwn.weights.data(),
                                      pwn.bias.data(), din->c, op.d.cout, pwn.d.cout, &e->weight_blob, &r);
               const uint64_t px2 = B * d2.h * d2.w, c42 = slices(d2.c) * 4;
               info.bytes = (in_px * in_c4 + px2 * c42 * (r.ep2.has_res ? 2 : 1) + static_cast<uint64_t>(din->c) * op.d.cout +
@@ -430,7 +635,7 @@ gi_status lower(const gi_graph& g, gi_exec* e) {
           const long long pc_tiles = (m_px_all_for_mm(e, din) + 127) / 128;
           const bool chain_auto = din->h * din->w > 64 && din->h * din->w <= 256 && op.d.cout <= 64 && din->c >= 192 && pc_tiles >= 2 * 148;
           if (pointwise && tc && e->opt.fuse && (e->opt.cross_op == GI_XOP_CHAIN || (e->opt.cross_op == GI_XOP_AUTO && chain_auto)) &&
-              chain_follows(g, e, i) &&
+              chain_follows(g, e, i) && !(grouped && group_of(e, i + 1)) &&
               pointwise_chain_supported(din->c, op.d.cout, g.ops[e->ops[i + 1].graph_op].d.cout, f.residual >= 0)) {
             const FusedOp& fb = e->ops[i + 1];
             const OpNode& nb = g.ops[fb.graph_op];
@@ -440,7 +645,7 @@ gi_status lower(const gi_graph& g, gi_exec* e) {
             r.Co2 = nb.d.cout;
             r.ep2.act_pre = fb.act_pre;
             r.out2 = loc_of(e, fb.out);
-            pointwise_chain_pack(op.weights.data(), op.bias.data(), nb.weights.data(), nb.bias.data(), din->c, op.d.cout, nb.d.cout,
+            if (pack) pointwise_chain_pack(op.weights.data(), op.bias.data(), nb.weights.data(), nb.bias.data(), din->c, op.d.cout, nb.d.cout,
                                  &e->weight_blob, &r);
             const uint64_t c42 = slices(d2.c) * 4;
             info.bytes = (in_px * in_c4 + out_px * out_c4 * (r.ep.has_res ? 2 : 1) + out_px * c42 +
@@ -478,13 +683,13 @@ gi_status lower(const gi_graph& g, gi_exec* e) {
           }
           if (pointwise && tc && wide_kernel && pointwise_mm_supported(din->c, op.d.cout)) {
             r.kernel = GI_KERNEL_POINTWISE_MM;
-            pointwise_mm_pack(op.weights.data(), op.bias.data(), din->c, op.d.cout, &e->weight_blob, &r);
+            if (pack) pointwise_mm_pack(op.weights.data(), op.bias.data(), din->c, op.d.cout, &e->weight_blob, &r);
           } else if (pointwise && tc && (lane_tab || (lane_kernel && !pair_tab)) && pointwise_ts_supported(din->c, op.d.cout)) {
             r.kernel = GI_KERNEL_POINTWISE_TS;
-            pointwise_ts_pack(op.weights.data(), op.bias.data(), din->c, op.d.cout, &e->weight_blob, &r);
+            if (pack) pointwise_ts_pack(op.weights.data(), op.bias.data(), din->c, op.d.cout, &e->weight_blob, &r);
           } else if (pointwise && tc && pointwise_tc_supported(din->c, op.d.cout)) {
             r.kernel = GI_KERNEL_POINTWISE_TC;
-            pointwise_tc_pack(op.weights.data(), op.bias.data(), din->c, op.d.cout, &e->weight_blob, &r);
+            if (pack) pointwise_tc_pack(op.weights.data(), op.bias.data(), din->c, op.d.cout, &e->weight_blob, &r);
           } else if (tc && conv3x3_tc_supported(din->c, op.d.cout, op.d.kh, op.d.kw, op.d.stride_h, op.d.stride_w,
                                           op.d.dilation_h, op.d.dilation_w)) {
             r.kernel = GI_KERNEL_CONV3X3_TC;
@@ -501,15 +706,15 @@ gi_status lower(const gi_graph& g, gi_exec* e) {
               e->op_info[pack_op].bytes = 0;
               info.bytes = (in_px * din->c + out_px * out_c4 * (r.ep.has_res ? 2 : 1)) * eb;
             }
-            conv3x3_tc_pack(op.weights.data(), op.bias.data(), din->c, op.d.cout, &e->weight_blob, &r);
+            if (pack) conv3x3_tc_pack(op.weights.data(), op.bias.data(), din->c, op.d.cout, &e->weight_blob, &r);
           } else if (tc && conv_kxk_tc_supported(din->c, op.d.cout, op.d.kh, op.d.kw, op.d.stride_h, op.d.stride_w,
                                                   op.d.dilation_h, op.d.dilation_w)) {
             // any other 1x1 (strided or padded), 2x2 or 3x3 convolution whose weights fit shared memory
             r.kernel = GI_KERNEL_CONV_TC;
-            conv_kxk_tc_pack(op.weights.data(), op.bias.data(), din->c, op.d.cout, op.d.kh, &e->weight_blob, &r);
+            if (pack) conv_kxk_tc_pack(op.weights.data(), op.bias.data(), din->c, op.d.cout, op.d.kh, &e->weight_blob, &r);
           } else {
             r.kernel = GI_KERNEL_CONV_SIMT;
-            pack_conv_simt(op, din->c, e->storage, &e->weight_blob, &r);
+            if (pack) pack_conv_simt(op, din->c, e->storage, &e->weight_blob, &r);
           }
           info.bytes += taps * din->c * op.d.cout * eb;
           info.flops = 2 * taps * out_px * din->c * op.d.cout;
@@ -564,6 +769,27 @@ gi_status lower(const gi_graph& g, gi_exec* e) {
   // keep the blob a whole number of 256-byte units so any tail read stays inside it
   e->weight_blob.resize(round_up_u64(e->weight_blob.size() + 1, 256), 0);
   return GI_OK;
+}
+
+// gi_exec_op describes the ops one by one - the kernel chosen for each and its own bytes; what gi_run launches is described
+// by run_info.  The two differ where ops are grouped.  Under the naive plan, the one under which a caller can find every
+// stored tensor after a run, gi_exec_op says what is launched: a tensor between the ops of a launch is not stored.
+gi_status lower(const gi_graph& g, gi_exec* e) {
+  std::vector<gi_op_info> one_by_one;
+  if (!e->groups.empty() && e->opt.planner != GI_PLAN_NAIVE) {
+    std::vector<uint64_t> run_offset;
+    run_offset.swap(e->run_offset);  // ops one by one: where the plan put the tensors
+    const gi_status s = lower_pass(g, e, false, false);
+    run_offset.swap(e->run_offset);
+    if (s != GI_OK) return s;
+    one_by_one.swap(e->op_info);
+    e->launches.clear();
+    e->weight_blob.clear();
+  }
+  const gi_status s = lower_pass(g, e, true, true);
+  e->run_info = e->op_info;
+  if (!one_by_one.empty()) e->op_info.swap(one_by_one);
+  return s;
 }
 
 }  // namespace gi

@@ -104,4 +104,10 @@ void inverted_residual_pack(const float* we, const float* be, const float* wd, c
 int launch_inverted_residual(const LaunchRec& r, const Ptrs& p, void* stream);
 unsigned int inverted_residual_error_word(int* cuda_err);
 
+// Depthwise 3x3 with the convolutions around it as one kernel, any plane size (fp16 storage; block_mma.cu).
+bool block_mma_choose(const LaunchRec& r, int kind, BlockCfg* best, double* us);
+void block_mma_pack(const float* we, const float* be, const float* wd, const float* bd, const float* wp, const float* bp, int cin,
+                    int chid, int cout, const BlockCfg& c, std::vector<uint8_t>* blob, LaunchRec* r);
+int launch_block_mma(const LaunchRec& r, const Ptrs& p, void* stream);
+
 }  // namespace gi

@@ -935,3 +935,61 @@ def test_bounded_wait_runs_out_and_the_context_survives():
     assert api.gi_device_status() == 0
     check_outputs(wl.separable_block(2), api.GI_F16)
     assert api.gi_device_status() == 0
+
+
+# ---------------------------------------------------------------------- depthwise and the convolutions around it as one kernel
+def _stem_block(batch, h, w, cmid, cout):
+    b = wl.GraphBuilder("stem_block", batch, 16)
+    y = b.activation(b.conv2d(b.input(h, w, 3), cmid, 3, 2), wl.ACT_RELU6)
+    y = b.activation(b.depthwise(y, 3, 1), wl.ACT_RELU)
+    b.output(b.conv2d(y, cout, 1))
+    return b.finish()
+
+
+BLOCK_MMA_CASES = {
+    # stem: even and odd images (rows that start on an odd half), one output slice short of a block, several tiles
+    "stem_even": lambda: _stem_block(2, 32, 32, 32, 16), "stem_odd": lambda: _stem_block(3, 33, 37, 32, 24),
+    "stem_w_odd": lambda: _stem_block(1, 64, 31, 24, 20), "stem_large": lambda: _stem_block(1, 225, 161, 32, 64),
+    # pairs: both layouts read and written by the kernel (channels a multiple of 4), conversions kept (they are not)
+    "pair": lambda: wl.depthwise_then_pointwise(1, 32, 32, 32, 64, pw_act=wl.ACT_RELU6), "pair_odd": lambda: wl.depthwise_then_pointwise(2, 9, 7, 20, 12),
+    "pair_ragged": lambda: wl.depthwise_then_pointwise(2, 13, 11, 21, 18), "pair_s2": lambda: wl.depthwise_then_pointwise(3, 21, 15, 48, 32, 2),
+    "pair_residual": lambda: wl.depthwise_then_pointwise(2, 17, 19, 24, 40, 1, residual=True, pw_act=wl.ACT_RELU, post_act=wl.ACT_RELU6),
+    # blocks: every width of the expansion, strides, residuals from shared and from global memory, ragged channels
+    "exp16_s2": lambda: wl.inverted_residual_block(2, 30, 26, 16, 96, 24, 2), "exp16": lambda: wl.inverted_residual_block(1, 7, 5, 10, 40, 10, 1),
+    "exp24": lambda: wl.inverted_residual_block(1, 56, 56, 24, 144, 24, 1), "exp24_odd": lambda: wl.inverted_residual_block(2, 29, 31, 21, 100, 21, 1, out_act=wl.ACT_RELU),
+    "exp32_s2": lambda: wl.inverted_residual_block(3, 29, 27, 32, 192, 64, 2), "exp32": lambda: wl.inverted_residual_block(5, 28, 28, 32, 192, 32, 1),
+    "wide": lambda: wl.inverted_residual_block(1, 14, 14, 64, 384, 64, 1), "wide_odd": lambda: wl.inverted_residual_block(2, 13, 9, 41, 130, 41, 1),
+    "wide_96": lambda: wl.inverted_residual_block(1, 33, 33, 96, 576, 96, 1, act=wl.ACT_RELU), "wide_s2": lambda: wl.inverted_residual_block(2, 14, 14, 96, 576, 160, 2),
+    "wide_160": lambda: wl.inverted_residual_block(1, 6, 6, 160, 960, 160, 1),
+}
+
+
+@pytest.mark.parametrize("case", list(BLOCK_MMA_CASES))
+def test_depthwise_with_its_neighbours_as_one_kernel(case):
+    """The library's own choice for small launches: one kernel, equal to the oracle within the tolerance of the ops one by one
+    (the hidden tensors are rounded to fp16 in both), and bit-identical from run to run."""
+    spec = BLOCK_MMA_CASES[case]()
+    xs = [wl.make_input(spec, index=i) for i in range(len(spec.inputs))]
+    run = DeviceRun(spec, api.GI_F16, guard_bytes=4096)
+    names = [api.KERNEL_NAMES[launch.kernel] for launch in run.ex.launches()]
+    assert names.count("block_mma") == 1 and "depthwise" not in names, names
+    if case in ("pair", "stem_even", "stem_odd"):  # no conversion of the input
+        assert names[0] == "block_mma" and "pack" not in names
+    outs = run.run(xs)
+    assert run.guard_intact()
+    ref = og.run(spec, xs, storage="f16", fused=True)
+    for t in spec.outputs:
+        assert_close(outs[t], ref[t], api.GI_F16, case)
+    again = run.run(xs)
+    assert all(np.array_equal(outs[t], again[t]) for t in spec.outputs)
+
+
+@pytest.mark.parametrize("batch,size", [(1, 224), (8, 130), (21, 205)])
+def test_mobilenet_v2_launches_few_kernels(batch, size):
+    spec = wl.mobilenet_v2(batch, size=size)
+    run, xs, outs = check_outputs(spec, api.GI_F16, images=list(range(min(batch, 3))))
+    names = [api.KERNEL_NAMES[launch.kernel] for launch in run.ex.launches()]
+    assert names.count("block_mma") >= 10
+    other = DeviceRun(spec, api.GI_F16, cross_op=api.GI_XOP_OFF).run(xs)
+    for t in spec.outputs:
+        assert_close(outs[t], other[t], api.GI_F16, "one kernel per op")

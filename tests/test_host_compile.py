@@ -689,3 +689,39 @@ def test_slice8_host_side():
     assert L.gi_slice8_pointwise_run(16, 32, 256, 1, 2, 2, 8, 8, 7, None) == api.GI_E_INVALID   # unknown activation
     assert L.gi_slice8_pointwise_run(16, 40, 256, 1, 2, 2, 8, 8, 0, None) == api.GI_E_INVALID   # output not 16-byte aligned
     assert L.gi_slice8_pointwise_run(16, 32, 128, 1, 2, 2, 8, 8, 0, None) == api.GI_E_INVALID   # blob not 256-byte aligned
+
+
+# ---------------------------------------------------------------------- runs of ops that are launched as one kernel
+def test_grouped_launches_host_side():
+    """gi_exec_launch says what gi_run launches; gi_exec_op keeps describing the ops one by one, except under the naive plan.
+    A group and the ops after it cover the list without gaps; asking for one kernel per op gives one."""
+    spec = wl.mobilenet_v2(1)
+    for planner in (api.GI_PLAN_GREEDY_BY_SIZE, api.GI_PLAN_NAIVE, api.GI_PLAN_GREEDY_SHARED_OBJECTS, api.GI_PLAN_MIN_COST_FLOW):
+        ex = api.graph_from_spec(spec, api.GI_F16)[0].compile(planner=planner)
+        launches = ex.launches()
+        names = [api.KERNEL_NAMES[x.kernel] for x in launches]
+        assert names.count("block_mma") >= 10 and names[0] == "block_mma"
+        i = 0
+        while i < len(launches):
+            assert launches[i].n_ops >= 1 and launches[i].bytes > 0
+            i += launches[i].n_ops
+        assert i == ex.info.n_ops
+        ops = [api.KERNEL_NAMES[o.kernel] for o in ex.ops()]
+        assert ("block_mma" in ops) == (planner == api.GI_PLAN_NAIVE)
+    off = api.graph_from_spec(spec, api.GI_F16)[0].compile(cross_op=api.GI_XOP_OFF)
+    assert [x.kernel for x in off.launches()] == [o.kernel for o in off.ops()]
+    assert "block_mma" not in [api.KERNEL_NAMES[x.kernel] for x in off.launches()]
+    with pytest.raises(api.GiError):
+        off.launch(off.info.n_ops)
+    # a tensor that something else reads, or that the caller asked for, stays stored: no group around it
+    b = wl.GraphBuilder("hidden_is_an_output", 1, 16)
+    y = b.activation(b.depthwise(b.input(16, 16, 32), 3, 1), wl.ACT_RELU6)
+    b.output(y)
+    b.output(b.conv2d(y, 32, 1))
+    ex = api.graph_from_spec(b.finish(), api.GI_F16)[0].compile()
+    assert "block_mma" not in [api.KERNEL_NAMES[x.kernel] for x in ex.launches()]
+    # fp32 storage and an activation that does not clamp at zero: the ops' own kernels
+    pair = wl.depthwise_then_pointwise(1, 16, 16, 32, 32, dw_act=None)
+    for storage, s in ((api.GI_F32, wl.depthwise_then_pointwise(1, 16, 16, 32, 32)), (api.GI_F16, pair)):
+        ex = api.graph_from_spec(s, storage)[0].compile()
+        assert "block_mma" not in [api.KERNEL_NAMES[x.kernel] for x in ex.launches()]
