@@ -52,6 +52,7 @@ struct Epilogue {
 // Configuration of the kernel that runs a depthwise convolution and the convolutions around it (block_mma.cu), chosen at
 // compile time.
 enum BlockKind { BLOCK_EXPANSION = 0, BLOCK_PAIR = 1, BLOCK_STEM = 2 };
+constexpr int GROUP_RESIZE = 3;  // an up-sampling and the layout conversion behind it (OpGroup::kind, beside the block kinds)
 struct BlockCfg {
   int s = 1, first = 0;         // stride of the depthwise operator; how the operator in front of it is computed
   int np = 2, tr = 2, hc = 1;   // 16-channel output blocks, output rows per warp, 16-channel sub-blocks per chunk
@@ -104,7 +105,7 @@ struct LaunchRec {
   // depthwise 3x3 and the convolutions around it as one kernel: `ep` is the first operator's epilogue, `ep_mid` the depthwise
   // one's behind it, `ep2` the projection's; Cmid / Co2, stride, pads and (Ho, Wo) as above; (H, W) the depthwise input
   BlockCfg block;
-  int nhwc_out = 0;  // it writes the caller's NHWC output itself
+  int nhwc_out = 0;  // the kernel writes the caller's NHWC output itself
   int lead = -1, dw_op = -1;  // executed ops: the convolution in front of the depthwise one (or -1), the depthwise one
   int stem_h = 0, stem_w = 0, stem_pt = 0, stem_pl = 0;  // image and padding of a stem in front of the depthwise operator
 };

@@ -347,6 +347,16 @@ static LaunchRec block_rec(const gi_graph& g, const gi_exec* e, const BlockOps& 
   return r;
 }
 
+// Executed op `i` up-samples into a tensor that nothing but the conversion behind it reads: the kernel can write the caller's
+// NHWC tensor itself.
+static bool resize_then_unpack(const gi_exec* e, size_t i) {
+  const FusedOp& a = e->ops[i];
+  if (a.kind != GI_OP_RESIZE_BILINEAR || i + 1 >= e->ops.size()) return false;
+  const TensorDesc& d = e->tensors[a.out];
+  return e->ops[i + 1].kind == GI_EXEC_UNPACK && e->ops[i + 1].in0 == a.out && private_to_next(e, a.out, i) &&
+         static_cast<int64_t>(d.w) * d.c < (1LL << 30);
+}
+
 // Estimated time of the run's ops as launches of their own: 4 us each (what a launch adds to a chain of them) plus their bytes
 // at the rates the kernels reach inside MobileNetV2 - 6 TB/s, 3.2 for a stencil on planes without a straight-line form, 4 for
 // the stem - plus 4 ns per input channel of a 1x1 convolution (its chain of matrix instructions).  Against the measured
@@ -384,6 +394,16 @@ void find_groups(const gi_graph& g, gi_exec* e) {
   e->groups.clear();
   if (e->storage != GI_F16 || !e->opt.fuse || e->opt.cross_op != GI_XOP_AUTO || e->opt.pointwise != GI_PW_AUTO) return;
   for (size_t i = 0; i < e->ops.size(); ++i) {
+    if (e->opt.planner != GI_PLAN_NAIVE && resize_then_unpack(e, i)) {
+      // bit for bit the two ops: gi_exec_op and the naive plan need not know
+      OpGroup gr;
+      gr.first = static_cast<int>(i);
+      gr.n = 2;
+      gr.kind = GROUP_RESIZE;
+      e->groups.push_back(gr);
+      ++i;
+      continue;
+    }
     const BlockOps b = block_ops_at(g, e, i);
     if (b.n == 0) continue;
     OpGroup gr;
@@ -433,7 +453,23 @@ static gi_status lower_pass(const gi_graph& g, gi_exec* e, bool grouped, bool pa
     info.act_pre = f.act_pre;
     info.act_post = f.act_post;
     if (const OpGroup* gr = grouped ? group_of(e, i) : nullptr) {
-      if (static_cast<int>(i) == gr->first) {
+      if (gr->kind == GROUP_RESIZE && static_cast<int>(i) == gr->first) {
+        const TensorDesc &d = e->tensors[f.in0], &o = e->tensors[f.out];
+        r.kernel = GI_KERNEL_RESIZE;
+        r.B = e->batch;
+        r.H = d.h;
+        r.W = d.w;
+        r.C = d.c;
+        r.Ho = o.h;
+        r.Wo = o.w;
+        r.Co = o.c;
+        r.align_corners = g.ops[f.graph_op].d.align_corners;
+        r.nhwc_out = 1;
+        r.in0 = loc_of(e, f.in0);
+        r.out = Loc{W_OUTPUT, e->ops[i + 1].io_index, 0};
+        info.bytes = (B * d.h * d.w * slices(d.c) * 4 + B * o.h * o.w * o.c) * eb;
+        info.flops = 8 * B * o.h * o.w * o.c;
+      } else if (static_cast<int>(i) == gr->first) {
         r = gr->rec;
         const int lead = r.lead;
         const FusedOp& d = e->ops[r.dw_op];

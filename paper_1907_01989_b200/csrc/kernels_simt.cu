@@ -6,6 +6,9 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
+#include <type_traits>
+
 #include "kernels.h"
 #include "pdl.cuh"
 
@@ -522,6 +525,122 @@ __global__ void __launch_bounds__(128) resize_kernel(const T* __restrict__ in, T
   }
 }
 
+// The same straight into the caller's NHWC tensor (fp16).  A warp owns 28 neighbouring groups of four values of an output row
+// (group k: values 4k .. 4k + 3 of the row's OW * C), walks down the source rows [y_lo, y_hi), interpolates its groups along x
+// once per source row and stores them in every output row of that interval, 8 bytes per lane.  Rows start on any half, so the
+// groups stored start `s` values later, on a 32-byte boundary, with values of up to four lanes further on (hence 28): a warp
+// then writes whole sectors only.  513x513x21 x 16 images (177 MB): 49 + 88 us as two kernels, 67 us so (46 M warp
+// instructions, issue slots 60 % busy: bound by issue; 82 us with stores of two values on 4-byte boundaries and one source
+// row per warp).  Values are those of the two kernels one after the other.
+template <typename I>
+__global__ void __launch_bounds__(128) resize_nhwc_kernel(const __half* __restrict__ in, __half* __restrict__ out, int B, int C, int H, int W,
+                                                          int Pin, int OH, int OW, int ny, int dy, int nx, int dx, int y_step) {
+  pdl_launch_dependents();
+  pdl_wait();
+  const int b = blockIdx.z, lane = threadIdx.x & 31;
+  const int n = OW * C;                                                       // values of an output row
+  const int k = (blockIdx.x * 4 + (static_cast<int>(threadIdx.x) >> 5)) * 28 + lane;  // this lane's group
+  const int y_lo = blockIdx.y * y_step, y_hi = min(H, y_lo + y_step);
+  const bool inner = k - lane >= 4 && 4 * (k - lane + 32) + 16 <= n;  // no group of the warp meets an end of the row
+  const __half* p0[4];  // the group's source values in row 0: left neighbour, and how far the right one is
+  int right[4];
+  float wx[4];
+  int ox = 4 * k / C, c = 4 * k - ox * C;
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    const bool in_row = 4 * k + e < n;
+    const I qx = static_cast<I>(in_row ? ox : 0) * static_cast<I>(nx);
+    int x0 = static_cast<int>(qx / static_cast<I>(dx));
+    wx[e] = static_cast<float>(qx - static_cast<I>(x0) * static_cast<I>(dx)) / static_cast<float>(dx);
+    if (x0 > W - 1) {
+      x0 = W - 1;
+      wx[e] = 0.f;
+    }
+    right[e] = x0 + 1 < W ? 4 : 0;
+    const int ch = in_row ? c : 0;
+    p0[e] = in + (static_cast<size_t>(ch >> 2) * B + b) * Pin * 4 + (ch & 3) + x0 * 4;
+    if (++c == C) {
+      c = 0;
+      ++ox;
+    }
+  }
+  __half raw[4][2];  // of the row below the current one
+  float bot[4];
+  auto fetch = [&](int y) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const __half* p = p0[e] + static_cast<size_t>(y) * W * 4;
+      raw[e][0] = __ldg(p);
+      raw[e][1] = __ldg(p + right[e]);
+    }
+  };
+  auto along_x = [&]() {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const float l = __half2float(raw[e][0]), r = __half2float(raw[e][1]);
+      bot[e] = fmaf(r - l, wx[e], l);
+    }
+  };
+  fetch(y_lo);
+  along_x();
+  fetch(min(y_lo + 1, H - 1));
+  for (int y0 = y_lo; y0 < y_hi; ++y0) {
+    const float top[4] = {bot[0], bot[1], bot[2], bot[3]};
+    along_x();
+    const float dif[4] = {bot[0] - top[0], bot[1] - top[1], bot[2] - top[2], bot[3] - top[3]};
+    if (y0 + 1 < y_hi) fetch(min(y0 + 2, H - 1));
+    // output rows oy with floor(oy * ny / dy) == y0
+    int oy_lo = 0, oy_hi = y0 == 0 ? OH : 0;
+    if (ny != 0) {
+      oy_lo = static_cast<int>((static_cast<I>(y0) * static_cast<I>(dy) + static_cast<I>(ny - 1)) / static_cast<I>(ny));
+      const I hi = (static_cast<I>(y0 + 1) * static_cast<I>(dy) + static_cast<I>(ny - 1)) / static_cast<I>(ny);
+      oy_hi = hi > static_cast<I>(OH) ? OH : static_cast<int>(hi);
+    }
+    for (int base = oy_lo; base < oy_hi; base += 32) {
+      const int cnt = min(32, oy_hi - base);
+      const I py = static_cast<I>(base + lane) * static_cast<I>(ny);
+      const float wy_lane = static_cast<float>(py - static_cast<I>(y0) * static_cast<I>(dy)) / static_cast<float>(dy);
+      const size_t first = (static_cast<size_t>(b) * OH + base) * n;  // the row's first value
+      __half* row = out + first + 4 * k;
+      unsigned s = static_cast<unsigned>(-static_cast<long long>(first)) & 15u;  // values before the row's first 32-byte boundary
+      auto rows = [&](auto edge) {
+#pragma unroll 2
+        for (int r = 0; r < cnt; ++r, row += n, s = (s - static_cast<unsigned>(n)) & 15u) {
+          const float wy = __shfl_sync(0xffffffffu, wy_lane, r);
+          const __half2 h0 = __floats2half2_rn(fmaf(dif[0], wy, top[0]), fmaf(dif[1], wy, top[1]));
+          const __half2 h1 = __floats2half2_rn(fmaf(dif[2], wy, top[2]), fmaf(dif[3], wy, top[3]));
+          const unsigned o0 = *reinterpret_cast<const unsigned*>(&h0), o1 = *reinterpret_cast<const unsigned*>(&h1);
+          const unsigned d = s >> 2;
+          const unsigned q0 = __shfl_down_sync(0xffffffffu, o0, d), q1 = __shfl_down_sync(0xffffffffu, o1, d);
+          const unsigned n0 = __shfl_down_sync(0xffffffffu, o0, d + 1), n1 = __shfl_down_sync(0xffffffffu, o1, d + 1);
+          const unsigned a0 = s & 2 ? q1 : q0, a1 = s & 2 ? n0 : q1, a2 = s & 2 ? n1 : n0, sh = (s & 1) * 16;
+          const unsigned w0 = __funnelshift_r(a0, a1, sh), w1 = __funnelshift_r(a1, a2, sh);
+          if (lane >= 28) continue;
+          unsigned short* at = reinterpret_cast<unsigned short*>(row + s);
+          const int left = decltype(edge)::value ? n - 4 * k - static_cast<int>(s) : 4;  // values of the row from this group on
+          if (left >= 4) {
+            *reinterpret_cast<uint2*>(at) = make_uint2(w0, w1);
+          } else if (left > 0) {
+            at[0] = static_cast<unsigned short>(w0);
+            if (left > 1) at[1] = static_cast<unsigned short>(w0 >> 16);
+            if (left > 2) at[2] = static_cast<unsigned short>(w1);
+          }
+          if (decltype(edge)::value && 4 * k < static_cast<int>(s)) {  // values before the first boundary
+            unsigned short* f = reinterpret_cast<unsigned short*>(row);
+            const int head = min(static_cast<int>(s), n) - 4 * k;
+            if (head > 0) f[0] = static_cast<unsigned short>(o0);
+            if (head > 1) f[1] = static_cast<unsigned short>(o0 >> 16);
+            if (head > 2) f[2] = static_cast<unsigned short>(o1);
+            if (head > 3) f[3] = static_cast<unsigned short>(o1 >> 16);
+          }
+        }
+      };
+      if (inner) rows(std::false_type{});
+      else rows(std::true_type{});
+    }
+  }
+}
+
 ConvGeom geom(const LaunchRec& r) {
   ConvGeom g;
   g.B = r.B;
@@ -690,9 +809,20 @@ int launch_resize(const LaunchRec& r, const Ptrs& p, int storage, void* stream) 
   }
   const int Pout = plane_pixels(r.Ho, r.Wo), Pin = plane_pixels(r.H, r.W);
   if (r.H > 65535 || r.B > 65535) return static_cast<int>(cudaErrorInvalidConfiguration);
-  const dim3 grid(blocks_for(r.Wo, 128), r.H, r.B);
   const bool narrow = (static_cast<long long>(r.Ho) + 1) * ny + static_cast<long long>(r.H + 1) * dy < (1LL << 31) &&
                       static_cast<long long>(r.Wo) * nx < (1LL << 31);
+  if (r.nhwc_out) {
+    const unsigned gx = blocks_for((static_cast<size_t>(r.Wo) * r.C + 3) / 4, 4 * 28);
+    // source rows per warp: as many as leave three waves of the eight CTAs an SM holds (1200 CTAs, one wave and a bit: 104 us)
+    const int y_step = static_cast<int>(std::max<long long>(1, std::min<long long>(8, static_cast<long long>(gx) * r.H * r.B / (148 * 24))));
+    const dim3 grid(gx, blocks_for(r.H, y_step), r.B);
+    const __half* in = static_cast<const __half*>(p.in0);
+    __half* out = static_cast<__half*>(p.out);
+    launch_pdl(narrow ? resize_nhwc_kernel<unsigned> : resize_nhwc_kernel<unsigned long long>, grid, 128, 0, st, in, out, r.B, r.C, r.H, r.W, Pin,
+               r.Ho, r.Wo, ny, dy, nx, dx, y_step);
+    return static_cast<int>(cudaGetLastError());
+  }
+  const dim3 grid(blocks_for(r.Wo, 128), r.H, r.B);
 #define GI_RESIZE(T, I)                                                                                                       \
   launch_pdl(resize_kernel<T, I>, grid, 128, 0, st, static_cast<const T*>(p.in0), static_cast<T*>(p.out), r.B, slices(r.C), r.H, r.W, \
              Pin, r.Ho, r.Wo, Pout, ny, dy, nx, dx)

@@ -993,3 +993,20 @@ def test_mobilenet_v2_launches_few_kernels(batch, size):
     other = DeviceRun(spec, api.GI_F16, cross_op=api.GI_XOP_OFF).run(xs)
     for t in spec.outputs:
         assert_close(outs[t], other[t], api.GI_F16, "one kernel per op")
+
+
+@pytest.mark.parametrize("case", [(9, 7, 70, 51, 5, True), (3, 3, 33, 33, 21, True), (5, 4, 9, 9, 3, False), (4, 6, 40, 16, 8, True), (8, 8, 3, 5, 1, False)])
+def test_resize_into_the_callers_layout(case):
+    """Up-sampling that writes the caller's NHWC tensor (odd rows start on an odd half) gives the bits of the two ops."""
+    h, w, oh, ow, c, align = case
+    b = wl.GraphBuilder("resize_out", 3, 17)
+    b.output(b.resize_bilinear(b.conv2d(b.input(h, w, 8), c, 1), oh, ow, align))
+    spec = b.finish()
+    run, xs, outs = check_outputs(spec, api.GI_F16)
+    names = [api.KERNEL_NAMES[launch.kernel] for launch in run.ex.launches()]
+    assert names[-2:] == ["resize", "none"], names
+    two = DeviceRun(spec, api.GI_F16, cross_op=api.GI_XOP_OFF)
+    assert api.KERNEL_NAMES[two.ex.launches()[-1].kernel] == "unpack"
+    other = two.run(xs)
+    for t in spec.outputs:
+        assert np.array_equal(outs[t], other[t])
