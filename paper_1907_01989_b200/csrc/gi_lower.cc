@@ -359,7 +359,7 @@ static bool resize_then_unpack(const gi_exec* e, size_t i) {
 
 // Estimated time of the run's ops as launches of their own: 4 us each (what a launch adds to a chain of them) plus their bytes
 // at the rates the kernels reach inside MobileNetV2 - 6 TB/s, 3.2 for a stencil on planes without a straight-line form, 4 for
-// the stem - plus 4 ns per input channel of a 1x1 convolution (its chain of matrix instructions).  Against the measured
+// the stem - plus 4 ns (1.2 ns where eight warps share the sum) per input channel of a 1x1 convolution, its chain of matrix instructions.  Against the measured
 // times of the network's ops at batch 1, 21 and 256 it is within 15 %.
 static double separate_us(const gi_exec* e, const OpGroup& gr) {
   double us = 0.0;
@@ -376,8 +376,13 @@ static double separate_us(const gi_exec* e, const OpGroup& gr) {
       if (gr.rec.lead >= 0 && gr.rec.stem_h > 0 && conv3x3_tc_reads_nhwc(d.c, d.h, d.w, 2, 1, gr.rec.stem_pt, gr.rec.stem_pl)) continue;
     }
     if (o.kind == GI_OP_CONV2D) {
+      LaunchRec pw;
+      pw.B = e->batch;
+      pw.H = e->tensors[o.in0].h;
+      pw.W = e->tensors[o.in0].w;
+      pw.Co = e->tensors[o.out].c;
       if (gr.rec.stem_h > 0 && i == gr.rec.lead) rate = 4.0e6;
-      else us += 0.004 * e->tensors[o.in0].c;
+      else us += (pointwise_mma_wanted(pw) ? 0.0012 : 0.004) * e->tensors[o.in0].c;
     }
     if (o.kind == GI_OP_DEPTHWISE_CONV2D) {
       const int w = e->tensors[o.out].w;
@@ -439,6 +444,7 @@ static const OpGroup* group_of(const gi_exec* e, size_t i) {
 static gi_status lower_pass(const gi_graph& g, gi_exec* e, bool grouped, bool pack) {
   const int eb = elem_bytes(e->storage);
   const uint64_t B = static_cast<uint64_t>(e->batch);
+  bool unpack_done = false;  // the next op, a layout conversion, runs inside the kernel of the op before it
   int absorbed = 0;  // this many following ops run inside the kernel of an op already lowered
   for (size_t i = 0; i < e->ops.size(); ++i) {
     const FusedOp& f = e->ops[i];
@@ -533,6 +539,11 @@ static gi_status lower_pass(const gi_graph& g, gi_exec* e, bool grouped, bool pa
         r.kernel = GI_KERNEL_UNPACK;
         r.out = Loc{W_OUTPUT, f.io_index, 0};
         info.bytes = in_px * in_c4 * eb + in_px * din->c * eb;
+        if (unpack_done) {
+          r.kernel = GI_KERNEL_NONE;
+          info.bytes = 0;
+          unpack_done = false;
+        }
         break;
       }
       case GI_OP_CONV2D:
@@ -606,6 +617,8 @@ static gi_status lower_pass(const gi_graph& g, gi_exec* e, bool grouped, bool pa
           const bool pointwise = op.d.kh == 1 && op.d.stride_h == 1 && op.d.stride_w == 1 && op.d.pad_t == 0 &&
                                  op.d.pad_l == 0 && op.d.pad_b == 0 && op.d.pad_r == 0;
           const bool tc = e->storage == GI_F16 && e->opt.pointwise != GI_PW_SIMT;
+          const bool unpack_next = grouped && e->opt.planner != GI_PLAN_NAIVE && i + 1 < e->ops.size() &&
+                                   e->ops[i + 1].kind == GI_EXEC_UNPACK && e->ops[i + 1].in0 == f.out && private_to_next(e, f.out, i);
           // Which tensor-core kernel: a rule distilled from measurements of the kernels on every 1x1 shape of
           // the benchmark networks (single launches whose input was written just before, as a producing kernel
           // leaves it, and confirmed inside the networks).  The lane-per-pixel kernel (dense weights, activations
@@ -717,7 +730,16 @@ static gi_status lower_pass(const gi_graph& g, gi_exec* e, bool grouped, bool pa
               pair_tab = lc->kernel == GI_KERNEL_POINTWISE_TC;
             }
           }
-          if (pointwise && tc && wide_kernel && pointwise_mm_supported(din->c, op.d.cout)) {
+          if (grouped && pointwise && tc && e->opt.fuse && e->opt.pointwise == GI_PW_AUTO && e->opt.cross_op == GI_XOP_AUTO &&
+              pointwise_mma_wanted(r)) {
+            r.kernel = GI_KERNEL_POINTWISE_MMA;
+            if (unpack_next) {
+              r.nhwc_out = 1;
+              r.out = Loc{W_OUTPUT, e->ops[i + 1].io_index, 0};
+              unpack_done = true;
+            }
+            if (pack) pointwise_mma_pack(op.weights.data(), op.bias.data(), din->c, op.d.cout, &e->weight_blob, &r);
+          } else if (pointwise && tc && wide_kernel && pointwise_mm_supported(din->c, op.d.cout)) {
             r.kernel = GI_KERNEL_POINTWISE_MM;
             if (pack) pointwise_mm_pack(op.weights.data(), op.bias.data(), din->c, op.d.cout, &e->weight_blob, &r);
           } else if (pointwise && tc && (lane_tab || (lane_kernel && !pair_tab)) && pointwise_ts_supported(din->c, op.d.cout)) {
@@ -812,7 +834,7 @@ static gi_status lower_pass(const gi_graph& g, gi_exec* e, bool grouped, bool pa
 // stored tensor after a run, gi_exec_op says what is launched: a tensor between the ops of a launch is not stored.
 gi_status lower(const gi_graph& g, gi_exec* e) {
   std::vector<gi_op_info> one_by_one;
-  if (!e->groups.empty() && e->opt.planner != GI_PLAN_NAIVE) {
+  if (e->opt.planner != GI_PLAN_NAIVE) {
     std::vector<uint64_t> run_offset;
     run_offset.swap(e->run_offset);  // ops one by one: where the plan put the tensors
     const gi_status s = lower_pass(g, e, false, false);

@@ -110,4 +110,10 @@ void block_mma_pack(const float* we, const float* be, const float* wd, const flo
                     int chid, int cout, const BlockCfg& c, std::vector<uint8_t>* blob, LaunchRec* r);
 int launch_block_mma(const LaunchRec& r, const Ptrs& p, void* stream);
 
+// Pointwise convolution for launches bound by latency (fp16 storage; pointwise_mma.cu)
+bool pointwise_mma_wanted(const LaunchRec& r);
+void pointwise_mma_pack(const float* w, const float* bias, int cin, int cout, std::vector<uint8_t>* blob, LaunchRec* r);
+int launch_pointwise_mma(const LaunchRec& r, const Ptrs& p, void** state, int launch_index, void* stream);
+unsigned int pointwise_mma_error_word(int* cuda_err);
+
 }  // namespace gi

@@ -1010,3 +1010,26 @@ def test_resize_into_the_callers_layout(case):
     other = two.run(xs)
     for t in spec.outputs:
         assert np.array_equal(outs[t], other[t])
+
+
+# (batch, plane, cin, cout, residual): one tile and less, remainders of every tile edge, more stages than shared memory holds
+# (1600 channels), single pixels (stored as two), odd planes into the caller's NHWC, the most tiles the kernel is taken for
+@pytest.mark.parametrize("case", [(1, 2, 4, 4, False), (3, 5, 37, 21, False), (2, 9, 20, 43, True), (5, 1, 1280, 1001, False), (64, 1, 64, 10, False),
+                                  (1, 7, 1600, 40, False), (4, 7, 129, 64, True), (37, 8, 16, 100, False), (2, 31, 136, 126, False)])
+def test_pointwise_of_few_tiles(case):
+    """1x1 convolutions whose 32 x 32 tiles fit on the chip at once, the conversion to the caller's layout included, against the
+    oracle, and against the one-op-per-kernel path within the same tolerance; bit-identical from run to run."""
+    batch, hw, cin, cout, residual = case
+    spec = wl.single_pointwise(batch, hw, cin, cout, residual, wl.ACT_RELU6 if hw > 2 else wl.ACT_NONE)
+    xs = [wl.make_input(spec, index=i) for i in range(len(spec.inputs))]
+    run = DeviceRun(spec, api.GI_F16, guard_bytes=4096)
+    names = [api.KERNEL_NAMES[launch.kernel] for launch in run.ex.launches()]
+    assert names[-2:] == ["pointwise_mma", "none"], names
+    outs = run.run(xs)
+    assert run.guard_intact()
+    ref = og.run(spec, xs, storage="f16", fused=True)
+    for t in spec.outputs:
+        assert_close(outs[t], ref[t], api.GI_F16, str(case))
+    again = run.run(xs)
+    assert all(np.array_equal(outs[t], again[t]) for t in spec.outputs)
+    assert api.gi_device_status() == 0
