@@ -23,17 +23,24 @@
 // permuted to match when the weights are packed.
 //
 // Walk.  A unit is a tile of output pixels of one image (or whole small images); its CTA - or cluster of CTAs, each taking
-// every ks-th chunk of the hidden channels, their partial sums added in rank order through distributed shared memory - walks
-// the hidden channels in chunks of 16 or 32: the first operator of chunk c+1 into one of two hidden tiles while the depthwise
+// every ks-th chunk of the hidden channels, their partial sums stored into the shared memory of the CTA that adds them up, in
+// rank order - walks the hidden channels in chunks of 16 or 32: the first operator of chunk c+1 into one of two hidden tiles while the depthwise
 // operator and the projection consume chunk c from the other; one barrier per chunk.  Weights arrive by cp.async, resident
 // when they fit, else through a ring of four chunks; they are requested before the previous kernel has finished.
 //
-// What bounds it.  Small launches: the chain of one unit (4.5 us for a pair, 6 to 10 us for a block at batch 1, against 4 us
-// for each of the two to four launches it replaces).  Large ones: nothing alone - on 56x56 24 -> 144 -> 24 at batch 256 a
+// Small launches.  Where there are fewer units than SMs the chain of one unit is what a launch takes: up to 16 sets of warps
+// then share a chunk, 16 hidden channels each (BlockCfg::wk), so that a warp's chain is one or two first operators, depthwise
+// slices and projections; where its pixels lie is worked out before the previous kernel has finished, only the copies are
+// issued behind it.  Of 8.3 us for 14x14 64 -> 384 -> 64 at batch 1 with a cluster alone, 0.9 were the addresses, 3.3 the three
+// chunks, 0.8 the cluster barrier and 3.0 reading the neighbours' sums one round trip after the other; sets of warps and
+// pushed sums: 7.7 against 10.5 us a launch, 7x7 160 -> 960 -> 160 10.3 against 19.  MobileNetV2 batch 1 169 -> 160 us, 8 x
+// 192 207 -> 186, segmentation batch 1 229 -> 211.
+//
+// What bounds it.  Small launches: that chain.  Large ones: nothing alone - on 56x56 24 -> 144 -> 24 at batch 256 a
 // chunk takes 1840 cycles of an SM for 800 of the matrix pipe, 770 of issue slots per scheduler and about 900 of shared
 // memory, with 16 warps to cover 21-cycle matrix and 30-cycle shared-memory latencies; 173 us against 194 us as three
-// kernels.  Measured on one B200, MobileNetV2: batch 1 225 -> 197 us, 21 images of 205 pixels 340 -> 288, batch 256 1413 ->
-// 1385; segmentation network batch 1 289 -> 246, batch 16 961 -> 874.
+// kernels.  Measured on one B200 against separate kernels, MobileNetV2: batch 1 225 -> 160 us, 21 images of 205
+// pixels 340 -> 278, batch 256 1413 -> 1385; segmentation network batch 1 289 -> 211, batch 16 961 -> 807.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
@@ -65,8 +72,8 @@ enum First { kNone = 0, kExp16 = 1, kExp24 = 2, kExp32 = 3, kExpWide = 4, kStem 
 
 // Bytes between the slices of a hidden tile: a constant, so that slices are immediate offsets.  32 modulo 128: the stores
 // of 4 pixels x 4 slices by half a warp meet 32 different banks.
-__host__ __device__ constexpr int slice_bytes(int first) { return first == kExpWide ? 18 * 128 + 32 : 36 * 128 + 32; }
-__host__ __device__ constexpr int tile_pixels(int first) { return slice_bytes(first) / 8 - 2; }
+__host__ __device__ constexpr int slice_bytes(int first, bool small) { return (small ? 9 : first == kExpWide ? 18 : 36) * 128 + 32; }
+__host__ __device__ constexpr int tile_pixels(int first, bool small) { return slice_bytes(first, small) / 8 - 2; }
 // warps an SM holds: 128 registers a thread for 16 warps, 255 for 8 (96 sums per thread and more; tr: output rows a warp
 // walks down)
 __host__ __device__ constexpr int max_warps(int s, int np, int tr) { return (s == 1 ? tr : 1) * np >= 6 || tr == 4 ? 8 : 16; }
@@ -96,9 +103,10 @@ struct BlockParams {
   int pw, ncols, ngroups;   // columns per band; columns and groups of 16 columns of a unit
   int eg, en;               // groups of 16 list pixels for a warp with / without a column group
   int nch, ks;              // chunks of hidden channels; CTAs sharing a unit
+  int wk, nwq;              // sets of warps that share a chunk's channels; warps of a set
   int resident;
   unsigned x_pitch;
-  unsigned off_bias, off_tab, off_x, off_raw, off_hid, off_red;
+  unsigned off_bias, off_tab, off_src, off_x, off_raw, off_hid, off_red;
   unsigned x_bytes, tab_bytes;  // of one of the two input tiles / tables (narrow expansions; otherwise there is one)
   unsigned mul_pitch, mul_w, mul_hw, mul_per, mul_tx;  // ceil(2^32 / d): division of a small number by d is one high multiplication
   unsigned hi_e, hi_d;  // upper clamp of the hidden activations, two halves (6 or infinity)
@@ -168,10 +176,8 @@ __device__ __forceinline__ void sts64(unsigned addr, unsigned a, unsigned b) {
 __device__ __forceinline__ void sts128(unsigned addr, unsigned a, unsigned b, unsigned c, unsigned d) {
   asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
-__device__ __forceinline__ float4 ld_cluster_f4(unsigned addr) {
-  float4 v;
-  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
-  return v;
+__device__ __forceinline__ void st_cluster_f4(unsigned addr, float a, float b, float c, float d) {
+  asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
 }
 __device__ __forceinline__ unsigned min_f16x2(unsigned a, unsigned b) {
   unsigned d;
@@ -348,19 +354,22 @@ __device__ __forceinline__ void store_col(const BlockParams& p, const UnitPos& u
 }
 
 // S: stride.  NP: 16-channel blocks of the output.  TR: output rows a warp walks down.  HC: 16-channel sub-blocks per chunk.
-template <int S, int FIRST, int NP, int TR, int HC>
+// SMALL: tiles of at most 146 list pixels, whose chunks several sets of warps share.
+template <int S, int FIRST, int NP, int TR, int HC, bool SMALL>
 __global__ void __launch_bounds__(32 * max_warps(S, NP, TR), 1) block_mma_kernel(const BlockParams p) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   const unsigned smem = smem_u32(smem_raw);
   const int tid = threadIdx.x, nthr = blockDim.x;
   const int warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
   constexpr bool kHasFirst = FIRST != kNone, kWideExp = FIRST == kExpWide;
-  constexpr int SL = slice_bytes(FIRST);
-  constexpr int kHidBytes = HC * 4 * SL;
+  constexpr int SL = slice_bytes(FIRST, SMALL);
+  constexpr int kSetBytes = HC * 4 * SL;
+  const int wk = SMALL ? p.wk : 1, wset = SMALL ? warp / p.nwq : 0, wq = SMALL ? warp - wset * p.nwq : warp;
+  const int hid_bytes = wk * kSetBytes;
   constexpr int NV = S == 1 ? TR : TR / 2;  // fragments of sums down a column: rows, or pairs of rows
   const int ke = kWideExp ? p.ke : FIRST == kNone ? 0 : FIRST == kExp16 ? 1 : 2;
   const int subb = ke * 512 + kSubFixed + NP * 512;
-  const int stage_bytes = HC * subb;
+  const int stage_bytes = wk * HC * subb;
   const int rank = p.ks > 1 ? static_cast<int>(cluster_ctarank()) : 0;
   const int unit0 = blockIdx.x / p.ks, ustep = gridDim.x / p.ks;
   const int nchl = (p.nch - rank + p.ks - 1) / p.ks;  // chunks of this CTA: rank, rank + ks, ...
@@ -386,8 +395,6 @@ __global__ void __launch_bounds__(32 * max_warps(S, NP, TR), 1) block_mma_kernel
     for (unsigned i = p.off_x + tid * 16; i < p.off_red; i += nthr * 16) sts128(smem + i, 0u, 0u, 0u, 0u);
   }
   for (int i = tid; i < NP * 4; i += nthr) cp_async16(smem + p.off_bias + i * 16, reinterpret_cast<const float4*>(p.bias) + i);
-  __syncthreads();
-  pdl_wait();
 
   const unsigned tab0 = smem + p.off_tab, xs0 = smem + p.off_x, raw = smem + p.off_raw, hid0 = smem + p.off_hid, red = smem + p.off_red;
   constexpr bool kTwoX = kHasFirst && !kWideExp && FIRST != kStem;  // the next unit's input arrives during this one
@@ -419,6 +426,28 @@ __global__ void __launch_bounds__(32 * max_warps(S, NP, TR), 1) block_mma_kernel
       else sts32(tab + i * 4, in ? p.hi_e : 0u);
     }
   };
+  // small tiles: the first unit's input in two steps: where its pixels lie is found out before the previous kernel has finished
+  auto find_x = [&](const UnitPos& u) {
+    for (int i = tid; i < p.mt * 16; i += nthr) {
+      const bool listed = i < p.n_list;
+      const ListPx l = list_pixel(p, u, S, listed ? i : 0);
+      const bool in = listed && l.in;
+      sts32(smem + p.off_src + i * 4, static_cast<unsigned>(in ? (u.img0 + l.im) * p.in_img + (l.y * p.W + l.x) * p.in_px : -1));
+      if (kWideExp) sts64(tab0 + i * 8, static_cast<unsigned>(listed ? l.hid : p.ni * p.sub_px) * 8u, in ? p.hi_e : 0u);
+      else sts32(tab0 + i * 4, in ? p.hi_e : 0u);
+    }
+  };
+  auto copy_x = [&]() {
+    const int px = p.n_list, parts = max(1, nthr / px), part = nthr >= 2 * px ? tid / px : 0;
+    if (part >= parts) return;
+    for (int i = tid - part * px; i < px; i += nthr) {
+      const int at = static_cast<int>(lds32(smem + p.off_src + i * 4));
+      const unsigned n = at >= 0 ? 8u : 0u, dst = xs0 + i * p.x_pitch;
+      const __half* src = p.in + max(at, 0);
+#pragma unroll 4
+      for (int s = part; s < p.sin; s += parts) cp_async8(dst + s * 8, at >= 0 ? src + s * p.in_sl : p.in, n);
+    }
+  };
   // no first operator: a chunk of the input goes straight into a hidden tile (a ring of them)
   auto load_hidden = [&](int run) {
     const int k = run / nchl, c = run - k * nchl, chunk = rank + c * p.ks;
@@ -429,13 +458,14 @@ __global__ void __launch_bounds__(32 * max_warps(S, NP, TR), 1) block_mma_kernel
         sts32(tab0 + i * 4, static_cast<unsigned>(l.in ? (u.img0 + l.im) * p.in_img + (l.y * p.W + l.x) * p.in_px : -1));
       }
     }
-    unsigned dst = hid0 + (run & (kRing - 1)) * kHidBytes + tid * 8;
-    const int s0 = chunk * HC * 4, ns = p.sin - s0;  // slices beyond the last one are zeros: their weights are, too
+    unsigned dst = hid0 + (run & (kRing - 1)) * hid_bytes + tid * 8;
+    const int s0 = chunk * wk * HC * 4, ns = p.sin - s0;  // slices beyond the last one are zeros: their weights are, too
     for (int i = tid; i < p.n_list; i += nthr, dst += nthr * 8) {
       const int at = static_cast<int>(lds32(tab0 + i * 4));
       const __half* src = p.in + (at < 0 ? 0 : at) + s0 * p.in_sl;
+      for (int w = 0; w < wk * HC * 4; w += HC * 4)
 #pragma unroll
-      for (int s = 0; s < HC * 4; ++s, src += p.in_sl) cp_async8(dst + s * SL, s < ns ? src : p.in, s < ns && at >= 0 ? 8u : 0u);
+        for (int s = w; s < w + HC * 4; ++s, src += p.in_sl) cp_async8(dst + s * SL, s < ns ? src : p.in, s < ns && at >= 0 ? 8u : 0u);
     }
   };
   // stem: the rows of the image under the unit's hidden tile, as 4-byte words from the aligned word that holds a row's first
@@ -497,11 +527,15 @@ __global__ void __launch_bounds__(32 * max_warps(S, NP, TR), 1) block_mma_kernel
       for (int q = 0; q < 4; ++q) sts128(xs0 + i * 80 + q * 16, o[q * 4], o[q * 4 + 1], o[q * 4 + 2], o[q * 4 + 3]);
     }
   };
+  if (SMALL && kHasFirst) find_x(unit_pos(p, unit0, th_rows));
+  __syncthreads();
+  pdl_wait();
   if (my_units > 0) {
     if (FIRST == kStem) {
       load_raw(unit_pos(p, unit0, th_rows));
     } else if (kHasFirst) {
-      load_x(unit_pos(p, unit0, th_rows), 0);
+      if (SMALL) copy_x();
+      else load_x(unit_pos(p, unit0, th_rows), 0);
     } else {
       load_hidden(0);
       cp_async_commit();
@@ -514,13 +548,13 @@ __global__ void __launch_bounds__(32 * max_warps(S, NP, TR), 1) block_mma_kernel
   unsigned dw_base;
   const unsigned row_b = p.pitch * 8;
   {
-    int col = warp * 16 + (lane & 15);
+    int col = wq * 16 + (lane & 15);
     if (col >= p.ncols) col = 0;
     int im, band, pos;
     column_pos(p, col, im, band, pos);
     dw_base = static_cast<unsigned>(im * p.sub_px + band * TR * S * p.pitch) * 8u + pos * 16u + (lane >> 4) * 16u;
   }
-  const unsigned col0 = lane_col(p, S, TR, warp * 16 + g), col1 = lane_col(p, S, TR, warp * 16 + g + 8);
+  const unsigned col0 = lane_col(p, S, TR, wq * 16 + g), col1 = lane_col(p, S, TR, wq * 16 + g + 8);
   const bool band_lane = (g >> 2) == (t & 1);
   const unsigned sel_a = !band_lane ? 0x4444u : ((g >> 1) & 1) ? 0x1044u : 0x4410u;
   const unsigned sel_b = !band_lane ? 0x4444u : ((g >> 1) & 1) ? 0x3244u : 0x4432u;
@@ -528,9 +562,9 @@ __global__ void __launch_bounds__(32 * max_warps(S, NP, TR), 1) block_mma_kernel
   const unsigned sel_a0 = odd ? 0x4444u : sel_a, sel_b0 = odd ? 0x4444u : sel_b;  // window rows of the first output row only
   const unsigned sel_a1 = odd ? sel_a : 0x4444u, sel_b1 = odd ? sel_b : 0x4444u;  // ... of the second only
   const unsigned dw_entry = ((t >> 1) * 8 + g) * 16;
-  const bool has_group = warp < p.ngroups;
+  const bool has_group = wq < p.ngroups;
   // this warp's groups of 16 list pixels
-  const int mt0 = has_group ? warp * p.eg : p.ngroups * p.eg + (warp - p.ngroups) * p.en;
+  const int mt0 = has_group ? wq * p.eg : p.ngroups * p.eg + (wq - p.ngroups) * p.en;
   const int mt1 = min(p.mt, mt0 + (has_group ? p.eg : p.en));
 
   if (kHasFirst) cp_async_wait<0>();
@@ -548,7 +582,7 @@ __global__ void __launch_bounds__(32 * max_warps(S, NP, TR), 1) block_mma_kernel
     float acc[NV][NP][2][2][4];  // sums start at the bias (a cluster's: in its first CTA)
 #pragma unroll
     for (int j = 0; j < NP; ++j) {
-      const uint4 q = rank ? make_uint4(0u, 0u, 0u, 0u) : lds128(smem + p.off_bias + (4 * j + t) * 16);
+      const uint4 q = rank || wset ? make_uint4(0u, 0u, 0u, 0u) : lds128(smem + p.off_bias + (4 * j + t) * 16);
 #pragma unroll
       for (int v = 0; v < NV; ++v)
 #pragma unroll
@@ -582,8 +616,8 @@ __global__ void __launch_bounds__(32 * max_warps(S, NP, TR), 1) block_mma_kernel
       // ---- first operator of chunk `it`
       if (kHasFirst && it < nchl && mt0 < mt1) {
         const int r = run + it;
-        const unsigned ws = smem + (p.resident ? it : r & (kRing - 1)) * stage_bytes;
-        const unsigned hb = hid0 + (r & 1) * kHidBytes + t * SL;
+        const unsigned ws = smem + (p.resident ? it : r & (kRing - 1)) * stage_bytes + wset * HC * subb;
+        const unsigned hb = hid0 + (r & 1) * hid_bytes + wset * kSetBytes + t * SL;
         if (!kWideExp) {
           const uint4 b0 = lds128(ws + lane * 16);
           const uint4 b1 = FIRST == kExp16 ? b0 : lds128(ws + 512 + lane * 16);
@@ -695,8 +729,8 @@ __global__ void __launch_bounds__(32 * max_warps(S, NP, TR), 1) block_mma_kernel
       const int dc = kHasFirst ? it - 1 : it;
       if (dc >= 0 && has_group) {
         const int r = run + dc;
-        const unsigned ws = smem + (p.resident ? dc : r & (kRing - 1)) * stage_bytes;
-        const unsigned hb = hid0 + (kHasFirst ? (r & 1) : (r & (kRing - 1))) * kHidBytes + dw_base;
+        const unsigned ws = smem + (p.resident ? dc : r & (kRing - 1)) * stage_bytes + wset * HC * subb;
+        const unsigned hb = hid0 + (kHasFirst ? (r & 1) : (r & (kRing - 1))) * hid_bytes + wset * kSetBytes + dw_base;
         constexpr int kRows = S == 1 ? TR + 2 : 2 * TR + 1;  // hidden rows under the column
         unsigned rb[kRows];
 #pragma unroll
@@ -769,48 +803,59 @@ __global__ void __launch_bounds__(32 * max_warps(S, NP, TR), 1) block_mma_kernel
     }
 
     const UnitPos u = unit_pos(p, unit, th_rows);
-    if (p.ks == 1) {
+    if (p.ks * wk == 1) {
       if (has_group) {
         store_col<S, 0, NV, NP>(p, u, xs, col0, 0, 0, t, acc);
         store_col<S, 1, NV, NP>(p, u, xs, col1, 0, 0, t, acc);
       }
     } else {
-      // partial sums of the cluster's CTAs: every CTA leaves its own in shared memory and adds up its share of the tiles
-      // over the ranks, in rank order
+      // partial sums of the cluster's CTAs and of the warp sets: every tile of 16 columns x 16 channels has an owner, the CTA
+      // tile % ks; everybody stores into the owner's shared memory, which then adds up its tiles in the order of the sources.
+      // (Reading the neighbours' shared memory instead took 2.5 us: eight round trips, one after the other.)
+      const int src = rank * wk + wset, n_src = p.ks * wk;
       if (has_group) {
 #pragma unroll
         for (int v = 0; v < NV; ++v)
 #pragma unroll
           for (int j = 0; j < NP; ++j) {
-            const unsigned at = red + ((warp * NV + v) * NP + j) * 2048 + lane * 16;
+            const int ti = (wq * NV + v) * NP + j, slot = ti / p.ks;
+            unsigned at = red + (slot * n_src + src) * 2048 + lane * 16;
+            if (p.ks > 1) at = mapa_shared(at, ti - slot * p.ks);
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
-              sts128(at + i * 512, __float_as_uint(acc[v][j][i >> 1][i & 1][0]), __float_as_uint(acc[v][j][i >> 1][i & 1][1]),
-                     __float_as_uint(acc[v][j][i >> 1][i & 1][2]), __float_as_uint(acc[v][j][i >> 1][i & 1][3]));
+            for (int i = 0; i < 4; ++i) {
+              const float(&f)[4] = acc[v][j][i >> 1][i & 1];
+              if (p.ks > 1) st_cluster_f4(at + i * 512, f[0], f[1], f[2], f[3]);
+              else sts128(at + i * 512, __float_as_uint(f[0]), __float_as_uint(f[1]), __float_as_uint(f[2]), __float_as_uint(f[3]));
+            }
           }
       }
-      cluster_sync();
+      if (p.ks > 1) cluster_sync();
+      else __syncthreads();
       const int tiles = p.ngroups * NV * NP;
-      for (int ti = warp * p.ks + rank; ti < tiles; ti += (nthr >> 5) * p.ks) {
+      for (int slot = warp; slot * p.ks + rank < tiles; slot += nthr >> 5) {
         float s[1][1][2][2][4];
 #pragma unroll
         for (int i = 0; i < 16; ++i) s[0][0][i >> 3][(i >> 2) & 1][i & 3] = 0.0f;
-        for (int r = 0; r < p.ks; ++r) {
-          const unsigned at = mapa_shared(red + ti * 2048 + lane * 16, r);
+        unsigned at = red + slot * n_src * 2048 + lane * 16;
+#pragma unroll 2
+        for (int r = 0; r < n_src; ++r, at += 2048) {
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
-            const float4 x = ld_cluster_f4(at + i * 512);
-            s[0][0][i >> 1][i & 1][0] += x.x;
-            s[0][0][i >> 1][i & 1][1] += x.y;
-            s[0][0][i >> 1][i & 1][2] += x.z;
-            s[0][0][i >> 1][i & 1][3] += x.w;
+            const uint4 x = lds128(at + i * 512);
+            s[0][0][i >> 1][i & 1][0] += __uint_as_float(x.x);
+            s[0][0][i >> 1][i & 1][1] += __uint_as_float(x.y);
+            s[0][0][i >> 1][i & 1][2] += __uint_as_float(x.z);
+            s[0][0][i >> 1][i & 1][3] += __uint_as_float(x.w);
           }
         }
-        const int j = ti % NP, gv = ti / NP, gid = gv / NV, v = gv % NV;
+        const int ti = slot * p.ks + rank, j = ti % NP, gv = ti / NP, gid = gv / NV, v = gv % NV;
         store_col<S, 0, 1, 1>(p, u, xs, lane_col(p, S, TR, gid * 16 + g), v, j, t, s);
         store_col<S, 1, 1, 1>(p, u, xs, lane_col(p, S, TR, gid * 16 + g + 8), v, j, t, s);
       }
-      cluster_sync();  // nobody overwrites or leaves while a neighbour still reads
+      if (k + 1 < my_units) {  // nobody overwrites what a neighbour still reads
+        if (p.ks > 1) cluster_sync();
+        else __syncthreads();
+      }
     }
   }
   cp_async_wait<0>();
@@ -820,7 +865,7 @@ __global__ void __launch_bounds__(32 * max_warps(S, NP, TR), 1) block_mma_kernel
 // Shared memory of one CTA under a configuration, and the offsets the kernel uses.
 struct Layout {
   int rows, pitch, sub_px, n_list, mt, compact, pw, ncols, ngroups, nw, eg, en;
-  unsigned x_pitch, x_bytes, tab_bytes, off_bias, off_tab, off_x, off_raw, off_hid, off_red, bytes;
+  unsigned x_pitch, x_bytes, tab_bytes, off_bias, off_tab, off_src, off_x, off_raw, off_hid, off_red, bytes;
   int stage_bytes, resident, nch, raw_rows, raw_words;
 };
 
@@ -842,17 +887,19 @@ bool layout_of(const LaunchRec& r, const BlockCfg& c, Layout* l) {
   l->compact = c.whole && c.first == kExpWide;
   l->n_list = l->compact ? c.ni * r.H * r.W : c.ni * l->sub_px;
   l->mt = (l->n_list + 15) / 16;
-  if (c.ni * l->sub_px > tile_pixels(c.first) || l->mt * 16 > tile_pixels(c.first) + 2) return false;
+  const bool small = c.wk > 0;
+  const int wk = std::max(1, c.wk);
+  if (c.ni * l->sub_px > tile_pixels(c.first, small) || l->mt * 16 > tile_pixels(c.first, small) + 2) return false;
   l->pw = c.s == 1 ? c.tw / 2 : c.tw;
   l->ncols = c.ni * c.nb * l->pw;
   l->ngroups = (l->ncols + 15) / 16;
   const int cap = max_warps(c.s, c.np, c.tr);
-  if (l->ngroups > cap) return false;
+  if (l->ngroups * wk > cap) return false;
   // warps without a column group still help with the first operator
-  l->nw = std::min(cap, std::max(l->ngroups, std::min(c.nw_min, c.first != kNone ? (l->mt + 1) / 2 : 4)));
+  l->nw = std::min(cap / wk, std::max(l->ngroups, std::min(c.nw_min / wk, c.first != kNone ? (small ? l->mt : (l->mt + 1) / 2) : small ? 1 : 4)));
   {
     const double gc = group_cost(r, c);
-    const double share = (l->mt + l->ngroups * gc) / l->nw;
+    const double share = (l->mt + l->ngroups * gc) / l->nw;  // (of a set)
     int eg = static_cast<int>(share - gc + 0.5);
     if (l->nw == l->ngroups) eg = (l->mt + l->nw - 1) / l->nw;
     l->eg = std::max(0, std::min(eg, (l->mt + l->nw - 1) / l->nw));
@@ -862,10 +909,10 @@ bool layout_of(const LaunchRec& r, const BlockCfg& c, Layout* l) {
   }
   const int ke = ke_of(r, c);
   const int chid = c.first == kNone ? r.C : r.Cmid;
-  l->nch = (chid + 16 * c.hc - 1) / (16 * c.hc);
+  l->nch = (chid + 16 * c.hc * wk - 1) / (16 * c.hc * wk);
   if (c.ks > l->nch) return false;
   const int nchl = (l->nch + c.ks - 1) / c.ks;
-  l->stage_bytes = c.hc * sub_bytes(ke, c.np);
+  l->stage_bytes = c.hc * wk * sub_bytes(ke, c.np);
   l->resident = nchl <= kRing || nchl * l->stage_bytes <= c.resident_kb * 1024;
   const int nslot = l->resident ? nchl : kRing;
   const int xw = ke * 2 - (c.first == kExp24 ? 1 : 0);  // 16-byte units of a list pixel; an odd number of them is free of conflicts
@@ -880,11 +927,14 @@ bool layout_of(const LaunchRec& r, const BlockCfg& c, Layout* l) {
   l->x_bytes = static_cast<unsigned>(round_up_u64(l->mt * 16 * l->x_pitch, 128));
   l->off_bias = static_cast<unsigned>(nslot * l->stage_bytes);
   l->off_tab = static_cast<unsigned>(round_up_u64(l->off_bias + c.np * 64, 128));
-  l->off_x = l->off_tab + two * l->tab_bytes;
+  l->off_src = l->off_tab + two * l->tab_bytes;
+  l->off_x = l->off_src + (c.first != kNone && small ? static_cast<unsigned>(round_up_u64(l->mt * 64, 128)) : 0u);
   l->off_raw = l->off_x + two * l->x_bytes;
   l->off_hid = static_cast<unsigned>(round_up_u64(l->off_raw + l->raw_rows * l->raw_words * 4 + (l->raw_rows ? 32 : 0), 128));
-  l->off_red = l->off_hid + (c.first == kNone ? kRing : 2) * c.hc * 4 * slice_bytes(c.first);
-  l->bytes = l->off_red + (c.ks > 1 ? l->ngroups * (c.s == 1 ? c.tr : c.tr / 2) * c.np * 2048 : 0);
+  l->off_red = l->off_hid + (c.first == kNone ? kRing : 2) * c.hc * wk * 4 * slice_bytes(c.first, small);
+  const int tiles = l->ngroups * (c.s == 1 ? c.tr : c.tr / 2) * c.np;
+  l->bytes = l->off_red + (c.ks * wk > 1 ? (tiles + c.ks - 1) / c.ks * c.ks * wk * 2048 : 0);
+  l->nw *= wk;
   return l->bytes <= kSmemPerSm - 1024;
 }
 
@@ -901,7 +951,7 @@ int cluster_slots(int ks) { return ks == 8 ? 15 : ks == 4 ? 33 : ks == 2 ? 73 : 
 // chunks one after the other, `lat`), and the throughput of an SM's matrix and shared-memory pipes under all its CTAs'
 // units (`thr`).  The coefficients are a least-squares fit to 6100 measured launches (110 shapes of MobileNetV2 at batch 1 to
 // 256 and image sizes 128 to 513, about 50 configurations each; rms error 13 %; the configuration it picks takes 1.07 times
-// the best one's time in the geometric mean).
+// the best one's time in the geometric mean), and to 3000 more for units that several CTAs or warp sets share (11 %, 1.04).
 double block_cost_us(const LaunchRec& r, const BlockCfg& c, const Layout& l) {
   const bool expansion = c.first != kNone && c.first != kStem;
   const int ke = ke_of(r, c), nv = c.s == 1 ? c.tr : c.tr / 2;
@@ -910,21 +960,29 @@ double block_cost_us(const LaunchRec& r, const BlockCfg& c, const Layout& l) {
   const double per_sm = (std::min(c.units, slots) * c.ks + 147) / 148;
   const double nchl = (l.nch + c.ks - 1) / c.ks, ew = std::max(l.eg, l.en), thr_n = l.nw * 32.0;
   const double dw = (4.0 * (c.s == 1 ? 3 : 5) * nv + 4.0 * c.np * nv) * c.hc;
-  double lat = 236.8 + (nchl + 1) * (443 + 34.49 * ew * ke * c.hc + 6.063 * dw + 521.9 * c.hc);
-  if (c.first == kStem) lat += 2432 * l.n_list / thr_n;
-  if (c.first == kNone) lat += (nchl + 1) * 14.16 * l.n_list * 4 / thr_n;
-  if (c.ks == 1) lat += 695.4 * c.np * nv;
-  else lat += 3492 + 1735 * l.ngroups * c.np * nv / (c.ks * static_cast<double>(l.nw));
-  double thr = 317.1 + 130.4 * l.ngroups * c.np * nv + nchl * (3.538 * l.mt * ke * 2 * c.hc + 4.459 * l.ngroups * dw + 74.9 * l.ngroups * c.hc);
+  const double wk = std::max(1, c.wk), src = c.ks * wk;
+  double lat;
+  if (src == 1) {
+    lat = 236.8 + (nchl + 1) * (443 + 34.49 * ew * ke * c.hc + 6.063 * dw + 521.9 * c.hc) + 695.4 * c.np * nv;
+    if (c.first == kStem) lat += 2432 * l.n_list / thr_n;
+    if (c.first == kNone) lat += (nchl + 1) * 14.16 * l.n_list * 4 / thr_n;
+  } else {
+    const int tiles = l.ngroups * nv * c.np, own = (tiles + c.ks - 1) / c.ks, rounds = (own + l.nw - 1) / l.nw;  // tiles a warp adds up
+    lat = (nchl + 1) * (459.1 + 68.17 * ew * ke * c.hc + 3.99 * dw + 75.98 * l.nw) + 78.48 * c.np * nv + rounds * (1581 + 96.46 * src);
+    if (c.first == kNone) lat += (nchl + 1) * 30.31 * l.n_list * 4 * wk / thr_n;
+    if (c.ks > 1) lat += 1561;
+  }
+  double thr = 317.1 + 130.4 * l.ngroups * c.np * nv * wk +
+               nchl * wk * (3.538 * l.mt * ke * 2 * c.hc + 4.459 * l.ngroups * dw + 74.9 * l.ngroups * c.hc);
   if (expansion) thr += 1.235 * l.n_list * slices(r.C);
   if (c.first == kStem) thr += 3.48 * l.n_list;
   const double a = upc * lat, b = upc * per_sm * thr;
   return 2.904 + std::cbrt(a * a * a + b * b * b) / 1965.0;
 }
 
-template <int S, int FIRST, int NP, int TR, int HC>
-int launch_t(const BlockParams& p, int nw, unsigned smem, int grid, cudaStream_t stream) {
-  auto kern = block_mma_kernel<S, FIRST, NP, TR, HC>;
+template <int S, int FIRST, int NP, int TR, int HC, bool SMALL>
+int launch_s(const BlockParams& p, int nw, unsigned smem, int grid, cudaStream_t stream) {
+  auto kern = block_mma_kernel<S, FIRST, NP, TR, HC, SMALL>;
   static bool attr_done_dev[kMaxDevices] = {};
   bool& attr_done = attr_done_dev[current_device_slot()];
   if (!attr_done) {
@@ -948,25 +1006,33 @@ int launch_t(const BlockParams& p, int nw, unsigned smem, int grid, cudaStream_t
   return static_cast<int>(cudaLaunchKernelEx(&cfg, kern, p));
 }
 
+template <int S, int FIRST, int NP, int TR, int HC>
+int launch_t(const BlockCfg& c, const BlockParams& p, int nw, unsigned smem, int grid, cudaStream_t stream) {
+  if constexpr (FIRST != kStem) {
+    if (c.wk > 0) return launch_s<S, FIRST, NP, TR, 1, true>(p, nw, smem, grid, stream);
+  }
+  return launch_s<S, FIRST, NP, TR, HC, false>(p, nw, smem, grid, stream);
+}
+
 // rows per warp and sub-blocks per chunk follow from the channel counts (each_config)
 template <int S, int FIRST>
 int launch_np(const BlockCfg& c, const BlockParams& p, int nw, unsigned smem, int grid, cudaStream_t st) {
   constexpr int HC = FIRST == kExpWide ? 2 : 1;
   if constexpr (S == 2) {
-    if (c.np == 2) return launch_t<2, FIRST, 2, 2, HC>(p, nw, smem, grid, st);
-    if (c.np == 4) return launch_t<2, FIRST, 4, 2, HC>(p, nw, smem, grid, st);
+    if (c.np == 2) return launch_t<2, FIRST, 2, 2, HC>(c, p, nw, smem, grid, st);
+    if (c.np == 4) return launch_t<2, FIRST, 4, 2, HC>(c, p, nw, smem, grid, st);
     if constexpr (FIRST == kExpWide) {
-      if (c.np == 6) return launch_t<2, FIRST, 6, 2, HC>(p, nw, smem, grid, st);
-      if (c.np == 10) return launch_t<2, FIRST, 10, 2, HC>(p, nw, smem, grid, st);
+      if (c.np == 6) return launch_t<2, FIRST, 6, 2, HC>(c, p, nw, smem, grid, st);
+      if (c.np == 10) return launch_t<2, FIRST, 10, 2, HC>(c, p, nw, smem, grid, st);
     }
   } else {
-    if (c.np == 2) return c.tr == 2 ? launch_t<1, FIRST, 2, 2, HC>(p, nw, smem, grid, st) : launch_t<1, FIRST, 2, 1, HC>(p, nw, smem, grid, st);
-    if (c.np == 4) return c.tr == 2 ? launch_t<1, FIRST, 4, 2, HC>(p, nw, smem, grid, st) : launch_t<1, FIRST, 4, 1, HC>(p, nw, smem, grid, st);
+    if (c.np == 2) return c.tr == 2 ? launch_t<1, FIRST, 2, 2, HC>(c, p, nw, smem, grid, st) : launch_t<1, FIRST, 2, 1, HC>(c, p, nw, smem, grid, st);
+    if (c.np == 4) return c.tr == 2 ? launch_t<1, FIRST, 4, 2, HC>(c, p, nw, smem, grid, st) : launch_t<1, FIRST, 4, 1, HC>(c, p, nw, smem, grid, st);
     if constexpr (FIRST == kExpWide) {
-      if (c.np == 6) return launch_t<1, FIRST, 6, 1, HC>(p, nw, smem, grid, st);
-      if (c.np == 10) return launch_t<1, FIRST, 10, 1, HC>(p, nw, smem, grid, st);
+      if (c.np == 6) return launch_t<1, FIRST, 6, 1, HC>(c, p, nw, smem, grid, st);
+      if (c.np == 10) return launch_t<1, FIRST, 10, 1, HC>(c, p, nw, smem, grid, st);
     } else {
-      if (c.np == 1) return c.tr == 4 ? launch_t<1, FIRST, 1, 4, HC>(p, nw, smem, grid, st) : launch_t<1, FIRST, 1, 2, HC>(p, nw, smem, grid, st);
+      if (c.np == 1) return c.tr == 4 ? launch_t<1, FIRST, 1, 4, HC>(c, p, nw, smem, grid, st) : launch_t<1, FIRST, 1, 2, HC>(c, p, nw, smem, grid, st);
     }
   }
   return static_cast<int>(cudaErrorInvalidConfiguration);
@@ -1026,17 +1092,25 @@ void each_config(const LaunchRec& r, int kind, F&& f) {
           const long long units = c.whole ? (r.B + c.ni - 1) / c.ni : static_cast<long long>(r.B) * c.tiles_x * c.tiles_y;
           if (units > (1 << 28) || static_cast<uint64_t>(units) * c.tiles_x * c.tiles_y >= (1ull << 32)) continue;
           c.units = static_cast<int>(units);
-          for (c.ks = 1; c.ks <= 8; c.ks *= 2) {
-            if (c.ks > 1 && units * c.ks > 148 * 2) break;  // a split pays only while SMs would be idle ...
-            for (c.nw_min = 8; c.nw_min <= max_warps(c.s, c.np, c.tr); c.nw_min += 8) {
-              for (int rk = 0; rk < 2; ++rk) {
-                c.resident_kb = rk ? 48 : 0;
-                Layout l;
-                if (!layout_of(r, c, &l) || (c.nw_min > 8 && l.nw <= 8)) break;  // nw_min 8 has given the same layout
-                if (rk && !l.resident) break;
-                // ... in one wave
-                if (c.ks == 1 || units <= cluster_slots(c.ks) * ctas_per_sm(c, l)) f(c, l);
-                if (l.resident) break;
+          // warp sets: small tiles, while there are no more of them than SMs
+          static const int kSets[] = {0, 1, 2, 3, 4, 6, 8, 12, 16};
+          const int hid = c.ni * (c.s * (th - 1) + 3) * (c.s * (c.tw - 1) + 3);
+          const bool sets = kind != BLOCK_STEM && units <= 148 && hid <= tile_pixels(c.first, true);
+          for (int wi = 0; wi < (sets ? 9 : 1); ++wi) {
+            c.wk = kSets[wi];
+            c.hc = c.first == kExpWide && c.wk == 0 ? 2 : 1;
+            for (c.ks = 1; c.ks <= 8; c.ks *= 2) {
+              if (c.ks > 1 && units * c.ks > 148 * 2) break;  // a split pays only while SMs would be idle ...
+              for (c.nw_min = 8; c.nw_min <= max_warps(c.s, c.np, c.tr); c.nw_min += 8) {
+                for (int rk = 0; rk < 2; ++rk) {
+                  c.resident_kb = rk ? 48 : 0;
+                  Layout l;
+                  if (!layout_of(r, c, &l) || (c.nw_min > 8 && l.nw <= 8)) break;  // nw_min 8 has given the same layout
+                  if (rk && !l.resident) break;
+                  // ... in one wave
+                  if (c.ks == 1 || units <= cluster_slots(c.ks) * ctas_per_sm(c, l)) f(c, l);
+                  if (l.resident) break;
+                }
               }
             }
           }
@@ -1070,7 +1144,7 @@ bool block_mma_choose(const LaunchRec& r, int kind, BlockCfg* best, double* us) 
 void block_mma_pack(const float* we, const float* be, const float* wd, const float* bd, const float* wp, const float* bp, int cin,
                     int chid, int cout, const BlockCfg& c, std::vector<uint8_t>* blob, LaunchRec* r) {
   const int ke = c.first == kNone ? 0 : c.first == kStem ? 2 : (cin + 15) / 16, np = c.np;
-  const int nsub = (chid + 16 * c.hc - 1) / (16 * c.hc) * c.hc;
+  const int per = c.hc * std::max(1, c.wk), nsub = (chid + 16 * per - 1) / (16 * per) * per;
   const size_t sb = sub_bytes(ke, np);
   const uint64_t woff = round_up_u64(blob->size(), 256);
   const uint64_t boff = round_up_u64(woff + nsub * sb, 256);
@@ -1179,12 +1253,15 @@ BlockParams params_of(const LaunchRec& r, const BlockCfg& c, const Layout& l) {
   p.en = l.en;
   p.nch = l.nch;
   p.ks = c.ks;
+  p.wk = std::max(1, c.wk);
+  p.nwq = l.nw / p.wk;
   p.resident = l.resident;
   p.x_pitch = l.x_pitch;
   p.off_bias = l.off_bias;
   p.x_bytes = l.x_bytes;
   p.tab_bytes = l.tab_bytes;
   p.off_tab = l.off_tab;
+  p.off_src = l.off_src;
   p.off_x = l.off_x;
   p.off_raw = l.off_raw;
   p.off_hid = l.off_hid;

@@ -59,6 +59,7 @@ struct BlockCfg {
   int tw = 2, nb = 1, ni = 1;   // output columns of a tile, bands of `tr` rows, images per unit
   int tiles_x = 1, tiles_y = 1, whole = 0, units = 1;
   int ks = 1;                   // CTAs (a cluster) that share a unit's hidden channels
+  int wk = 0;                   // > 0: small tiles, sets of warps that share a chunk's channels, 16 each (`hc` is 1)
   int nw_min = 8;               // warps of a CTA, if the first operator has work for them
   int resident_kb = 0;          // weights of at most this size stay in shared memory
 };
