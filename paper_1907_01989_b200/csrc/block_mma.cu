@@ -1,6 +1,6 @@
 // A depthwise 3x3 convolution with the convolutions around it as ONE kernel, for any plane size:
 //   1x1 expansion -> depthwise 3x3 -> 1x1 projection (+ residual)   an inverted-residual block
-//   3x3 stride-2 stem on a 3-channel NHWC image -> depthwise 3x3 -> 1x1   the first layers of the MobileNets
+//   3x3 stride-2 stem on a 3-channel NHWC image -> depthwise 3x3 -> 1x1   the first layers of the MobileNets: stem_block.cu
 //   depthwise 3x3 -> 1x1                                            a depthwise-separable pair
 // The tensors between the operators - up to six times as wide as the block's ends - never reach memory; they are rounded to
 // fp16 exactly where the separate kernels would have stored them.
@@ -51,6 +51,7 @@
 #include <type_traits>
 
 #include "kernels.h"
+#include "mma_frag.cuh"
 #include "pdl.cuh"
 #include "sm100_ptx.cuh"
 
@@ -58,17 +59,15 @@ namespace gi {
 namespace {
 
 using namespace ptx;
+using namespace frag;
 
-constexpr int kTableBytes = 1024;  // banded depthwise operands of 4 slices: [slice][16 lanes][3 window rows + pad] x 4 bytes
-constexpr int kBiasBytes = 64;     // 16 floats
-constexpr int kDwBiasBytes = 256;  // bias of 16 channels, each four times: the start value of a fragment of sums
 constexpr int kSubFixed = kBiasBytes + kTableBytes + kDwBiasBytes;
 constexpr int kRing = 4;
 constexpr int kSmemPerSm = 227 * 1024;
 
 // How the first operator is computed: none (the input is the hidden tensor), a 1x1 expansion from up to 16 / 24 / 32 / 160
-// channels, or the stem
-enum First { kNone = 0, kExp16 = 1, kExp24 = 2, kExp32 = 3, kExpWide = 4, kStem = 5 };
+// channels
+enum First { kNone = 0, kExp16 = 1, kExp24 = 2, kExp32 = 3, kExpWide = 4 };
 
 // Bytes between the slices of a hidden tile: a constant, so that slices are immediate offsets.  32 modulo 128: the stores
 // of 4 pixels x 4 slices by half a warp meet 32 different banks.
@@ -106,7 +105,7 @@ struct BlockParams {
   int wk, nwq;              // sets of warps that share a chunk's channels; warps of a set
   int resident;
   unsigned x_pitch;
-  unsigned off_bias, off_tab, off_src, off_x, off_raw, off_hid, off_red;
+  unsigned off_bias, off_tab, off_src, off_x, off_hid, off_red;
   unsigned x_bytes, tab_bytes;  // of one of the two input tiles / tables (narrow expansions; otherwise there is one)
   unsigned mul_pitch, mul_w, mul_hw, mul_per, mul_tx;  // ceil(2^32 / d): division of a small number by d is one high multiplication
   unsigned hi_e, hi_d;  // upper clamp of the hidden activations, two halves (6 or infinity)
@@ -114,7 +113,6 @@ struct BlockParams {
   int res_x;            // the residual is the block's input: it is still in shared memory
   int wide;             // both pixels of a pair are one aligned 16-byte store
   int pad_px;           // an odd plane holds one more pixel: zero it
-  int Hi, Wi, spt, spl, raw_rows, raw_words;  // stem: image, its padding, the staged rows
 };
 
 __device__ __forceinline__ void cp_async16(unsigned dst, const void* src) {
@@ -131,67 +129,9 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-__device__ __forceinline__ void ldsm4(unsigned addr, unsigned (&r)[4]) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
-}
-__device__ __forceinline__ void ldsm2(unsigned addr, unsigned& a, unsigned& b) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0, %1}, [%2];" : "=r"(a), "=r"(b) : "r"(addr) : "memory");
-}
-__device__ __forceinline__ void mma16816(float (&d)[4], const unsigned (&a)[4], unsigned b0, unsigned b1) {
-  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
-      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-// the same with the sum started from c0..c3 (a bias): saves copying it into the accumulators
-__device__ __forceinline__ void mma16816c(float (&d)[4], const unsigned (&a)[4], unsigned b0, unsigned b1, float c0, float c1, float c2,
-                                          float c3) {
-  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%10, %11, %12, %13};"
-      : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(c0), "f"(c1), "f"(c2), "f"(c3));
-}
-__device__ __forceinline__ void mma1688(float (&d)[4], unsigned a0, unsigned a1, unsigned b0) {
-  asm("mma.sync.aligned.m16n8k8.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5}, {%6}, {%0, %1, %2, %3};"
-      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-      : "r"(a0), "r"(a1), "r"(b0));
-}
-__device__ __forceinline__ uint4 lds128(unsigned addr) {
-  uint4 v;
-  asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
-  return v;
-}
-__device__ __forceinline__ uint2 lds64(unsigned addr) {
-  uint2 v;
-  asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(addr) : "memory");
-  return v;
-}
-__device__ __forceinline__ unsigned lds32(unsigned addr) {
-  unsigned v;
-  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
-  return v;
-}
-__device__ __forceinline__ void sts32(unsigned addr, unsigned a) { asm volatile("st.shared.u32 [%0], %1;" ::"r"(addr), "r"(a) : "memory"); }
-__device__ __forceinline__ void sts64(unsigned addr, unsigned a, unsigned b) {
-  asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(addr), "r"(a), "r"(b) : "memory");
-}
-__device__ __forceinline__ void sts128(unsigned addr, unsigned a, unsigned b, unsigned c, unsigned d) {
-  asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
-}
 __device__ __forceinline__ void st_cluster_f4(unsigned addr, float a, float b, float c, float d) {
   asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
 }
-__device__ __forceinline__ unsigned min_f16x2(unsigned a, unsigned b) {
-  unsigned d;
-  asm("min.f16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
-  return d;
-}
-__device__ __forceinline__ unsigned prmt(unsigned a, unsigned sel) { return __byte_perm(a, 0u, sel); }
-
-__device__ __forceinline__ float act_f(float v, int act) {
-  if (act != GI_ACT_NONE) v = fmaxf(v, 0.0f);
-  if (act == GI_ACT_RELU6) v = fminf(v, 6.0f);
-  return v;
-}
-
 // Four consecutive channels (one pixel-slice) of the projection, bias included: activation, residual, activation, fp16.
 __device__ __forceinline__ uint2 finish4(const BlockParams& p, float v0, float v1, float v2, float v3, const uint2& r) {
   if (p.act_pre != GI_ACT_NONE) {
@@ -215,14 +155,6 @@ __device__ __forceinline__ uint2 finish4(const BlockParams& p, float v0, float v
     }
   }
   return make_uint2(pack_f16x2<false>(v0, v1), pack_f16x2<false>(v2, v3));
-}
-
-__host__ __device__ __forceinline__ int div_by(int i, unsigned mul) {
-#ifdef __CUDA_ARCH__
-  return static_cast<int>(__umulhi(static_cast<unsigned>(i), mul));
-#else
-  return static_cast<int>((static_cast<uint64_t>(i) * mul) >> 32);
-#endif
 }
 
 struct UnitPos {
@@ -391,13 +323,13 @@ __global__ void __launch_bounds__(32 * max_warps(S, NP, TR), 1) block_mma_kernel
     if (1 < total) load_weights(1, 1 % nchl);
   }
   // shared memory that must start at zero: borders of compact tiles, channels beyond the input's last slice
-  if (FIRST != kStem && (p.compact || (p.sin & 1))) {
+  if (p.compact || (p.sin & 1)) {
     for (unsigned i = p.off_x + tid * 16; i < p.off_red; i += nthr * 16) sts128(smem + i, 0u, 0u, 0u, 0u);
   }
   for (int i = tid; i < NP * 4; i += nthr) cp_async16(smem + p.off_bias + i * 16, reinterpret_cast<const float4*>(p.bias) + i);
 
-  const unsigned tab0 = smem + p.off_tab, xs0 = smem + p.off_x, raw = smem + p.off_raw, hid0 = smem + p.off_hid, red = smem + p.off_red;
-  constexpr bool kTwoX = kHasFirst && !kWideExp && FIRST != kStem;  // the next unit's input arrives during this one
+  const unsigned tab0 = smem + p.off_tab, xs0 = smem + p.off_x, hid0 = smem + p.off_hid, red = smem + p.off_red;
+  constexpr bool kTwoX = kHasFirst && !kWideExp;  // the next unit's input arrives during this one
 
   // expansion: the unit's input tile, [list pixel][channel].  The table says what a list pixel's hidden value is clamped to
   // (zero outside the image); for a wide expansion, whose list may leave out the border, also where it goes
@@ -468,72 +400,11 @@ __global__ void __launch_bounds__(32 * max_warps(S, NP, TR), 1) block_mma_kernel
         for (int s = w; s < w + HC * 4; ++s, src += p.in_sl) cp_async8(dst + s * SL, s < ns ? src : p.in, s < ns && at >= 0 ? 8u : 0u);
     }
   };
-  // stem: the rows of the image under the unit's hidden tile, as 4-byte words from the aligned word that holds a row's first
-  // value; rows outside the image are zeros, columns outside it hold neighbours' values that build_x masks
-  const long long halves = static_cast<long long>(p.B) * p.Hi * p.Wi * 3;
-  auto load_raw = [&](const UnitPos& u) {
-    const int iy0 = 2 * (u.y0 - p.pad_t) - p.spt, ix0 = 2 * (u.x0 - p.pad_l) - p.spl;
-    for (int r = warp; r < p.raw_rows; r += nthr >> 5) {
-      const int iy = iy0 + r;
-      const bool row_in = static_cast<unsigned>(iy) < static_cast<unsigned>(p.Hi);
-      const long long first = ((static_cast<long long>(u.img0) * p.Hi + iy) * p.Wi + ix0) * 3;
-      const long long word0 = first >> 1;
-      for (int w = lane; w < p.raw_words; w += 32) {
-        const long long h = (word0 + w) * 2;
-        const unsigned n = !row_in || h < 0 || h >= halves ? 0u : h + 1 < halves ? 4u : 2u;
-        cp_async4(raw + (r * p.raw_words + w) * 4, n ? p.in + h : p.in, n);
-      }
-    }
-  };
-  // stem: [list pixel][10 ky + 3 kx + c], the 9 values of a window row from 5 words
-  auto build_x = [&](const UnitPos& u) {
-    const int iy0 = 2 * (u.y0 - p.pad_t) - p.spt, ix0 = 2 * (u.x0 - p.pad_l) - p.spl;
-    const unsigned par0 = static_cast<unsigned>(((static_cast<long long>(u.img0) * p.Hi + iy0) * p.Wi + ix0) & 1);
-    for (int i = tid; i < p.mt * 16; i += nthr) {
-      if (i >= p.n_list) {
-        sts32(tab0 + i * 4, 0u);
-        continue;
-      }
-      const int r = div_by(i, p.mul_pitch), c = i - r * p.pitch;
-      const int ix = ix0 + 2 * c;
-      sts32(tab0 + i * 4, static_cast<unsigned>(u.y0 - p.pad_t + r) < static_cast<unsigned>(p.H) &&
-                                 static_cast<unsigned>(u.x0 - p.pad_l + c) < static_cast<unsigned>(p.W)
-                             ? p.hi_e : 0u);
-      unsigned o[16];
-#pragma unroll
-      for (int ky = 0; ky < 3; ++ky) {
-        const unsigned at = raw + ((2 * r + ky) * p.raw_words + 3 * c) * 4;
-        unsigned w[5];
-#pragma unroll
-        for (int q = 0; q < 5; ++q) w[q] = lds32(at + q * 4);
-        const unsigned sh = ((par0 + (ky & 1) * p.Wi) & 1) * 16;  // an even number of rows further on the parity is the same
-#pragma unroll
-        for (int q = 0; q < 4; ++q) o[ky * 5 + q] = __funnelshift_r(w[q], w[q + 1], sh);
-        o[ky * 5 + 4] = (w[4] >> sh) & 0xffffu;
-        if (ix < 0 || ix + 2 >= p.Wi) {
-          if (static_cast<unsigned>(ix) >= static_cast<unsigned>(p.Wi)) {
-            o[ky * 5] = 0u;
-            o[ky * 5 + 1] &= 0xffff0000u;
-          }
-          if (static_cast<unsigned>(ix + 1) >= static_cast<unsigned>(p.Wi)) {
-            o[ky * 5 + 1] &= 0xffffu;
-            o[ky * 5 + 2] = 0u;
-          }
-          if (static_cast<unsigned>(ix + 2) >= static_cast<unsigned>(p.Wi)) o[ky * 5 + 3] = o[ky * 5 + 4] = 0u;
-        }
-      }
-      o[15] = 0u;
-#pragma unroll
-      for (int q = 0; q < 4; ++q) sts128(xs0 + i * 80 + q * 16, o[q * 4], o[q * 4 + 1], o[q * 4 + 2], o[q * 4 + 3]);
-    }
-  };
   if (SMALL && kHasFirst) find_x(unit_pos(p, unit0, th_rows));
   __syncthreads();
   pdl_wait();
   if (my_units > 0) {
-    if (FIRST == kStem) {
-      load_raw(unit_pos(p, unit0, th_rows));
-    } else if (kHasFirst) {
+    if (kHasFirst) {
       if (SMALL) copy_x();
       else load_x(unit_pos(p, unit0, th_rows), 0);
     } else {
@@ -573,12 +444,6 @@ __global__ void __launch_bounds__(32 * max_warps(S, NP, TR), 1) block_mma_kernel
   int run = 0;
   for (int k = 0; k < my_units; ++k, run += nchl) {
     const int unit = unit0 + k * ustep;
-    if (FIRST == kStem) {
-      cp_async_wait<0>();
-      __syncthreads();
-      build_x(unit_pos(p, unit, th_rows));
-    }
-
     float acc[NV][NP][2][2][4];  // sums start at the bias (a cluster's: in its first CTA)
 #pragma unroll
     for (int j = 0; j < NP; ++j) {
@@ -603,7 +468,6 @@ __global__ void __launch_bounds__(32 * max_warps(S, NP, TR), 1) block_mma_kernel
       if (kHasFirst) {
         if (!p.resident && it < nchl && run + it + 2 < total) load_weights(run + it + 2, it + 2 >= nchl ? (it + 2) % nchl : it + 2);
         if (k + 1 < my_units) {
-          if (FIRST == kStem && it == 0) load_raw(unit_pos(p, unit + ustep, th_rows));
           if (kTwoX && it == 0) load_x(unit_pos(p, unit + ustep, th_rows), (k + 1) & 1);
           if (kWideExp && it == nchl) load_x(unit_pos(p, unit + ustep, th_rows), 0);
         }
@@ -635,7 +499,7 @@ __global__ void __launch_bounds__(32 * max_warps(S, NP, TR), 1) block_mma_kernel
             for (int i = 0; i < N; ++i) {
               ldsm4(xa + i * 16 * XP, a[i]);
               if (FIRST == kExp24) ldsm2(xh + i * 16 * XP, a2[i][0], a2[i][1]);
-              if (FIRST == kExp32 || FIRST == kStem) ldsm4(xa + i * 16 * XP + 32, a2[i]);
+              if (FIRST == kExp32) ldsm4(xa + i * 16 * XP + 32, a2[i]);
               hi[i][0] = lds32(tb + i * 64);
               hi[i][1] = lds32(tb + i * 64 + 32);
             }
@@ -647,7 +511,7 @@ __global__ void __launch_bounds__(32 * max_warps(S, NP, TR), 1) block_mma_kernel
                 mma1688(c[i][0], a2[i][0], a2[i][1], b1.x);
                 mma1688(c[i][1], a2[i][0], a2[i][1], b1.z);
               }
-              if (FIRST == kExp32 || FIRST == kStem) {
+              if (FIRST == kExp32) {
                 mma16816(c[i][0], a2[i], b1.x, b1.y);
                 mma16816(c[i][1], a2[i], b1.z, b1.w);
               }
@@ -865,11 +729,11 @@ __global__ void __launch_bounds__(32 * max_warps(S, NP, TR), 1) block_mma_kernel
 // Shared memory of one CTA under a configuration, and the offsets the kernel uses.
 struct Layout {
   int rows, pitch, sub_px, n_list, mt, compact, pw, ncols, ngroups, nw, eg, en;
-  unsigned x_pitch, x_bytes, tab_bytes, off_bias, off_tab, off_src, off_x, off_raw, off_hid, off_red, bytes;
-  int stage_bytes, resident, nch, raw_rows, raw_words;
+  unsigned x_pitch, x_bytes, tab_bytes, off_bias, off_tab, off_src, off_x, off_hid, off_red, bytes;
+  int stage_bytes, resident, nch;
 };
 
-int ke_of(const LaunchRec& r, const BlockCfg& c) { return c.first == kNone ? 0 : c.first == kStem ? 2 : (r.C + 15) / 16; }
+int ke_of(const LaunchRec& r, const BlockCfg& c) { return c.first == kNone ? 0 : (r.C + 15) / 16; }
 
 // cost of a column group's depthwise and projection relative to a group of 16 list pixels; it only divides the list between
 // warps that have a column group and warps that have none
@@ -916,21 +780,15 @@ bool layout_of(const LaunchRec& r, const BlockCfg& c, Layout* l) {
   l->resident = nchl <= kRing || nchl * l->stage_bytes <= c.resident_kb * 1024;
   const int nslot = l->resident ? nchl : kRing;
   const int xw = ke * 2 - (c.first == kExp24 ? 1 : 0);  // 16-byte units of a list pixel; an odd number of them is free of conflicts
-  l->x_pitch = c.first == kNone ? 0u : c.first == kStem ? 80u : static_cast<unsigned>((xw % 2 ? xw : xw + 1) * 16);
-  l->raw_rows = l->raw_words = 0;
-  if (c.first == kStem) {
-    l->raw_rows = 2 * l->rows + 1;
-    l->raw_words = ((2 * l->pitch + 1) * 3 + 2) / 2 + 1;
-  }
-  const int two = c.first != kNone && c.first != kExpWide && c.first != kStem ? 2 : 1;
+  l->x_pitch = c.first == kNone ? 0u : static_cast<unsigned>((xw % 2 ? xw : xw + 1) * 16);
+  const int two = c.first != kNone && c.first != kExpWide ? 2 : 1;
   l->tab_bytes = static_cast<unsigned>(round_up_u64(l->mt * (c.first == kExpWide ? 128 : 64), 128));
   l->x_bytes = static_cast<unsigned>(round_up_u64(l->mt * 16 * l->x_pitch, 128));
   l->off_bias = static_cast<unsigned>(nslot * l->stage_bytes);
   l->off_tab = static_cast<unsigned>(round_up_u64(l->off_bias + c.np * 64, 128));
   l->off_src = l->off_tab + two * l->tab_bytes;
   l->off_x = l->off_src + (c.first != kNone && small ? static_cast<unsigned>(round_up_u64(l->mt * 64, 128)) : 0u);
-  l->off_raw = l->off_x + two * l->x_bytes;
-  l->off_hid = static_cast<unsigned>(round_up_u64(l->off_raw + l->raw_rows * l->raw_words * 4 + (l->raw_rows ? 32 : 0), 128));
+  l->off_hid = static_cast<unsigned>(round_up_u64(l->off_x + two * l->x_bytes, 128));
   l->off_red = l->off_hid + (c.first == kNone ? kRing : 2) * c.hc * wk * 4 * slice_bytes(c.first, small);
   const int tiles = l->ngroups * (c.s == 1 ? c.tr : c.tr / 2) * c.np;
   l->bytes = l->off_red + (c.ks * wk > 1 ? (tiles + c.ks - 1) / c.ks * c.ks * wk * 2048 : 0);
@@ -953,7 +811,6 @@ int cluster_slots(int ks) { return ks == 8 ? 15 : ks == 4 ? 33 : ks == 2 ? 73 : 
 // 256 and image sizes 128 to 513, about 50 configurations each; rms error 13 %; the configuration it picks takes 1.07 times
 // the best one's time in the geometric mean), and to 3000 more for units that several CTAs or warp sets share (11 %, 1.04).
 double block_cost_us(const LaunchRec& r, const BlockCfg& c, const Layout& l) {
-  const bool expansion = c.first != kNone && c.first != kStem;
   const int ke = ke_of(r, c), nv = c.s == 1 ? c.tr : c.tr / 2;
   const int occ = ctas_per_sm(c, l), slots = cluster_slots(c.ks) * occ;
   const double upc = (c.units + std::min(c.units, slots) - 1) / std::min(c.units, slots);  // units per CTA
@@ -964,7 +821,6 @@ double block_cost_us(const LaunchRec& r, const BlockCfg& c, const Layout& l) {
   double lat;
   if (src == 1) {
     lat = 236.8 + (nchl + 1) * (443 + 34.49 * ew * ke * c.hc + 6.063 * dw + 521.9 * c.hc) + 695.4 * c.np * nv;
-    if (c.first == kStem) lat += 2432 * l.n_list / thr_n;
     if (c.first == kNone) lat += (nchl + 1) * 14.16 * l.n_list * 4 / thr_n;
   } else {
     const int tiles = l.ngroups * nv * c.np, own = (tiles + c.ks - 1) / c.ks, rounds = (own + l.nw - 1) / l.nw;  // tiles a warp adds up
@@ -974,8 +830,7 @@ double block_cost_us(const LaunchRec& r, const BlockCfg& c, const Layout& l) {
   }
   double thr = 317.1 + 130.4 * l.ngroups * c.np * nv * wk +
                nchl * wk * (3.538 * l.mt * ke * 2 * c.hc + 4.459 * l.ngroups * dw + 74.9 * l.ngroups * c.hc);
-  if (expansion) thr += 1.235 * l.n_list * slices(r.C);
-  if (c.first == kStem) thr += 3.48 * l.n_list;
+  if (c.first != kNone) thr += 1.235 * l.n_list * slices(r.C);
   const double a = upc * lat, b = upc * per_sm * thr;
   return 2.904 + std::cbrt(a * a * a + b * b * b) / 1965.0;
 }
@@ -1008,9 +863,7 @@ int launch_s(const BlockParams& p, int nw, unsigned smem, int grid, cudaStream_t
 
 template <int S, int FIRST, int NP, int TR, int HC>
 int launch_t(const BlockCfg& c, const BlockParams& p, int nw, unsigned smem, int grid, cudaStream_t stream) {
-  if constexpr (FIRST != kStem) {
-    if (c.wk > 0) return launch_s<S, FIRST, NP, TR, 1, true>(p, nw, smem, grid, stream);
-  }
+  if (c.wk > 0) return launch_s<S, FIRST, NP, TR, 1, true>(p, nw, smem, grid, stream);
   return launch_s<S, FIRST, NP, TR, HC, false>(p, nw, smem, grid, stream);
 }
 
@@ -1045,25 +898,19 @@ int launch_first(const BlockCfg& c, const BlockParams& p, int nw, unsigned smem,
     case kExp16: return launch_np<S, kExp16>(c, p, nw, smem, grid, st);
     case kExp24: return launch_np<S, kExp24>(c, p, nw, smem, grid, st);
     case kExp32: return launch_np<S, kExp32>(c, p, nw, smem, grid, st);
-    case kStem:
-      if constexpr (S == 1) return launch_np<1, kStem>(c, p, nw, smem, grid, st);
-      return static_cast<int>(cudaErrorInvalidConfiguration);
     default: return launch_np<S, kExpWide>(c, p, nw, smem, grid, st);
   }
 }
-
-unsigned magic(uint64_t d) { return static_cast<unsigned>(std::min<uint64_t>(0xffffffffull, (0xffffffffull + d) / d)); }
 
 // Calls f(configuration, layout) for every configuration that runs the block in `r`.
 template <class F>
 void each_config(const LaunchRec& r, int kind, F&& f) {
   if (r.kh != 3 || r.kw != 3 || r.sh != r.sw || (r.sh != 1 && r.sh != 2) || r.dh != 1 || r.dw != 1) return;
   if (r.pt < 0 || r.pt > 2 || r.pl < 0 || r.pl > 2 || r.W < 2 || r.H < 1) return;
-  if (kind == BLOCK_STEM && (r.sh != 1 || r.C != 3)) return;
-  if ((kind == BLOCK_STEM || kind == BLOCK_EXPANSION) && r.Cmid < 16) return;
+  if (kind == BLOCK_EXPANSION && r.Cmid < 16) return;
   BlockCfg c;
   c.s = r.sh;
-  c.first = kind == BLOCK_STEM ? kStem : kind == BLOCK_PAIR ? kNone : r.C <= 16 ? kExp16 : r.C <= 24 ? kExp24 : r.C <= 32 ? kExp32 : kExpWide;
+  c.first = kind == BLOCK_PAIR ? kNone : r.C <= 16 ? kExp16 : r.C <= 24 ? kExp24 : r.C <= 32 ? kExp32 : kExpWide;
   const int np_raw = (r.Co2 + 15) / 16;
   if (c.first == kExpWide) {
     c.np = np_raw <= 2 ? 2 : np_raw <= 4 ? 4 : np_raw <= 6 ? 6 : np_raw <= 10 ? 10 : 0;
@@ -1072,7 +919,7 @@ void each_config(const LaunchRec& r, int kind, F&& f) {
     c.np = np_raw == 1 && c.s == 1 ? 1 : np_raw <= 2 ? 2 : np_raw <= 4 ? 4 : 0;
   }
   if (c.np == 0) return;
-  const int64_t in_plane = kind == BLOCK_STEM ? static_cast<int64_t>(r.stem_h) * r.stem_w * 3 : static_cast<int64_t>(plane_pixels(r.H, r.W)) * 4;
+  const int64_t in_plane = static_cast<int64_t>(plane_pixels(r.H, r.W)) * 4;
   if (r.B * in_plane * (kind == BLOCK_PAIR ? (r.C + 3) / 4 : 1) >= (1LL << 31)) return;  // offsets inside the input are 32-bit
   if (static_cast<int64_t>(r.Ho) * r.Wo * std::max(4, r.Co2) >= (1LL << 31)) return;
   c.hc = c.first == kExpWide ? 2 : 1;
@@ -1088,14 +935,14 @@ void each_config(const LaunchRec& r, int kind, F&& f) {
         if (th - c.tr >= r.Ho) break;
         c.tiles_y = (r.Ho + th - 1) / th;
         c.whole = c.tiles_x == 1 && c.tiles_y == 1;
-        for (c.ni = 1; c.ni <= (c.whole && kind != BLOCK_STEM ? 8 : 1) && c.ni <= r.B; ++c.ni) {
+        for (c.ni = 1; c.ni <= (c.whole ? 8 : 1) && c.ni <= r.B; ++c.ni) {
           const long long units = c.whole ? (r.B + c.ni - 1) / c.ni : static_cast<long long>(r.B) * c.tiles_x * c.tiles_y;
           if (units > (1 << 28) || static_cast<uint64_t>(units) * c.tiles_x * c.tiles_y >= (1ull << 32)) continue;
           c.units = static_cast<int>(units);
           // warp sets: small tiles, while there are no more of them than SMs
           static const int kSets[] = {0, 1, 2, 3, 4, 6, 8, 12, 16};
           const int hid = c.ni * (c.s * (th - 1) + 3) * (c.s * (c.tw - 1) + 3);
-          const bool sets = kind != BLOCK_STEM && units <= 148 && hid <= tile_pixels(c.first, true);
+          const bool sets = units <= 148 && hid <= tile_pixels(c.first, true);
           for (int wi = 0; wi < (sets ? 9 : 1); ++wi) {
             c.wk = kSets[wi];
             c.hc = c.first == kExpWide && c.wk == 0 ? 2 : 1;
@@ -1128,6 +975,7 @@ uint16_t half_bits(float v) { return f32_to_f16_rne(v); }
 bool block_mma_choose(const LaunchRec& r, int kind, BlockCfg* best, double* us) {
   double best_cost = 0.0;
   bool found = false;
+  if (kind == BLOCK_STEM) return stem_block_choose(r, best, us);
   each_config(r, kind, [&](const BlockCfg& c, const Layout& l) {
     const double cost = block_cost_us(r, c, l);
     if (found && cost >= best_cost) return;
@@ -1143,21 +991,13 @@ bool block_mma_choose(const LaunchRec& r, int kind, BlockCfg* best, double* us) 
 // we: [chid][cin], for the stem [chid][3][3][3], null for a pair; wd [9][chid], wp [cout][chid].
 void block_mma_pack(const float* we, const float* be, const float* wd, const float* bd, const float* wp, const float* bp, int cin,
                     int chid, int cout, const BlockCfg& c, std::vector<uint8_t>* blob, LaunchRec* r) {
-  const int ke = c.first == kNone ? 0 : c.first == kStem ? 2 : (cin + 15) / 16, np = c.np;
+  if (c.stem) return stem_block_pack(we, be, wd, bd, wp, bp, chid, cout, c, blob, r);
+  const int ke = c.first == kNone ? 0 : (cin + 15) / 16, np = c.np;
   const int per = c.hc * std::max(1, c.wk), nsub = (chid + 16 * per - 1) / (16 * per) * per;
   const size_t sb = sub_bytes(ke, np);
   const uint64_t woff = round_up_u64(blob->size(), 256);
   const uint64_t boff = round_up_u64(woff + nsub * sb, 256);
   blob->resize(boff + static_cast<size_t>(np) * 16 * sizeof(float), 0);
-  auto hid_of = [](int sub, int f, int n) { return 16 * sub + 4 * (n >> 1) + 2 * f + (n & 1); };
-  // weight of hidden channel h at position k of the first operator's sum
-  auto first_weight = [&](int h, int k) -> float {
-    if (c.first == kStem) {
-      const int ky = k / 10, e = k % 10;
-      return ky < 3 && e < 9 ? we[(static_cast<size_t>(h) * 3 + ky) * 9 + e] : 0.0f;
-    }
-    return k < cin ? we[static_cast<size_t>(h) * cin + k] : 0.0f;
-  };
   for (int sub = 0; sub < nsub; ++sub) {
     uint8_t* base = blob->data() + woff + sub * sb;
     uint16_t* e = reinterpret_cast<uint16_t*>(base);
@@ -1166,8 +1006,8 @@ void block_mma_pack(const float* we, const float* be, const float* wd, const flo
         for (int w = 0; w < 8; ++w) {  // halves of {frag 0: b0, b1; frag 1: b0, b1}
           const int f = w >> 2, hi8 = (w >> 1) & 1, lo = w & 1;
           const int n = lane >> 2, t = lane & 3;
-          const int k = kk * 16 + hi8 * 8 + 2 * t + lo, h = hid_of(sub, f, n);
-          if (h < chid) e[(kk * 32 + lane) * 8 + w] = half_bits(first_weight(h, k));
+          const int k = kk * 16 + hi8 * 8 + 2 * t + lo, h = channel_of(sub, f, n);
+          if (h < chid && k < cin) e[(kk * 32 + lane) * 8 + w] = half_bits(we[static_cast<size_t>(h) * cin + k]);
         }
     float* ebias = reinterpret_cast<float*>(base + ke * 512);
     uint16_t* tabl = reinterpret_cast<uint16_t*>(base + ke * 512 + kBiasBytes);
@@ -1198,7 +1038,7 @@ void block_mma_pack(const float* we, const float* be, const float* wd, const flo
         for (int w = 0; w < 8; ++w) {
           const int f = w >> 2, hi8 = (w >> 1) & 1, lo = w & 1;
           const int n = lane >> 2, t = lane & 3;
-          const int h = sub * 16 + hi8 * 8 + lo * 4 + t, co = hid_of(j, f, n);
+          const int h = sub * 16 + hi8 * 8 + lo * 4 + t, co = channel_of(j, f, n);
           if (h < chid && co < cout) q[(j * 32 + lane) * 8 + w] = half_bits(wp[static_cast<size_t>(co) * chid + h]);
         }
   }
@@ -1219,10 +1059,9 @@ BlockParams params_of(const LaunchRec& r, const BlockCfg& c, const Layout& l) {
   p.Ho = r.Ho;
   p.Wo = r.Wo;
   const int P = plane_pixels(r.H, r.W), Po = plane_pixels(r.Ho, r.Wo);
-  const bool nhwc_in = r.nhwc_in && c.first != kStem;
-  p.in_px = nhwc_in ? r.C : 4;
-  p.in_img = nhwc_in ? r.H * r.W * r.C : P * 4;
-  p.in_sl = nhwc_in ? 4 : static_cast<long long>(r.B) * P * 4;
+  p.in_px = r.nhwc_in ? r.C : 4;
+  p.in_img = r.nhwc_in ? r.H * r.W * r.C : P * 4;
+  p.in_sl = r.nhwc_in ? 4 : static_cast<long long>(r.B) * P * 4;
   p.o_px = r.nhwc_out ? r.Co2 : 4;
   p.o_img = r.nhwc_out ? static_cast<long long>(r.Ho) * r.Wo * r.Co2 : Po * 4;
   p.o_sl = r.nhwc_out ? 4 : static_cast<long long>(r.B) * Po * 4;
@@ -1263,7 +1102,6 @@ BlockParams params_of(const LaunchRec& r, const BlockCfg& c, const Layout& l) {
   p.off_tab = l.off_tab;
   p.off_src = l.off_src;
   p.off_x = l.off_x;
-  p.off_raw = l.off_raw;
   p.off_hid = l.off_hid;
   p.off_red = l.off_red;
   p.mul_pitch = magic(l.pitch);
@@ -1279,18 +1117,13 @@ BlockParams params_of(const LaunchRec& r, const BlockCfg& c, const Layout& l) {
   p.has_res = r.ep2.has_res;
   p.wide = !r.nhwc_out && r.Wo % 2 == 0;
   p.pad_px = !r.nhwc_out && (r.Ho * r.Wo) % 2;
-  p.Hi = r.stem_h;
-  p.Wi = r.stem_w;
-  p.spt = r.stem_pt;
-  p.spl = r.stem_pl;
-  p.raw_rows = l.raw_rows;
-  p.raw_words = l.raw_words;
   return p;
 }
 }  // namespace
 
 int launch_block_mma(const LaunchRec& r, const Ptrs& ptr, void* stream) {
   const BlockCfg& c = r.block;
+  if (c.stem) return launch_stem_block(r, ptr, stream);
   Layout l;
   if (!layout_of(r, c, &l)) return static_cast<int>(cudaErrorInvalidConfiguration);
   BlockParams p = params_of(r, c, l);
@@ -1299,7 +1132,7 @@ int launch_block_mma(const LaunchRec& r, const Ptrs& ptr, void* stream) {
   p.out = static_cast<__half*>(ptr.out);
   p.wts = static_cast<const unsigned char*>(ptr.wts);
   p.bias = static_cast<const float*>(ptr.bias);
-  p.res_x = p.has_res && ptr.res == ptr.in0 && !r.nhwc_in && c.s == 1 && c.first != kNone && c.first != kExpWide && c.first != kStem;
+  p.res_x = p.has_res && ptr.res == ptr.in0 && !r.nhwc_in && c.s == 1 && c.first != kNone && c.first != kExpWide;
   const long long slots = c.ks > 1 ? c.units : static_cast<long long>(device_sm_count()) * ctas_per_sm(c, l);
   const int grid = static_cast<int>(std::min<long long>(c.units, std::max<long long>(1, slots))) * c.ks;
   cudaStream_t st = static_cast<cudaStream_t>(stream);

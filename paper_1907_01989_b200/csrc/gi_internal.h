@@ -54,6 +54,7 @@ struct Epilogue {
 enum BlockKind { BLOCK_EXPANSION = 0, BLOCK_PAIR = 1, BLOCK_STEM = 2 };
 constexpr int GROUP_RESIZE = 3;  // an up-sampling and the layout conversion behind it (OpGroup::kind, beside the block kinds)
 struct BlockCfg {
+  int stem = 0;                 // the stem kernel (stem_block.cu): only np, tw, nb, tiles_x, tiles_y, units count
   int s = 1, first = 0;         // stride of the depthwise operator; how the operator in front of it is computed
   int np = 2, tr = 2, hc = 1;   // 16-channel output blocks, output rows per warp, 16-channel sub-blocks per chunk
   int tw = 2, nb = 1, ni = 1;   // output columns of a tile, bands of `tr` rows, images per unit

@@ -110,6 +110,13 @@ void block_mma_pack(const float* we, const float* be, const float* wd, const flo
                     int chid, int cout, const BlockCfg& c, std::vector<uint8_t>* blob, LaunchRec* r);
 int launch_block_mma(const LaunchRec& r, const Ptrs& p, void* stream);
 
+// The same for a stem, its depthwise and its 1x1 convolution (stem_block.cu); reached through the three above.
+bool stem_block_choose(const LaunchRec& r, BlockCfg* best, double* us);
+void stem_block_pack(const float* ws, const float* bs, const float* wd, const float* bd, const float* wp, const float* bp, int chid, int cout,
+                     const BlockCfg& c, std::vector<uint8_t>* blob, LaunchRec* r);
+int launch_stem_block(const LaunchRec& r, const Ptrs& p, void* stream);
+unsigned int stem_block_error_word(int* cuda_err);
+
 // Pointwise convolution for launches bound by latency (fp16 storage; pointwise_mma.cu)
 bool pointwise_mma_wanted(const LaunchRec& r);
 void pointwise_mma_pack(const float* w, const float* bias, int cin, int cout, std::vector<uint8_t>* blob, LaunchRec* r);

@@ -984,6 +984,25 @@ def test_depthwise_with_its_neighbours_as_one_kernel(case):
     assert all(np.array_equal(outs[t], again[t]) for t in spec.outputs)
 
 
+# (batch, h, w, hidden, cout): one row of tiles, a single pixel column, ends of the tensor that are no multiple of 16 bytes, rows
+# on every 16-byte remainder, more tiles than two per SM (three and more rounds of the two staging buffers)
+@pytest.mark.parametrize("case", [(1, 3, 5, 32, 16), (1, 9, 4, 20, 8), (2, 31, 33, 32, 64), (3, 45, 63, 16, 96), (5, 129, 127, 32, 16), (48, 97, 122, 32, 24)])
+def test_stem_block_edges(case):
+    batch, h, w, cmid, cout = case
+    spec = _stem_block(batch, h, w, cmid, cout)
+    xs = [wl.make_input(spec)]
+    run = DeviceRun(spec, api.GI_F16, guard_bytes=4096)
+    assert "block_mma" in [api.KERNEL_NAMES[launch.kernel] for launch in run.ex.launches()]
+    outs = run.run(xs)
+    assert run.guard_intact()
+    t = spec.outputs[0]
+    if batch <= 5:
+        assert_close(outs[t], og.run(spec, xs, storage="f16", fused=True)[t], api.GI_F16, str(case))
+    assert_close(outs[t], DeviceRun(spec, api.GI_F16, cross_op=api.GI_XOP_OFF).run(xs)[t], api.GI_F16, "one kernel per op")
+    assert np.array_equal(outs[t], run.run(xs)[t])
+    assert api.gi_device_status() == 0
+
+
 @pytest.mark.parametrize("batch,size", [(1, 224), (8, 130), (21, 205)])
 def test_mobilenet_v2_launches_few_kernels(batch, size):
     spec = wl.mobilenet_v2(batch, size=size)
