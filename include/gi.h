@@ -217,7 +217,8 @@ enum {
   GI_KERNEL_POINTWISE_MM = 16,        /* 1x1 convolution, wide tiles for tensor-bound shapes */
   GI_KERNEL_POINTWISE_CHAIN = 17,     /* this op (1x1) and the next one (1x1) as one kernel; both outputs are stored */
   GI_KERNEL_BLOCK_MMA = 18,           /* gi_exec_launch only: a depthwise 3x3 op with the ops around it as one kernel */
-  GI_KERNEL_POINTWISE_MMA = 19        /* gi_exec_launch only: 1x1 convolution for launches bound by latency (and the layout conversion behind it) */
+  GI_KERNEL_POINTWISE_MMA = 19,       /* gi_exec_launch only: 1x1 convolution for launches bound by latency (and the layout conversion behind it) */
+  GI_KERNEL_CONV_MMA = 20             /* gi_exec_launch only: k x k convolution with few channels, or a whole fire module */
 };
 
 /* ---- graph construction (Section 3.1, "Initialization": the sub-graph given to the GPU backend) ---- */

@@ -52,8 +52,11 @@ struct Epilogue {
 // Configuration of the kernel that runs a depthwise convolution and the convolutions around it (block_mma.cu), chosen at
 // compile time.
 enum BlockKind { BLOCK_EXPANSION = 0, BLOCK_PAIR = 1, BLOCK_STEM = 2 };
-constexpr int GROUP_RESIZE = 3;  // an up-sampling and the layout conversion behind it (OpGroup::kind, beside the block kinds)
+// (OpGroup::kind, beside the block kinds) an up-sampling and the layout conversion behind it; a k x k convolution with or without
+// the conversion in front of it, or a fire module
+constexpr int GROUP_RESIZE = 3, GROUP_CONV = 4;
 struct BlockCfg {
+  // (conv_mma.cu: only tw and nb, the tile's rows, count)
   int stem = 0;                 // the stem kernel (stem_block.cu): only np, tw, nb, tiles_x, tiles_y, units count
   int s = 1, first = 0;         // stride of the depthwise operator; how the operator in front of it is computed
   int np = 2, tr = 2, hc = 1;   // 16-channel output blocks, output rows per warp, 16-channel sub-blocks per chunk
@@ -109,6 +112,9 @@ struct LaunchRec {
   BlockCfg block;
   int nhwc_out = 0;  // the kernel writes the caller's NHWC output itself
   int lead = -1, dw_op = -1;  // executed ops: the convolution in front of the depthwise one (or -1), the depthwise one
+  // a convolution group: `lead` the squeeze (or -1); the convolutions in the order of their output channels (the second or -1);
+  // the sum behind the concatenation (or -1).  `ep` is the squeeze's epilogue, `ep2` what happens to the result
+  int conv_a = -1, conv_b = -1, sum_op = -1;
   int stem_h = 0, stem_w = 0, stem_pt = 0, stem_pl = 0;  // image and padding of a stem in front of the depthwise operator
 };
 

@@ -357,11 +357,121 @@ static bool resize_then_unpack(const gi_exec* e, size_t i) {
          static_cast<int64_t>(d.w) * d.c < (1LL << 30);
 }
 
+// A run that conv_mma.cu may run as one kernel: a k x k convolution (with the conversion of a small NHWC image in front of it),
+// or squeeze, two expansions of the squeezed tensor, their concatenation and the sum behind it.
+struct ConvOps {
+  int n = 0;
+  int pack = 0, squeeze = -1, a = -1, b = -1;  // executed ops: the squeeze, the convolution(s) in the output's channel order
+  int last = -1, sum = -1;
+};
+
+static int readers(const gi_exec* e, int t) {
+  int n = 0;
+  for (const FusedOp& o : e->ops) n += (o.in0 == t) + (o.in1 == t) + (o.residual == t);
+  return n;
+}
+
+// Only the run's own ops read tensor `t`, `n` of them, and no caller sees it.
+static bool inside_run(const gi_exec* e, int t, int n) {
+  return t >= 0 && e->tensors[t].output_index < 0 && e->tensors[t].input_index < 0 && readers(e, t) == n;
+}
+
+static ConvOps fire_at(const gi_graph& g, const gi_exec* e, size_t i) {
+  ConvOps c;
+  if (i + 3 >= e->ops.size()) return c;
+  const FusedOp &s = e->ops[i], &x = e->ops[i + 1], &y = e->ops[i + 2], &cat = e->ops[i + 3];
+  if (s.kind != GI_OP_CONV2D || x.kind != GI_OP_CONV2D || y.kind != GI_OP_CONV2D || cat.kind != GI_OP_CONCAT || cat.in1 < 0) return c;
+  if (!is_plain_pointwise(g.ops[s.graph_op].d) || s.residual >= 0 || s.act_post != GI_ACT_NONE) return c;
+  if (x.in0 != s.out || y.in0 != s.out || x.residual >= 0 || y.residual >= 0 || x.act_pre != y.act_pre || x.act_post != GI_ACT_NONE ||
+      y.act_post != GI_ACT_NONE)
+    return c;
+  if (!inside_run(e, s.out, 2) || !inside_run(e, x.out, 1) || !inside_run(e, y.out, 1)) return c;
+  const bool in_order = cat.in0 == x.out && cat.in1 == y.out, swapped = cat.in0 == y.out && cat.in1 == x.out;
+  if (!in_order && !swapped) return c;
+  int dilation = 0;
+  for (const FusedOp* f : {&x, &y}) {
+    const gi_op_desc& d = g.ops[f->graph_op].d;
+    if (is_plain_pointwise(d)) continue;
+    if (d.kh != 3 || d.kw != 3 || d.stride_h != 1 || d.stride_w != 1 || d.dilation_h != d.dilation_w || d.pad_t != d.dilation_h ||
+        d.pad_l != d.dilation_w || d.pad_b != d.pad_t || d.pad_r != d.pad_l)
+      return c;
+    if (dilation != 0 && dilation != d.dilation_h) return c;
+    dilation = d.dilation_h;
+  }
+  if (dilation == 0) return c;
+  c.squeeze = static_cast<int>(i);
+  c.a = static_cast<int>(in_order ? i + 1 : i + 2);
+  c.b = static_cast<int>(in_order ? i + 2 : i + 1);
+  c.last = static_cast<int>(i + 3);
+  c.n = 4;
+  if (i + 4 < e->ops.size()) {
+    const FusedOp& sum = e->ops[i + 4];
+    const int other = sum.in0 == cat.out ? sum.in1 : sum.in0;
+    if (sum.kind == GI_OP_ADD && sum.in1 >= 0 && (sum.in0 == cat.out || sum.in1 == cat.out) && other != cat.out && inside_run(e, cat.out, 1)) {
+      c.sum = c.last = static_cast<int>(i + 4);
+      c.n = 5;
+    }
+  }
+  return c;
+}
+
+static ConvOps conv_at(const gi_graph& g, const gi_exec* e, size_t i) {
+  ConvOps c;
+  size_t k = i;
+  if (e->ops[k].kind == GI_EXEC_PACK) {
+    const int t = e->ops[k].out;
+    if (k + 1 >= e->ops.size() || e->ops[k + 1].in0 != t || e->tensors[t].output_index >= 0 || readers(e, t) != 1) return c;
+    c.pack = 1;
+    ++k;
+  }
+  const FusedOp& f = e->ops[k];
+  if (f.kind != GI_OP_CONV2D || is_plain_pointwise(g.ops[f.graph_op].d)) return c;
+  c.a = c.last = static_cast<int>(k);
+  c.n = static_cast<int>(k - i) + 1;
+  return c;
+}
+
+static LaunchRec conv_rec(const gi_graph& g, const gi_exec* e, const ConvOps& c) {
+  const FusedOp& a = e->ops[c.a];
+  const FusedOp& first = e->ops[c.squeeze >= 0 ? c.squeeze : c.a];
+  const bool window_b = c.b >= 0 && is_plain_pointwise(g.ops[a.graph_op].d);
+  const gi_op_desc& d = g.ops[e->ops[window_b ? c.b : c.a].graph_op].d;
+  const TensorDesc &in = e->tensors[first.in0], &out = e->tensors[e->ops[c.last].out];
+  LaunchRec r;
+  r.kernel = GI_KERNEL_CONV_MMA;
+  r.B = e->batch;
+  r.H = in.h;
+  r.W = in.w;
+  r.C = in.c;
+  r.Ho = out.h;
+  r.Wo = out.w;
+  r.Co = out.c;
+  r.Cmid = c.squeeze >= 0 ? e->tensors[first.out].c : 0;
+  r.kh = d.kh;
+  r.kw = d.kw;
+  r.sh = d.stride_h;
+  r.sw = d.stride_w;
+  r.dh = d.dilation_h;
+  r.dw = d.dilation_w;
+  r.pt = d.pad_t;
+  r.pl = d.pad_l;
+  r.nhwc_in = c.pack;
+  r.ep.act_pre = c.squeeze >= 0 ? first.act_pre : GI_ACT_NONE;
+  r.ep2.act_pre = a.act_pre;
+  r.ep2.has_res = c.sum >= 0 || a.residual >= 0;
+  r.ep2.act_post = c.sum >= 0 ? GI_ACT_NONE : a.act_post;
+  r.lead = c.squeeze;
+  r.conv_a = c.a;
+  r.conv_b = c.b;
+  r.sum_op = c.sum;
+  return r;
+}
+
 // Estimated time of the run's ops as launches of their own: 4 us each (what a launch adds to a chain of them) plus their bytes
 // at the rates the kernels reach inside MobileNetV2 - 6 TB/s, 3.2 for a stencil on planes without a straight-line form, 4 for
 // the stem - plus 4 ns (1.2 ns where eight warps share the sum) per input channel of a 1x1 convolution, its chain of matrix instructions.  Against the measured
 // times of the network's ops at batch 1, 21 and 256 it is within 15 %.
-static double separate_us(const gi_exec* e, const OpGroup& gr) {
+static double separate_us(const gi_graph& g, const gi_exec* e, const OpGroup& gr) {
   double us = 0.0;
   auto bytes = [&](int t) {
     return t < 0 ? 0.0 : 2.0 * e->batch * e->tensors[t].h * e->tensors[t].w * slices(e->tensors[t].c) * 4;
@@ -381,6 +491,14 @@ static double separate_us(const gi_exec* e, const OpGroup& gr) {
       pw.H = e->tensors[o.in0].h;
       pw.W = e->tensors[o.in0].w;
       pw.Co = e->tensors[o.out].c;
+      const gi_op_desc& d = g.ops[o.graph_op].d;
+      if (gr.kind == GROUP_CONV && !is_plain_pointwise(d)) {
+        // conv_tc.cu: every window position gathered at 5.3 TB/s or the output written at 2.3, 10 ns per 1 x 1 x 1 of the sum
+        const double px = static_cast<double>(e->batch) * e->tensors[o.out].h * e->tensors[o.out].w, taps = d.kh * d.kw;
+        us += 4.0 + 0.01 * taps * e->tensors[o.in0].c +
+              std::max(8 * px * taps * slices(e->tensors[o.in0].c) / 5.3e6, 8 * px * slices(e->tensors[o.out].c) / 2.3e6);
+        continue;
+      }
       if (gr.rec.stem_h > 0 && i == gr.rec.lead) rate = 4.0e6;
       else us += (pointwise_mma_wanted(pw) ? 0.0012 : 0.004) * e->tensors[o.in0].c;
     }
@@ -409,6 +527,24 @@ void find_groups(const gi_graph& g, gi_exec* e) {
       ++i;
       continue;
     }
+    if (e->opt.planner != GI_PLAN_NAIVE) {
+      ConvOps c = fire_at(g, e, i);
+      if (c.n == 0) c = conv_at(g, e, i);
+      if (c.n != 0) {
+        OpGroup gr;
+        gr.first = static_cast<int>(i);
+        gr.n = c.n;
+        gr.kind = GROUP_CONV;
+        gr.rec = conv_rec(g, e, c);
+        // the 3-channel stem has a kernel of its own
+        const bool stem = conv3x3_tc_supported(gr.rec.C, gr.rec.Co, gr.rec.kh, gr.rec.kw, gr.rec.sh, gr.rec.sw, gr.rec.dh, gr.rec.dw);
+        if (!stem && conv_mma_choose(gr.rec, &gr.rec.block, &gr.us) && gr.us <= separate_us(g, e, gr)) {
+          e->groups.push_back(gr);
+          i += c.n - 1;
+          continue;
+        }
+      }
+    }
     const BlockOps b = block_ops_at(g, e, i);
     if (b.n == 0) continue;
     OpGroup gr;
@@ -425,7 +561,7 @@ void find_groups(const gi_graph& g, gi_exec* e) {
         us = o.us;
       }
     if (us == 0.0 && !block_mma_choose(gr.rec, b.kind, &gr.rec.block, &us)) continue;
-    if (us > separate_us(e, gr)) continue;
+    if (us > separate_us(g, e, gr)) continue;
     gr.kind = b.kind;
     gr.us = us;
     e->groups.push_back(gr);
@@ -475,6 +611,33 @@ static gi_status lower_pass(const gi_graph& g, gi_exec* e, bool grouped, bool pa
         r.out = Loc{W_OUTPUT, e->ops[i + 1].io_index, 0};
         info.bytes = (B * d.h * d.w * slices(d.c) * 4 + B * o.h * o.w * o.c) * eb;
         info.flops = 8 * B * o.h * o.w * o.c;
+      } else if (gr->kind == GROUP_CONV && static_cast<int>(i) == gr->first) {
+        r = gr->rec;
+        const FusedOp& a = e->ops[r.conv_a];
+        const FusedOp& last = e->ops[gr->first + gr->n - 1];
+        const OpNode* ws = r.lead >= 0 ? &g.ops[e->ops[r.lead].graph_op] : nullptr;
+        const OpNode& wa = g.ops[a.graph_op];
+        const OpNode* wb = r.conv_b >= 0 ? &g.ops[e->ops[r.conv_b].graph_op] : nullptr;
+        const int in = r.lead >= 0 ? e->ops[r.lead].in0 : a.in0;
+        int res = a.residual;
+        if (r.sum_op >= 0) {
+          const int cat = e->ops[r.sum_op - 1].out;
+          res = e->ops[r.sum_op].in0 == cat ? e->ops[r.sum_op].in1 : e->ops[r.sum_op].in0;
+        }
+        r.in0 = r.nhwc_in ? Loc{W_INPUT, e->tensors[in].input_index, 0} : loc_of(e, in);
+        r.out = loc_of(e, last.out);
+        r.res = loc_of(e, res);
+        if (pack)
+          conv_mma_pack(ws ? ws->weights.data() : nullptr, ws ? ws->bias.data() : nullptr, wa.weights.data(), wa.bias.data(), wa.d.kh, wa.d.cout,
+                        wb ? wb->weights.data() : nullptr, wb ? wb->bias.data() : nullptr, wb ? wb->d.kh : 0, r.C, r.Cmid, r.Co, r.kh,
+                        &e->weight_blob, &r);
+        const uint64_t px_in = B * r.H * r.W, px_out = B * r.Ho * r.Wo, cz = r.Cmid ? r.Cmid : r.C;
+        uint64_t per_px = 0;  // multiply-adds of an output pixel
+        for (const OpNode* w : {&wa, wb})
+          if (w) per_px += static_cast<uint64_t>(w->d.kh) * w->d.kw * w->d.cout * cz;
+        info.bytes = (px_in * (r.nhwc_in ? r.C : slices(r.C) * 4) + px_out * slices(r.Co) * 4 * (r.ep2.has_res ? 2 : 1) + per_px +
+                      static_cast<uint64_t>(r.C) * r.Cmid) * eb;
+        info.flops = 2 * px_out * per_px + 2 * px_in * r.C * r.Cmid;
       } else if (static_cast<int>(i) == gr->first) {
         r = gr->rec;
         const int lead = r.lead;

@@ -112,6 +112,7 @@ static gi_status run_impl(gi_exec* e, const void* const* dev_inputs, void* const
       case GI_KERNEL_POINTWISE_CHAIN: err = launch_pointwise_chain(r, p, &e->tc_state, static_cast<int>(i), stream); break;
       case GI_KERNEL_BLOCK_MMA: err = launch_block_mma(r, p, stream); break;
       case GI_KERNEL_POINTWISE_MMA: err = launch_pointwise_mma(r, p, &e->tc_state, static_cast<int>(i), stream); break;
+      case GI_KERNEL_CONV_MMA: err = launch_conv_mma(r, p, stream); break;
       case GI_KERNEL_NONE: break;  // computed by the previous launch
       case GI_KERNEL_ELTWISE:
         if (r.ep.has_res && !p.in1) p.in1 = p.res;
@@ -146,6 +147,7 @@ gi_status gi_device_status(uint32_t* flags) {
   if (err == 0) *flags |= pointwise_chain_error_word(&err) << 12;
   if (err == 0) *flags |= pointwise_mma_error_word(&err) << 3;
   if (err == 0) *flags |= stem_block_error_word(&err) << 3;
+  if (err == 0) *flags |= conv_mma_error_word(&err) << 3;
   if (err != 0) return fail(GI_E_CUDA, std::string("gi_device_status: ") + cudaGetErrorString(static_cast<cudaError_t>(err)));
   return GI_OK;
 }

@@ -117,6 +117,13 @@ void stem_block_pack(const float* ws, const float* bs, const float* wd, const fl
 int launch_stem_block(const LaunchRec& r, const Ptrs& p, void* stream);
 unsigned int stem_block_error_word(int* cuda_err);
 
+// k x k convolution with few channels, alone or as a fire module (fp16 storage; conv_mma.cu)
+bool conv_mma_choose(const LaunchRec& r, BlockCfg* cfg, double* us);
+void conv_mma_pack(const float* sq, const float* sqb, const float* wa, const float* ba, int ka, int c1, const float* wb, const float* bb, int kb,
+                   int cin, int csq, int cout, int k, std::vector<uint8_t>* blob, LaunchRec* r);
+int launch_conv_mma(const LaunchRec& r, const Ptrs& p, void* stream);
+unsigned int conv_mma_error_word(int* cuda_err);
+
 // Pointwise convolution for launches bound by latency (fp16 storage; pointwise_mma.cu)
 bool pointwise_mma_wanted(const LaunchRec& r);
 void pointwise_mma_pack(const float* w, const float* bias, int cin, int cout, std::vector<uint8_t>* blob, LaunchRec* r);

@@ -1052,3 +1052,56 @@ def test_pointwise_of_few_tiles(case):
     again = run.run(xs)
     assert all(np.array_equal(outs[t], again[t]) for t in spec.outputs)
     assert api.gi_device_status() == 0
+
+
+def _fire_module(batch, h, w, cin, squeeze, e1, e3, residual, swap=False, dilation=1):
+    b = wl.GraphBuilder("fire_module", batch, 18)
+    x = b.activation(b.conv2d(b.input(h, w, 4), cin, 1), wl.ACT_RELU)
+    s = b.activation(b.conv2d(x, squeeze, 1), wl.ACT_RELU)
+    one = b.activation(b.conv2d(s, e1, 1), wl.ACT_RELU6)
+    three = b.activation(b.conv2d(s, e3, 3, 1, dilation), wl.ACT_RELU6)
+    y = b.concat(three, one) if swap else b.concat(one, three)
+    b.output(b.add(x, y) if residual else y)
+    return b.finish()
+
+
+def _window_conv(batch, h, w, cin, cout, k, stride, dilation=1, residual=False, nhwc=False):
+    b = wl.GraphBuilder("window_conv", batch, 19)
+    x = b.input(h, w, cin)
+    if not nhwc:
+        x = b.conv2d(x, cin, 1)
+    y = b.activation(b.conv2d(x, cout, k, stride, dilation), wl.ACT_RELU)
+    b.output(b.add(x, y) if residual else y)
+    return b.finish()
+
+
+CONV_MMA_CASES = {
+    # channel counts off every multiple, both orders of the parts, planes smaller than a tile, odd, several tiles, many units
+    "fire": lambda: _fire_module(2, 24, 24, 24, 8, 16, 16, False), "fire_ragged": lambda: _fire_module(3, 13, 9, 21, 5, 7, 14, False),
+    "fire_sum": lambda: _fire_module(2, 16, 16, 48, 12, 23, 25, True), "fire_swap": lambda: _fire_module(1, 31, 33, 32, 16, 9, 30, False, swap=True),
+    "fire_dilated": lambda: _fire_module(1, 20, 22, 16, 8, 8, 8, True, dilation=2), "fire_many": lambda: _fire_module(80, 40, 41, 8, 8, 10, 6, False),
+    "fire_tiny": lambda: _fire_module(1, 3, 2, 64, 3, 1, 2, False),
+    # window, stride and padding; the caller's NHWC image; a residual; few and many output channels
+    "conv2": lambda: _window_conv(2, 30, 31, 48, 64, 2, 1), "conv3_s3": lambda: _window_conv(4, 48, 47, 32, 48, 3, 3),
+    "conv3_s2": lambda: _window_conv(2, 17, 19, 10, 20, 3, 2), "conv1_s2": lambda: _window_conv(2, 15, 16, 12, 9, 1, 2),
+    "conv3_dilated": lambda: _window_conv(1, 19, 21, 8, 16, 3, 1, 2), "conv3_sum": lambda: _window_conv(2, 18, 15, 12, 12, 3, 1, residual=True),
+    "conv2_image": lambda: _window_conv(3, 33, 35, 3, 24, 2, 2, nhwc=True), "conv3_image4": lambda: _window_conv(2, 21, 20, 4, 33, 3, 1, nhwc=True),
+}
+
+
+@pytest.mark.parametrize("case", list(CONV_MMA_CASES))
+def test_window_convolutions_and_fire_modules_as_one_kernel(case):
+    spec = CONV_MMA_CASES[case]()
+    xs = [wl.make_input(spec)]
+    run = DeviceRun(spec, api.GI_F16, guard_bytes=4096)
+    names = [api.KERNEL_NAMES[launch.kernel] for launch in run.ex.launches()]
+    if case != "conv3_image4":  # (one input slice, 3x3: the stem's kernel)
+        assert "conv_mma" in names and "concat" not in names and "eltwise" not in names, names
+    outs = run.run(xs)
+    assert run.guard_intact()
+    t = spec.outputs[0]
+    if spec.batch <= 4:
+        assert_close(outs[t], og.run(spec, xs, storage="f16", fused=True)[t], api.GI_F16, case)
+    assert_close(outs[t], DeviceRun(spec, api.GI_F16, cross_op=api.GI_XOP_OFF).run(xs)[t], api.GI_F16, "one kernel per op")
+    assert np.array_equal(outs[t], run.run(xs)[t])
+    assert api.gi_device_status() == 0
