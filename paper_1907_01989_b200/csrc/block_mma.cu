@@ -74,8 +74,9 @@ enum First { kNone = 0, kExp16 = 1, kExp24 = 2, kExp32 = 3, kExpWide = 4 };
 __host__ __device__ constexpr int slice_bytes(int first, bool small) { return (small ? 9 : first == kExpWide ? 18 : 36) * 128 + 32; }
 __host__ __device__ constexpr int tile_pixels(int first, bool small) { return slice_bytes(first, small) / 8 - 2; }
 // warps an SM holds: 128 registers a thread for 16 warps, 255 for 8 (96 sums per thread and more; tr: output rows a warp
-// walks down)
-__host__ __device__ constexpr int max_warps(int s, int np, int tr) { return (s == 1 ? tr : 1) * np >= 6 || tr == 4 ? 8 : 16; }
+// walks down), 168 for 12 where 64 sums and the fragments of four rows do not fit 128 (28x28 32 -> 192 -> 32 at batch 256: 77 us
+// with 416 bytes of spills in the loop, 69 with 12 warps; 26x26 at batch 21 18.7 -> 16.9)
+__host__ __device__ constexpr int max_warps(int s, int np, int tr) { return (s == 1 ? tr : 1) * np >= 6 || tr == 4 ? 8 : s == 1 && tr == 2 && np == 2 ? 12 : 16; }
 // bytes of one 16-channel sub-block of packed weights: first operator's fragments and bias, banded depthwise operands and
 // bias, projection fragments
 __host__ __device__ constexpr int sub_bytes(int ke, int np) { return ke * 512 + kSubFixed + np * 512; }
@@ -807,9 +808,9 @@ int cluster_slots(int ks) { return ks == 8 ? 15 : ks == 4 ? 33 : ks == 2 ? 73 : 
 
 // Estimated time of a launch, for choosing a configuration.  Two bounds, both in SM cycles: the chain of one CTA's units (its
 // chunks one after the other, `lat`), and the throughput of an SM's matrix and shared-memory pipes under all its CTAs'
-// units (`thr`).  The coefficients are a least-squares fit to 6100 measured launches (110 shapes of MobileNetV2 at batch 1 to
-// 256 and image sizes 128 to 513, about 50 configurations each; rms error 13 %; the configuration it picks takes 1.07 times
-// the best one's time in the geometric mean), and to 3000 more for units that several CTAs or warp sets share (11 %, 1.04).
+// units (`thr`).  The coefficients are least-squares fits: of units that one CTA computes to 2060 measured launches (ten shapes at
+// batch 2 to 256 and image sizes 128 to 513; rms error 8 %), of units that several CTAs or warp sets share to 3000 more (11 %;
+// the configuration it picks takes 1.04 times the best one's time in the geometric mean).
 double block_cost_us(const LaunchRec& r, const BlockCfg& c, const Layout& l) {
   const int ke = ke_of(r, c), nv = c.s == 1 ? c.tr : c.tr / 2;
   const int occ = ctas_per_sm(c, l), slots = cluster_slots(c.ks) * occ;
@@ -818,16 +819,23 @@ double block_cost_us(const LaunchRec& r, const BlockCfg& c, const Layout& l) {
   const double nchl = (l.nch + c.ks - 1) / c.ks, ew = std::max(l.eg, l.en), thr_n = l.nw * 32.0;
   const double dw = (4.0 * (c.s == 1 ? 3 : 5) * nv + 4.0 * c.np * nv) * c.hc;
   const double wk = std::max(1, c.wk), src = c.ks * wk;
-  double lat;
   if (src == 1) {
-    lat = 236.8 + (nchl + 1) * (443 + 34.49 * ew * ke * c.hc + 6.063 * dw + 521.9 * c.hc) + 695.4 * c.np * nv;
-    if (c.first == kNone) lat += (nchl + 1) * 14.16 * l.n_list * 4 / thr_n;
-  } else {
-    const int tiles = l.ngroups * nv * c.np, own = (tiles + c.ks - 1) / c.ks, rounds = (own + l.nw - 1) / l.nw;  // tiles a warp adds up
-    lat = (nchl + 1) * (459.1 + 68.17 * ew * ke * c.hc + 3.99 * dw + 75.98 * l.nw) + 78.48 * c.np * nv + rounds * (1581 + 96.46 * src);
-    if (c.first == kNone) lat += (nchl + 1) * 30.31 * l.n_list * 4 * wk / thr_n;
-    if (c.ks > 1) lat += 1561;
+    const int first = c.first != kNone;
+    const double e = c.hc * (4.17 + 76 * ke), d = 82.5 + 3.83 * dw + 977 * c.hc;  // a group of list pixels, of columns
+    const double step = 353 + std::max(l.eg * e + d, l.en * e);                   // from one chunk's barrier to the next
+    double lat = 815 + (l.nch + first) * step + 520 * c.np * nv;
+    lat += first ? 4.47 * l.n_list * slices(r.C) / thr_n : 82.0 * l.nch * c.hc * l.n_list * 4 / thr_n;
+    const double rows = 4.0 * (c.s == 1 ? c.tr + 2 : 2 * c.tr + 1);  // fragments of a column group's hidden rows
+    double thr = 43.4 + 121 * l.ngroups * c.np * nv;
+    thr += l.nch * c.hc * (l.mt * (3.75 * first + 10.74 * ke) + l.ngroups * (0.47 * dw / c.hc + 0.57 * rows + 124.9));
+    thr += first ? 0.43 * l.n_list * slices(r.C) : 0.26 * l.n_list * l.nch * c.hc * 4;
+    const double a = upc * lat, b = upc * per_sm * thr;
+    return 3.02 + std::cbrt(a * a * a + b * b * b) / 1900.0;
   }
+  const int tiles = l.ngroups * nv * c.np, own = (tiles + c.ks - 1) / c.ks, rounds = (own + l.nw - 1) / l.nw;  // tiles a warp adds up
+  double lat = (nchl + 1) * (459.1 + 68.17 * ew * ke * c.hc + 3.99 * dw + 75.98 * l.nw) + 78.48 * c.np * nv + rounds * (1581 + 96.46 * src);
+  if (c.first == kNone) lat += (nchl + 1) * 30.31 * l.n_list * 4 * wk / thr_n;
+  if (c.ks > 1) lat += 1561;
   double thr = 317.1 + 130.4 * l.ngroups * c.np * nv * wk +
                nchl * wk * (3.538 * l.mt * ke * 2 * c.hc + 4.459 * l.ngroups * dw + 74.9 * l.ngroups * c.hc);
   if (c.first != kNone) thr += 1.235 * l.n_list * slices(r.C);
@@ -948,7 +956,7 @@ void each_config(const LaunchRec& r, int kind, F&& f) {
             c.hc = c.first == kExpWide && c.wk == 0 ? 2 : 1;
             for (c.ks = 1; c.ks <= 8; c.ks *= 2) {
               if (c.ks > 1 && units * c.ks > 148 * 2) break;  // a split pays only while SMs would be idle ...
-              for (c.nw_min = 8; c.nw_min <= max_warps(c.s, c.np, c.tr); c.nw_min += 8) {
+              for (c.nw_min = 8; c.nw_min <= max_warps(c.s, c.np, c.tr); c.nw_min += max_warps(c.s, c.np, c.tr) == 12 ? 4 : 8) {
                 for (int rk = 0; rk < 2; ++rk) {
                   c.resident_kb = rk ? 48 : 0;
                   Layout l;
