@@ -413,29 +413,28 @@ __global__ void concat_kernel(const T* __restrict__ a, const T* __restrict__ b, 
 }
 
 // ------------------------------------------------------------------ global average pool
-// eight lanes per (slice, image), four planes per warp: a lane strides over the pixels with all its
+// eight lanes (or a whole warp, launch_pool) per (slice, image): a lane strides over the pixels with all its
 // loads independent (many small planes are latency-bound otherwise), then a shuffle reduction over
-// the eight lanes in a fixed order
-template <typename T>
+// the lanes in a fixed order
+template <typename T, int L>
 __global__ void pool_kernel(const T* __restrict__ in, T* __restrict__ out, int planes, int HW, int Pin, int Pout) {
   pdl_launch_dependents();
   pdl_wait();
-  const int lane = threadIdx.x & 31, sub = lane & 7;
-  const int plane_id = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 4 + (lane >> 3);
+  const int sub = threadIdx.x % L, plane_id = (blockIdx.x * blockDim.x + threadIdx.x) / L;
   const bool live = plane_id < planes;
   float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
   if (live) {
     const T* plane = in + static_cast<size_t>(plane_id) * Pin * 4;
     int p = sub;
-    for (; p + 24 < HW; p += 32) {  // four loads in flight
-      const float4 x0 = Px<T>::load(plane + static_cast<size_t>(p) * 4), x1 = Px<T>::load(plane + static_cast<size_t>(p + 8) * 4);
-      const float4 x2 = Px<T>::load(plane + static_cast<size_t>(p + 16) * 4), x3 = Px<T>::load(plane + static_cast<size_t>(p + 24) * 4);
+    for (; p + 3 * L < HW; p += 4 * L) {  // four loads in flight
+      const float4 x0 = Px<T>::load(plane + static_cast<size_t>(p) * 4), x1 = Px<T>::load(plane + static_cast<size_t>(p + L) * 4);
+      const float4 x2 = Px<T>::load(plane + static_cast<size_t>(p + 2 * L) * 4), x3 = Px<T>::load(plane + static_cast<size_t>(p + 3 * L) * 4);
       s.x += (x0.x + x1.x) + (x2.x + x3.x);
       s.y += (x0.y + x1.y) + (x2.y + x3.y);
       s.z += (x0.z + x1.z) + (x2.z + x3.z);
       s.w += (x0.w + x1.w) + (x2.w + x3.w);
     }
-    for (; p < HW; p += 8) {
+    for (; p < HW; p += L) {
       const float4 x = Px<T>::load(plane + static_cast<size_t>(p) * 4);
       s.x += x.x;
       s.y += x.y;
@@ -443,11 +442,11 @@ __global__ void pool_kernel(const T* __restrict__ in, T* __restrict__ out, int p
       s.w += x.w;
     }
   }
-  for (int d = 4; d > 0; d >>= 1) {
-    s.x += __shfl_down_sync(0xffffffffu, s.x, d, 8);
-    s.y += __shfl_down_sync(0xffffffffu, s.y, d, 8);
-    s.z += __shfl_down_sync(0xffffffffu, s.z, d, 8);
-    s.w += __shfl_down_sync(0xffffffffu, s.w, d, 8);
+  for (int d = L / 2; d > 0; d >>= 1) {
+    s.x += __shfl_down_sync(0xffffffffu, s.x, d, L);
+    s.y += __shfl_down_sync(0xffffffffu, s.y, d, L);
+    s.z += __shfl_down_sync(0xffffffffu, s.z, d, L);
+    s.w += __shfl_down_sync(0xffffffffu, s.w, d, L);
   }
   if (live && sub < Pout) {
     const float inv = 1.0f / static_cast<float>(HW);
@@ -784,12 +783,18 @@ int launch_concat(const LaunchRec& r, const Ptrs& p, int storage, void* stream) 
 
 int launch_pool(const LaunchRec& r, const Ptrs& p, int storage, void* stream) {
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const int planes = slices(r.C) * r.B;
-  const unsigned blocks = blocks_for(static_cast<size_t>(planes) * 8, 256);
-  GI_BY_STORAGE((launch_pdl(pool_kernel<__half>, blocks, 256, 0, st, static_cast<const __half*>(p.in0), static_cast<__half*>(p.out), planes,
-                                                            r.H * r.W, plane_pixels(r.H, r.W), plane_pixels(1, 1))),
-                (launch_pdl(pool_kernel<float>, blocks, 256, 0, st, static_cast<const float*>(p.in0), static_cast<float*>(p.out), planes,
-                                                           r.H * r.W, plane_pixels(r.H, r.W), plane_pixels(1, 1))));
+  const int planes = slices(r.C) * r.B, HW = r.H * r.W, Pin = plane_pixels(r.H, r.W), Pout = plane_pixels(1, 1);
+  // a whole warp for a plane of 128 pixels and more while eight lanes each would leave SMs without work (64 images of 16x16x64,
+  // 32 CTAs: 10.2 us between events, 128 CTAs: 7.0)
+  const bool warp = HW >= 128 && planes <= 148 * 32;
+  const unsigned blocks = blocks_for(static_cast<size_t>(planes) * (warp ? 32 : 8), 256);
+#define GI_POOL(T, L) (launch_pdl(pool_kernel<T, L>, blocks, 256, 0, st, static_cast<const T*>(p.in0), static_cast<T*>(p.out), planes, HW, Pin, Pout))
+  if (warp) {
+    GI_BY_STORAGE(GI_POOL(__half, 32), GI_POOL(float, 32));
+  } else {
+    GI_BY_STORAGE(GI_POOL(__half, 8), GI_POOL(float, 8));
+  }
+#undef GI_POOL
   return static_cast<int>(cudaGetLastError());
 }
 

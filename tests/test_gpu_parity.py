@@ -1105,3 +1105,13 @@ def test_window_convolutions_and_fire_modules_as_one_kernel(case):
     assert_close(outs[t], DeviceRun(spec, api.GI_F16, cross_op=api.GI_XOP_OFF).run(xs)[t], api.GI_F16, "one kernel per op")
     assert np.array_equal(outs[t], run.run(xs)[t])
     assert api.gi_device_status() == 0
+
+
+# eight lanes a plane; a warp a plane (128 pixels and more, up to 4736 planes): the smallest plane, odd ones, the largest count
+@pytest.mark.parametrize("case", [(2, 7, 9, 20), (1, 8, 16, 12), (3, 33, 35, 7), (37, 16, 16, 512), (38, 16, 16, 512)])
+@pytest.mark.parametrize("storage", [api.GI_F16, api.GI_F32])
+def test_average_pool_lanes(case, storage):
+    batch, h, w, c = case
+    b = wl.GraphBuilder("pool", batch, 20)
+    b.output(b.global_avg_pool(b.input(h, w, c)))
+    check_outputs(b.finish(), storage, images=list(range(min(batch, 3))))
