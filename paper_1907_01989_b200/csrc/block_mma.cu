@@ -830,7 +830,10 @@ double block_cost_us(const LaunchRec& r, const BlockCfg& c, const Layout& l) {
     thr += l.nch * c.hc * (l.mt * (3.75 * first + 10.74 * ke) + l.ngroups * (0.47 * dw / c.hc + 0.57 * rows + 124.9));
     thr += first ? 0.43 * l.n_list * slices(r.C) : 0.26 * l.n_list * l.nch * c.hc * 4;
     const double a = upc * lat, b = upc * per_sm * thr;
-    return 3.02 + std::cbrt(a * a * a + b * b * b) / 1900.0;
+    const double us = 3.02 + std::cbrt(a * a * a + b * b * b) / 1900.0;
+    // what the fit leaves on narrow expansions: long rows read and write better (56x56 24 -> 144 -> 24 at batch 256, tiles 28
+    // wide 175 us, 14 wide 202), a ring of weights costs its copies; the choice is then within 1.02 of the best, else 1.05
+    return c.first == kNone || c.first == kExpWide ? us : us * 0.965 * (1 + 1.0 / c.tw) * (l.resident ? 1 : 1.03);
   }
   const int tiles = l.ngroups * nv * c.np, own = (tiles + c.ks - 1) / c.ks, rounds = (own + l.nw - 1) / l.nw;  // tiles a warp adds up
   double lat = (nchl + 1) * (459.1 + 68.17 * ew * ke * c.hc + 3.99 * dw + 75.98 * l.nw) + 78.48 * c.np * nv + rounds * (1581 + 96.46 * src);
@@ -931,7 +934,7 @@ void each_config(const LaunchRec& r, int kind, F&& f) {
   if (r.B * in_plane * (kind == BLOCK_PAIR ? (r.C + 3) / 4 : 1) >= (1LL << 31)) return;  // offsets inside the input are 32-bit
   if (static_cast<int64_t>(r.Ho) * r.Wo * std::max(4, r.Co2) >= (1LL << 31)) return;
   c.hc = c.first == kExpWide ? 2 : 1;
-  const int wo_even = (r.Wo + 1) / 2 * 2;
+  const int wo_even = (r.Wo + 1) / 2 * 2, chid = kind == BLOCK_PAIR ? r.C : r.Cmid;
   const int tr_hi = c.s == 2 ? 2 : c.np == 1 ? 4 : c.np <= 4 ? 2 : 1, tr_lo = c.s == 2 ? 2 : c.np == 1 ? 2 : 1;
   for (c.tr = tr_lo; c.tr <= tr_hi; c.tr *= 2)
     for (int tx = 1; tx <= 32; ++tx) {
@@ -953,6 +956,7 @@ void each_config(const LaunchRec& r, int kind, F&& f) {
           const bool sets = units <= 148 && hid <= tile_pixels(c.first, true);
           for (int wi = 0; wi < (sets ? 9 : 1); ++wi) {
             c.wk = kSets[wi];
+            if ((c.wk - 1) * 16 >= chid) break;  // a set without channels
             c.hc = c.first == kExpWide && c.wk == 0 ? 2 : 1;
             for (c.ks = 1; c.ks <= 8; c.ks *= 2) {
               if (c.ks > 1 && units * c.ks > 148 * 2) break;  // a split pays only while SMs would be idle ...
