@@ -39,8 +39,9 @@
 // What bounds it.  Small launches: that chain.  Large ones: nothing alone - on 56x56 24 -> 144 -> 24 at batch 256 a
 // chunk takes 1840 cycles of an SM for 800 of the matrix pipe, 770 of issue slots per scheduler and about 900 of shared
 // memory, with 16 warps to cover 21-cycle matrix and 30-cycle shared-memory latencies; 173 us against 194 us as three
-// kernels.  Measured on one B200 against separate kernels, MobileNetV2: batch 1 225 -> 160 us, 21 images of 205
-// pixels 340 -> 278, batch 256 1413 -> 1385; segmentation network batch 1 289 -> 211, batch 16 961 -> 807.
+// kernels.  Measured on one B200 against separate kernels, stem included
+// (stem_block.cu), MobileNetV2: batch 1 225 -> 155 us, 21 images of 205 pixels 340 -> 270, batch 256 1413 -> 1298;
+// segmentation network batch 1 289 -> 207, batch 16 961 -> 748.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
