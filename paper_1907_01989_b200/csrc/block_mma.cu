@@ -1138,7 +1138,7 @@ int launch_block_mma(const LaunchRec& r, const Ptrs& ptr, void* stream) {
   const BlockCfg& c = r.block;
   if (c.stem) return launch_stem_block(r, ptr, stream);
   Layout l;
-  if (!layout_of(r, c, &l)) return static_cast<int>(cudaErrorInvalidConfiguration);
+  if (r.dh != 1 || r.dw != 1 || !layout_of(r, c, &l)) return static_cast<int>(cudaErrorInvalidConfiguration);
   BlockParams p = params_of(r, c, l);
   p.in = static_cast<const __half*>(ptr.in0);
   p.res = static_cast<const __half*>(ptr.res);

@@ -553,14 +553,10 @@ void find_groups(const gi_graph& g, gi_exec* e) {
     gr.rec = block_rec(g, e, b);
     gr.rec.lead = b.first;
     gr.rec.dw_op = b.dw;
+    // Every block is asked about by itself: what the kernel runs depends on more than its sizes (dilation, padding, residual, the
+    // caller's layout), and the search takes 0.1 ms.
     double us = 0.0;
-    for (const OpGroup& o : e->groups)  // blocks of a network repeat: the same geometry, the same choice
-      if (o.kind == b.kind && o.rec.H == gr.rec.H && o.rec.W == gr.rec.W && o.rec.C == gr.rec.C && o.rec.Cmid == gr.rec.Cmid &&
-          o.rec.Co2 == gr.rec.Co2 && o.rec.sh == gr.rec.sh && o.rec.Ho == gr.rec.Ho && o.rec.Wo == gr.rec.Wo) {
-        gr.rec.block = o.rec.block;
-        us = o.us;
-      }
-    if (us == 0.0 && !block_mma_choose(gr.rec, b.kind, &gr.rec.block, &us)) continue;
+    if (!block_mma_choose(gr.rec, b.kind, &gr.rec.block, &us)) continue;
     if (us > separate_us(g, e, gr)) continue;
     gr.kind = b.kind;
     gr.us = us;

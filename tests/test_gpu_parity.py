@@ -1115,3 +1115,13 @@ def test_average_pool_lanes(case, storage):
     b = wl.GraphBuilder("pool", batch, 20)
     b.output(b.global_avg_pool(b.input(h, w, c)))
     check_outputs(b.finish(), storage, images=list(range(min(batch, 3))))
+
+
+# ---------------------------------------------------------------------- blocks of one geometry with and without dilation
+@pytest.mark.parametrize("batch,hw,c,hidden,dilations", [(1, 14, 64, 384, [1, 2]), (1, 33, 64, 384, [1, 2, 1, 4]), (1, 17, 160, 960, [1, 2]), (2, 33, 64, 0, [1, 2])])
+def test_dilated_blocks_behind_equal_undilated_ones(batch, hw, c, hidden, dilations):
+    from test_host_compile import equal_blocks
+    run, _, _ = check_outputs(equal_blocks(batch, hw, c, hidden, dilations), api.GI_F16)
+    names = [api.KERNEL_NAMES[launch.kernel] for launch in run.ex.launches()]
+    assert names.count("block_mma") == dilations.count(1) and names.count("depthwise") == len(dilations) - dilations.count(1), names
+    assert api.gi_device_status() == 0

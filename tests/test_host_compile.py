@@ -725,3 +725,32 @@ def test_grouped_launches_host_side():
     for storage, s in ((api.GI_F32, wl.depthwise_then_pointwise(1, 16, 16, 32, 32)), (api.GI_F16, pair)):
         ex = api.graph_from_spec(s, storage)[0].compile()
         assert "block_mma" not in [api.KERNEL_NAMES[x.kernel] for x in ex.launches()]
+
+
+def _launch_names(spec, **kw):
+    return [api.KERNEL_NAMES[x.kernel] for x in api.graph_from_spec(spec, api.GI_F16)[0].compile(**kw).launches()]
+
+
+def equal_blocks(batch, hw, c, hidden, dilations, workload_id=31):
+    """Residual blocks c -> hidden -> c (hidden 0: depthwise-separable pairs c -> c) of one geometry whose depthwise operators
+    differ in dilation alone."""
+    b = wl.GraphBuilder("equal_blocks", batch, workload_id)
+    x = b.activation(b.conv2d(b.input(hw, hw, 8), c, 1), wl.ACT_RELU6)
+    for d in dilations:
+        y = b.activation(b.conv2d(x, hidden, 1), wl.ACT_RELU6) if hidden else x
+        y = b.conv2d(b.activation(b.depthwise(y, 3, 1, d), wl.ACT_RELU6), c, 1)
+        x = b.add(x, y) if hidden else b.activation(y, wl.ACT_RELU6)
+    b.output(x)
+    return b.finish()
+
+
+@pytest.mark.parametrize("planner", PLANNERS)
+@pytest.mark.parametrize("batch,hw,c,hidden", [(1, 14, 64, 384), (1, 33, 64, 384), (1, 33, 96, 576), (1, 65, 32, 192), (1, 17, 160, 960), (1, 33, 64, 0), (8, 33, 64, 0)])
+def test_a_dilated_block_behind_an_equal_undilated_one_keeps_its_own_kernels(batch, hw, c, hidden, planner):
+    """The kernel that runs a whole block has no dilation: whatever stands in front of it, a dilated depthwise operator runs as a
+    launch of its own, and the choice for a block does not depend on the blocks before it."""
+    alone = [_launch_names(equal_blocks(batch, hw, c, hidden, [d]), planner=planner) for d in (1, 2)]
+    assert alone[0].count("block_mma") == 1 and alone[1].count("block_mma") == 0 and alone[1].count("depthwise") == 1
+    for dilations in ([1, 2], [2, 1], [1, 2, 1, 4]):
+        names = _launch_names(equal_blocks(batch, hw, c, hidden, dilations), planner=planner)
+        assert names.count("block_mma") == dilations.count(1) and names.count("depthwise") == len(dilations) - dilations.count(1), names
