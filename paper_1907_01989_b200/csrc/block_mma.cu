@@ -312,6 +312,7 @@ __global__ void __launch_bounds__(32 * max_warps(S, NP, TR), 1) block_mma_kernel
   const int total = nchl * my_units;
 
   pdl_launch_dependents();
+  if (p.ks > 1) cluster_arrive();  // (waited for before the first store into a neighbour's shared memory)
 
   auto load_weights = [&](int run, int c) {
     const unsigned dst = smem + (p.resident ? run : run & (kRing - 1)) * stage_bytes;
@@ -679,6 +680,7 @@ __global__ void __launch_bounds__(32 * max_warps(S, NP, TR), 1) block_mma_kernel
       // tile % ks; everybody stores into the owner's shared memory, which then adds up its tiles in the order of the sources.
       // (Reading the neighbours' shared memory instead took 2.5 us: eight round trips, one after the other.)
       const int src = rank * wk + wset, n_src = p.ks * wk;
+      if (p.ks > 1 && k == 0) cluster_wait();  // every CTA of the cluster has started
       if (has_group) {
 #pragma unroll
         for (int v = 0; v < NV; ++v)

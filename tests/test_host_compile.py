@@ -754,3 +754,12 @@ def test_a_dilated_block_behind_an_equal_undilated_one_keeps_its_own_kernels(bat
     for dilations in ([1, 2], [2, 1], [1, 2, 1, 4]):
         names = _launch_names(equal_blocks(batch, hw, c, hidden, dilations), planner=planner)
         assert names.count("block_mma") == dilations.count(1) and names.count("depthwise") == len(dilations) - dilations.count(1), names
+
+
+def test_block_kernel_knows_its_cluster_has_started_before_it_stores_into_it():
+    """The shared memory of another CTA may be touched only once that CTA is known to run.  Nothing in a result shows whether a
+    kernel made sure of it, so its source is read: an arrival at the start, the wait for it in front of the first such store."""
+    text = open(os.path.join(ROOT, "paper_1907_01989_b200", "csrc", "block_mma.cu")).read()
+    body = text[text.index("block_mma_kernel(const BlockParams p) {"):]
+    arrive, wait, store = (body.index(s) for s in ("cluster_arrive();", "cluster_wait();", "st_cluster_f4(at"))
+    assert arrive < body.index("pdl_wait();") < wait < store < body.index("cluster_sync();")
