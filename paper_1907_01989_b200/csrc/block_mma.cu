@@ -325,8 +325,10 @@ __global__ void __launch_bounds__(32 * max_warps(S, NP, TR), 1) block_mma_kernel
     load_weights(0, 0);
     if (1 < total) load_weights(1, 1 % nchl);
   }
-  // shared memory that must start at zero: borders of compact tiles, channels beyond the input's last slice
-  if (p.compact || (p.sin & 1)) {
+  // shared memory that must start at zero: borders of compact tiles, and the slices beyond the input's last one that the first
+  // operator's steps of 16 channels read (their weights are zero, but 0 x NaN is not)
+  const int step_slices = FIRST == kExp24 ? 6 : 4 * ke;
+  if (p.compact || p.sin < step_slices) {
     for (unsigned i = p.off_x + tid * 16; i < p.off_red; i += nthr * 16) sts128(smem + i, 0u, 0u, 0u, 0u);
   }
   for (int i = tid; i < NP * 4; i += nthr) cp_async16(smem + p.off_bias + i * 16, reinterpret_cast<const float4*>(p.bias) + i);

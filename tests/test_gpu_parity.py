@@ -1125,3 +1125,27 @@ def test_dilated_blocks_behind_equal_undilated_ones(batch, hw, c, hidden, dilati
     names = [api.KERNEL_NAMES[launch.kernel] for launch in run.ex.launches()]
     assert names.count("block_mma") == dilations.count(1) and names.count("depthwise") == len(dilations) - dilations.count(1), names
     assert api.gi_device_status() == 0
+
+
+def fill_shared_memory_with_nan():
+    """Leaves NaN in the shared memory of (nearly) every SM: a 1x1 convolution of 1536 channels of NaN on 145 tiles, whose stages
+    take 209 KB of each."""
+    spec = wl.single_pointwise(1, 68, 1536, 32)
+    run = DeviceRun(spec, api.GI_F16)
+    assert "pointwise_mma" in [api.KERNEL_NAMES[launch.kernel] for launch in run.ex.launches()]
+    run.run([np.full((1, 68, 68, 1536), np.nan, dtype=np.float32)])
+
+
+# widths of the expansion's input that leave two of the four slices of its last 16-channel step without channels (MobileNetV2's own
+# at other multipliers among them), on planes whose tile is not cleared for its border
+@pytest.mark.parametrize("batch,hw,cin", [(1, 33, 8), (40, 33, 8), (1, 33, 40), (30, 33, 40), (2, 33, 56), (1, 31, 72), (2, 33, 88), (1, 33, 136)])
+def test_blocks_whose_input_ends_inside_a_step_of_channels(batch, hw, cin):
+    spec = wl.inverted_residual_block(batch, hw, hw, cin, 6 * cin, cin, 1)
+    xs = [wl.make_input(spec)]
+    run = DeviceRun(spec, api.GI_F16)
+    names = [api.KERNEL_NAMES[launch.kernel] for launch in run.ex.launches()]
+    assert names.count("block_mma") == 1, names
+    fill_shared_memory_with_nan()
+    t = spec.outputs[0]
+    sel = [0, batch - 1]
+    assert_close(run.run(xs)[t][sel], og.run(spec, [xs[0][sel]], storage="f16", fused=True)[t], api.GI_F16, str((batch, hw, cin)))
