@@ -249,6 +249,15 @@ static int nhwc_pack_feeding_only(const gi_exec* e, int t, size_t reader) {
   return pack;
 }
 
+// Two activations with no sum between them are one: both clamp at zero, and a bound of 6 holds whichever of them brings it.  The
+// kernels on mma.sync look at the second one only behind a sum.
+static Epilogue one_activation(Epilogue ep) {
+  if (ep.has_res || ep.act_post == GI_ACT_NONE) return ep;
+  if (ep.act_pre != GI_ACT_RELU6) ep.act_pre = ep.act_post;
+  ep.act_post = GI_ACT_NONE;
+  return ep;
+}
+
 static bool clamps_at_zero(int act) { return act == GI_ACT_RELU || act == GI_ACT_RELU6; }
 
 // A run of executed ops that block_mma.cu may run as one kernel: `n` ops of which the first `lead` stand in front of the
@@ -335,6 +344,7 @@ static LaunchRec block_rec(const gi_graph& g, const gi_exec* e, const BlockOps& 
   r.ep2.act_pre = c.act_pre;
   r.ep2.has_res = c.residual >= 0;
   r.ep2.act_post = c.act_post;
+  r.ep2 = one_activation(r.ep2);
   r.nhwc_in = b.pack;
   r.nhwc_out = b.unpack;
   if (b.kind == BLOCK_STEM) {
@@ -460,6 +470,7 @@ static LaunchRec conv_rec(const gi_graph& g, const gi_exec* e, const ConvOps& c)
   r.ep2.act_pre = a.act_pre;
   r.ep2.has_res = c.sum >= 0 || a.residual >= 0;
   r.ep2.act_post = c.sum >= 0 ? GI_ACT_NONE : a.act_post;
+  r.ep2 = one_activation(r.ep2);
   r.lead = c.squeeze;
   r.conv_a = c.a;
   r.conv_b = c.b;
@@ -892,6 +903,7 @@ static gi_status lower_pass(const gi_graph& g, gi_exec* e, bool grouped, bool pa
           if (grouped && pointwise && tc && e->opt.fuse && e->opt.pointwise == GI_PW_AUTO && e->opt.cross_op == GI_XOP_AUTO &&
               pointwise_mma_wanted(r)) {
             r.kernel = GI_KERNEL_POINTWISE_MMA;
+            r.ep = one_activation(r.ep);
             if (unpack_next) {
               r.nhwc_out = 1;
               r.out = Loc{W_OUTPUT, e->ops[i + 1].io_index, 0};

@@ -1149,3 +1149,38 @@ def test_blocks_whose_input_ends_inside_a_step_of_channels(batch, hw, cin):
     t = spec.outputs[0]
     sel = [0, batch - 1]
     assert_close(run.run(xs)[t][sel], og.run(spec, [xs[0][sel]], storage="f16", fused=True)[t], api.GI_F16, str((batch, hw, cin)))
+
+
+def _twice_activated(kind, first, second):
+    b = wl.GraphBuilder("twice_activated", 2, 32)
+    if kind == "stem":
+        y = b.activation(b.conv2d(b.input(33, 30, 3), 32, 3, 2), wl.ACT_RELU)
+    else:
+        y = b.input(15, 14, 32)
+    if kind == "block":
+        y = b.activation(b.conv2d(y, 96, 1), wl.ACT_RELU)
+    if kind in ("stem", "block", "pair"):
+        y = b.activation(b.depthwise(y, 3, 1), wl.ACT_RELU)
+    if kind == "fire":
+        s = b.activation(b.conv2d(b.conv2d(y, 16, 1), 8, 1), wl.ACT_RELU)
+        y = b.concat(b.activation(b.conv2d(s, 8, 1), first), b.activation(b.conv2d(s, 8, 3), first))
+        b.output(b.activation(y, second))
+        return b.finish()
+    y = b.conv2d(b.conv2d(y, 32, 1) if kind == "window" else y, 24, 3 if kind == "window" else 1)
+    b.output(b.activation(b.activation(y, first), second))
+    return b.finish()
+
+
+@pytest.mark.parametrize("first,second", [(wl.ACT_RELU, wl.ACT_RELU6), (wl.ACT_RELU6, wl.ACT_RELU), (wl.ACT_RELU, wl.ACT_RELU)])
+@pytest.mark.parametrize("kind,kernel", [("pointwise", "pointwise_mma"), ("window", "conv_mma"), ("fire", "conv_mma"), ("pair", "block_mma"), ("block", "block_mma"),
+                                         ("stem", "block_mma")])
+def test_a_second_activation_without_a_sum_between(kind, kernel, first, second):
+    """conv -> activation -> activation is one operator; inputs 32 times as large as elsewhere bring values above 6."""
+    spec = _twice_activated(kind, first, second)
+    x = wl.make_input(spec) * 32
+    run = DeviceRun(spec, api.GI_F16)
+    assert kernel in [api.KERNEL_NAMES[launch.kernel] for launch in run.ex.launches()]
+    t = spec.outputs[0]
+    ref = og.run(spec, [x], storage="f16", fused=True)[t]
+    assert ref.max() == 6.0 if wl.ACT_RELU6 in (first, second) else ref.max() > 6.0
+    assert_close(run.run([x])[t], ref, api.GI_F16, kind)
