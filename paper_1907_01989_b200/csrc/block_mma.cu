@@ -937,6 +937,7 @@ void each_config(const LaunchRec& r, int kind, F&& f) {
   if (c.np == 0) return;
   const int64_t in_plane = static_cast<int64_t>(plane_pixels(r.H, r.W)) * 4;
   if (r.B * in_plane * (kind == BLOCK_PAIR ? (r.C + 3) / 4 : 1) >= (1LL << 31)) return;  // offsets inside the input are 32-bit
+  if (r.nhwc_in && static_cast<int64_t>(r.H) * r.W * r.C >= (1LL << 31)) return;  // and so is an image of the caller's tensor
   if (static_cast<int64_t>(r.Ho) * r.Wo * std::max(4, r.Co2) >= (1LL << 31)) return;
   c.hc = c.first == kExpWide ? 2 : 1;
   const int wo_even = (r.Wo + 1) / 2 * 2, chid = kind == BLOCK_PAIR ? r.C : r.Cmid;

@@ -763,3 +763,12 @@ def test_block_kernel_knows_its_cluster_has_started_before_it_stores_into_it():
     body = text[text.index("block_mma_kernel(const BlockParams p) {"):]
     arrive, wait, store = (body.index(s) for s in ("cluster_arrive();", "cluster_wait();", "st_cluster_f4(at"))
     assert arrive < body.index("pdl_wait();") < wait < store < body.index("cluster_sync();")
+
+
+@pytest.mark.parametrize("hidden,cout", [(16, 16), (64, 32), (960, 160)])
+@pytest.mark.parametrize("c,w", [(32, 2048), (152, 1400), (160, 60), (160, 700)])
+def test_no_block_reads_an_image_of_the_callers_layout_beyond_32_bit_offsets(c, w, hidden, cout):
+    """Offsets inside an image of the caller's NHWC tensor are 32-bit: from 2^31 values on it is converted first (a slice of it is
+    small enough)."""
+    names = _launch_names(wl.inverted_residual_block(1, 2 ** 31 // (w * c) + 2, w, c, hidden, cout, 1))
+    assert names[0] == "pack", names
