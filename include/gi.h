@@ -26,7 +26,9 @@
  * follow one another: element (b,h,w,c) is at element index
  *     ((c/4 * B + b) * plane + h*W + w) * 4 + c%4,      plane = H*W rounded up to even.
  * The extra pixel of an odd plane must hold finite values (the library writes zeros or
- * finite values there).  Caller-visible tensors can instead be plain NHWC, in which case
+ * finite values there).  Inputs are expected to be finite altogether: several kernels multiply
+ * the pixels and channels beside a value by structural zeros, so what an infinity or a NaN in a
+ * stored tensor does to the values next to it depends on the kernel.  Caller-visible tensors can instead be plain NHWC, in which case
  * the executable starts / ends with a layout conversion kernel (Section 3, "Running
  * Inference").
  */
@@ -195,7 +197,9 @@ typedef struct gi_op_info {
 /* What gi_run launches at an executed op.  gi_op_info describes the ops one by one, each with the kernel chosen for it
  * alone; with GI_XOP_AUTO, GI_PW_AUTO, `fuse` set and fp16 storage, gi_run launches a depthwise 3x3 op with the ops
  * around it as ONE kernel where that is faster: the tensors between them are then never stored (their place in the arena
- * may hold anything), and results are those of the ops one after the other up to the order of fp32 sums.  Under
+ * may hold anything), and results are those of the ops one after the other up to the order of fp32 sums (a value of such a
+ * tensor beyond the range of fp16 is the largest finite one instead of infinity where its neighbours are multiplied by
+ * structural zeros: what a window convolution reads).  Under
  * GI_PLAN_NAIVE gi_op_info itself says so: its `kernel` is then that of the launch, and GI_KERNEL_NONE marks the ops inside
  * one.  (GI_XOP_OFF keeps one kernel per op.) */
 typedef struct gi_launch_info {

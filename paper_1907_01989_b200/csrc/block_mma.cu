@@ -110,7 +110,7 @@ struct BlockParams {
   unsigned off_bias, off_tab, off_src, off_x, off_hid, off_red;
   unsigned x_bytes, tab_bytes;  // of one of the two input tiles / tables (narrow expansions; otherwise there is one)
   unsigned mul_pitch, mul_w, mul_hw, mul_per, mul_tx;  // ceil(2^32 / d): division of a small number by d is one high multiplication
-  unsigned hi_e, hi_d;  // upper clamp of the hidden activations, two halves (6 or infinity)
+  unsigned hi_e, hi_d;  // upper clamp of the hidden activations, two halves (6; hi_e: or the largest finite value, hi_d: or infinity)
   int act_pre, act_post, has_res;
   int res_x;            // the residual is the block's input: it is still in shared memory
   int wide;             // both pixels of a pair are one aligned 16-byte store
@@ -1127,7 +1127,7 @@ BlockParams params_of(const LaunchRec& r, const BlockCfg& c, const Layout& l) {
   p.mul_hw = magic(static_cast<uint64_t>(r.H) * r.W);
   p.mul_per = magic(static_cast<uint64_t>(c.tiles_x) * c.tiles_y);
   p.mul_tx = magic(c.tiles_x);
-  p.hi_e = r.ep.act_pre == GI_ACT_RELU6 ? 0x46004600u : 0x7c007c00u;
+  p.hi_e = r.ep.act_pre == GI_ACT_RELU6 ? 0x46004600u : kMaxFinite;  // the banded operand multiplies neighbours by zero
   const int dact = c.first != kNone ? r.ep_mid.act_pre : r.ep.act_pre;
   p.hi_d = dact == GI_ACT_RELU6 ? 0x46004600u : 0x7c007c00u;
   p.act_pre = r.ep2.act_pre;

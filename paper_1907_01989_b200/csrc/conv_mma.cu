@@ -4,7 +4,8 @@
 // A fire module's two expansions read the same squeezed tensor: they are one convolution whose output channels are both
 // parts', the 1x1 part with zero weights outside the window's middle, so that the concatenation is where the results are stored
 // and costs nothing, at any channel count.  The squeezed tensor never leaves the SM (rounded to fp16 where a kernel of its own
-// would have stored it).
+// would have stored it; beyond the range of fp16 it is the largest finite value, not infinity, so that the zero weights around a
+// 1x1's middle stay zeros).
 //
 // A unit is a tile of output pixels of one image.  Its input is staged as [pixel][channels] rows of 16-byte units of 8
 // channels; all sums are mma.sync.m16n8k16.  The K axis is (window position, 8 channels) taken in pairs: the two halves of an
@@ -150,8 +151,9 @@ __global__ void __launch_bounds__(kThreads, NB * MG > 4 ? 2 : 3) conv_mma_kernel
         for (int h = 0; h < 2; ++h) {
           const int i = m * 16 + g + h * 8, r = div_by(i, p.mul_cols), x = ix0 + i - r * p.cols;
           const bool in = static_cast<unsigned>(iy0 + r) < static_cast<unsigned>(p.H) && static_cast<unsigned>(x) < static_cast<unsigned>(p.W);
-          const unsigned lo = pack_f16x2<false>(act_f(c[0][h * 2], p.act_sq), act_f(c[0][h * 2 + 1], p.act_sq));
-          const unsigned hi = pack_f16x2<false>(act_f(c[1][h * 2], p.act_sq), act_f(c[1][h * 2 + 1], p.act_sq));
+          // finite: the 1x1 part meets its neighbours with zero weights
+          const unsigned lo = finite_f16x2(pack_f16x2<false>(act_f(c[0][h * 2], p.act_sq), act_f(c[0][h * 2 + 1], p.act_sq)));
+          const unsigned hi = finite_f16x2(pack_f16x2<false>(act_f(c[1][h * 2], p.act_sq), act_f(c[1][h * 2 + 1], p.act_sq)));
           if (t < 2 * p.u_z) sts64(zs + i * p.z_pitch + t * 8, in ? lo : 0u, in ? hi : 0u);
         }
       }

@@ -18,6 +18,11 @@ constexpr int kTableBytes = 1024;  // banded depthwise operands of 4 slices: [sl
 constexpr int kBiasBytes = 64;     // 16 floats
 constexpr int kDwBiasBytes = 256;  // bias of 16 channels, each four times: the start value of a fragment of sums
 
+// The largest finite fp16 value, twice.  A tensor that stays on the SM and is multiplied by structural zeros - the banded operand of
+// a depthwise convolution, a 1x1 evaluated as a window - holds it in the place of infinity: 0 x infinity would reach pixels and
+// channels that the value has nothing to do with.
+constexpr unsigned kMaxFinite = 0x7bff7bffu;
+
 __device__ __forceinline__ void ldsm4(unsigned addr, unsigned (&r)[4]) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
 }
@@ -66,6 +71,13 @@ __device__ __forceinline__ void sts128(unsigned addr, unsigned a, unsigned b, un
 __device__ __forceinline__ unsigned min_f16x2(unsigned a, unsigned b) {
   unsigned d;
   asm("min.f16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
+  return d;
+}
+// both halves between the largest finite values; NaN stays NaN
+__device__ __forceinline__ unsigned finite_f16x2(unsigned a) {
+  unsigned d;
+  asm("min.NaN.f16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(kMaxFinite));
+  asm("max.NaN.f16x2 %0, %1, %2;" : "=r"(d) : "r"(d), "r"(kMaxFinite | 0x80008000u));
   return d;
 }
 __device__ __forceinline__ unsigned prmt(unsigned a, unsigned sel) { return __byte_perm(a, 0u, sel); }

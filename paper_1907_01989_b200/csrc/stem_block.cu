@@ -65,7 +65,7 @@ struct Params {
   int o_px, sout;
   unsigned off_raw, off_hid, off_bar;
   unsigned mul_gpr, mul_per, mul_tx;
-  unsigned hi_s, hi_d, hi_p;  // upper clamps behind the three operators, two halves (6 or infinity)
+  unsigned hi_s, hi_d, hi_p;  // upper clamps behind the three operators, two halves (6; hi_s: or the largest finite value, the others: or infinity)
   int wide, pad_px;     // a pair of pixels is one aligned 16-byte store; an odd plane holds one more pixel: zero it
 };
 
@@ -511,7 +511,7 @@ int launch_stem_block(const LaunchRec& r, const Ptrs& ptr, void* stream) {
   p.mul_gpr = magic(p.gpr);
   p.mul_per = magic(static_cast<uint64_t>(c.tiles_x) * c.tiles_y);
   p.mul_tx = magic(c.tiles_x);
-  p.hi_s = r.ep.act_pre == GI_ACT_RELU6 ? 0x46004600u : 0x7c007c00u;
+  p.hi_s = r.ep.act_pre == GI_ACT_RELU6 ? 0x46004600u : kMaxFinite;  // the banded operand multiplies neighbours by zero
   p.hi_d = r.ep_mid.act_pre == GI_ACT_RELU6 ? 0x46004600u : 0x7c007c00u;
   p.hi_p = r.ep2.act_pre == GI_ACT_RELU6 ? 0x46004600u : 0x7c007c00u;
   p.wide = !r.nhwc_out && r.Wo % 2 == 0;

@@ -1184,3 +1184,47 @@ def test_a_second_activation_without_a_sum_between(kind, kernel, first, second):
     ref = og.run(spec, [x], storage="f16", fused=True)[t]
     assert ref.max() == 6.0 if wl.ACT_RELU6 in (first, second) else ref.max() > 6.0
     assert_close(run.run([x])[t], ref, api.GI_F16, kind)
+
+
+def _hidden_overflow(kind):
+    """A graph whose first convolution takes a few large pixels beyond the range of fp16; (spec, input, its tensor)."""
+    b = wl.GraphBuilder("hidden_overflow", 1, 33)
+    if kind == "stem":
+        h = b.conv2d(b.input(40, 42, 3), 32, 3, 2)
+    else:
+        h = b.conv2d(b.input(20, 21, {"exp16": 16, "exp32": 32, "wide": 96}.get(kind, 24)), 8 if kind.startswith("fire") else 192, 1)
+    if kind != "fire_linear":
+        h = b.activation(h, wl.ACT_RELU)
+    if kind.startswith("fire"):
+        b.output(b.concat(b.conv2d(h, 10, 1), b.conv2d(h, 9, 3)))
+    else:
+        b.output(b.conv2d(b.activation(b.depthwise(h, 3, 1), wl.ACT_RELU6), 24, 1))
+    spec = b.finish()
+    x = wl.make_input(spec)
+    h0, w0 = x.shape[1] // 2, x.shape[2] // 2
+    x[0, h0 - 1:h0 + 2, w0 - 1:w0 + 2, :] = 65504.0
+    return spec, x, h
+
+
+@pytest.mark.parametrize("kind", ["exp16", "exp24", "exp32", "wide", "stem", "fire", "fire_linear"])
+def test_an_overflow_inside_a_launch_reaches_only_its_own_window(kind):
+    """A hidden value beyond the range of fp16 must not change pixels it has nothing to do with, and what its own window holds is
+    a number (behind ReLU6) or infinity."""
+    spec, x, hidden = _hidden_overflow(kind)
+    run = DeviceRun(spec, api.GI_F16)
+    names = [api.KERNEL_NAMES[launch.kernel] for launch in run.ex.launches()]
+    assert ("conv_mma" if kind.startswith("fire") else "block_mma") in names, names
+    with np.errstate(all="ignore"):
+        ref = og.run(spec, [x], storage="f16", fused=True, keep_all=True)
+        assert np.isinf(ref[hidden]).any()
+        quiet = x.copy()
+        quiet[np.abs(quiet) > 1] = 0
+        t = spec.outputs[0]
+        same = og.run(spec, [quiet], storage="f16", fused=True)[t] == ref[t]
+    if not kind.startswith("fire"):  # (of a fire module the 1x1 part's window is one pixel, the 3x3 part's nine)
+        same = same.all(axis=-1)
+    assert same.mean() > 0.9
+    got = run.run([x])[t]
+    assert_close(got[same], ref[t][same], api.GI_F16, kind)
+    if not kind.startswith("fire"):
+        assert np.isfinite(got).all()
