@@ -28,9 +28,9 @@
  * The extra pixel of an odd plane must hold finite values (the library writes zeros or
  * finite values there).  Inputs are expected to be finite altogether: several kernels multiply
  * the pixels and channels beside a value by structural zeros, so what an infinity or a NaN in a
- * stored tensor does to the values next to it depends on the kernel.  Caller-visible tensors can instead be plain NHWC, in which case
- * the executable starts / ends with a layout conversion kernel (Section 3, "Running
- * Inference").
+ * stored tensor does to the values next to it depends on the kernel.  Caller-visible tensors
+ * can instead be plain NHWC, in which case the executable starts / ends with a layout
+ * conversion kernel (Section 3, "Running Inference").
  */
 #ifndef GI_H_
 #define GI_H_
@@ -329,8 +329,8 @@ GI_API gi_status gi_run_timed(gi_exec* e, const void* const* dev_inputs, void* c
  * (1 producer, 2 MMA issuer, 4 epilogue, 8 drain; 0x10000 depthwise staging copy;
  * 0x100000 / 0x200000 / 0x400000 gather / MMA issuer / epilogue of the k x k tensor-core kernels; 0x1000000..0x8000000
  * producer / MMA issuer / data warps / drain of the lane-per-pixel 1x1 kernel; 0x10000000..
- * 0x80000000 copy warp / MMA issuer / compute warps / drain of the depthwise + pointwise kernel; 0x8 / 0x10 / 0x20 also copies,
- * computing warps and shutdown of the kernels on the warp-level matrix instruction), lets the
+ * 0x80000000 copy warp / MMA issuer / compute warps / drain of the depthwise + pointwise kernel; 0x20000 / 0x40000 / 0x80000
+ * copies / computing warps / shutdown of the kernels on the warp-level matrix instruction), lets the
  * kernel finish without its results
  * and leaves the CUDA context usable.  Sticky until the process exits.  Synchronous: copies
  * the word from the current device. */

@@ -145,9 +145,9 @@ gi_status gi_device_status(uint32_t* flags) {
   if (err == 0) *flags |= inverted_residual_error_word(&err) << 4;
   if (err == 0) *flags |= pointwise_mm_error_word(&err) << 8;
   if (err == 0) *flags |= pointwise_chain_error_word(&err) << 12;
-  if (err == 0) *flags |= pointwise_mma_error_word(&err) << 3;
-  if (err == 0) *flags |= stem_block_error_word(&err) << 3;
-  if (err == 0) *flags |= conv_mma_error_word(&err) << 3;
+  if (err == 0) *flags |= pointwise_mma_error_word(&err) << 17;
+  if (err == 0) *flags |= stem_block_error_word(&err) << 17;
+  if (err == 0) *flags |= conv_mma_error_word(&err) << 17;
   if (err != 0) return fail(GI_E_CUDA, std::string("gi_device_status: ") + cudaGetErrorString(static_cast<cudaError_t>(err)));
   return GI_OK;
 }

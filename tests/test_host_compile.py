@@ -772,3 +772,21 @@ def test_no_block_reads_an_image_of_the_callers_layout_beyond_32_bit_offsets(c, 
     small enough)."""
     names = _launch_names(wl.inverted_residual_block(1, 2 ** 31 // (w * c) + 2, w, c, hidden, cout, 1))
     assert names[0] == "pack", names
+
+
+def test_device_status_bits_name_their_kernels():
+    """Where each kernel's error codes lie in the status word: the kernels on the warp-level matrix instruction share three bits that
+    no other kernel's codes fall on (as the two window convolutions on tcgen05 share theirs)."""
+    csrc = os.path.join(ROOT, "paper_1907_01989_b200", "csrc")
+    shift = {m.group(1): int(m.group(2) or 0) for m in re.finditer(r"(\w+)_error_word\(&err\)(?: << (\d+))?;", open(os.path.join(csrc, "gi_run.cu")).read())}
+    warp_level = {"pointwise_mma", "stem_block", "conv_mma"}
+    assert warp_level < set(shift) and {shift[k] for k in warp_level} == {17}
+    bits = {}
+    for name, at in shift.items():
+        text = open(os.path.join(csrc, name.replace("conv_kxk_tc", "conv_tc") + ".cu")).read()
+        codes = {int(c) for c in re.findall(r"kErr\w+ = (\d+)u", text)} | {int(c) for c in re.findall(r"&g_\w+_error, (\d+)u", text)}
+        assert codes and max(codes) << at < 1 << 32, name
+        bits[name] = {c << at for c in codes}
+    taken = set().union(*(b for name, b in bits.items() if name not in warp_level))
+    for name in warp_level:
+        assert not bits[name] & taken and bits[name] <= {0x20000, 0x40000, 0x80000}, name
