@@ -93,8 +93,12 @@ __global__ void __launch_bounds__(kThreads, NB * MG > 4 ? 2 : 3) conv_mma_kernel
   if (tid < 4) sts32(xs + p.mt * 16 * p.x_pitch + tid * 4, 0u);
   __syncthreads();
   pdl_wait();
-  bool ok = mbar_wait(bar, 0u, abort_flag, kWaitNs, &g_cm_error, 1u);
-  ok = __syncthreads_and(ok);
+  // a wait that ran out: nothing is stored, and the weights' copy lands before the CTA leaves (bounded as well)
+  if (!__syncthreads_and(mbar_wait(bar, 0u, abort_flag, kWaitNs, &g_cm_error, 1u))) {
+    unsigned none = 0;
+    if (tid == 0) mbar_wait(bar, 0u, &none, kWaitNs, &g_cm_error, 4u);
+    return;
+  }
 
   const int per = p.tiles_x * p.tiles_y;
   for (int unit = blockIdx.x; unit < p.units; unit += gridDim.x) {
@@ -199,7 +203,6 @@ __global__ void __launch_bounds__(kThreads, NB * MG > 4 ? 2 : 3) conv_mma_kernel
           }
         }
       }
-      if (!ok) continue;
 #pragma unroll
       for (int k = 0; k < MG; ++k)
 #pragma unroll

@@ -151,6 +151,7 @@ __global__ void __launch_bounds__(kThreads + 32, 2) pointwise_mma_kernel(const _
 #pragma unroll
   for (int i = 0; i < 32; ++i) acc[i / 16][i / 8 % 2][i / 4 % 2][i % 4] = 0.0f;
 
+  int asked = 0;  // stages the copying thread has requested
   if (warp == kSplit) {
     if (lane == 0) {
       auto load_w = [&](int st, int slot) {
@@ -162,10 +163,11 @@ __global__ void __launch_bounds__(kThreads + 32, 2) pointwise_mma_kernel(const _
       for (int st = 0; st < ahead; ++st) load_w(st, st);
       pdl_wait();
       for (int st = 0; st < ahead; ++st) load_a(st, st);
-      for (int st = ahead, slot = 0, round = 0; st < n_st; ++st) {
+      asked = ahead;
+      for (int slot = 0, round = 0; asked < n_st; ++asked) {
         if (!mbar_wait(empty + slot * 8, round & 1, abort_flag, kWaitNs, &g_pm_error, 1u)) break;
-        load_w(st, slot);
-        load_a(st, slot);
+        load_w(asked, slot);
+        load_a(asked, slot);
         if (++slot == p.stages) slot = 0, ++round;
       }
     }
@@ -196,11 +198,10 @@ __global__ void __launch_bounds__(kThreads + 32, 2) pointwise_mma_kernel(const _
   }
   // a wait that ran out: the copies in flight land before the CTA leaves (bounded as well), nothing is stored
   if (__syncthreads_or(static_cast<int>(*abort_flag))) {
-    if (tid == 0)
-      for (int st = max(0, n_st - p.stages); st < n_st; ++st) {
-        unsigned none = 0;
-        mbar_wait(full + st % p.stages * 8, (st / p.stages) & 1, &none, kWaitNs, &g_pm_error, 4u);
-      }
+    for (int st = max(0, asked - p.stages); st < asked; ++st) {
+      unsigned none = 0;
+      mbar_wait(full + st % p.stages * 8, (st / p.stages) & 1, &none, kWaitNs, &g_pm_error, 4u);
+    }
     return;
   }
   if (warp == kSplit) return;

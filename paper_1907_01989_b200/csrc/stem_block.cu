@@ -154,11 +154,18 @@ __global__ void __launch_bounds__(kWarps * 32 + 32, 2) stem_block_kernel(const P
       bulk_load(smem, p.wts, p.wts_bytes, bar_w);
     }
     pdl_wait();
-    for (int k = 0; k < my_units; ++k) {
+    int k = 0;  // units whose rows have been requested
+    for (; k < my_units; ++k) {
       if (k > 1 && !mbar_wait_warp(bar_empty + (k & 1) * 8, (k / 2 - 1) & 1, abort_flag, kWaitNs, &g_stem_error, 1u)) break;
       load_rows(p, unit_pos(p, blockIdx.x + k * gridDim.x), smem + p.off_raw + (k & 1) * p.raw_bytes, bar_full + (k & 1) * 8, lane);
     }
-    return;  // every copy is waited for by the warps that compute
+    // the warps that compute stop waiting once a wait has run out: the copies in flight land before this warp leaves (bounded as well)
+    if (lane == 0) {
+      unsigned none = 0;
+      mbar_wait(bar_w, 0u, &none, kWaitNs, &g_stem_error, 4u);
+      for (int i = max(0, k - 2); i < k; ++i) mbar_wait(bar_full + (i & 1) * 8, (i / 2) & 1, &none, kWaitNs, &g_stem_error, 4u);
+    }
+    return;
   }
 
   pdl_wait();
