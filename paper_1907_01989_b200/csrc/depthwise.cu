@@ -161,7 +161,8 @@ __global__ void __launch_bounds__(256, (PLANE > 0 && !PAIR) ? 3 : 2) depthwise_f
     const int in_y1 = min(H, (oy1 - 1) * stride - pt + 2 * g.dil + 1);
     start_px = in_y0 * W;
     start_px -= start_px & 1;  // copies start on a 16-byte boundary: at most one pixel early
-    const int end_px = min((in_y1 * W + 1) & ~1, g.Pin);
+    // (packed: one copy brings whole planes, rows that no window reaches included)
+    const int end_px = PACKED ? g.Pin : min((in_y1 * W + 1) & ~1, g.Pin);
     bytes = static_cast<unsigned>(end_px - start_px) * 8u;
     last_band = band == g.bands - 1;
   };

@@ -1228,3 +1228,15 @@ def test_an_overflow_inside_a_launch_reaches_only_its_own_window(kind):
     assert_close(got[same], ref[t][same], api.GI_F16, kind)
     if not kind.startswith("fire"):
         assert np.isfinite(got).all()
+
+
+# (batch, h, w, c, pads top, left, bottom, right): stride 2 on small planes whose last row or column no window reaches
+@pytest.mark.parametrize("case", [(17, 4, 16, 43, (0, 1, 0, 0)), (40, 5, 31, 80, (1, 0, 0, 1)), (40, 8, 33, 14, (0, 0, 0, 0)), (9, 14, 14, 8, (0, 0, 0, 0)), (300, 6, 6, 4, (1, 1, 0, 0))])
+def test_depthwise_planes_with_rows_that_no_window_reaches(case):
+    batch, h, w, c, pads = case
+    b = wl.GraphBuilder("depthwise_valid", batch, 34)
+    y = b.depthwise(b.input(h, w, c), 3, 2)
+    b.g.ops[-1].pads = pads
+    b.g.shapes[y] = ((h + pads[0] + pads[2] - 3) // 2 + 1, (w + pads[1] + pads[3] - 3) // 2 + 1, c)
+    b.output(b.activation(y, wl.ACT_RELU6))
+    check_outputs(b.finish(), api.GI_F16)
