@@ -450,11 +450,16 @@ void plan_run(gi_exec* e) {
   std::vector<int> step(e->ops.size());
   std::vector<char> inside(e->tensors.size(), 0);
   for (size_t i = 0; i < e->ops.size(); ++i) step[i] = static_cast<int>(i);
-  for (const OpGroup& gr : e->groups)
+  for (const OpGroup& gr : e->groups) {
+    // a launch from the caller's input straight to the caller's output keeps the converted input's place: the caller may have
+    // handed over overlapping buffers (gi_run copies the input there, then)
+    const int last = e->ops[gr.first + gr.n - 1].out;
+    const bool in_place = gr.rec.nhwc_in && (last < 0 || (e->tensors[last].output_index >= 0 && e->tensors[last].output_layout == GI_PHWC4));
     for (int k = 0; k < gr.n; ++k) {
       step[gr.first + k] = gr.first;
-      if (k + 1 < gr.n) inside[e->ops[gr.first + k].out] = 1;
+      if (k + 1 < gr.n && !(in_place && k == 0)) inside[e->ops[gr.first + k].out] = 1;
     }
+  }
   const std::vector<TensorPlan> planned = e->plan;
   for (size_t t = 0; t < e->plan.size(); ++t) {
     e->plan[t].first = static_cast<int>(e->ops.size());

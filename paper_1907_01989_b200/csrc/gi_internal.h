@@ -111,6 +111,10 @@ struct LaunchRec {
   // one's behind it, `ep2` the projection's; Cmid / Co2, stride, pads and (Ho, Wo) as above; (H, W) the depthwise input
   BlockCfg block;
   int nhwc_out = 0;  // the kernel writes the caller's NHWC output itself
+  // a launch that reads the caller's NHWC input while it writes a caller's output: arena bytes for a copy of the input where the
+  // caller handed over overlapping buffers, and the sizes of both
+  Loc spare;
+  uint64_t in_bytes = 0, out_bytes = 0;
   int lead = -1, dw_op = -1;  // executed ops: the convolution in front of the depthwise one (or -1), the depthwise one
   // a convolution group: `lead` the squeeze (or -1); the convolutions in the order of their output channels (the second or -1);
   // the sum behind the concatenation (or -1).  `ep` is the squeeze's epilogue, `ep2` what happens to the result

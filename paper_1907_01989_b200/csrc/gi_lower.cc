@@ -666,6 +666,12 @@ static gi_status lower_pass(const gi_graph& g, gi_exec* e, bool grouped, bool pa
       } else {
         r.kernel = GI_KERNEL_NONE;
       }
+      if (r.nhwc_in && r.out.where == W_OUTPUT) {
+        const TensorDesc &d = e->tensors[f.out], &o = e->tensors[g.outputs[r.out.index]];
+        r.spare = loc_of(e, f.out);
+        r.in_bytes = B * d.h * d.w * d.c * eb;
+        r.out_bytes = r.nhwc_out ? B * o.h * o.w * o.c * eb : gi_tensor_bytes(e->batch, o.h, o.w, o.c, e->storage, 256);
+      }
       info.kernel = r.kernel;
       e->launches.push_back(r);
       e->op_info.push_back(info);

@@ -98,7 +98,15 @@ static gi_status run_impl(gi_exec* e, const void* const* dev_inputs, void* const
     p.bias2 = resolve(r.bias2);
     p.out2 = resolve(r.out2);
     int err = 0;
-    switch (r.kernel) {
+    if (r.spare.where == W_ARENA) {
+      const uintptr_t in = reinterpret_cast<uintptr_t>(p.in0), out = reinterpret_cast<uintptr_t>(p.out);
+      if (in < out + r.out_bytes && out < in + r.in_bytes) {
+        void* copy = resolve(r.spare);
+        err = static_cast<int>(cudaMemcpyAsync(copy, p.in0, r.in_bytes, cudaMemcpyDeviceToDevice, static_cast<cudaStream_t>(stream)));
+        p.in0 = copy;
+      }
+    }
+    switch (err == 0 ? r.kernel : GI_KERNEL_NONE) {
       case GI_KERNEL_PACK: err = launch_pack(r, p, e->storage, stream); break;
       case GI_KERNEL_UNPACK: err = launch_unpack(r, p, e->storage, stream); break;
       case GI_KERNEL_CONV_SIMT: err = launch_conv_simt(r, p, e->storage, stream); break;

@@ -1240,3 +1240,31 @@ def test_depthwise_planes_with_rows_that_no_window_reaches(case):
     b.g.shapes[y] = ((h + pads[0] + pads[2] - 3) // 2 + 1, (w + pads[1] + pads[3] - 3) // 2 + 1, c)
     b.output(b.activation(y, wl.ACT_RELU6))
     check_outputs(b.finish(), api.GI_F16)
+
+
+# (graph, layout of its output, bytes between the start of the output and that of the input): one launch from the caller's input to
+# the caller's output
+@pytest.mark.parametrize("make,out_layout,shift", [(lambda: wl.separable_block(2, 40, 38, 32, 32), api.GI_NHWC, 0), (lambda: wl.separable_block(2, 40, 38, 32, 32), api.GI_NHWC, 4096),
+                                                   (lambda: wl.separable_block(1, 17, 19, 16, 24), api.GI_PHWC4, 0), (lambda: _window_conv(2, 33, 35, 3, 24, 2, 1, nhwc=True), api.GI_PHWC4, 256),
+                                                   (lambda: _stem_block(1, 64, 62, 32, 64), api.GI_NHWC, 0)],
+                         ids=["block", "block_shifted", "block_phwc4", "window_phwc4", "stem"])
+@pytest.mark.parametrize("planner", [api.GI_PLAN_GREEDY_BY_SIZE, api.GI_PLAN_MIN_COST_FLOW])
+def test_one_launch_into_the_buffer_it_reads(make, out_layout, shift, planner):
+    """The output lies on the input's bytes, as it may where a conversion reads the whole input first: the same bits as with buffers
+    of their own."""
+    import torch
+    spec = make()
+    ex = api.graph_from_spec(spec, api.GI_F16, out_layout=out_layout)[0].compile(planner=planner)
+    assert sum(api.KERNEL_NAMES[launch.kernel] != "none" for launch in ex.launches()) == 1
+    ex.bind()
+    x = torch.from_numpy(wl.make_input(spec)).to("cuda:0").half().contiguous()
+    H, W, Cc = spec.shapes[spec.outputs[0]]
+    n_in, n_out = x.numel(), spec.batch * H * W * Cc if out_layout == api.GI_NHWC else api.gi_tensor_bytes(spec.batch, H, W, Cc) // 2
+    apart = torch.zeros(n_out, dtype=torch.float16, device="cuda:0")
+    ex.run([x], [apart])
+    both = torch.zeros(max(n_out, n_in + shift // 2), dtype=torch.float16, device="cuda:0")
+    for _ in range(3):
+        both[shift // 2:shift // 2 + n_in] = x.flatten()
+        ex.run([both[shift // 2:]], [both])
+        torch.cuda.synchronize()
+        assert torch.equal(both[:n_out], apart)
