@@ -349,7 +349,7 @@ def run_sweep(args):
         g, _ = api.graph_from_spec(spec, api.GI_F16, io_layout=in_layout, out_layout=api.GI_PHWC4)
         ex = g.compile(pointwise=PW_MODES[args.pointwise], cross_op=XOP_MODES[args.cross_op])
         ex.bind(dev)
-        ops = ex.ops()
+        ops = ex.launches()  # what one run launches at each executed op
         assert len(ops) == {"dwpw": 2, "stem": 2, "block": 3, "pair": 2}.get(args.sweep, 1)
         # seeded images (the workload recipe), at most 8 distinct ones: image k of the batch is drawn image k % 8
         n_img = min(b, 8)
@@ -504,7 +504,7 @@ def run_slice8_sweep(args):
             ins = [sliced(x, 4, api.gi_tensor_bytes(b, hw, hw, cin) // 2)]
             outs = [torch.full((api.gi_tensor_bytes(b, hw, hw, cout) // 2,), float("nan"), dtype=torch.float16, device=dev)]
             ms = timed(lambda: ex.run(ins, outs, stream))
-            kernel = "+".join(api.KERNEL_NAMES[q.kernel] for q in ex.ops())
+            kernel = "+".join(api.KERNEL_NAMES[q.kernel] for q in ex.launches())
             report("slices of 4 channels, " + ("the library's choice" if mode == "auto" else "wide-tile kernel"), kernel, ms, outs[0], 4)
         conv = [o for o in spec.ops if o.kind == wl.CONV2D][0]
         blob = torch.from_numpy(api.gi_slice8_pointwise_pack(conv.weights.reshape(cout, cin), conv.bias)).to(dev)

@@ -113,10 +113,11 @@ enum {
  * memory plan is not affected: those tensors keep their place in the arena, unused; operators whose input and output the
  * planner placed on the same bytes (legal for separate kernels, not for one that reads while it writes) stay separate. */
 enum {
-  GI_XOP_AUTO = 0,  /* the library's choice, from whole-network measurements (default): (3) for seams on planes of 65 to 256
-                       pixels with at most 64 channels between the two convolutions, at least 192 into the first and two
-                       pixel tiles per SM; never (1) or (2), which have not measured faster than separate kernels inside
-                       the benchmark networks */
+  GI_XOP_AUTO = 0,  /* the library's choice (default): a depthwise op with the ops around it, a fire module or a convolution and
+                       the conversion beside it as one launch wherever a fitted estimate of its time is below that of separate
+                       launches (gi_launch_info); (3) for seams on planes of 65 to 256 pixels with at most 64 channels between
+                       the two convolutions, at least 192 into the first and two pixel tiles per SM; never the kernels of (1)
+                       and (2), which have not measured faster than separate ones inside the benchmark networks */
   GI_XOP_OFF = 1,   /* one kernel per fused op */
   GI_XOP_ON = 2,    /* (1) wherever the block kernel supports the three ops, else (2) wherever the pair kernel does */
   GI_XOP_CHAIN = 3  /* (3) wherever that kernel supports the two ops; neither (1) nor (2) */
@@ -161,7 +162,8 @@ typedef struct gi_compile_options {
 } gi_compile_options;
 
 typedef struct gi_exec_info {
-  int32_t n_ops;           /* executed ops: layout conversions + fused ops = kernel launches per gi_run */
+  int32_t n_ops;           /* executed ops: layout conversions + fused ops.  gi_run launches at most one kernel for each; how many
+                              it does launch: gi_exec_launch */
   int32_t n_fused_ops;     /* fused ops only */
   int32_t n_tensors;       /* tensors of the graph (ids 0 .. n_tensors-1) */
   int32_t batch, storage;
@@ -178,7 +180,9 @@ typedef struct gi_tensor_info {
                            that needs no copy: `offset` then points into that tensor) */
   int32_t first_op, last_op; /* executed-op indices, inclusive; -1 if not alive */
   uint64_t bytes;       /* physical size under the size formula */
-  uint64_t offset;      /* arena offset (intermediate tensors only) */
+  uint64_t offset;      /* arena offset (intermediate tensors only) under the chosen planner, ops run one by one.  Where gi_run
+                           launches several ops as one kernel (gi_exec_launch), the tensors that remain are placed anew inside the
+                           same arena: only under GI_PLAN_NAIVE is a tensor that gi_run stores found at this offset */
 } gi_tensor_info;
 
 typedef struct gi_op_info {
@@ -189,19 +193,20 @@ typedef struct gi_op_info {
   gi_tensor output;     /* tensor written (-1 = caller buffer) */
   int32_t act_pre;      /* activation applied before the residual add */
   int32_t act_post;     /* activation applied after the residual add */
-  int32_t kernel;       /* GI_KERNEL_* that runs this op */
+  int32_t kernel;       /* GI_KERNEL_* chosen for this op by itself; what gi_run launches: gi_exec_launch */
   uint64_t bytes;       /* algorithmic bytes: inputs + residual + output once, weights once */
   uint64_t flops;       /* algorithmic flops (2 per multiply-add) */
 } gi_op_info;
 
 /* What gi_run launches at an executed op.  gi_op_info describes the ops one by one, each with the kernel chosen for it
  * alone; with GI_XOP_AUTO, GI_PW_AUTO, `fuse` set and fp16 storage, gi_run launches a depthwise 3x3 op with the ops
- * around it as ONE kernel where that is faster: the tensors between them are then never stored (their place in the arena
- * may hold anything), and results are those of the ops one after the other up to the order of fp32 sums (a value of such a
- * tensor beyond the range of fp16 is the largest finite one instead of infinity where its neighbours are multiplied by
- * structural zeros: what a window convolution reads).  Under
- * GI_PLAN_NAIVE gi_op_info itself says so: its `kernel` is then that of the launch, and GI_KERNEL_NONE marks the ops inside
- * one.  (GI_XOP_OFF keeps one kernel per op.) */
+ * around it as ONE kernel where that is faster, a fire module or a window convolution of few channels likewise, and lets
+ * a kernel read or write the caller's NHWC tensor itself.  The tensors inside a launch are then never stored (their place in
+ * the arena may hold anything), and results are those of the ops one after the other up to the order of fp32 sums (a value
+ * of such a tensor beyond the range of fp16 is the largest finite one instead of infinity where its neighbours are
+ * multiplied by structural zeros: what a window convolution reads).  Under GI_PLAN_NAIVE gi_op_info itself says what is
+ * launched: its `kernel` is then that of the launch, and GI_KERNEL_NONE marks the ops inside one; that plan with GI_XOP_OFF
+ * (one kernel per op) stores every tensor of the graph where gi_exec_tensor says. */
 typedef struct gi_launch_info {
   int32_t kernel;       /* GI_KERNEL_*; GI_KERNEL_NONE: no launch here, another op's kernel runs this op */
   int32_t n_ops;        /* executed ops up to the next launch (0 for GI_KERNEL_NONE) */
@@ -265,7 +270,7 @@ GI_API void gi_graph_destroy(gi_graph* g);
  * Two tables generated from measurements on the device (the counterpart of the paper's table of optimal work-group sizes,
  * Section 4) are consulted: which 1x1 kernel runs a shape, and how much the depthwise stencil stages at a time.  The
  * environment variables GI_DW_BUF_KB and GI_DW_CTA_KB, read here, override the second table for every depthwise operator of
- * the graph (largest staging buffer and shared memory of one CTA, in KB); they exist for the tuner that generates it. */
+ * the graph that is launched by itself (largest staging buffer and shared memory of one CTA, in KB); they exist for the tuner that generates it. */
 GI_API gi_status gi_compile(const gi_graph* g, const gi_compile_options* opt, gi_exec** out);
 
 GI_API gi_status gi_exec_query(const gi_exec* e, gi_exec_info* info);

@@ -69,7 +69,7 @@ def time_graph(torch, api, spec, dev, stream, flush, iters, **compile_kw):
         z.record(stream)
         z.synchronize()
         ms.append(a.elapsed_time(z))
-    return statistics.median(ms), [api.KERNEL_NAMES[o.kernel] for o in ex.ops()]
+    return statistics.median(ms), [api.KERNEL_NAMES[x.kernel] for x in ex.launches()]
 
 
 def tune_depthwise(args):
@@ -162,7 +162,7 @@ def main():
         for name, mode, kernel, _ in VARIANTS + [("rule", 5, None, 0)]:
             g, _ids = api.graph_from_spec(spec, api.GI_F16, io_layout=api.GI_PHWC4)
             ex = g.compile(pointwise=mode)
-            ran = api.KERNEL_NAMES[ex.ops()[0].kernel]
+            ran = api.KERNEL_NAMES[ex.launches()[0].kernel]
             if kernel is not None and ran != kernel:
                 continue  # this variant does not support the shape
             ex.bind(dev)

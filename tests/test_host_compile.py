@@ -203,7 +203,8 @@ def test_expected_fused_counts_and_arena():
 
 
 def test_kernels_of_the_benchmark_step():
-    """Which kernel runs which layer of MobileNetV2-224 at batch 256 (the bench configuration): the generated launch
+    """Which kernel is chosen for which layer of MobileNetV2-224 at batch 256 (the bench configuration) by itself, which is what
+    runs with one kernel per op but for the chains: the generated launch
     table and the cross-operator rule decide at compile time, so the mix is checked without a GPU.  The expansion
     layers from 24 input channels on and the 14x14 / 7x7 projections run on the lane-per-pixel kernel, the 112x112
     layers and the 56x56 / 28x28 projections on the pixel-pair kernel, the 7x7 layers with 576 or more input channels on
@@ -227,6 +228,21 @@ def test_kernels_of_the_benchmark_step():
                 assert name == "pointwise_ts", (tin.h, tin.c, tout.c)  # an expansion layer
             if tin.h == 112:
                 assert name == "pointwise_tc", (tin.h, tin.c, tout.c)
+
+
+def test_launches_of_the_benchmark_step():
+    """What one step of that configuration launches: the stem with the depthwise and the 1x1 operator behind it as one kernel, blocks
+    of the larger planes whole, four 14x14 seams as one kernel each, every other operator by itself on the kernel chosen for it."""
+    from collections import Counter
+    ex = api.graph_from_spec(wl.mobilenet_v2(256), api.GI_F16)[0].compile()
+    launches, ops = ex.launches(), ex.ops()
+    mix = Counter(api.KERNEL_NAMES[x.kernel] for x in launches)
+    assert sum(v for k, v in mix.items() if k != "none") <= 43 and sum(x.n_ops for x in launches) == ex.info.n_ops
+    assert mix["block_mma"] >= 4 and launches[0].n_ops == 4 and api.KERNEL_NAMES[launches[0].kernel] == "block_mma"
+    assert mix["conv3x3_tc"] == 0 and mix["depthwise"] + mix["block_mma"] == 17 and mix["pointwise_chain"] == 4
+    inside = {k for i, x in enumerate(launches) if api.KERNEL_NAMES[x.kernel] == "block_mma" for k in range(i, i + x.n_ops)}
+    for i, (x, o) in enumerate(zip(launches, ops)):
+        assert i in inside or x.kernel == o.kernel, (i, api.KERNEL_NAMES[x.kernel], api.KERNEL_NAMES[o.kernel])
 
 
 # ---------------------------------------------------------------------- error behaviour
