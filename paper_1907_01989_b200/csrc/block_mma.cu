@@ -31,10 +31,10 @@
 // Small launches.  Where there are fewer units than SMs the chain of one unit is what a launch takes: up to 16 sets of warps
 // then share a chunk, 16 hidden channels each (BlockCfg::wk), so that a warp's chain is one or two first operators, depthwise
 // slices and projections; where its pixels lie is worked out before the previous kernel has finished, only the copies are
-// issued behind it.  Of 8.3 us for 14x14 64 -> 384 -> 64 at batch 1 with a cluster alone, 0.9 were the addresses, 3.3 the three
-// chunks, 0.8 the cluster barrier and 3.0 reading the neighbours' sums one round trip after the other; sets of warps and
-// pushed sums: 7.7 against 10.5 us a launch, 7x7 160 -> 960 -> 160 10.3 against 19.  MobileNetV2 batch 1 169 -> 160 us, 8 x
-// 192 207 -> 186, segmentation batch 1 229 -> 211.
+// issued behind it.  Of a launch of 14x14 64 -> 384 -> 64 at batch 1 with a cluster alone (8.7 us in a chain of such launches), 0.9
+// us were the addresses, 3.3 the three chunks, 0.8 the cluster barrier and 3.0 reading the neighbours' sums one round trip after
+// the other; with sets of warps and pushed sums 8.0 us a launch, 14x14 96 -> 576 -> 96 8.2 against 9.5.  Inside the networks:
+// MobileNetV2 batch 1 169 -> 160 us, 8 x 192 207 -> 186, segmentation batch 1 229 -> 211.
 //
 // What bounds it.  Small launches: that chain.  Large ones: nothing alone - on 56x56 24 -> 144 -> 24 at batch 256 a
 // chunk takes 1840 cycles of an SM for 800 of the matrix pipe, 770 of issue slots per scheduler and about 900 of shared
@@ -120,12 +120,9 @@ struct BlockParams {
 __device__ __forceinline__ void cp_async16(unsigned dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
-// 8 (4) bytes of which the first `bytes` are read and the others written as zeros
+// 8 bytes of which the first `bytes` are read and the others written as zeros
 __device__ __forceinline__ void cp_async8(unsigned dst, const void* src, unsigned bytes) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void cp_async4(unsigned dst, const void* src, unsigned bytes) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>

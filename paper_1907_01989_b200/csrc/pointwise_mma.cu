@@ -21,6 +21,7 @@
 #include <cstring>
 
 #include "kernels.h"
+#include "mma_frag.cuh"
 #include "pdl.cuh"
 #include "sm100_ptx.cuh"
 #include "tma_host.h"
@@ -29,6 +30,7 @@ namespace gi {
 namespace {
 
 using namespace ptx;
+using namespace frag;
 
 constexpr int kThreads = 256;  // threads that compute; one more warp issues the copies
 constexpr int kMaxStages = 12;
@@ -60,30 +62,6 @@ struct Params {
 };
 
 __device__ unsigned g_pm_error = 0;
-
-__device__ __forceinline__ uint4 lds128(unsigned addr) {
-  uint4 v;
-  asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
-  return v;
-}
-__device__ __forceinline__ uint2 lds64(unsigned addr) {
-  uint2 v;
-  asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(addr) : "memory");
-  return v;
-}
-__device__ __forceinline__ void sts128(unsigned addr, const float* v) {
-  asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]) : "memory");
-}
-__device__ __forceinline__ void mma16816(float (&d)[4], unsigned a0, unsigned a1, unsigned a2, unsigned a3, unsigned b0, unsigned b1) {
-  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
-      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-__device__ __forceinline__ float act_f(float v, int act) {
-  if (act != GI_ACT_NONE) v = fmaxf(v, 0.0f);
-  if (act == GI_ACT_RELU6) v = fminf(v, 6.0f);
-  return v;
-}
 
 // One pixel-slice of the result: bias, activation, residual, activation, fp16; stored as a slice or into the caller's tensor.
 __device__ __forceinline__ void finish(const Params& p, int row, int slice, const float4& bias, float v0, float v1, float v2, float v3) {
@@ -178,16 +156,20 @@ __global__ void __launch_bounds__(kThreads + 32, 2) pointwise_mma_kernel(const _
       if (!mbar_wait_warp(full + slot * 8, round & 1, abort_flag, kWaitNs, &g_pm_error, 2u)) break;
       if (st * kSplit + warp < p.k16) {
         const unsigned a_at = smem + slot * kStage + (warp * 4 + t) * kSlicePitch + g * 8, b_at = smem + slot * kStage + kABytes + warp * 512 + lane * 16;
-        uint2 a[2][2];
+        unsigned a[2][4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) a[i >> 1][i & 1] = lds64(a_at + i * 64);
+        for (int i = 0; i < 4; ++i) {
+          const uint2 v = lds64(a_at + i * 64);
+          a[i >> 1][i & 1] = v.x;
+          a[i >> 1][2 + (i & 1)] = v.y;
+        }
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
           const uint4 b = lds128(b_at + j * kSplit * 512);
 #pragma unroll
           for (int i = 0; i < 2; ++i) {
-            mma16816(acc[i][j][0], a[i][0].x, a[i][1].x, a[i][0].y, a[i][1].y, b.x, b.y);
-            mma16816(acc[i][j][1], a[i][0].x, a[i][1].x, a[i][0].y, a[i][1].y, b.z, b.w);
+            mma16816(acc[i][j][0], a[i], b.x, b.y);
+            mma16816(acc[i][j][1], a[i], b.z, b.w);
           }
         }
       }
@@ -212,10 +194,12 @@ __global__ void __launch_bounds__(kThreads + 32, 2) pointwise_mma_kernel(const _
 #pragma unroll
   for (int i = 0; i < 2; ++i)
 #pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      sts128(mine + (i * 2 + j) * 1024, acc[i][j][0]);
-      sts128(mine + (i * 2 + j) * 1024 + 512, acc[i][j][1]);
-    }
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+      for (int f = 0; f < 2; ++f) {
+        const float(&v)[4] = acc[i][j][f];
+        sts128(mine + (i * 2 + j) * 1024 + f * 512, __float_as_uint(v[0]), __float_as_uint(v[1]), __float_as_uint(v[2]), __float_as_uint(v[3]));
+      }
   asm volatile("bar.sync 1, %0;" ::"n"(kThreads) : "memory");  // the warps that compute
   const int gr = warp >> 1, half = warp & 1;
   const unsigned at = smem + gr * 1024 + lane * 16 + half * 8;
@@ -257,7 +241,7 @@ void pointwise_mma_pack(const float* w, const float* bias, int cin, int cout, st
           for (int lane = 0; lane < 32; ++lane)
             for (int e = 0; e < 8; ++e, ++q) {  // {fragment 0: b0, b1; fragment 1: b0, b1}
               const int f = e >> 2, hi8 = (e >> 1) & 1, lo = e & 1, n = lane >> 2, t = lane & 3;
-              const int co = 16 * j + 4 * (n >> 1) + 2 * f + (n & 1), ci = 16 * kk + 4 * t + 2 * hi8 + lo;
+              const int co = channel_of(j, f, n), ci = 16 * kk + 4 * t + 2 * hi8 + lo;
               if (co < cout && ci < cin) *q = f32_to_f16_rne(w[static_cast<size_t>(co) * cin + ci]);
             }
   std::memcpy(blob->data() + boff, bias, static_cast<size_t>(cout) * sizeof(float));
