@@ -36,10 +36,7 @@
 // the other; with sets of warps and pushed sums 8.0 us a launch, 14x14 96 -> 576 -> 96 8.2 against 9.5.  Inside the networks:
 // MobileNetV2 batch 1 169 -> 160 us, 8 x 192 207 -> 186, segmentation batch 1 229 -> 211.
 //
-// What bounds it.  Small launches: that chain.  Large ones: nothing alone - on 56x56 24 -> 144 -> 24 at batch 256 a
-// chunk takes 1840 cycles of an SM for 800 of the matrix pipe, 770 of issue slots per scheduler and about 900 of shared
-// memory, with 16 warps to cover 21-cycle matrix and 30-cycle shared-memory latencies; 173 us against 194 us as three
-// kernels.  Measured on one B200 against separate kernels, stem included
+// What bounds it.  Small launches: that chain.  Large ones: block_ws_kernel.  Measured on one B200 against separate kernels, stem included
 // (stem_block.cu), MobileNetV2: batch 1 225 -> 155 us, 21 images of 205 pixels 340 -> 270, batch 256 1413 -> 1298;
 // segmentation network batch 1 289 -> 207, batch 16 961 -> 748.
 #include <cuda_fp16.h>
@@ -77,10 +74,16 @@ __host__ __device__ constexpr int tile_pixels(int first, bool small) { return sl
 // warps an SM holds: 128 registers a thread for 16 warps, 255 for 8 (96 sums per thread and more; tr: output rows a warp
 // walks down), 168 for 12 where 64 sums and the fragments of four rows do not fit 128 (28x28 32 -> 192 -> 32 at batch 256: 77 us
 // with 416 bytes of spills in the loop, 69 with 12 warps; 26x26 at batch 21 18.7 -> 16.9)
-__host__ __device__ constexpr int max_warps(int s, int np, int tr) { return (s == 1 ? tr : 1) * np >= 6 || tr == 4 ? 8 : s == 1 && tr == 2 && np == 2 ? 12 : 16; }
+// ws: the kernel with specialised warps; 96 sums then fit 168 registers
+__host__ __device__ constexpr int max_warps(int s, int np, int tr, bool ws = false) {
+  return ws && np == 6 && (s == 2 || tr == 1) ? 12 : (s == 1 ? tr : 1) * np >= 6 || tr == 4 ? 8 : s == 1 && tr == 2 && np == 2 ? 12 : 16;
+}
 // bytes of one 16-channel sub-block of packed weights: first operator's fragments and bias, banded depthwise operands and
 // bias, projection fragments
 __host__ __device__ constexpr int sub_bytes(int ke, int np) { return ke * 512 + kSubFixed + np * 512; }
+// ... of the kernel with specialised warps: behind it the expansion's bias as B operand, [fragment][column][two words]
+constexpr int kOnesBytes = 128;
+__host__ __device__ constexpr int ws_sub_bytes(int ke, int np) { return sub_bytes(ke, np) + kOnesBytes; }
 
 struct BlockParams {
   const __half* in;
@@ -120,13 +123,19 @@ struct BlockParams {
 __device__ __forceinline__ void cp_async16(unsigned dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
-// 8 bytes of which the first `bytes` are read and the others written as zeros
-__device__ __forceinline__ void cp_async8(unsigned dst, const void* src, unsigned bytes) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+// 8 bytes, or zeros in their place where there is nothing to read.  (A predicate: a size in a register costs 14 more instructions.)
+__device__ __forceinline__ void cp_async8(unsigned dst, const void* src, bool in) {
+  asm volatile("{\n\t.reg .pred none;\n\tsetp.eq.u32 none, %2, 0;\n\tcp.async.ca.shared.global [%0], [%1], 8, none;\n\t}" ::"r"(dst), "l"(src),
+               "r"(static_cast<unsigned>(in))
+               : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// A barrier of `n` threads of the CTA that some only arrive at
+__device__ __forceinline__ void named_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+__device__ __forceinline__ void named_arrive(int id, int n) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory"); }
 
 __device__ __forceinline__ void st_cluster_f4(unsigned addr, float a, float b, float c, float d) {
   asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
@@ -284,6 +293,153 @@ __device__ __forceinline__ void store_col(const BlockParams& p, const UnitPos& u
   }
 }
 
+// Which half of a banded weight word a lane takes, where its words lie, and whether it is a lane of the second output row (stride 2).
+struct BandSel {
+  unsigned a, b, a0, b0, a1, b1, entry;
+  bool odd;
+};
+__device__ __forceinline__ BandSel band_sel(int lane) {
+  const int g = lane >> 2, t = lane & 3;
+  const bool band_lane = (g >> 2) == (t & 1);
+  BandSel s;
+  s.a = !band_lane ? 0x4444u : ((g >> 1) & 1) ? 0x1044u : 0x4410u;
+  s.b = !band_lane ? 0x4444u : ((g >> 1) & 1) ? 0x3244u : 0x4432u;
+  s.odd = g & 1;
+  s.a0 = s.odd ? 0x4444u : s.a;  // window rows of the first output row only
+  s.b0 = s.odd ? 0x4444u : s.b;
+  s.a1 = s.odd ? s.a : 0x4444u;  // ... of the second only
+  s.b1 = s.odd ? s.b : 0x4444u;
+  s.entry = ((t >> 1) * 8 + g) * 16;
+  return s;
+}
+
+// Depthwise operator and projection of HC sub-blocks of 16 hidden channels for one group of 16 columns, added to `acc`.  ws: the
+// chunk's packed weights; hb: the lane's place in the hidden tile's first slice; row_b: bytes between hidden rows.
+template <int S, int NP, int TR, int HC, int SL>
+__device__ __forceinline__ void depthwise_project(unsigned ws, int ke, int subb, unsigned hb, unsigned row_b, int lane, unsigned hi_d,
+                                                  const BandSel& sel, float (&acc)[S == 1 ? TR : TR / 2][NP][2][2][4]) {
+  constexpr int NV = S == 1 ? TR : TR / 2;
+  const int t = lane & 3;
+  constexpr int kRows = S == 1 ? TR + 2 : 2 * TR + 1;  // hidden rows under the column
+  unsigned rb[kRows];
+#pragma unroll
+  for (int i = 0; i < kRows; ++i) rb[i] = hb + i * row_b;
+#pragma unroll
+  for (int h = 0; h < HC; ++h) {
+    const unsigned wd = ws + h * subb + ke * 512 + kBiasBytes;
+    unsigned af[NV][2][4];
+#pragma unroll
+    for (int sp = 0; sp < 2; ++sp) {
+      float d[2][NV][4], bd[2];
+#pragma unroll
+      for (int s2 = 0; s2 < 2; ++s2) {
+        const int sl = sp * 2 + s2;
+        const uint4 w = lds128(wd + sl * 256 + sel.entry);
+        bd[s2] = __uint_as_float(lds32(wd + kTableBytes + sl * 64 + t * 16));
+        if (S == 1) {
+          const unsigned b0[3] = {prmt(w.x, sel.a), prmt(w.y, sel.a), prmt(w.z, sel.a)};
+          const unsigned b1[3] = {prmt(w.x, sel.b), prmt(w.y, sel.b), prmt(w.z, sel.b)};
+#pragma unroll
+          for (int rr = 0; rr < kRows; ++rr) {
+            unsigned a[4];
+            ldsm4(rb[rr] + (h * 4 + sl) * SL, a);
+#pragma unroll
+            for (int ky = 0; ky < 3; ++ky) {
+              const int v = rr - ky;
+              if (v < 0 || v >= TR) continue;
+              if (ky == 0) mma16816z(d[s2][v], a, b0[ky], b1[ky]);
+              else mma16816(d[s2][v], a, b0[ky], b1[ky]);
+            }
+          }
+        } else {
+          const unsigned wm = sel.odd ? w.x : w.z;
+          const unsigned b0[5] = {prmt(w.x, sel.a0), prmt(w.y, sel.a0), prmt(wm, sel.a), prmt(w.y, sel.a1), prmt(w.z, sel.a1)};
+          const unsigned b1[5] = {prmt(w.x, sel.b0), prmt(w.y, sel.b0), prmt(wm, sel.b), prmt(w.y, sel.b1), prmt(w.z, sel.b1)};
+#pragma unroll
+          for (int rr = 0; rr < kRows; ++rr) {
+            unsigned a[4];
+            ldsm4(rb[rr] + (h * 4 + sl) * SL, a);
+            const int v = rr >> 2, q = rr & 3;
+            if (v < NV && q == 0) mma16816z(d[s2][v < NV ? v : 0], a, b0[q], b1[q]);
+            else if (v < NV) mma16816(d[s2][v < NV ? v : 0], a, b0[q], b1[q]);
+            if (q == 0 && v > 0) mma16816(d[s2][v > 0 ? v - 1 : 0], a, b0[4], b1[4]);
+          }
+        }
+      }
+#pragma unroll
+      for (int v = 0; v < NV; ++v)
+#pragma unroll
+        for (int s2 = 0; s2 < 2; ++s2) {  // the bias behind the sum: as its start value it would be moved into the accumulators
+          add2(d[s2][v][0], d[s2][v][1], bd[s2], bd[s2]);
+          add2(d[s2][v][2], d[s2][v][3], bd[s2], bd[s2]);
+        }
+#pragma unroll
+      for (int v = 0; v < NV; ++v)
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          af[v][q][sp * 2] = min_f16x2(pack_f16x2<true>(d[0][v][q], d[1][v][q]), hi_d);
+          af[v][q][sp * 2 + 1] = min_f16x2(pack_f16x2<true>(d[0][v][2 + q], d[1][v][2 + q]), hi_d);
+        }
+    }
+    const unsigned wp = wd + kTableBytes + kDwBiasBytes + lane * 16;
+#pragma unroll
+    for (int j = 0; j < NP; ++j) {
+      const uint4 b = lds128(wp + j * 512);
+#pragma unroll
+      for (int v = 0; v < NV; ++v)
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          mma16816(acc[v][j][q][0], af[v][q], b.x, b.y);
+          mma16816(acc[v][j][q][1], af[v][q], b.z, b.w);
+        }
+    }
+  }
+}
+
+// Partial sums of a cluster's CTAs and of warp sets: every tile of 16 columns x 16 channels has an owner, the CTA tile % ks;
+// everybody stores into the owner's shared memory (source `src` of `n_src`), which then adds up its tiles in the order of the
+// sources.  (Reading the neighbours' shared memory instead took 2.5 us: eight round trips, one after the other.)
+// push_sums calls store(address, four sums).
+template <int NV, int NP, class F>
+__device__ __forceinline__ void push_sums(const BlockParams& p, unsigned red, int group, int src, int n_src, int lane,
+                                          const float (&acc)[NV][NP][2][2][4], F&& store) {
+#pragma unroll
+  for (int v = 0; v < NV; ++v)
+#pragma unroll
+    for (int j = 0; j < NP; ++j) {
+      const int ti = (group * NV + v) * NP + j, slot = ti / p.ks;
+      unsigned at = red + (slot * n_src + src) * 2048 + lane * 16;
+      if (p.ks > 1) at = mapa_shared(at, ti - slot * p.ks);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) store(at + i * 512, acc[v][j][i >> 1][i & 1]);
+    }
+}
+template <int S, int TR, int NV, int NP>
+__device__ __forceinline__ void add_sums(const BlockParams& p, const UnitPos& u, unsigned xs, unsigned red, int rank, int n_src, int warp,
+                                         int warps, int lane) {
+  const int g = lane >> 2, t = lane & 3, tiles = p.ngroups * NV * NP;
+  for (int slot = warp; slot * p.ks + rank < tiles; slot += warps) {
+    float s[1][1][2][2][4];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) s[0][0][i >> 3][(i >> 2) & 1][i & 3] = 0.0f;
+    unsigned at = red + slot * n_src * 2048 + lane * 16;
+#pragma unroll 2
+    for (int r = 0; r < n_src; ++r, at += 2048) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const uint4 x = lds128(at + i * 512);
+        s[0][0][i >> 1][i & 1][0] += __uint_as_float(x.x);
+        s[0][0][i >> 1][i & 1][1] += __uint_as_float(x.y);
+        s[0][0][i >> 1][i & 1][2] += __uint_as_float(x.z);
+        s[0][0][i >> 1][i & 1][3] += __uint_as_float(x.w);
+      }
+    }
+    const int ti = slot * p.ks + rank, j = ti % NP, gv = ti / NP, gid = gv / NV, v = gv % NV;
+    store_col<S, 0, 1, 1>(p, u, xs, lane_col(p, S, TR, gid * 16 + g), v, j, t, s);
+    store_col<S, 1, 1, 1>(p, u, xs, lane_col(p, S, TR, gid * 16 + g + 8), v, j, t, s);
+  }
+}
+
 // S: stride.  NP: 16-channel blocks of the output.  TR: output rows a warp walks down.  HC: 16-channel sub-blocks per chunk.
 // SMALL: tiles of at most 146 list pixels, whose chunks several sets of warps share.
 template <int S, int FIRST, int NP, int TR, int HC, bool SMALL>
@@ -345,15 +501,14 @@ __global__ void __launch_bounds__(32 * max_warps(S, NP, TR), 1) block_mma_kernel
       if (listed) {
         const __half* src = p.in;
         if (in) src += static_cast<long long>(u.img0 + l.im) * p.in_img + static_cast<long long>(l.y * p.W + l.x) * p.in_px;
-        const unsigned n = in ? 8u : 0u;
         const long long step = in ? p.in_sl : 0;
         unsigned dst = xs + i * p.x_pitch;
         if (kTwoX) {
 #pragma unroll
           for (int s = 0; s < kSlices; ++s, src += step)
-            if (s < p.sin) cp_async8(dst + s * 8, src, n);
+            if (s < p.sin) cp_async8(dst + s * 8, src, in);
         } else {
-          for (int s = 0; s < p.sin; ++s, src += step, dst += 8) cp_async8(dst, src, n);
+          for (int s = 0; s < p.sin; ++s, src += step, dst += 8) cp_async8(dst, src, in);
         }
       }
       if (kWideExp) sts64(tab + i * 8, static_cast<unsigned>(listed ? l.hid : p.ni * p.sub_px) * 8u, in ? p.hi_e : 0u);
@@ -376,10 +531,10 @@ __global__ void __launch_bounds__(32 * max_warps(S, NP, TR), 1) block_mma_kernel
     if (part >= parts) return;
     for (int i = tid - part * px; i < px; i += nthr) {
       const int at = static_cast<int>(lds32(smem + p.off_src + i * 4));
-      const unsigned n = at >= 0 ? 8u : 0u, dst = xs0 + i * p.x_pitch;
+      const unsigned dst = xs0 + i * p.x_pitch;
       const __half* src = p.in + max(at, 0);
 #pragma unroll 4
-      for (int s = part; s < p.sin; s += parts) cp_async8(dst + s * 8, at >= 0 ? src + s * p.in_sl : p.in, n);
+      for (int s = part; s < p.sin; s += parts) cp_async8(dst + s * 8, at >= 0 ? src + s * p.in_sl : p.in, at >= 0);
     }
   };
   // no first operator: a chunk of the input goes straight into a hidden tile (a ring of them)
@@ -399,7 +554,7 @@ __global__ void __launch_bounds__(32 * max_warps(S, NP, TR), 1) block_mma_kernel
       const __half* src = p.in + (at < 0 ? 0 : at) + s0 * p.in_sl;
       for (int w = 0; w < wk * HC * 4; w += HC * 4)
 #pragma unroll
-        for (int s = w; s < w + HC * 4; ++s, src += p.in_sl) cp_async8(dst + s * SL, s < ns ? src : p.in, s < ns && at >= 0 ? 8u : 0u);
+        for (int s = w; s < w + HC * 4; ++s, src += p.in_sl) cp_async8(dst + s * SL, s < ns ? src : p.in, s < ns && at >= 0);
     }
   };
   if (SMALL && kHasFirst) find_x(unit_pos(p, unit0, th_rows));
@@ -428,13 +583,7 @@ __global__ void __launch_bounds__(32 * max_warps(S, NP, TR), 1) block_mma_kernel
     dw_base = static_cast<unsigned>(im * p.sub_px + band * TR * S * p.pitch) * 8u + pos * 16u + (lane >> 4) * 16u;
   }
   const unsigned col0 = lane_col(p, S, TR, wq * 16 + g), col1 = lane_col(p, S, TR, wq * 16 + g + 8);
-  const bool band_lane = (g >> 2) == (t & 1);
-  const unsigned sel_a = !band_lane ? 0x4444u : ((g >> 1) & 1) ? 0x1044u : 0x4410u;
-  const unsigned sel_b = !band_lane ? 0x4444u : ((g >> 1) & 1) ? 0x3244u : 0x4432u;
-  const bool odd = g & 1;
-  const unsigned sel_a0 = odd ? 0x4444u : sel_a, sel_b0 = odd ? 0x4444u : sel_b;  // window rows of the first output row only
-  const unsigned sel_a1 = odd ? sel_a : 0x4444u, sel_b1 = odd ? sel_b : 0x4444u;  // ... of the second only
-  const unsigned dw_entry = ((t >> 1) * 8 + g) * 16;
+  const BandSel sel = band_sel(lane);
   const bool has_group = wq < p.ngroups;
   // this warp's groups of 16 list pixels
   const int mt0 = has_group ? wq * p.eg : p.ngroups * p.eg + (wq - p.ngroups) * p.en;
@@ -597,74 +746,7 @@ __global__ void __launch_bounds__(32 * max_warps(S, NP, TR), 1) block_mma_kernel
         const int r = run + dc;
         const unsigned ws = smem + (p.resident ? dc : r & (kRing - 1)) * stage_bytes + wset * HC * subb;
         const unsigned hb = hid0 + (kHasFirst ? (r & 1) : (r & (kRing - 1))) * hid_bytes + wset * kSetBytes + dw_base;
-        constexpr int kRows = S == 1 ? TR + 2 : 2 * TR + 1;  // hidden rows under the column
-        unsigned rb[kRows];
-#pragma unroll
-        for (int i = 0; i < kRows; ++i) rb[i] = hb + i * row_b;
-#pragma unroll
-        for (int h = 0; h < HC; ++h) {
-          const unsigned wd = ws + h * subb + ke * 512 + kBiasBytes;
-          unsigned af[NV][2][4];
-#pragma unroll
-          for (int sp = 0; sp < 2; ++sp) {
-            float d[2][NV][4];
-#pragma unroll
-            for (int s2 = 0; s2 < 2; ++s2) {
-              const int sl = sp * 2 + s2;
-              const uint4 w = lds128(wd + sl * 256 + dw_entry);
-              const uint4 bq = lds128(wd + kTableBytes + sl * 64 + t * 16);
-              const float bd[4] = {__uint_as_float(bq.x), __uint_as_float(bq.y), __uint_as_float(bq.z), __uint_as_float(bq.w)};
-              if (S == 1) {
-                const unsigned b0[3] = {prmt(w.x, sel_a), prmt(w.y, sel_a), prmt(w.z, sel_a)};
-                const unsigned b1[3] = {prmt(w.x, sel_b), prmt(w.y, sel_b), prmt(w.z, sel_b)};
-#pragma unroll
-                for (int rr = 0; rr < kRows; ++rr) {
-                  unsigned a[4];
-                  ldsm4(rb[rr] + (h * 4 + sl) * SL, a);
-#pragma unroll
-                  for (int ky = 0; ky < 3; ++ky) {
-                    const int v = rr - ky;
-                    if (v < 0 || v >= TR) continue;
-                    if (ky == 0) mma16816c(d[s2][v], a, b0[ky], b1[ky], bd[0], bd[1], bd[2], bd[3]);
-                    else mma16816(d[s2][v], a, b0[ky], b1[ky]);
-                  }
-                }
-              } else {
-                const unsigned wm = odd ? w.x : w.z;
-                const unsigned b0[5] = {prmt(w.x, sel_a0), prmt(w.y, sel_a0), prmt(wm, sel_a), prmt(w.y, sel_a1), prmt(w.z, sel_a1)};
-                const unsigned b1[5] = {prmt(w.x, sel_b0), prmt(w.y, sel_b0), prmt(wm, sel_b), prmt(w.y, sel_b1), prmt(w.z, sel_b1)};
-#pragma unroll
-                for (int rr = 0; rr < kRows; ++rr) {
-                  unsigned a[4];
-                  ldsm4(rb[rr] + (h * 4 + sl) * SL, a);
-                  const int v = rr >> 2, q = rr & 3;
-                  if (v < NV && q == 0) mma16816c(d[s2][v < NV ? v : 0], a, b0[q], b1[q], bd[0], bd[1], bd[2], bd[3]);
-                  else if (v < NV) mma16816(d[s2][v < NV ? v : 0], a, b0[q], b1[q]);
-                  if (q == 0 && v > 0) mma16816(d[s2][v > 0 ? v - 1 : 0], a, b0[4], b1[4]);
-                }
-              }
-            }
-#pragma unroll
-            for (int v = 0; v < NV; ++v)
-#pragma unroll
-              for (int q = 0; q < 2; ++q) {
-                af[v][q][sp * 2] = min_f16x2(pack_f16x2<true>(d[0][v][q], d[1][v][q]), p.hi_d);
-                af[v][q][sp * 2 + 1] = min_f16x2(pack_f16x2<true>(d[0][v][2 + q], d[1][v][2 + q]), p.hi_d);
-              }
-          }
-          const unsigned wp = wd + kTableBytes + kDwBiasBytes + lane * 16;
-#pragma unroll
-          for (int j = 0; j < NP; ++j) {
-            const uint4 b = lds128(wp + j * 512);
-#pragma unroll
-            for (int v = 0; v < NV; ++v)
-#pragma unroll
-              for (int q = 0; q < 2; ++q) {
-                mma16816(acc[v][j][q][0], af[v][q], b.x, b.y);
-                mma16816(acc[v][j][q][1], af[v][q], b.z, b.w);
-              }
-          }
-        }
+        depthwise_project<S, NP, TR, HC, SL>(ws, ke, subb, hb, row_b, lane, p.hi_d, sel, acc);
       }
     }
 
@@ -675,50 +757,16 @@ __global__ void __launch_bounds__(32 * max_warps(S, NP, TR), 1) block_mma_kernel
         store_col<S, 1, NV, NP>(p, u, xs, col1, 0, 0, t, acc);
       }
     } else {
-      // partial sums of the cluster's CTAs and of the warp sets: every tile of 16 columns x 16 channels has an owner, the CTA
-      // tile % ks; everybody stores into the owner's shared memory, which then adds up its tiles in the order of the sources.
-      // (Reading the neighbours' shared memory instead took 2.5 us: eight round trips, one after the other.)
       const int src = rank * wk + wset, n_src = p.ks * wk;
       if (p.ks > 1 && k == 0) cluster_wait();  // every CTA of the cluster has started
-      if (has_group) {
-#pragma unroll
-        for (int v = 0; v < NV; ++v)
-#pragma unroll
-          for (int j = 0; j < NP; ++j) {
-            const int ti = (wq * NV + v) * NP + j, slot = ti / p.ks;
-            unsigned at = red + (slot * n_src + src) * 2048 + lane * 16;
-            if (p.ks > 1) at = mapa_shared(at, ti - slot * p.ks);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              const float(&f)[4] = acc[v][j][i >> 1][i & 1];
-              if (p.ks > 1) st_cluster_f4(at + i * 512, f[0], f[1], f[2], f[3]);
-              else sts128(at + i * 512, __float_as_uint(f[0]), __float_as_uint(f[1]), __float_as_uint(f[2]), __float_as_uint(f[3]));
-            }
-          }
-      }
+      if (has_group)
+        push_sums<NV, NP>(p, red, wq, src, n_src, lane, acc, [&](unsigned at, const float(&f)[4]) {
+          if (p.ks > 1) st_cluster_f4(at, f[0], f[1], f[2], f[3]);
+          else sts128(at, __float_as_uint(f[0]), __float_as_uint(f[1]), __float_as_uint(f[2]), __float_as_uint(f[3]));
+        });
       if (p.ks > 1) cluster_sync();
       else __syncthreads();
-      const int tiles = p.ngroups * NV * NP;
-      for (int slot = warp; slot * p.ks + rank < tiles; slot += nthr >> 5) {
-        float s[1][1][2][2][4];
-#pragma unroll
-        for (int i = 0; i < 16; ++i) s[0][0][i >> 3][(i >> 2) & 1][i & 3] = 0.0f;
-        unsigned at = red + slot * n_src * 2048 + lane * 16;
-#pragma unroll 2
-        for (int r = 0; r < n_src; ++r, at += 2048) {
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const uint4 x = lds128(at + i * 512);
-            s[0][0][i >> 1][i & 1][0] += __uint_as_float(x.x);
-            s[0][0][i >> 1][i & 1][1] += __uint_as_float(x.y);
-            s[0][0][i >> 1][i & 1][2] += __uint_as_float(x.z);
-            s[0][0][i >> 1][i & 1][3] += __uint_as_float(x.w);
-          }
-        }
-        const int ti = slot * p.ks + rank, j = ti % NP, gv = ti / NP, gid = gv / NV, v = gv % NV;
-        store_col<S, 0, 1, 1>(p, u, xs, lane_col(p, S, TR, gid * 16 + g), v, j, t, s);
-        store_col<S, 1, 1, 1>(p, u, xs, lane_col(p, S, TR, gid * 16 + g + 8), v, j, t, s);
-      }
+      add_sums<S, TR, NV, NP>(p, u, xs, red, rank, n_src, warp, nthr >> 5, lane);
       if (k + 1 < my_units) {  // nobody overwrites what a neighbour still reads
         if (p.ks > 1) cluster_sync();
         else __syncthreads();
@@ -726,6 +774,313 @@ __global__ void __launch_bounds__(32 * max_warps(S, NP, TR), 1) block_mma_kernel
     }
   }
   cp_async_wait<0>();
+}
+
+// The same with the two halves of a chunk on warps of their own: the first p.ngroups warps each own a group of columns and run its
+// depthwise operator and projection, the others compute the expansion of the chunk after it and bring weights and the next tile's
+// input.  A pair of barriers per hidden tile (complete, free) lets the two run up to two chunks apart.  For units that one CTA or a
+// cluster computes, with four chunks of hidden channels or more; blocks without an expansion and small tiles, whose chunks sets of
+// warps share, stay on the kernel above.
+//
+// What it is for: with both halves in one warp the projection's sums stay live through the expansion, the register file makes the
+// compiler move them, and a warp that waits for its shared memory has nobody to take its place.  Of 33.4 M warp instructions of 112x112
+// 16 -> 96 -> 24, stride 2, at batch 64 are left 24.8 M (3 M of them because a bias as a sum's start value costs four moves a
+// matrix instruction: the expansion's comes as a product with ones, the depthwise operator's as one two-wide addition behind the
+// sum).  Kernel above -> this one, us on one B200: that block 63.4 -> 52.3, 56x56 24 -> 144 -> 24 at batch 64 51.4 -> 43.7, 14x14
+// 64 -> 384 -> 64 at batch 64 22.2 -> 17.7, 33x33 64 -> 384 -> 64 at batch 16 29.9 -> 25.3.  MobileNetV2 at batch 256 1299 -> 1192, 21
+// images of 205 pixels 271 -> 250, segmentation at batch 16 748 -> 713.  What bounds it now: shared memory's pipe (62 % of its
+// wavefronts on the first of these) and the latency from ldmatrix to store with 12 to 16 warps; the matrix pipe is 27 % busy.
+template <int S, int FIRST, int NP, int TR>
+__global__ void __launch_bounds__(32 * max_warps(S, NP, TR, true), 1) block_ws_kernel(const BlockParams p) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  const unsigned smem = smem_u32(smem_raw);
+  const int tid = threadIdx.x, nthr = blockDim.x;
+  const int warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+  constexpr bool kWide = FIRST == kExpWide;
+  constexpr int SL = slice_bytes(FIRST, false), HC = kWide ? 2 : 1;
+  constexpr int kHidBytes = HC * 4 * SL, kSlices = FIRST == kExp16 ? 4 : FIRST == kExp24 ? 6 : 8;
+  constexpr int NV = S == 1 ? TR : TR / 2;
+  const int ke = kWide ? p.ke : FIRST == kExp16 ? 1 : 2;
+  const int subb = ws_sub_bytes(ke, NP), stage_bytes = HC * subb;
+  const unsigned XP = kWide ? p.x_pitch : FIRST == kExp32 ? 80u : 48u;  // bytes of a list pixel
+  const int th_rows = p.nb * TR;
+  const int rank = p.ks > 1 ? static_cast<int>(cluster_ctarank()) : 0;
+  const int unit0 = p.ks > 1 ? blockIdx.x / p.ks : blockIdx.x, ustep = p.ks > 1 ? gridDim.x / p.ks : gridDim.x;
+  const int nch = p.ks > 1 ? (p.nch - rank + p.ks - 1) / p.ks : p.nch;  // chunks of this CTA: rank, rank + ks, ...
+  const int my_units = (p.units - unit0 + ustep - 1) / ustep;           // (of a cluster: one)
+  const int total = nch * my_units;
+  const unsigned tab0 = smem + p.off_tab, xs0 = smem + p.off_x, hid0 = smem + p.off_hid, red = smem + p.off_red;
+
+  pdl_launch_dependents();
+  if (p.ks > 1) cluster_arrive();  // (waited for before the first store into a neighbour's shared memory)
+  auto load_weights = [&](int run, int c, int i0, int n) {
+    const unsigned dst = smem + (p.resident ? c : run & (kRing - 1)) * stage_bytes;
+    const unsigned char* src = p.wts + static_cast<size_t>(rank + c * p.ks) * stage_bytes;
+    for (int i = i0 * 16; i < stage_bytes; i += n * 16) cp_async16(dst + i, src + i);
+  };
+  // a unit's input tile, [list pixel][channel], and what its hidden pixels are clamped to (zero outside the image); for a wide
+  // expansion, whose list may leave out the border, also where they go
+  auto load_x = [&](const UnitPos& u, int buf, int i0, int n) {
+    const int yb = u.y0 * S - p.pad_t, xb = u.x0 * S - p.pad_l;
+    const __half* base = p.in + static_cast<long long>(u.img0) * p.in_img;
+    const unsigned xs = xs0 + buf * p.x_bytes, tab = tab0 + buf * p.tab_bytes;
+    for (int i = i0; i < p.mt * 16; i += n) {
+      int at, hid = i;
+      bool in;
+      if (kWide) {
+        const bool listed = i < p.n_list;
+        const ListPx l = list_pixel(p, u, S, listed ? i : 0);
+        in = listed && l.in;
+        hid = listed ? l.hid : p.ni * p.sub_px;
+        at = l.im * p.in_img + (l.y * p.W + l.x) * p.in_px;
+      } else {
+        const int q = div_by(i, p.mul_pitch), x = xb + (i - q * p.pitch), y = yb + q;
+        in = i < p.n_list && static_cast<unsigned>(y) < static_cast<unsigned>(p.H) && static_cast<unsigned>(x) < static_cast<unsigned>(p.W);
+        at = (y * p.W + x) * p.in_px;
+      }
+      const __half* src = in ? base + at : p.in;
+      const long long step = in ? p.in_sl : 0;
+      unsigned dst = xs + i * XP;
+      if (kWide) {
+#pragma unroll 4
+        for (int s = 0; s < p.sin; ++s, src += step, dst += 8) cp_async8(dst, src, in);
+        sts64(tab + i * 8, hid * 8u, in ? p.hi_e : 0u);
+      } else {
+#pragma unroll
+        for (int s = 0; s < kSlices; ++s, src += step)
+          if (s < p.sin) cp_async8(dst + s * 8, src, in);
+        sts32(tab + i * 4, in ? p.hi_e : 0u);
+      }
+    }
+  };
+  for (int c = 0; c < (p.resident ? nch : 2); ++c) load_weights(c, c, tid, nthr);
+  for (int i = tid; i < NP * 4; i += nthr) cp_async16(smem + p.off_bias + i * 16, reinterpret_cast<const float4*>(p.bias) + i);
+  // shared memory that must start at zero: borders of compact tiles, and the slices beyond the input's last one that the
+  // expansion's steps of 16 channels read (their weights are zero, but 0 x NaN is not)
+  if (p.compact || p.sin < (FIRST == kExp24 ? 6 : 4 * ke)) {
+    for (unsigned i = p.off_x + tid * 16; i < p.off_red; i += nthr * 16) sts128(smem + i, 0u, 0u, 0u, 0u);
+    __syncthreads();
+  }
+  pdl_wait();
+  load_x(unit_pos(p, unit0, th_rows), 0, tid, nthr);
+  cp_async_commit();
+  cp_async_wait<0>();
+  __syncthreads();
+
+  const int ncons = p.ngroups;
+  if (warp >= ncons) {
+    // ---- expansion: groups of 16 list pixels; of a wide one, every second warp takes the second 16 channels of the chunk
+    const int nprod = (nthr >> 5) - ncons, w = warp - ncons, ptid = tid - ncons * 32, np = nprod * 32;
+    const int half_chunk = kWide ? w & 1 : 0, wg = kWide ? w >> 1 : w, nwg = kWide ? nprod >> 1 : nprod;
+    const int mt0 = wg * p.mt / nwg, cnt = (wg + 1) * p.mt / nwg - mt0;
+    const unsigned a_off = (mt0 * 16 + (lane & 15)) * XP + (lane >> 4) * 16, h_off = (mt0 * 16 + (lane & 15)) * XP + 32;
+    const unsigned t_off = (mt0 * 16 + g) * (kWide ? 8 : 4), ones = ones_word(t);
+    int r = 0;
+#pragma unroll 1
+    for (int k = 0; k < my_units; ++k) {
+      const unsigned xs = xs0 + (k & 1) * p.x_bytes, tab = tab0 + (k & 1) * p.tab_bytes + t_off;
+      unsigned edge = 0u;  // groups (of the first 32) with pixels outside the image
+#pragma unroll 1
+      for (int c = 0; c < nch; ++c, ++r) {
+        cp_async_wait<1>();
+        if (r >= 2) named_sync(3 + (r & 1), nthr);  // the hidden tile is free, and the copies of all these warps have arrived
+        if (!p.resident && r + 2 < total) load_weights(r + 2, c + 2 >= nch ? c + 2 - nch : c + 2, ptid, np);
+        // (the columns' warps have finished the unit before this one: its tile may be overwritten)
+        if (c == 2 && k + 1 < my_units) load_x(unit_pos(p, unit0 + (k + 1) * ustep, th_rows), (k + 1) & 1, ptid, np);
+        cp_async_commit();
+        const unsigned ws = smem + (p.resident ? c : r & (kRing - 1)) * stage_bytes + half_chunk * subb;
+        const unsigned hid = hid0 + (r & 1) * kHidBytes + (half_chunk * 4 + t) * SL;
+        unsigned one[2] = {0u, 0u};  // the bias as B operand of one more step (24 channels: in the second step)
+        if (FIRST != kExp24) {
+          one[0] = lds32(ws + sub_bytes(ke, NP) + g * 8 + (t & 1) * 4);
+          one[1] = lds32(ws + sub_bytes(ke, NP) + 64 + g * 8 + (t & 1) * 4);
+        }
+        if constexpr (kWide) {
+          auto some = [&](auto count, int n) {  // `count` groups in flight
+            constexpr int N = decltype(count)::value;
+            float d[N][2][4];
+            unsigned xa = xs + a_off + n * 16 * XP, wk = ws + lane * 16;
+            const unsigned step = 16 * XP;
+#pragma unroll
+            for (int i = 0; i < N; ++i)
+#pragma unroll
+              for (int f = 0; f < 2; ++f) {
+                d[i][f][0] = d[i][f][1] = d[i][f][2] = d[i][f][3] = 0.0f;
+                mma1688(d[i][f], ones, ones, one[f]);
+              }
+            unsigned a[2][N][4];
+            uint4 b[2];
+            auto load = [&](int s) {  // (the next step's operands are under way while this one's are multiplied)
+#pragma unroll
+              for (int i = 0; i < N; ++i) ldsm4(xa + i * step, a[s][i]);
+              b[s] = lds128(wk);
+              xa += 32;
+              wk += 512;
+            };
+            auto mul = [&](int s) {
+#pragma unroll
+              for (int i = 0; i < N; ++i) {
+                mma16816(d[i][0], a[s][i], b[s].x, b[s].y);
+                mma16816(d[i][1], a[s][i], b[s].z, b[s].w);
+              }
+            };
+            load(0);
+            int kk = 1;
+#pragma unroll 1
+            for (; kk + 2 <= ke; kk += 2) {
+              load(1);
+              mul(0);
+              load(0);
+              mul(1);
+            }
+            if (kk < ke) {
+              load(1);
+              mul(0);
+              mul(1);
+            } else {
+              mul(0);
+            }
+#pragma unroll
+            for (int i = 0; i < N; ++i)
+#pragma unroll
+              for (int half = 0; half < 2; ++half) {
+                const uint2 e = lds64(tab + (n + i) * 128 + half * 64);
+                sts64(hid + e.x, min_f16x2(pack_f16x2<true>(d[i][0][half * 2], d[i][0][half * 2 + 1]), e.y),
+                      min_f16x2(pack_f16x2<true>(d[i][1][half * 2], d[i][1][half * 2 + 1]), e.y));
+              }
+          };
+          int n = 0;
+#pragma unroll 1
+          for (; n + 3 <= cnt; n += 3) some(std::integral_constant<int, 3>{}, n);
+          if (n + 2 <= cnt) some(std::integral_constant<int, 2>{}, n);
+          else if (n < cnt) some(std::integral_constant<int, 1>{}, n);
+        } else {
+          if (c == 0) {
+            edge = 0u;
+            for (int n = 0; n < min(cnt, 32); ++n) {
+              const bool out = lds32(tab + n * 64) != p.hi_e || lds32(tab + n * 64 + 32) != p.hi_e;
+              edge |= __any_sync(0xffffffffu, out) ? 1u << n : 0u;
+            }
+          }
+          const uint4 b0 = lds128(ws + lane * 16);
+          const uint4 b1 = FIRST == kExp16 ? b0 : lds128(ws + 512 + lane * 16);
+          unsigned xa = xs + a_off, xh = xs + h_off, tb = tab, at = hid + (mt0 * 16 + g) * 8;
+          auto some = [&](auto count, auto masked) {  // `count` groups in flight
+            constexpr int N = decltype(count)::value;
+            constexpr bool kMasked = decltype(masked)::value;
+            unsigned a[N][4], a2[N][4], hi[N][2];
+            float d[N][2][4];
+#pragma unroll
+            for (int i = 0; i < N; ++i) {
+              ldsm4(xa + i * 16 * XP, a[i]);
+              if (FIRST == kExp24) {
+                ldsm2(xh + i * 16 * XP, a2[i][0], a2[i][1]);
+                a2[i][2] = a2[i][3] = ones;
+              }
+              if (FIRST == kExp32) ldsm4(xa + i * 16 * XP + 32, a2[i]);
+              hi[i][0] = kMasked ? lds32(tb + i * 64) : p.hi_e;
+              hi[i][1] = kMasked ? lds32(tb + i * 64 + 32) : p.hi_e;
+            }
+#pragma unroll
+            for (int i = 0; i < N; ++i) {
+              mma16816z(d[i][0], a[i], b0.x, b0.y);
+              mma16816z(d[i][1], a[i], b0.z, b0.w);
+            }
+            if (FIRST != kExp16) {
+#pragma unroll
+              for (int i = 0; i < N; ++i) {
+                mma16816(d[i][0], a2[i], b1.x, b1.y);
+                mma16816(d[i][1], a2[i], b1.z, b1.w);
+              }
+            }
+            if (FIRST != kExp24) {
+#pragma unroll
+              for (int i = 0; i < N; ++i) {
+                mma1688(d[i][0], ones, ones, one[0]);
+                mma1688(d[i][1], ones, ones, one[1]);
+              }
+            }
+#pragma unroll
+            for (int i = 0; i < N; ++i)
+#pragma unroll
+              for (int half = 0; half < 2; ++half)
+                sts64(at + i * 128 + half * 64, min_f16x2(pack_f16x2<true>(d[i][0][half * 2], d[i][0][half * 2 + 1]), hi[i][half]),
+                      min_f16x2(pack_f16x2<true>(d[i][1][half * 2], d[i][1][half * 2 + 1]), hi[i][half]));
+            xa += N * 16 * XP;
+            xh += N * 16 * XP;
+            at += N * 128;
+            tb += N * 64;
+          };
+          auto groups = [&](auto count, unsigned edges) {
+            if (edges) some(count, std::true_type{});
+            else some(count, std::false_type{});
+          };
+          int n = 0;
+#pragma unroll 1
+          for (; n + 4 <= cnt; n += 4) groups(std::integral_constant<int, 4>{}, n < 29 ? edge >> n & 15u : 1u);
+          if (n + 2 <= cnt) {
+            groups(std::integral_constant<int, 2>{}, n < 31 ? edge >> n & 3u : 1u);
+            n += 2;
+          }
+          if (n < cnt) groups(std::integral_constant<int, 1>{}, n < 32 ? edge >> n & 1u : 1u);
+        }
+        named_arrive(1 + (r & 1), nthr);
+      }
+    }
+    cp_async_wait<0>();
+    if (p.ks == 1) return;
+    cluster_wait();
+  } else {
+    // ---- depthwise operator and projection of this warp's columns
+    unsigned dw_base;
+    const unsigned row_b = p.pitch * 8;
+    {
+      int col = warp * 16 + (lane & 15);
+      if (col >= p.ncols) col = 0;
+      int im, band, pos;
+      column_pos(p, col, im, band, pos);
+      dw_base = static_cast<unsigned>(im * p.sub_px + band * TR * S * p.pitch) * 8u + pos * 16u + (lane >> 4) * 16u;
+    }
+    const BandSel sel = band_sel(lane);
+    int r = 0;
+#pragma unroll 1
+    for (int k = 0; k < my_units; ++k) {
+      float acc[NV][NP][2][2][4];
+#pragma unroll
+      for (int j = 0; j < NP; ++j) {
+        const uint4 q = rank ? make_uint4(0u, 0u, 0u, 0u) : lds128(smem + p.off_bias + (4 * j + t) * 16);
+#pragma unroll
+        for (int v = 0; v < NV; ++v)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            acc[v][j][i >> 1][0][(i & 1) * 2] = __uint_as_float(q.x);
+            acc[v][j][i >> 1][0][(i & 1) * 2 + 1] = __uint_as_float(q.y);
+            acc[v][j][i >> 1][1][(i & 1) * 2] = __uint_as_float(q.z);
+            acc[v][j][i >> 1][1][(i & 1) * 2 + 1] = __uint_as_float(q.w);
+          }
+      }
+#pragma unroll 1
+      for (int c = 0; c < nch; ++c, ++r) {
+        named_sync(1 + (r & 1), nthr);  // the hidden tile is complete
+        const unsigned ws = smem + (p.resident ? c : r & (kRing - 1)) * stage_bytes;
+        depthwise_project<S, NP, TR, HC, SL>(ws, ke, subb, hid0 + (r & 1) * kHidBytes + dw_base, row_b, lane, p.hi_d, sel, acc);
+        if (r + 2 < total) named_arrive(3 + (r & 1), nthr);
+      }
+      if (p.ks == 1) {
+        const UnitPos u = unit_pos(p, unit0 + k * ustep, th_rows);
+        const unsigned xs = xs0 + (k & 1) * p.x_bytes;
+        store_col<S, 0, NV, NP>(p, u, xs, lane_col(p, S, TR, warp * 16 + g), 0, 0, t, acc);
+        store_col<S, 1, NV, NP>(p, u, xs, lane_col(p, S, TR, warp * 16 + g + 8), 0, 0, t, acc);
+      } else {
+        cluster_wait();  // every CTA of the cluster has started
+        push_sums<NV, NP>(p, red, warp, rank, p.ks, lane, acc,
+                          [](unsigned at, const float(&f)[4]) { st_cluster_f4(at, f[0], f[1], f[2], f[3]); });
+      }
+    }
+    if (p.ks == 1) return;
+  }
+  cluster_sync();
+  add_sums<S, TR, NV, NP>(p, unit_pos(p, unit0, th_rows), xs0, red, rank, p.ks, warp, nthr >> 5, lane);
 }
 
 // ---------------------------------------------------------------- host side
@@ -760,7 +1115,7 @@ bool layout_of(const LaunchRec& r, const BlockCfg& c, Layout* l) {
   l->pw = c.s == 1 ? c.tw / 2 : c.tw;
   l->ncols = c.ni * c.nb * l->pw;
   l->ngroups = (l->ncols + 15) / 16;
-  const int cap = max_warps(c.s, c.np, c.tr);
+  const int cap = max_warps(c.s, c.np, c.tr, c.ws);
   if (l->ngroups * wk > cap) return false;
   // warps without a column group still help with the first operator
   l->nw = std::min(cap / wk, std::max(l->ngroups, std::min(c.nw_min / wk, c.first != kNone ? (small ? l->mt : (l->mt + 1) / 2) : small ? 1 : 4)));
@@ -774,17 +1129,23 @@ bool layout_of(const LaunchRec& r, const BlockCfg& c, Layout* l) {
     l->en = l->nw > l->ngroups ? std::max(0, (rest + l->nw - l->ngroups - 1) / (l->nw - l->ngroups)) : 0;
     if (c.first == kNone) l->eg = l->en = 0;
   }
+  if (c.ws) {
+    l->nw = c.nw_min;
+    if (l->ngroups >= l->nw || l->nw > cap || (c.first == kExpWide && (l->nw - l->ngroups) % 2)) return false;
+    l->eg = 0;
+    l->en = (l->mt + l->nw - l->ngroups - 1) / (l->nw - l->ngroups);
+  }
   const int ke = ke_of(r, c);
   const int chid = c.first == kNone ? r.C : r.Cmid;
   l->nch = (chid + 16 * c.hc * wk - 1) / (16 * c.hc * wk);
-  if (c.ks > l->nch) return false;
+  if (c.ks > l->nch || (c.ws && l->nch / c.ks < 4)) return false;
   const int nchl = (l->nch + c.ks - 1) / c.ks;
-  l->stage_bytes = c.hc * wk * sub_bytes(ke, c.np);
+  l->stage_bytes = c.hc * wk * (c.ws ? ws_sub_bytes(ke, c.np) : sub_bytes(ke, c.np));
   l->resident = nchl <= kRing || nchl * l->stage_bytes <= c.resident_kb * 1024;
   const int nslot = l->resident ? nchl : kRing;
   const int xw = ke * 2 - (c.first == kExp24 ? 1 : 0);  // 16-byte units of a list pixel; an odd number of them is free of conflicts
   l->x_pitch = c.first == kNone ? 0u : static_cast<unsigned>((xw % 2 ? xw : xw + 1) * 16);
-  const int two = c.first != kNone && c.first != kExpWide ? 2 : 1;
+  const int two = c.first != kNone && (c.first != kExpWide || c.ws) ? 2 : 1;
   l->tab_bytes = static_cast<unsigned>(round_up_u64(l->mt * (c.first == kExpWide ? 128 : 64), 128));
   l->x_bytes = static_cast<unsigned>(round_up_u64(l->mt * 16 * l->x_pitch, 128));
   l->off_bias = static_cast<unsigned>(nslot * l->stage_bytes);
@@ -801,7 +1162,7 @@ bool layout_of(const LaunchRec& r, const BlockCfg& c, Layout* l) {
 
 // (two CTAs that together ask for exactly 227 KB do not share an SM: measured)
 int ctas_per_sm(const BlockCfg& c, const Layout& l) {
-  return std::max(1, std::min<int>((kSmemPerSm - 1024) / (static_cast<int>(l.bytes) + 1024), max_warps(c.s, c.np, c.tr) / l.nw));
+  return std::max(1, std::min<int>((kSmemPerSm - 1024) / (static_cast<int>(l.bytes) + 1024), max_warps(c.s, c.np, c.tr, c.ws) / l.nw));
 }
 
 // Clusters of `ks` CTAs that run at the same time with one CTA per SM: a cluster stays inside one of the chip's GPCs.  Found
@@ -813,7 +1174,23 @@ int cluster_slots(int ks) { return ks == 8 ? 15 : ks == 4 ? 33 : ks == 2 ? 73 : 
 // units (`thr`).  The coefficients are least-squares fits: of units that one CTA computes to 2060 measured launches (ten shapes at
 // batch 2 to 256 and image sizes 128 to 513; rms error 8 %), of units that several CTAs or warp sets share to 3000 more (11 %;
 // the configuration it picks takes 1.04 times the best one's time in the geometric mean).
+// Specialised warps, from 35578 launches of 46 shapes (batch 1 to 256, planes of 10 to 257): within 6 % (rms) near the best; the
+// configuration it picks takes 1.03 times the best one's time in the geometric mean, 1.10 at worst.  A chunk takes what the slower of
+// the two kinds of warps takes.
+double ws_cost_us(const LaunchRec& r, const BlockCfg& c, const Layout& l) {
+  const int ke = ke_of(r, c), nv = c.s == 1 ? c.tr : c.tr / 2, nprod = l.nw - l.ngroups, nwg = c.hc == 2 ? nprod / 2 : nprod;
+  const int slots = cluster_slots(c.ks) * ctas_per_sm(c, l), act = std::min(c.units, slots);
+  const double upc = (c.units + act - 1) / act, per_sm = (act * c.ks + 147) / 148, nchl = (l.nch + c.ks - 1) / c.ks;
+  const double rows = 4.0 * (c.s == 1 ? c.tr + 2 : 2 * c.tr + 1);
+  const double first = 90.4 + 13.05 * ((l.mt + nwg - 1) / nwg) * ke, second = 29.0 + c.hc * (73.6 * c.np * nv + 7.73 * rows);
+  double lat = (nchl + 1) * (44.4 + 18.7 * l.nw + std::max(first, second)) + 134.8 * c.np * nv +
+               209.5 * l.n_list * slices(r.C) / (nprod * 32.0) + (c.ks > 1 ? 53.0 : 0.0);
+  const double thr = nchl * c.hc * (7.83 * l.mt * ke + 116.9 * l.ngroups) + 60.0 * l.ngroups * c.np * nv;
+  const double edge = 1 + 0.45 / c.tw, a = upc * lat * edge, b = upc * per_sm * thr * edge;
+  return 3.8 + std::pow(std::pow(a, 1.314) + std::pow(b, 1.314), 1 / 1.314) / 1900.0;
+}
 double block_cost_us(const LaunchRec& r, const BlockCfg& c, const Layout& l) {
+  if (c.ws) return ws_cost_us(r, c, l);
   const int ke = ke_of(r, c), nv = c.s == 1 ? c.tr : c.tr / 2;
   const int occ = ctas_per_sm(c, l), slots = cluster_slots(c.ks) * occ;
   const double upc = (c.units + std::min(c.units, slots) - 1) / std::min(c.units, slots);  // units per CTA
@@ -848,9 +1225,8 @@ double block_cost_us(const LaunchRec& r, const BlockCfg& c, const Layout& l) {
   return 2.904 + std::cbrt(a * a * a + b * b * b) / 1965.0;
 }
 
-template <int S, int FIRST, int NP, int TR, int HC, bool SMALL>
-int launch_s(const BlockParams& p, int nw, unsigned smem, int grid, cudaStream_t stream) {
-  auto kern = block_mma_kernel<S, FIRST, NP, TR, HC, SMALL>;
+template <void (*kern)(BlockParams)>
+int launch_k(const BlockParams& p, int nw, unsigned smem, int grid, cudaStream_t stream) {
   static bool attr_done_dev[kMaxDevices] = {};
   bool& attr_done = attr_done_dev[current_device_slot()];
   if (!attr_done) {
@@ -876,8 +1252,11 @@ int launch_s(const BlockParams& p, int nw, unsigned smem, int grid, cudaStream_t
 
 template <int S, int FIRST, int NP, int TR, int HC>
 int launch_t(const BlockCfg& c, const BlockParams& p, int nw, unsigned smem, int grid, cudaStream_t stream) {
-  if (c.wk > 0) return launch_s<S, FIRST, NP, TR, 1, true>(p, nw, smem, grid, stream);
-  return launch_s<S, FIRST, NP, TR, HC, false>(p, nw, smem, grid, stream);
+  if constexpr (FIRST != kNone) {
+    if (c.ws) return launch_k<block_ws_kernel<S, FIRST, NP, TR>>(p, nw, smem, grid, stream);
+  }
+  if (c.wk > 0) return launch_k<block_mma_kernel<S, FIRST, NP, TR, 1, true>>(p, nw, smem, grid, stream);
+  return launch_k<block_mma_kernel<S, FIRST, NP, TR, HC, false>>(p, nw, smem, grid, stream);
 }
 
 // rows per warp and sub-blocks per chunk follow from the channel counts (each_config)
@@ -946,7 +1325,7 @@ void each_config(const LaunchRec& r, int kind, F&& f) {
       if (c.tiles_x != tx) continue;
       for (c.nb = 1; c.nb <= 28; ++c.nb) {
         const int th = c.nb * c.tr;
-        if (th - c.tr >= r.Ho) break;
+        if (th - c.tr >= r.Ho || (c.s * (th - 1) + 3) * (c.s * (c.tw - 1) + 3) > tile_pixels(c.first, false)) break;
         c.tiles_y = (r.Ho + th - 1) / th;
         c.whole = c.tiles_x == 1 && c.tiles_y == 1;
         for (c.ni = 1; c.ni <= (c.whole ? 8 : 1) && c.ni <= r.B; ++c.ni) {
@@ -961,7 +1340,31 @@ void each_config(const LaunchRec& r, int kind, F&& f) {
             c.wk = kSets[wi];
             if ((c.wk - 1) * 16 >= chid) break;  // a set without channels
             c.hc = c.first == kExpWide && c.wk == 0 ? 2 : 1;
-            for (c.ks = 1; c.ks <= 8; c.ks *= 2) {
+            // specialised warps: as many as fit one, two or three CTAs of an SM, or one less (a wide expansion's warps work in
+            // pairs); wide ones, of which there are few tiles, any number.  Narrow ones stay in one CTA: their clusters are small
+            // tiles for the kernel below.
+            bool specialised = false;
+            if (c.wk == 0 && c.first != kNone && (c.ni == 1 || c.first == kExpWide)) {
+              const int cap = max_warps(c.s, c.np, c.tr, true);
+              c.ws = 1;
+              for (c.ks = 1; c.ks <= (c.first == kExpWide ? 8 : 1); c.ks *= 2) {
+                if (c.ks > 1 && units * c.ks > 148) break;
+                for (c.nw_min = cap; c.nw_min >= 2; --c.nw_min) {
+                  if (c.first != kExpWide && cap / (cap / c.nw_min) != c.nw_min && cap / (cap / (c.nw_min + 1)) != c.nw_min + 1) continue;
+                  for (int rk = 0; rk < 2; ++rk) {
+                    c.resident_kb = rk ? 64 : 0;
+                    Layout l;
+                    if (!layout_of(r, c, &l) || (rk && !l.resident)) continue;
+                    specialised = true;
+                    if (c.ks == 1 || units <= cluster_slots(c.ks) * ctas_per_sm(c, l)) f(c, l);
+                    if (l.resident) break;
+                  }
+                }
+              }
+              c.ws = 0;
+            }
+            if (specialised && c.first == kExpWide) continue;
+            for (c.ks = specialised ? 2 : 1; c.ks <= 8; c.ks *= 2) {
               if (c.ks > 1 && units * c.ks > 148 * 2) break;  // a split pays only while SMs would be idle ...
               for (c.nw_min = 8; c.nw_min <= max_warps(c.s, c.np, c.tr); c.nw_min += max_warps(c.s, c.np, c.tr) == 12 ? 4 : 8) {
                 for (int rk = 0; rk < 2; ++rk) {
@@ -1009,7 +1412,7 @@ void block_mma_pack(const float* we, const float* be, const float* wd, const flo
   if (c.stem) return stem_block_pack(we, be, wd, bd, wp, bp, chid, cout, c, blob, r);
   const int ke = c.first == kNone ? 0 : (cin + 15) / 16, np = c.np;
   const int per = c.hc * std::max(1, c.wk), nsub = (chid + 16 * per - 1) / (16 * per) * per;
-  const size_t sb = sub_bytes(ke, np);
+  const size_t sb = c.ws ? ws_sub_bytes(ke, np) : sub_bytes(ke, np);
   const uint64_t woff = round_up_u64(blob->size(), 256);
   const uint64_t boff = round_up_u64(woff + nsub * sb, 256);
   blob->resize(boff + static_cast<size_t>(np) * 16 * sizeof(float), 0);
@@ -1024,6 +1427,19 @@ void block_mma_pack(const float* we, const float* be, const float* wd, const flo
           const int k = kk * 16 + hi8 * 8 + 2 * t + lo, h = channel_of(sub, f, n);
           if (h < chid && k < cin) e[(kk * 32 + lane) * 8 + w] = half_bits(we[static_cast<size_t>(h) * cin + k]);
         }
+    if (c.ws) {
+      uint16_t* words = reinterpret_cast<uint16_t*>(base + sub_bytes(ke, np));
+      for (int f = 0; f < 2; ++f)
+        for (int n = 0; n < 8; ++n) {
+          const int h = channel_of(sub, f, n);
+          uint16_t part[4] = {};
+          if (h < chid) bias_parts(be[h], part);
+          std::copy(part, part + 4, words + (f * 8 + n) * 4);
+          // up to 24 channels: the second step's last four values are free
+          if (c.first == kExp24)
+            for (int i = 0; i < 4; ++i) e[(32 + n * 4 + i / 2) * 8 + f * 4 + 2 + i % 2] = part[i];
+        }
+    }
     float* ebias = reinterpret_cast<float*>(base + ke * 512);
     uint16_t* tabl = reinterpret_cast<uint16_t*>(base + ke * 512 + kBiasBytes);
     float* dbias = reinterpret_cast<float*>(base + ke * 512 + kBiasBytes + kTableBytes);

@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstdint>
 
 #include "gi_internal.h"
@@ -34,7 +35,14 @@ __device__ __forceinline__ void mma16816(float (&d)[4], const unsigned (&a)[4], 
       : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
-// the same with the sum started from c0..c3 (a bias): saves copying it into the accumulators
+// the same with the sum started from zero
+__device__ __forceinline__ void mma16816z(float (&d)[4], const unsigned (&a)[4], unsigned b0, unsigned b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%10, %10, %10, %10};"
+      : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.0f));
+}
+// the same with the sum started from c0..c3 (a bias).  The compiler copies them into the accumulators: four moves, where the
+// values are used again
 __device__ __forceinline__ void mma16816c(float (&d)[4], const unsigned (&a)[4], unsigned b0, unsigned b1, float c0, float c1, float c2,
                                           float c3) {
   asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%10, %11, %12, %13};"
@@ -45,6 +53,12 @@ __device__ __forceinline__ void mma1688(float (&d)[4], unsigned a0, unsigned a1,
   asm("mma.sync.aligned.m16n8k8.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5}, {%6}, {%0, %1, %2, %3};"
       : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
       : "r"(a0), "r"(a1), "r"(b0));
+}
+// a += c, b += d in one instruction
+__device__ __forceinline__ void add2(float& a, float& b, float c, float d) {
+  asm("{\n\t.reg .b64 x, y;\n\tmov.b64 x, {%0, %1};\n\tmov.b64 y, {%2, %3};\n\tadd.rn.f32x2 x, x, y;\n\tmov.b64 {%0, %1}, x;\n\t}"
+      : "+f"(a), "+f"(b)
+      : "f"(c), "f"(d));
 }
 __device__ __forceinline__ uint4 lds128(unsigned addr) {
   uint4 v;
@@ -98,6 +112,33 @@ __host__ __device__ __forceinline__ int div_by(int i, unsigned mul) {
 
 // division of a small number by d > 1 is one high multiplication (div_by)
 inline unsigned magic(uint64_t d) { return static_cast<unsigned>(std::min<uint64_t>(0xffffffffull, (0xffffffffull + d) / d)); }
+
+// A bias as four products in the K steps of a matrix instruction: the A operand holds ones_word in each of its rows, the B operand the
+// bias in four fp16 parts, whose products and sum are exact in fp32 (11 bits each; the last part is for values beyond fp16's range).
+// A word of A: what lane t of a quad holds, two halves.
+__host__ __device__ constexpr unsigned ones_word(int t) { return t == 0 ? 0x10003c00u : t == 1 ? 0x78000004u : 0u; }  // 1, 2^-11; 2^-22, 2^15
+inline void bias_parts(float b, uint16_t (&part)[4]) {
+  auto value = [](uint16_t h) {
+    __half_raw raw;
+    raw.x = h;
+    return static_cast<double>(__half2float(__half(raw)));
+  };
+  auto take = [&](double& rest, double scale) {
+    const uint16_t h = f32_to_f16_rne(static_cast<float>(rest * scale));
+    rest -= value(h) / scale;
+    return h;
+  };
+  double rest = b;
+  part[0] = part[1] = part[2] = part[3] = 0;
+  if (!(std::fabs(b) < 2.0e9f)) {  // (infinity and what is as good as it for a tensor stored in fp16)
+    part[0] = f32_to_f16_rne(b);
+    return;
+  }
+  if (std::fabs(b) > 65504.0f) part[3] = take(rest, 1.0 / 32768.0);
+  part[0] = take(rest, 1.0);
+  part[1] = take(rest, 2048.0);
+  part[2] = take(rest, 4194304.0);
+}
 
 // channel of column n of fragment f in 16-channel block j: lane t of a quad holds the 4 channels of slice 4 j + t
 inline int channel_of(int j, int f, int n) { return 16 * j + 4 * (n >> 1) + 2 * f + (n & 1); }

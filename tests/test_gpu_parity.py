@@ -1151,6 +1151,42 @@ def test_blocks_whose_input_ends_inside_a_step_of_channels(batch, hw, cin):
     assert_close(run.run(xs)[t][sel], og.run(spec, [xs[0][sel]], storage="f16", fused=True)[t], api.GI_F16, str((batch, hw, cin)))
 
 
+# (batch, h, w, cin, hidden, cout, stride) of blocks whose expansion and depthwise operator run on warps of their own: the fewest
+# chunks of hidden channels it takes (four, the last one not full), more tiles than CTAs (two and more rounds of both hidden tiles),
+# rings and resident weights, one and two CTAs of an SM, tiles with and without pixels outside the image, clusters, several
+# images a tile, every width of the expansion and of the output
+WARP_ROLES_CASES = [(3, 129, 131, 16, 96, 24, 2), (40, 33, 35, 10, 50, 12, 1), (6, 131, 67, 16, 64, 40, 2), (8, 65, 67, 24, 144, 24, 1),
+                    (24, 57, 55, 21, 100, 21, 2), (40, 56, 56, 24, 144, 24, 1), (16, 65, 63, 32, 192, 32, 1), (33, 29, 27, 30, 200, 64, 2),
+                    (16, 33, 33, 64, 384, 64, 1), (21, 13, 13, 64, 384, 64, 1), (24, 13, 13, 96, 576, 96, 1), (24, 14, 14, 96, 576, 160, 2),
+                    (40, 14, 15, 41, 130, 41, 1), (300, 7, 7, 40, 160, 40, 1)]
+
+
+@pytest.mark.parametrize("case", WARP_ROLES_CASES)
+@pytest.mark.parametrize("bias", [None, 7.0e4])
+def test_blocks_with_roles_for_warps(case, bias):
+    """Equal to the oracle (first and last image) and to one kernel per op (all) within the tolerance; the same bits again.  Biases of
+    the expansion beyond the range of fp16, and far below its smallest number, are as good as others."""
+    batch, h, w, cin, hidden, cout, stride = case
+    spec = wl.inverted_residual_block(batch, h, w, cin, hidden, cout, stride)
+    if bias is not None:
+        conv = spec.ops[0]
+        conv.bias[::5] = bias
+        conv.bias[1::5] = -bias
+        conv.bias[2::5] = 3.0e-9
+    xs = [wl.make_input(spec)]
+    run = DeviceRun(spec, api.GI_F16, guard_bytes=4096)
+    names = [api.KERNEL_NAMES[launch.kernel] for launch in run.ex.launches()]
+    assert names.count("block_mma") == 1, names
+    outs = run.run(xs)
+    assert run.guard_intact()
+    t = spec.outputs[0]
+    sel = [0, batch - 1]
+    assert_close(outs[t][sel], og.run(spec, [xs[0][sel]], storage="f16", fused=True)[t], api.GI_F16, str(case))
+    assert_close(outs[t], DeviceRun(spec, api.GI_F16, cross_op=api.GI_XOP_OFF).run(xs)[t], api.GI_F16, "one kernel per op")
+    assert np.array_equal(outs[t], run.run(xs)[t])
+    assert api.gi_device_status() == 0
+
+
 def _twice_activated(kind, first, second):
     b = wl.GraphBuilder("twice_activated", 2, 32)
     if kind == "stem":
