@@ -15,6 +15,8 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "kernels.h"
 #include "pdl.cuh"
 
@@ -98,11 +100,11 @@ __device__ __forceinline__ Row widen(const uint2* u) {
 // MODE 1: stride 2, dilation 1, same padding limit - the last row of an output is the first row
 //         of the next
 // MODE 2: anything else - three rows fetched per output row, each tap tested
-// MODE 3: stride 1, dilation d > 1, padding d on every side (the dilated blocks of a segmentation backbone), whole planes
-//         staged by one copy: the rows of one residue class modulo d form an ordinary 3-row stencil among themselves
-//         (output row y reads rows y - d, y, y + d), so a thread owns (plane, residue, column) and walks its class
-//         with the three running accumulators of mode 0 - every staged pixel is fetched and widened three times, as in
-//         mode 0, instead of nine times as in mode 2
+// MODE 3: stride 1, dilation d >= 1, padding d on every side (the dilated blocks of a segmentation backbone, and planes of sizes
+//         that have no straight-line form), whole planes staged by one copy: the rows of one residue class modulo d form an
+//         ordinary 3-row stencil among themselves (output row y reads rows y - d, y, y + d), so a thread owns (plane, segment
+//         of a residue class, columns x and x + d) and walks its rows with the running accumulators of mode 0.  The two windows
+//         share two of their four pixels a row: 4 loads and 16 conversions for two outputs instead of 6 and 24.
 // PACKED (modes 0/1, small planes): a work item is a run of whole planes, which are contiguous in
 //         memory, so ONE bulk copy stages them back to back (many small copies are slow); the
 //         rows above and below a plane are then its neighbours' rows, so row validity is tested
@@ -220,7 +222,7 @@ __global__ void __launch_bounds__(256, (PLANE > 0 && !PAIR) ? 3 : 2) depthwise_f
   }
   __syncthreads();
   // column (pair of columns) owned by this thread in the first pass over an item's columns: (plane, sub-band, x)
-  const int wcols = PAIR ? Wo >> 1 : Wo;
+  const int wcols = MODE == 3 ? Wo / (2 * g.dil) * g.dil + min(g.dil, Wo % (2 * g.dil)) : PAIR ? Wo >> 1 : Wo;
   const int vp_first = static_cast<int>(threadIdx.x) / wcols;
   const int x_first = static_cast<int>(threadIdx.x) - vp_first * wcols;
   const int pi_first = vp_first / g.sub, sb_first = vp_first - pi_first * g.sub;
@@ -313,8 +315,10 @@ __global__ void __launch_bounds__(256, (PLANE > 0 && !PAIR) ? 3 : 2) depthwise_f
         sb = vp - pi * g.sub;
       }
       if (PAIR) x *= 2;
-      // (mode 3: `sb` is the residue class, whose first row is row sb)
-      const int ya = MODE == 3 ? sb : oy0 + sb * g.tr, yb = MODE == 3 ? H : min(oy1, ya + g.tr);
+      // mode 3: `sb` is a segment of a residue class, whose first row is row res_class; columns come in pairs g.dil apart
+      const int seg = MODE == 3 ? sb / g.dil : 0, res_class = sb - seg * g.dil;
+      if (MODE == 3) x += x / g.dil * g.dil;
+      const int ya = MODE == 3 ? res_class + seg * g.tr * g.dil : oy0 + sb * g.tr, yb = MODE == 3 ? H : min(oy1, ya + g.tr);
       if (ya >= yb) continue;
       // plane_zero: a pixel of the zero head; data: where pixel (0,0) of the plane would be staged
       const unsigned plane_zero = PACKED ? buf_addr : buf_addr + static_cast<unsigned>(pi) * g.plane_stride_px * 8u;
@@ -549,54 +553,85 @@ __global__ void __launch_bounds__(256, (PLANE > 0 && !PAIR) ? 3 : 2) depthwise_f
           if (j < kRowsOut) acc[j % 3] = fma_row_from(bias_acc, r, wlo, whi);
         }
       } else if (MODE == 3) {
-        const int d = g.dil;
-        const bool vl = x - d >= 0, vr = x + d < W;
-        unsigned at = data + static_cast<unsigned>((ya * W + x) * 8);
+        // columns x and x + d (the latter may lie outside the image): their windows share two of four pixels a row.  Row k of the
+        // residue class is kernel row 2 of the class's output row k - 1, row 1 of output row k, row 0 of output row k + 1.
+        const int d = g.dil, k0 = seg * g.tr, n = (H - res_class + d - 1) / d, k1 = min(n, k0 + g.tr);
+        if (k0 >= k1) continue;
+        const bool vl = x >= d, v2 = x + d < W, v3 = x + 2 * d < W;
         const unsigned row_step = static_cast<unsigned>(d * W) * 8u, dx = static_cast<unsigned>(d) * 8u;
-        auto next_row = [&]() {
-          uint2 u[3];
-          u[0] = make_uint2(0u, 0u);
-          u[2] = make_uint2(0u, 0u);
+        unsigned at = data + static_cast<unsigned>(((res_class + k0 * d) * W + x) * 8);
+        float2 plo[4], phi[4];
+        auto next4 = [&]() {
+          uint2 u[4];
+          u[0] = u[2] = u[3] = make_uint2(0u, 0u);
           if (vl) u[0] = lds64(at - dx);
           u[1] = lds64(at);
-          if (vr) u[2] = lds64(at + dx);
+          if (v2) u[2] = lds64(at + dx);
+          if (v3) u[3] = lds64(at + 2 * dx);
           at += row_step;
-          return widen(u);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            plo[i] = __half22float2(*reinterpret_cast<const __half2*>(&u[i].x));
+            phi[i] = __half22float2(*reinterpret_cast<const __half2*>(&u[i].y));
+          }
         };
-        const int n = (H - ya + d - 1) / d;  // rows of this residue class
-        // class row k is kernel row 2 of the class's output row k - 1, row 1 of output row k, row 0 of output row k + 1
-        Acc a0 = bias_acc, a1, a2;
-        Row r = next_row();
-        fma_row(a0, r, wlo + 3, whi + 3);
-        a1 = fma_row_from(bias_acc, r, wlo, whi);
-        for (int k = 1;; k += 3) {
-          if (k >= n) {
-            emit(a0);
-            break;
+        auto fma2 = [&](Acc* a, int kr) {
+#pragma unroll
+          for (int k = 0; k < 3; ++k) {
+            a[0].lo = __ffma2_rn(plo[k], wlo[kr * 3 + k], a[0].lo);
+            a[0].hi = __ffma2_rn(phi[k], whi[kr * 3 + k], a[0].hi);
+            a[1].lo = __ffma2_rn(plo[k + 1], wlo[kr * 3 + k], a[1].lo);
+            a[1].hi = __ffma2_rn(phi[k + 1], whi[kr * 3 + k], a[1].hi);
           }
-          r = next_row();
-          fma_row(a0, r, wlo + 6, whi + 6);
-          emit(a0);
-          fma_row(a1, r, wlo + 3, whi + 3);
-          a2 = fma_row_from(bias_acc, r, wlo, whi);
-          if (k + 1 >= n) {
-            emit(a1);
-            break;
+        };
+        auto start2 = [&](Acc* a) {
+          a[0] = a[1] = bias_acc;
+          fma2(a, 0);
+        };
+        auto emit2 = [&](const Acc* a) {
+          __half* const first = op;
+          emit(a[0]);
+          __half* const next = op;
+          op = first + d * 4;
+          if (v2) emit(a[1]);
+          op = next;
+        };
+        Acc a0[2], a1[2], a2[2];
+        a0[0] = a0[1] = bias_acc;
+        if (k0 > 0) {
+          at -= row_step;
+          next4();
+          fma2(a0, 0);
+        }
+        next4();
+        fma2(a0, 1);
+        start2(a1);
+        // rows beyond the segment's last output row end it; beyond the plane's last row there is nothing to add
+        for (int k = k0 + 1;; k += 3) {
+          if (k < n) {
+            next4();
+            fma2(a0, 2);
           }
-          r = next_row();
-          fma_row(a1, r, wlo + 6, whi + 6);
-          emit(a1);
-          fma_row(a2, r, wlo + 3, whi + 3);
-          a0 = fma_row_from(bias_acc, r, wlo, whi);
-          if (k + 2 >= n) {
-            emit(a2);
-            break;
+          emit2(a0);
+          if (k >= k1) break;
+          fma2(a1, 1);
+          start2(a2);
+          if (k + 1 < n) {
+            next4();
+            fma2(a1, 2);
           }
-          r = next_row();
-          fma_row(a2, r, wlo + 6, whi + 6);
-          emit(a2);
-          fma_row(a0, r, wlo + 3, whi + 3);
-          a1 = fma_row_from(bias_acc, r, wlo, whi);
+          emit2(a1);
+          if (k + 1 >= k1) break;
+          fma2(a2, 1);
+          start2(a0);
+          if (k + 2 < n) {
+            next4();
+            fma2(a2, 2);
+          }
+          emit2(a2);
+          if (k + 2 >= k1) break;
+          fma2(a0, 1);
+          start2(a1);
         }
       } else if (MODE == 1 && !PACKED && PLANE > 0) {
         // stride 2 without padding above / left on PLANE-wide planes, bands of exactly kRowsOut output rows: the band's
@@ -801,7 +836,7 @@ static int depthwise_f16_impl(const LaunchRec& r, const Ptrs& p, void* stream, b
   // 0.1055 -> 0.0901 ms, 112x112x96 (batch 128) 0.1393 -> 0.1290 ms, 56x56x144 0.1208 -> 0.1024 ms; 28x28 and
   // smaller planes are 2-12 % slower that way and keep one column per thread.
   const bool pair = g.stride == 1 && g.dil == 1 && g.pl == 1 && g.pt <= 1 && g.W % 2 == 0 && g.Wo == g.W && g.W >= 56;
-  const int wcols = pair ? g.Wo / 2 : g.Wo;
+  int wcols = pair ? g.Wo / 2 : g.Wo;
   // thread groups: as many "virtual planes" (plane x sub-band) as fit in ~256 threads
   int vp = 256 / wcols;
   if (vp < 1) vp = 1;
@@ -850,26 +885,16 @@ static int depthwise_f16_impl(const LaunchRec& r, const Ptrs& p, void* stream, b
     g.bands = (total_sub + g.sub - 1) / g.sub;
     g.plane_stride_px = smem_for(g);
   }
-  // dilated, stride 1, padded by the dilation, planes small enough to stage a few whole: the residue-class walk
-  const bool dilated = g.stride == 1 && g.dil > 1 && g.pt == g.dil && g.pl == g.dil && g.Ho == g.H && g.Wo == g.W && g.dil <= g.H &&
-                       static_cast<long long>(g.Pin) * 8 <= budget;
-  if (dilated) {
-    g.sub = g.dil;                          // residue classes
-    g.tr = (g.H + g.dil - 1) / g.dil;       // rows of the longest class
-    g.bands = 1;
-    long long planes = budget / (static_cast<long long>(g.Pin) * 8);
-    if (planes > 8) planes = 8;
-    g.nb = planes < g.B ? static_cast<int>(planes) : g.B;
-    g.plane_stride_px = smem_for(g);
-  }
+  const bool same = g.stride == 1 && g.pt == g.dil && g.pl == g.dil && g.Ho == g.H && g.Wo == g.W && g.dil <= g.H;
+  const bool dilated = same && g.dil > 1 && static_cast<long long>(g.Pin) * 8 <= budget;
   // the fast paths need the rows above and below the image to be at most one (zero rows in the buffer)
   const int overshoot = (g.Ho - 1) * g.stride - g.pt + 2 - (g.H - 1);
   const bool edge_ok = g.dil == 1 && g.pt <= 1 && overshoot <= 1;
-  const int mode = dilated ? 3 : (edge_ok && g.stride == 1) ? 0 : (edge_ok && g.stride == 2) ? 1 : 2;
+  int mode = dilated ? 3 : (edge_ok && g.stride == 1) ? 0 : (edge_ok && g.stride == 2) ? 1 : 2;
   // small planes, several per item, each walked top to bottom by its threads: stage them with one copy
-  const bool packed = mode == 3 || (mode != 2 && g.bands == 1 && g.sub == 1 && g.nb > 4 && !pair);
+  bool packed = mode == 3 || (mode != 2 && g.bands == 1 && g.sub == 1 && g.nb > 4 && !pair);
   g.packed = packed ? 1 : 0;
-  const size_t buf_bytes = packed ? static_cast<size_t>(g.Pin) * 8 * g.nb + 16 : static_cast<size_t>(g.plane_stride_px) * 8 * g.nb;
+  size_t buf_bytes = packed ? static_cast<size_t>(g.Pin) * 8 * g.nb + 16 : static_cast<size_t>(g.plane_stride_px) * 8 * g.nb;
   // bytes in flight hide the HBM latency: two CTAs per SM (the register file allows no more),
   // each with up to three items requested ahead of the one it computes
   // small square planes, stride 1, one padding row / column on every side, a thread per whole column: straight-line stencil
@@ -886,10 +911,35 @@ static int depthwise_f16_impl(const LaunchRec& r, const Ptrs& p, void* stream, b
   const int plane = whole_plane && g.H == 28 ? 28 : whole_plane && g.H == 14 ? 14 : whole_plane && g.H == 7 ? 7 : band28 ? 28 : pair14 ? g.W : down ? g.W : down14 ? 14 : 0;
   // the one-column straight-line variants need 80 registers: three CTAs per SM, so each gets a third of the shared memory
   const bool three_ctas = plane > 0 && !pair;
+  // Mode 3 for undilated planes as well where there is no straight-line form: half the threads, each with a third less to fetch and
+  // widen per output.  Not below 9 columns (5x5x1024 at batch 32 4.05 us with a column a thread, 4.39 with two) nor above 30 KB a plane
+  // (61x61x192 at batch 16 15.6 and 15.0, the largest measured).  us before and after: 33x33x960 batch 16 24.6, 21.0 (dilated by two 30,
+  // 21); 20x20x256 batch 32 7.5, 6.2; 40x40x128 batch 64 18.1, 15.9; 10x10x512 batch 256 17.9, 14.4; 26x26x192 batch 64 12.4, 11.9.
+  const bool walk = dilated || (mode == 0 && plane == 0 && !pair && same && g.W >= 9 && static_cast<long long>(g.Pin) * 8 <= 30 * 1024);
+  if (walk) {
+    mode = 3;
+    packed = true;
+    wcols = g.Wo / (2 * g.dil) * g.dil + std::min(g.dil, g.Wo % (2 * g.dil));
+    // a walk of at most 17 rows, shorter ones (down to five) until an SM has 256; items of about 120 walks
+    const int rows = (g.H + g.dil - 1) / g.dil;
+    int nseg = (rows + 16) / 17;
+    while (static_cast<long long>(g.S) * g.B * wcols * g.dil * nseg < 148 * 256 && rows >= 5 * (nseg + 1)) ++nseg;
+    const int per_plane = wcols * g.dil * nseg;
+    long long nb = std::max(1, (120 + per_plane / 2) / per_plane);
+    nb = std::max(1LL, std::min({nb, budget / (static_cast<long long>(g.Pin) * 8), static_cast<long long>(g.B)}));
+    const long long chunks = (g.B + nb - 1) / nb;
+    g.nb = static_cast<int>((g.B + chunks - 1) / chunks);
+    g.tr = (rows + nseg - 1) / nseg;
+    g.sub = g.dil * nseg;
+    g.bands = 1;
+    g.packed = 1;
+    buf_bytes = static_cast<size_t>(g.Pin) * 8 * g.nb + 16;
+  }
   const size_t per_cta = r.dw_cta_kb > 0 ? static_cast<size_t>(r.dw_cta_kb) * 1024
                                           : three_ctas ? static_cast<size_t>(73 * 1024) : static_cast<size_t>(kSmemPerCta);
   int nbuf = static_cast<int>(per_cta / buf_bytes);
   g.nbuf = nbuf > 4 ? 4 : nbuf < 2 ? 2 : nbuf;
+  if (walk) g.nbuf = 2;  // (three and four measured the same or slower: 33x33x960 21.0 us, 24)
   const size_t smem = buf_bytes * g.nbuf;
   if (smem > static_cast<size_t>(kMaxSmem)) return static_cast<int>(cudaErrorInvalidConfiguration);
   g.bchunks = (g.B + g.nb - 1) / g.nb;

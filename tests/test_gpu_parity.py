@@ -1278,6 +1278,24 @@ def test_depthwise_planes_with_rows_that_no_window_reaches(case):
     check_outputs(b.finish(), api.GI_F16)
 
 
+# (batch, h, w, c, dilation): planes without a straight-line form, two columns a thread: odd and even widths around whole and broken
+# groups of 2 d columns, one to four segments of a class of rows, classes of one row, the smallest width, the largest plane, more
+# items than CTAs and a last item with fewer planes
+@pytest.mark.parametrize("case", [(1, 9, 9, 4, 1), (3, 33, 33, 20, 1), (2, 10, 17, 12, 1), (41, 13, 12, 7, 1), (2, 5, 61, 8, 1), (300, 20, 20, 16, 1), (7, 61, 61, 64, 1),
+                                  (2, 34, 10, 260, 1), (2, 33, 35, 12, 4), (5, 33, 33, 96, 2), (1, 9, 33, 8, 9), (3, 7, 14, 8, 3), (2, 11, 3, 8, 2), (17, 61, 13, 8, 5)])
+@pytest.mark.parametrize("residual", [False, True])
+def test_depthwise_two_columns_a_thread(case, residual):
+    batch, h, w, c, d = case
+    b = wl.GraphBuilder("depthwise_walk", batch, 35)
+    x = b.input(h, w, c)
+    y = b.activation(b.depthwise(x, 3, 1, d), wl.ACT_RELU6)
+    b.output(b.activation(b.add(x, y), wl.ACT_RELU) if residual else y)
+    run, xs, outs = check_outputs(b.finish(), api.GI_F16, images=sorted({0, batch // 2, batch - 1}))
+    assert "depthwise" in [api.KERNEL_NAMES[launch.kernel] for launch in run.ex.launches()]
+    assert all(np.array_equal(v, run.run(xs)[t]) for t, v in outs.items())
+    assert api.gi_device_status() == 0
+
+
 # (graph, layout of its output, bytes between the start of the output and that of the input): one launch from the caller's input to
 # the caller's output
 @pytest.mark.parametrize("make,out_layout,shift", [(lambda: wl.separable_block(2, 40, 38, 32, 32), api.GI_NHWC, 0), (lambda: wl.separable_block(2, 40, 38, 32, 32), api.GI_NHWC, 4096),
