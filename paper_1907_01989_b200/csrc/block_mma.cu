@@ -48,6 +48,7 @@
 #include <cstring>
 #include <type_traits>
 
+#include "bias_split.h"
 #include "kernels.h"
 #include "mma_frag.cuh"
 #include "pdl.cuh"
@@ -1342,9 +1343,9 @@ void each_config(const LaunchRec& r, int kind, F&& f) {
             c.hc = c.first == kExpWide && c.wk == 0 ? 2 : 1;
             // specialised warps: as many as fit one, two or three CTAs of an SM, or one less (a wide expansion's warps work in
             // pairs); wide ones, of which there are few tiles, any number.  Narrow ones stay in one CTA: their clusters are small
-            // tiles for the kernel below.
+            // tiles for the older kernel.  Not with a bias of the expansion that has no parts (bias_split.h).
             bool specialised = false;
-            if (c.wk == 0 && c.first != kNone && (c.ni == 1 || c.first == kExpWide)) {
+            if (c.wk == 0 && c.first != kNone && r.split_bias && (c.ni == 1 || c.first == kExpWide)) {
               const int cap = max_warps(c.s, c.np, c.tr, true);
               c.ws = 1;
               for (c.ks = 1; c.ks <= (c.first == kExpWide ? 8 : 1); c.ks *= 2) {

@@ -111,6 +111,7 @@ struct LaunchRec {
   // depthwise 3x3 and the convolutions around it as one kernel: `ep` is the first operator's epilogue, `ep_mid` the depthwise
   // one's behind it, `ep2` the projection's; Cmid / Co2, stride, pads and (Ho, Wo) as above; (H, W) the depthwise input
   BlockCfg block;
+  int split_bias = 1;  // the first operator's biases can be written as fp16 parts (bias_split.h)
   int nhwc_out = 0;  // the kernel writes the caller's NHWC output itself
   // a launch that reads the caller's NHWC input while it writes a caller's output: arena bytes for a copy of the input where the
   // caller handed over overlapping buffers, and the sizes of both

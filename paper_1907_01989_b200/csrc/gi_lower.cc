@@ -5,6 +5,7 @@
 #include <cstdlib>
 #include <cstring>
 
+#include "bias_split.h"
 #include "gi_internal.h"
 #include "kernels.h"
 
@@ -564,6 +565,10 @@ void find_groups(const gi_graph& g, gi_exec* e) {
     gr.rec = block_rec(g, e, b);
     gr.rec.lead = b.first;
     gr.rec.dw_op = b.dw;
+    if (b.kind == BLOCK_EXPANSION) {
+      const std::vector<float>& bias = g.ops[e->ops[b.first].graph_op].bias;
+      gr.rec.split_bias = std::all_of(bias.begin(), bias.end(), bias_splits);
+    }
     // Every block is asked about by itself: what the kernel runs depends on more than its sizes (dilation, padding, residual, the
     // caller's layout), and the search takes 0.1 ms.
     double us = 0.0;

@@ -6,7 +6,6 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <cmath>
 #include <cstdint>
 
 #include "gi_internal.h"
@@ -113,32 +112,8 @@ __host__ __device__ __forceinline__ int div_by(int i, unsigned mul) {
 // division of a small number by d > 1 is one high multiplication (div_by)
 inline unsigned magic(uint64_t d) { return static_cast<unsigned>(std::min<uint64_t>(0xffffffffull, (0xffffffffull + d) / d)); }
 
-// A bias as four products in the K steps of a matrix instruction: the A operand holds ones_word in each of its rows, the B operand the
-// bias in four fp16 parts, whose products and sum are exact in fp32 (11 bits each; the last part is for values beyond fp16's range).
-// A word of A: what lane t of a quad holds, two halves.
+// The A operand that a bias in four parts (bias_split.h) is multiplied by: what lane t of a quad holds, two halves.
 __host__ __device__ constexpr unsigned ones_word(int t) { return t == 0 ? 0x10003c00u : t == 1 ? 0x78000004u : 0u; }  // 1, 2^-11; 2^-22, 2^15
-inline void bias_parts(float b, uint16_t (&part)[4]) {
-  auto value = [](uint16_t h) {
-    __half_raw raw;
-    raw.x = h;
-    return static_cast<double>(__half2float(__half(raw)));
-  };
-  auto take = [&](double& rest, double scale) {
-    const uint16_t h = f32_to_f16_rne(static_cast<float>(rest * scale));
-    rest -= value(h) / scale;
-    return h;
-  };
-  double rest = b;
-  part[0] = part[1] = part[2] = part[3] = 0;
-  if (!(std::fabs(b) < 2.0e9f)) {  // (infinity and what is as good as it for a tensor stored in fp16)
-    part[0] = f32_to_f16_rne(b);
-    return;
-  }
-  if (std::fabs(b) > 65504.0f) part[3] = take(rest, 1.0 / 32768.0);
-  part[0] = take(rest, 1.0);
-  part[1] = take(rest, 2048.0);
-  part[2] = take(rest, 4194304.0);
-}
 
 // channel of column n of fragment f in 16-channel block j: lane t of a quad holds the 4 channels of slice 4 j + t
 inline int channel_of(int j, int f, int n) { return 16 * j + 4 * (n >> 1) + 2 * f + (n & 1); }

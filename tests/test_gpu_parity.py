@@ -1187,6 +1187,39 @@ def test_blocks_with_roles_for_warps(case, bias):
     assert api.gi_device_status() == 0
 
 
+# biases of an expansion: around the limits of fp16 and of what its parts hold, masked channels up to infinity
+LARGE_BIASES = [v * s for v in (65504.0, 65520.0, 1.0e5, 1.3e8, 2.0 ** 27, 1.5e8, 2.8e8, 3.0e8, 1.0e9, 2.0e9, 3.0e9, 1.0e20, 3.4028235e38, float("inf")) for s in (-1.0, 1.0)]
+
+
+@pytest.mark.parametrize("case", [(3, 129, 131, 16, 96, 24, 2), (40, 56, 56, 24, 144, 24, 1), (16, 65, 63, 32, 192, 32, 1), (16, 33, 33, 64, 384, 64, 1)])
+@pytest.mark.parametrize("biases", ["all", "finite", "negative", "products"])
+def test_expansion_biases_of_any_size(case, biases):
+    """Equal to the oracle and to one kernel per op, for each width of the expansion: a hidden channel whose bias is far beyond what
+    products can reach holds 0 or the activation's limit, and its neighbours what they always hold; one whose products take its bias
+    away again ("products") holds the difference to fp32's precision."""
+    batch, h, w, cin, hidden, cout, stride = case
+    spec = wl.inverted_residual_block(batch, h, w, cin, hidden, cout, stride)
+    conv, x = spec.ops[0], wl.make_input(spec)
+    if biases == "products":
+        values = [12345.678, 60000.3, 1000.0007, 70003.0, 130000.5]
+        x[..., 0:2] = 1.0
+        for i, v in enumerate(values):
+            half = np.float32(np.float16(v / 2 if v > 65504 else v))  # (the largest need two inputs)
+            conv.bias[3 * i:: 3 * len(values)] = v
+            conv.weights.reshape(hidden, cin)[3 * i:: 3 * len(values), 0] = -half
+            conv.weights.reshape(hidden, cin)[3 * i:: 3 * len(values), 1] = -half if v > 65504 else 0.0
+    else:
+        values = [v for v in LARGE_BIASES if biases == "all" or (abs(v) <= 2.0 ** 27 if biases == "finite" else v < 0)]
+        for i, v in enumerate(values):
+            conv.bias[2 * i:: 2 * len(values)] = v
+    run = DeviceRun(spec, api.GI_F16)
+    names = [api.KERNEL_NAMES[launch.kernel] for launch in run.ex.launches()]
+    assert names.count("block_mma") == 1, names
+    got, t, sel = run.run([x])[spec.outputs[0]], spec.outputs[0], [0, batch - 1]
+    assert_close(got[sel], og.run(spec, [x[sel]], storage="f16", fused=True)[t], api.GI_F16, str((case, biases)))
+    assert_close(got, DeviceRun(spec, api.GI_F16, cross_op=api.GI_XOP_OFF).run([x])[t], api.GI_F16, "one kernel per op")
+
+
 def _twice_activated(kind, first, second):
     b = wl.GraphBuilder("twice_activated", 2, 32)
     if kind == "stem":

@@ -4,6 +4,7 @@ import ctypes as C
 import os
 import random
 import re
+import subprocess
 
 import numpy as np
 import pytest
@@ -788,6 +789,44 @@ def test_no_block_reads_an_image_of_the_callers_layout_beyond_32_bit_offsets(c, 
     small enough)."""
     names = _launch_names(wl.inverted_residual_block(1, 2 ** 31 // (w * c) + 2, w, c, hidden, cout, 1))
     assert names[0] == "pack", names
+
+
+BIAS_SPLIT_MAIN = r"""
+#include <cstdio>
+#include <cstring>
+#include "bias_split.h"
+int main() {  // floats from standard input -> whether they split, and their four parts
+  float b;
+  while (std::fread(&b, 4, 1, stdin) == 1) {
+    uint16_t out[5] = {gi::bias_splits(b), 0, 0, 0, 0}, part[4];
+    if (out[0]) gi::bias_parts(b, part), std::memcpy(out + 1, part, 8);
+    std::fwrite(out, 2, 5, stdout);
+  }
+}
+"""
+
+
+def test_bias_in_four_fp16_parts(tmp_path):
+    """Over the whole range of fp32: a bias that is said to split does so into finite parts whose products with 1, 2^-11, 2^-22 and 2^15
+    add up to it (below 2^-22: to within 2^-47); every other one - beyond 2^27, infinite, NaN - is refused."""
+    csrc = os.path.join(ROOT, "paper_1907_01989_b200", "csrc")
+    (tmp_path / "main.cc").write_text(BIAS_SPLIT_MAIN)
+    exe = str(tmp_path / "bias_split")
+    subprocess.check_call(["g++", "-std=c++17", "-O1", "-I", csrc, "-I", os.path.join(ROOT, "include"), str(tmp_path / "main.cc"), os.path.join(csrc, "gi_graph.cc"), "-o", exe])
+    rng = np.random.Generator(np.random.PCG64(11))
+    bits = np.concatenate([rng.integers(0, 2 ** 32, 200000, dtype=np.uint64),  # any pattern, NaN and infinities among them
+                           rng.integers(0x30000000, 0x4f800000, 200000, dtype=np.uint64)])  # 2^-31 .. 2^32
+    edge = [0.0, 65504.0, 65519.99, 65520.0, 70000.0, 2.0 ** 27, 2.0 ** 27 + 16, 1.5e8, 2.8e8, 1e9, 2e9, 3e9, 3.4028235e38, np.inf, np.nan, 3e-9, 1e-30, 1e-45]
+    b = np.concatenate([bits.astype(np.uint32).view(np.float32), np.float32(edge), -np.float32(edge)])
+    out = np.frombuffer(subprocess.run([exe], input=b.tobytes(), stdout=subprocess.PIPE, check=True).stdout, dtype=np.uint16).reshape(-1, 5)
+    splits = out[:, 0] != 0
+    assert np.array_equal(splits, np.abs(b) <= 2.0 ** 27)
+    parts = np.ascontiguousarray(out[splits, 1:]).view(np.float16).astype(np.float64)
+    assert np.isfinite(parts).all()
+    total, want = parts @ np.array([1.0, 2.0 ** -11, 2.0 ** -22, 2.0 ** 15]), b[splits].astype(np.float64)
+    large = np.abs(want) >= 2.0 ** -22
+    assert np.array_equal(total[large], want[large])
+    assert np.abs(total - want).max() <= 2.0 ** -47
 
 
 def test_device_status_bits_name_their_kernels():
