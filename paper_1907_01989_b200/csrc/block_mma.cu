@@ -1295,7 +1295,8 @@ int launch_first(const BlockCfg& c, const BlockParams& p, int nw, unsigned smem,
   }
 }
 
-// Calls f(configuration, layout) for every configuration that runs the block in `r`.
+// Calls f(configuration, layout, spare) for every configuration that runs the block in `r`.  spare: the older kernel beside the
+// specialised one (block_mma_choose).
 template <class F>
 void each_config(const LaunchRec& r, int kind, F&& f) {
   if (r.kh != 3 || r.kw != 3 || r.sh != r.sw || (r.sh != 1 && r.sh != 2) || r.dh != 1 || r.dw != 1) return;
@@ -1344,7 +1345,7 @@ void each_config(const LaunchRec& r, int kind, F&& f) {
             // specialised warps: as many as fit one, two or three CTAs of an SM, or one less (a wide expansion's warps work in
             // pairs); wide ones, of which there are few tiles, any number.  Narrow ones stay in one CTA: their clusters are small
             // tiles for the older kernel.  Not with a bias of the expansion that has no parts (bias_split.h).
-            bool specialised = false;
+            int specialised = 0;  // cluster sizes with such a layout
             if (c.wk == 0 && c.first != kNone && r.split_bias && (c.ni == 1 || c.first == kExpWide)) {
               const int cap = max_warps(c.s, c.np, c.tr, true);
               c.ws = 1;
@@ -1356,16 +1357,17 @@ void each_config(const LaunchRec& r, int kind, F&& f) {
                     c.resident_kb = rk ? 64 : 0;
                     Layout l;
                     if (!layout_of(r, c, &l) || (rk && !l.resident)) continue;
-                    specialised = true;
-                    if (c.ks == 1 || units <= cluster_slots(c.ks) * ctas_per_sm(c, l)) f(c, l);
+                    specialised |= c.ks;
+                    if (c.ks == 1 || units <= cluster_slots(c.ks) * ctas_per_sm(c, l)) f(c, l, false);
                     if (l.resident) break;
                   }
                 }
               }
               c.ws = 0;
             }
-            if (specialised && c.first == kExpWide) continue;
-            for (c.ks = specialised ? 2 : 1; c.ks <= 8; c.ks *= 2) {
+            const bool spare = specialised && c.first == kExpWide;
+            for (c.ks = 1; c.ks <= 8; c.ks *= 2) {
+              if (specialised & c.ks) continue;
               if (c.ks > 1 && units * c.ks > 148 * 2) break;  // a split pays only while SMs would be idle ...
               for (c.nw_min = 8; c.nw_min <= max_warps(c.s, c.np, c.tr); c.nw_min += max_warps(c.s, c.np, c.tr) == 12 ? 4 : 8) {
                 for (int rk = 0; rk < 2; ++rk) {
@@ -1373,8 +1375,9 @@ void each_config(const LaunchRec& r, int kind, F&& f) {
                   Layout l;
                   if (!layout_of(r, c, &l) || (c.nw_min > 8 && l.nw <= 8)) break;  // nw_min 8 has given the same layout
                   if (rk && !l.resident) break;
+                  if (spare && !l.resident) continue;
                   // ... in one wave
-                  if (c.ks == 1 || units <= cluster_slots(c.ks) * ctas_per_sm(c, l)) f(c, l);
+                  if (c.ks == 1 || units <= cluster_slots(c.ks) * ctas_per_sm(c, l)) f(c, l, spare);
                   if (l.resident) break;
                 }
               }
@@ -1392,16 +1395,29 @@ uint16_t half_bits(float v) { return f32_to_f16_rne(v); }
 // Chooses tile, image and cluster split for the block in `r` (C -> Cmid -> Co2, or C -> Co2 for BLOCK_PAIR; stride r.sh, output
 // Ho x Wo).  False if no configuration runs it; `us` receives the estimate the choice was made by.
 bool block_mma_choose(const LaunchRec& r, int kind, BlockCfg* best, double* us) {
-  double best_cost = 0.0;
-  bool found = false;
+  double best_cost = 0.0, spare_cost = 0.0;
+  BlockCfg spare_cfg;
+  bool found = false, spare_found = false;
   if (kind == BLOCK_STEM) return stem_block_choose(r, best, us);
-  each_config(r, kind, [&](const BlockCfg& c, const Layout& l) {
+  each_config(r, kind, [&](const BlockCfg& c, const Layout& l, bool spare) {
     const double cost = block_cost_us(r, c, l);
-    if (found && cost >= best_cost) return;
-    found = true;
-    best_cost = cost;
-    *best = c;
+    bool& any = spare ? spare_found : found;
+    double& least = spare ? spare_cost : best_cost;
+    if (any && cost >= least) return;
+    any = true;
+    least = cost;
+    (spare ? spare_cfg : *best) = c;
   });
+  // Wide expansions on tiles for which there are specialised warps, at the cluster sizes for which there are none (fewer than four
+  // chunks a CTA): the older kernel, where its weights stay in shared memory, stands in for warp sets, not for specialised warps.
+  // us, it and the choice without it: 6x6 80-480-80 batch 54 10.9, 13.3; 10x10 64-384-64 batch 28 11.0, 12.1; 12x12 64-384-96 batch
+  // 15 10.3, 11.3; the other way 5x5 64-384-64 batch 108 12.2, 11.7; 10x10 64-384-64 batch 17 11.6, 10.2.  Of 4000 random blocks
+  // it changes the choice for 65: 0.93 times the time (geometric mean), six slower.  Set against specialised warps too it would
+  // take their place where they are faster (6x6 160-960-160 batch 55 30.6, 22.1), and with a ring of weights it is slower than sets.
+  if (found && spare_found && !best->ws && spare_cost < best_cost) {
+    *best = spare_cfg;
+    best_cost = spare_cost;
+  }
   if (us) *us = best_cost;
   return found;
 }

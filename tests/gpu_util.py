@@ -94,6 +94,17 @@ class DeviceRun:
         return self.arena[ti.offset: ti.offset + ti.bytes].cpu().numpy().view(np_dtype(self.storage))
 
 
+def device_kernels(run: DeviceRun, inputs):
+    """Names of this library's kernels that a run launched, in order, with their template arguments: "block_ws_kernel<1, 4, 4, 1>"."""
+    import re
+    from torch.profiler import ProfilerActivity, profile
+    run.run(inputs)
+    with profile(activities=[ProfilerActivity.CUDA], acc_events=True) as prof:
+        run.run(inputs)
+    events = sorted((e for e in prof.events() if "gi::" in e.name), key=lambda e: e.time_range.start)
+    return [m.group(1) for m in (re.search(r"gi::(?:\(anonymous namespace\)::)?(\w+(?:<[^>]*>)?)\(", e.name) for e in events) if m]
+
+
 def error_report(got: np.ndarray, ref: np.ndarray, storage):
     atol, rtol = TOL[storage]
     norm = np.abs(got.astype(np.float64) - ref.astype(np.float64)) / (atol + rtol * np.abs(ref.astype(np.float64)))

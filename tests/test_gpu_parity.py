@@ -9,7 +9,7 @@ from oracle import ops as oops
 from paper_1907_01989_b200 import api
 from paper_1907_01989_b200 import workloads as wl
 
-from gpu_util import DeviceRun, assert_close
+from gpu_util import DeviceRun, assert_close, device_kernels
 
 pytestmark = pytest.mark.gpu
 
@@ -1218,6 +1218,27 @@ def test_expansion_biases_of_any_size(case, biases):
     got, t, sel = run.run([x])[spec.outputs[0]], spec.outputs[0], [0, batch - 1]
     assert_close(got[sel], og.run(spec, [x[sel]], storage="f16", fused=True)[t], api.GI_F16, str((case, biases)))
     assert_close(got, DeviceRun(spec, api.GI_F16, cross_op=api.GI_XOP_OFF).run([x])[t], api.GI_F16, "one kernel per op")
+
+
+# (batch, h, w, cin, hidden, cout, stride): wide expansions on tiles whose only cluster of specialised warps is too small for the launch;
+# one, two and four images a tile, strides, planes with a broken last tile
+@pytest.mark.parametrize("case", [(28, 10, 10, 64, 384, 64, 1), (54, 6, 6, 80, 480, 80, 1), (14, 10, 10, 72, 432, 120, 2), (15, 12, 12, 64, 384, 96, 1)])
+def test_small_tiles_whose_weights_stay_in_a_cluster(case):
+    """These run on the kernel with one kind of warps, a cluster of CTAs whose weights are resident: not on sets of warps (last
+    template argument: small tiles)."""
+    batch, h, w, cin, hidden, cout, stride = case
+    spec = wl.inverted_residual_block(batch, h, w, cin, hidden, cout, stride)
+    xs = [wl.make_input(spec)]
+    run = DeviceRun(spec, api.GI_F16, guard_bytes=4096)
+    kernels = [k for k in device_kernels(run, xs) if k.startswith("block")]
+    assert len(kernels) == 1 and kernels[0].startswith("block_mma_kernel<") and kernels[0].endswith("false>"), kernels
+    t, sel = spec.outputs[0], [0, batch - 1]
+    outs = run.run(xs)
+    assert run.guard_intact()
+    assert_close(outs[t][sel], og.run(spec, [xs[0][sel]], storage="f16", fused=True)[t], api.GI_F16, str(case))
+    assert_close(outs[t], DeviceRun(spec, api.GI_F16, cross_op=api.GI_XOP_OFF).run(xs)[t], api.GI_F16, "one kernel per op")
+    assert np.array_equal(outs[t], run.run(xs)[t])
+    assert api.gi_device_status() == 0
 
 
 def _twice_activated(kind, first, second):
