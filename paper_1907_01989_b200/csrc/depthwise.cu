@@ -102,9 +102,10 @@ __device__ __forceinline__ Row widen(const uint2* u) {
 // MODE 2: anything else - three rows fetched per output row, each tap tested
 // MODE 3: stride 1, dilation d >= 1, padding d on every side (the dilated blocks of a segmentation backbone, and planes of sizes
 //         that have no straight-line form), whole planes staged by one copy: the rows of one residue class modulo d form an
-//         ordinary 3-row stencil among themselves (output row y reads rows y - d, y, y + d), so a thread owns (plane, segment
-//         of a residue class, columns x and x + d) and walks its rows with the running accumulators of mode 0.  The two windows
-//         share two of their four pixels a row: 4 loads and 16 conversions for two outputs instead of 6 and 24.
+//         ordinary 3-row stencil among themselves (output row y reads rows y - d, y, y + d), so a thread owns (plane,
+//         residue class, column x) and walks its class with the running accumulators of mode 0.  With PAIR it owns a segment of
+//         the class and columns x and x + d: the two windows share two of their four pixels a row, 4 loads and 16 conversions for
+//         two outputs instead of 6 and 24.
 // PACKED (modes 0/1, small planes): a work item is a run of whole planes, which are contiguous in
 //         memory, so ONE bulk copy stages them back to back (many small copies are slow); the
 //         rows above and below a plane are then its neighbours' rows, so row validity is tested
@@ -222,7 +223,7 @@ __global__ void __launch_bounds__(256, (PLANE > 0 && !PAIR) ? 3 : 2) depthwise_f
   }
   __syncthreads();
   // column (pair of columns) owned by this thread in the first pass over an item's columns: (plane, sub-band, x)
-  const int wcols = MODE == 3 ? Wo / (2 * g.dil) * g.dil + min(g.dil, Wo % (2 * g.dil)) : PAIR ? Wo >> 1 : Wo;
+  const int wcols = !PAIR ? Wo : MODE == 3 ? Wo / (2 * g.dil) * g.dil + min(g.dil, Wo % (2 * g.dil)) : Wo >> 1;
   const int vp_first = static_cast<int>(threadIdx.x) / wcols;
   const int x_first = static_cast<int>(threadIdx.x) - vp_first * wcols;
   const int pi_first = vp_first / g.sub, sb_first = vp_first - pi_first * g.sub;
@@ -314,10 +315,9 @@ __global__ void __launch_bounds__(256, (PLANE > 0 && !PAIR) ? 3 : 2) depthwise_f
         pi = vp / g.sub;
         sb = vp - pi * g.sub;
       }
-      if (PAIR) x *= 2;
       // mode 3: `sb` is a segment of a residue class, whose first row is row res_class; columns come in pairs g.dil apart
-      const int seg = MODE == 3 ? sb / g.dil : 0, res_class = sb - seg * g.dil;
-      if (MODE == 3) x += x / g.dil * g.dil;
+      if (PAIR) x += MODE == 3 ? x / g.dil * g.dil : x;
+      const int seg = MODE == 3 && PAIR ? sb / g.dil : 0, res_class = sb - seg * g.dil;
       const int ya = MODE == 3 ? res_class + seg * g.tr * g.dil : oy0 + sb * g.tr, yb = MODE == 3 ? H : min(oy1, ya + g.tr);
       if (ya >= yb) continue;
       // plane_zero: a pixel of the zero head; data: where pixel (0,0) of the plane would be staged
@@ -553,15 +553,16 @@ __global__ void __launch_bounds__(256, (PLANE > 0 && !PAIR) ? 3 : 2) depthwise_f
           if (j < kRowsOut) acc[j % 3] = fma_row_from(bias_acc, r, wlo, whi);
         }
       } else if (MODE == 3) {
-        // columns x and x + d (the latter may lie outside the image): their windows share two of four pixels a row.  Row k of the
-        // residue class is kernel row 2 of the class's output row k - 1, row 1 of output row k, row 0 of output row k + 1.
-        const int d = g.dil, k0 = seg * g.tr, n = (H - res_class + d - 1) / d, k1 = min(n, k0 + g.tr);
+        // column x, or x and x + d (the latter may lie outside the image): their windows share two of four pixels a row.  Row k of
+        // the residue class is kernel row 2 of the class's output row k - 1, row 1 of output row k, row 0 of output row k + 1.
+        constexpr int kCols = PAIR ? 2 : 1;
+        const int d = g.dil, k0 = PAIR ? seg * g.tr : 0, n = (H - res_class + d - 1) / d, k1 = PAIR ? min(n, k0 + g.tr) : n;
         if (k0 >= k1) continue;
-        const bool vl = x >= d, v2 = x + d < W, v3 = x + 2 * d < W;
+        const bool vl = x >= d, v2 = x + d < W, v3 = PAIR && x + 2 * d < W;
         const unsigned row_step = static_cast<unsigned>(d * W) * 8u, dx = static_cast<unsigned>(d) * 8u;
         unsigned at = data + static_cast<unsigned>(((res_class + k0 * d) * W + x) * 8);
-        float2 plo[4], phi[4];
-        auto next4 = [&]() {
+        float2 plo[kCols + 2], phi[kCols + 2];
+        auto next_row = [&]() {
           uint2 u[4];
           u[0] = u[2] = u[3] = make_uint2(0u, 0u);
           if (vl) u[0] = lds64(at - dx);
@@ -570,68 +571,86 @@ __global__ void __launch_bounds__(256, (PLANE > 0 && !PAIR) ? 3 : 2) depthwise_f
           if (v3) u[3] = lds64(at + 2 * dx);
           at += row_step;
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
+          for (int i = 0; i < kCols + 2; ++i) {
             plo[i] = __half22float2(*reinterpret_cast<const __half2*>(&u[i].x));
             phi[i] = __half22float2(*reinterpret_cast<const __half2*>(&u[i].y));
           }
         };
-        auto fma2 = [&](Acc* a, int kr) {
+        auto fma_cols = [&](Acc* a, int kr) {
 #pragma unroll
-          for (int k = 0; k < 3; ++k) {
-            a[0].lo = __ffma2_rn(plo[k], wlo[kr * 3 + k], a[0].lo);
-            a[0].hi = __ffma2_rn(phi[k], whi[kr * 3 + k], a[0].hi);
-            a[1].lo = __ffma2_rn(plo[k + 1], wlo[kr * 3 + k], a[1].lo);
-            a[1].hi = __ffma2_rn(phi[k + 1], whi[kr * 3 + k], a[1].hi);
-          }
+          for (int k = 0; k < 3; ++k)
+#pragma unroll
+            for (int i = 0; i < kCols; ++i) {
+              a[i].lo = __ffma2_rn(plo[k + i], wlo[kr * 3 + k], a[i].lo);
+              a[i].hi = __ffma2_rn(phi[k + i], whi[kr * 3 + k], a[i].hi);
+            }
         };
-        auto start2 = [&](Acc* a) {
-          a[0] = a[1] = bias_acc;
-          fma2(a, 0);
+        auto start = [&](Acc* a) {
+#pragma unroll
+          for (int i = 0; i < kCols; ++i) a[i] = bias_acc;
         };
-        auto emit2 = [&](const Acc* a) {
+        auto emit_cols = [&](const Acc* a) {
           __half* const first = op;
           emit(a[0]);
-          __half* const next = op;
-          op = first + d * 4;
-          if (v2) emit(a[1]);
-          op = next;
+          if (PAIR) {
+            __half* const next = op;
+            op = first + d * 4;
+            if (v2) emit(a[kCols - 1]);
+            op = next;
+          }
         };
-        Acc a0[2], a1[2], a2[2];
-        a0[0] = a0[1] = bias_acc;
+        Acc a0[kCols], a1[kCols], a2[kCols];
+        start(a0);
         if (k0 > 0) {
           at -= row_step;
-          next4();
-          fma2(a0, 0);
+          next_row();
+          fma_cols(a0, 0);
         }
-        next4();
-        fma2(a0, 1);
-        start2(a1);
+        next_row();
+        fma_cols(a0, 1);
+        start(a1);
+        fma_cols(a1, 0);
         // rows beyond the segment's last output row end it; beyond the plane's last row there is nothing to add
         for (int k = k0 + 1;; k += 3) {
-          if (k < n) {
-            next4();
-            fma2(a0, 2);
+          if (!PAIR && k >= n) {
+            emit_cols(a0);
+            break;
           }
-          emit2(a0);
-          if (k >= k1) break;
-          fma2(a1, 1);
-          start2(a2);
-          if (k + 1 < n) {
-            next4();
-            fma2(a1, 2);
+          if (!PAIR || k < n) {
+            next_row();
+            fma_cols(a0, 2);
           }
-          emit2(a1);
-          if (k + 1 >= k1) break;
-          fma2(a2, 1);
-          start2(a0);
-          if (k + 2 < n) {
-            next4();
-            fma2(a2, 2);
+          emit_cols(a0);
+          if (PAIR && k >= k1) break;
+          fma_cols(a1, 1);
+          start(a2);
+          fma_cols(a2, 0);
+          if (!PAIR && k + 1 >= n) {
+            emit_cols(a1);
+            break;
           }
-          emit2(a2);
-          if (k + 2 >= k1) break;
-          fma2(a0, 1);
-          start2(a1);
+          if (!PAIR || k + 1 < n) {
+            next_row();
+            fma_cols(a1, 2);
+          }
+          emit_cols(a1);
+          if (PAIR && k + 1 >= k1) break;
+          fma_cols(a2, 1);
+          start(a0);
+          fma_cols(a0, 0);
+          if (!PAIR && k + 2 >= n) {
+            emit_cols(a2);
+            break;
+          }
+          if (!PAIR || k + 2 < n) {
+            next_row();
+            fma_cols(a2, 2);
+          }
+          emit_cols(a2);
+          if (PAIR && k + 2 >= k1) break;
+          fma_cols(a0, 1);
+          start(a1);
+          fma_cols(a1, 0);
         }
       } else if (MODE == 1 && !PACKED && PLANE > 0) {
         // stride 2 without padding above / left on PLANE-wide planes, bands of exactly kRowsOut output rows: the band's
@@ -911,35 +930,64 @@ static int depthwise_f16_impl(const LaunchRec& r, const Ptrs& p, void* stream, b
   const int plane = whole_plane && g.H == 28 ? 28 : whole_plane && g.H == 14 ? 14 : whole_plane && g.H == 7 ? 7 : band28 ? 28 : pair14 ? g.W : down ? g.W : down14 ? 14 : 0;
   // the one-column straight-line variants need 80 registers: three CTAs per SM, so each gets a third of the shared memory
   const bool three_ctas = plane > 0 && !pair;
-  // Mode 3 for undilated planes as well where there is no straight-line form: half the threads, each with a third less to fetch and
-  // widen per output.  Not below 9 columns (5x5x1024 at batch 32 4.05 us with a column a thread, 4.39 with two) nor above 30 KB a plane
-  // (61x61x192 at batch 16 15.6 and 15.0, the largest measured).  us before and after: 33x33x960 batch 16 24.6, 21.0 (dilated by two 30,
-  // 21); 20x20x256 batch 32 7.5, 6.2; 40x40x128 batch 64 18.1, 15.9; 10x10x512 batch 256 17.9, 14.4; 26x26x192 batch 64 12.4, 11.9.
-  const bool walk = dilated || (mode == 0 && plane == 0 && !pair && same && g.W >= 9 && static_cast<long long>(g.Pin) * 8 <= 30 * 1024);
-  if (walk) {
-    mode = 3;
-    packed = true;
-    wcols = g.Wo / (2 * g.dil) * g.dil + std::min(g.dil, g.Wo % (2 * g.dil));
-    // a walk of at most 17 rows, shorter ones (down to five) until an SM has 256; items of about 120 walks
+  // Two columns a thread (mode 3) on dilated planes, and on undilated ones of at most 30 KB that have no straight-line form: they share
+  // a third of what each has to fetch and widen, but a row of such a walk takes 0.14 us where a row of one column takes 0.06 (small
+  // launches, one walk a thread).  Walks are cut into segments of rows until an SM has 256 of them.
+  //   Undilated, items in the one-column form that fill the SMs: always, but for whole planes of 17 to 28 rows, which that form
+  //   stages with one copy too (us, one column and two: 21x21x192 batch 106 11.2, 14.0; 25x25x576 batch 49 18.4, 22.9).
+  //   33x33x960 batch 16 24.6, 22.1; 10x10x576 batch 57 0.88 times; 42x42x96 batch 66 0.86 times; 9x9 planes 0.87 times.
+  //   Undilated and fewer items: where the walk is a quarter of a column's, or 5 / 12 and the busiest SM gets at most 1.2 times the
+  //   warps.  9x9x1024 batch 1 3.03, 2.82; 33x33x960 batch 1 6.1, 4.0; 17x17x576 batch 1 stays: 2.93, 3.41.
+  //   Dilated: where the one-column form's items (up to eight planes) take its threads more than one pass, or the walk is a quarter of
+  //   a column's.  33x33x960 dilated by two batch 16 30, 21; batch 1 5.0, 3.8; 9x9x576 batch 1 stays: 2.5, 3.0.
+  // Over 708 random undilated planes of the networks (9 to 61 wide, batch 1 to 256) 0.95 times the time of one column a thread, 30 slower
+  // by more than 3 %; over 292 dilated ones 0.95 times, 21 slower by more than 6 %.  Two columns everywhere were 1.01 and 1.02 times,
+  // 315 and 173 slower by more than 3 %.
+  const bool walk_fits = mode == 0 && plane == 0 && !pair && same && g.W >= 9 && static_cast<long long>(g.Pin) * 8 <= 30 * 1024;
+  bool two = false;
+  if (dilated || walk_fits) {
     const int rows = (g.H + g.dil - 1) / g.dil;
+    const long long most = std::max(1LL, std::min(budget / (static_cast<long long>(g.Pin) * 8), static_cast<long long>(g.B)));
+    if (dilated) {
+      g.nb = static_cast<int>(std::min(8LL, most));
+      g.sub = g.dil;
+      g.tr = rows;
+      g.bands = 1;
+      buf_bytes = static_cast<size_t>(g.Pin) * 8 * g.nb + 16;
+    }
+    const long long items = static_cast<long long>(g.S) * ((g.B + g.nb - 1) / g.nb) * g.bands;
+    const int columns = g.nb * g.sub * wcols;
+    const bool many = items > 148 * (buf_bytes * 2 + 1024 > kSmemPerSm / 2 ? 1 : 2), tall = packed && g.H > 16 && g.H <= 28;
+    const int pairs = (g.Wo / (2 * g.dil) * g.dil + std::min(g.dil, g.Wo % (2 * g.dil))) * g.dil, min_rows = many && !dilated ? 5 : 3;
     int nseg = (rows + 16) / 17;
-    while (static_cast<long long>(g.S) * g.B * wcols * g.dil * nseg < 148 * 256 && rows >= 5 * (nseg + 1)) ++nseg;
-    const int per_plane = wcols * g.dil * nseg;
-    long long nb = std::max(1, (120 + per_plane / 2) / per_plane);
-    nb = std::max(1LL, std::min({nb, budget / (static_cast<long long>(g.Pin) * 8), static_cast<long long>(g.B)}));
+    while (static_cast<long long>(g.S) * g.B * pairs * nseg < 148 * 256 && rows >= min_rows * (nseg + 1) && pairs * (nseg + 1) <= 256) ++nseg;
+    // items of about 120 walks
+    const int tr = (rows + nseg - 1) / nseg;
+    long long nb = std::min<long long>(std::max(1, (120 + pairs * nseg / 2) / (pairs * nseg)), most);
     const long long chunks = (g.B + nb - 1) / nb;
-    g.nb = static_cast<int>((g.B + chunks - 1) / chunks);
-    g.tr = (rows + nseg - 1) / nseg;
-    g.sub = g.dil * nseg;
-    g.bands = 1;
-    g.packed = 1;
-    buf_bytes = static_cast<size_t>(g.Pin) * 8 * g.nb + 16;
+    nb = (g.B + chunks - 1) / chunks;
+    const auto warps = [](long long n, long long threads) { return (n + 147) / 148 * ((std::min(threads, 256LL) + 31) / 32); };
+    two = g.tr >= 4 * tr;
+    if (dilated) two = two || columns > 256;
+    else if (many) two = !tall;
+    else two = two || (g.tr * 5 >= tr * 12 && warps(g.S * chunks, nb * pairs * nseg) * 5 <= warps(items, columns) * 6);
+    if (two) {
+      mode = 3;
+      packed = true;
+      wcols = pairs / g.dil;
+      g.nb = static_cast<int>(nb);
+      g.tr = tr;
+      g.sub = g.dil * nseg;
+      g.bands = 1;
+      g.packed = 1;
+      buf_bytes = static_cast<size_t>(g.Pin) * 8 * g.nb + 16;
+    }
   }
   const size_t per_cta = r.dw_cta_kb > 0 ? static_cast<size_t>(r.dw_cta_kb) * 1024
                                           : three_ctas ? static_cast<size_t>(73 * 1024) : static_cast<size_t>(kSmemPerCta);
   int nbuf = static_cast<int>(per_cta / buf_bytes);
   g.nbuf = nbuf > 4 ? 4 : nbuf < 2 ? 2 : nbuf;
-  if (walk) g.nbuf = 2;  // (three and four measured the same or slower: 33x33x960 21.0 us, 24)
+  if (two) g.nbuf = 2;  // (three and four measured the same or slower: 33x33x960 21.0 us, 24)
   const size_t smem = buf_bytes * g.nbuf;
   if (smem > static_cast<size_t>(kMaxSmem)) return static_cast<int>(cudaErrorInvalidConfiguration);
   g.bchunks = (g.B + g.nb - 1) / g.nb;
@@ -1010,6 +1058,8 @@ static int depthwise_f16_impl(const LaunchRec& r, const Ptrs& p, void* stream, b
   do {                                      \
     if (M == 0 && P == 0 && pair) {         \
       GI_DW_LAUNCH2(0, A, T, 0, 1);         \
+    } else if (M == 3 && P == 1 && two) {   \
+      GI_DW_LAUNCH2(3, A, T, 1, 1);         \
     } else {                                \
       GI_DW_LAUNCH2(M, A, T, P, 0);         \
     }                                       \

@@ -1332,9 +1332,8 @@ def test_depthwise_planes_with_rows_that_no_window_reaches(case):
     check_outputs(b.finish(), api.GI_F16)
 
 
-# (batch, h, w, c, dilation): planes without a straight-line form, two columns a thread: odd and even widths around whole and broken
-# groups of 2 d columns, one to four segments of a class of rows, classes of one row, the smallest width, the largest plane, more
-# items than CTAs and a last item with fewer planes
+# (batch, h, w, c, dilation): planes without a straight-line form: odd and even widths around whole and broken groups of 2 d columns,
+# one and more segments of a class of rows, classes of one row, the smallest width, the largest plane, a last item with fewer planes
 @pytest.mark.parametrize("case", [(1, 9, 9, 4, 1), (3, 33, 33, 20, 1), (2, 10, 17, 12, 1), (41, 13, 12, 7, 1), (2, 5, 61, 8, 1), (300, 20, 20, 16, 1), (7, 61, 61, 64, 1),
                                   (2, 34, 10, 260, 1), (2, 33, 35, 12, 4), (5, 33, 33, 96, 2), (1, 9, 33, 8, 9), (3, 7, 14, 8, 3), (2, 11, 3, 8, 2), (17, 61, 13, 8, 5)])
 @pytest.mark.parametrize("residual", [False, True])
@@ -1346,6 +1345,23 @@ def test_depthwise_two_columns_a_thread(case, residual):
     b.output(b.activation(b.add(x, y), wl.ACT_RELU) if residual else y)
     run, xs, outs = check_outputs(b.finish(), api.GI_F16, images=sorted({0, batch // 2, batch - 1}))
     assert "depthwise" in [api.KERNEL_NAMES[launch.kernel] for launch in run.ex.launches()]
+    assert all(np.array_equal(v, run.run(xs)[t]) for t, v in outs.items())
+    assert api.gi_device_status() == 0
+
+
+# (batch, h, w, c, dilation, two columns a thread): launches of few planes cut into many segments (three rows and more), whole planes
+# in one, three items a CTA and more (a buffer is filled again, the parity of its wait flips, the slice changes) with a last item
+# of fewer planes, classes of one row; one column: one and several items a CTA, a width below the dilation
+@pytest.mark.parametrize("case", [(1, 33, 33, 960, 1, True), (2, 9, 9, 260, 1, True), (41, 13, 12, 7, 1, True), (16, 33, 33, 576, 1, True), (1003, 10, 10, 260, 1, True),
+                                  (16, 33, 33, 96, 2, True), (1, 33, 33, 960, 2, True), (9, 61, 13, 8, 5, True), (299, 20, 20, 256, 2, True), (40, 14, 15, 130, 4, True),
+                                  (3, 7, 14, 8, 3, False), (1, 9, 33, 8, 9, True), (2, 11, 3, 8, 5, False), (9, 12, 13, 131, 2, False), (500, 5, 6, 300, 2, False)])
+def test_depthwise_walks(case):
+    batch, h, w, c, d, two = case
+    b = wl.GraphBuilder("depthwise_walk", batch, 36)
+    b.output(b.activation(b.depthwise(b.input(h, w, c), 3, 1, d), wl.ACT_RELU6))
+    run, xs, outs = check_outputs(b.finish(), api.GI_F16, images=sorted({0, batch // 2, batch - 1}))
+    kernels = [k for k in device_kernels(run, xs) if k.startswith("depthwise")]
+    assert kernels == [f"depthwise_f16_kernel<3, 2, false, true, {str(two).lower()}, 0>"], kernels
     assert all(np.array_equal(v, run.run(xs)[t]) for t, v in outs.items())
     assert api.gi_device_status() == 0
 
