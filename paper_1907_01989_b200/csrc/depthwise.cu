@@ -987,7 +987,7 @@ static int depthwise_f16_impl(const LaunchRec& r, const Ptrs& p, void* stream, b
                                           : three_ctas ? static_cast<size_t>(73 * 1024) : static_cast<size_t>(kSmemPerCta);
   int nbuf = static_cast<int>(per_cta / buf_bytes);
   g.nbuf = nbuf > 4 ? 4 : nbuf < 2 ? 2 : nbuf;
-  if (two) g.nbuf = 2;  // (three and four measured the same or slower: 33x33x960 21.0 us, 24)
+  if (two && r.dw_cta_kb == 0) g.nbuf = 2;  // (three and four measured the same or slower: 33x33x960 dilated by two 21.0 us, 24)
   const size_t smem = buf_bytes * g.nbuf;
   if (smem > static_cast<size_t>(kMaxSmem)) return static_cast<int>(cudaErrorInvalidConfiguration);
   g.bchunks = (g.B + g.nb - 1) / g.nb;

@@ -1,6 +1,8 @@
 """GPU parity: the CUDA path, called through the C ABI, against the CPU oracle on the same
 seeded inputs.  Tolerances: fp16 storage |gpu-oracle| <= 1e-2 + 1e-2*|oracle|; fp32 storage
 <= 1e-4 + 1e-4*|oracle| (element-wise)."""
+import json
+
 import numpy as np
 import pytest
 
@@ -1364,6 +1366,27 @@ def test_depthwise_walks(case):
     assert kernels == [f"depthwise_f16_kernel<3, 2, false, true, {str(two).lower()}, 0>"], kernels
     assert all(np.array_equal(v, run.run(xs)[t]) for t, v in outs.items())
     assert api.gi_device_status() == 0
+
+
+@pytest.mark.parametrize("cta_kb,buffers", [(None, 2), (56, 2), (110, 3), (150, 4)])
+def test_staging_sizes_of_two_column_walks(monkeypatch, tmp_path, cta_kb, buffers):
+    """The shared memory of one CTA that the environment asks for decides how many items are staged ahead, as for every other form
+    of the stencil: what the launch takes is a whole number of buffers of four planes."""
+    from torch.profiler import ProfilerActivity, profile
+    if cta_kb:
+        monkeypatch.setenv("GI_DW_CTA_KB", str(cta_kb))
+    run = DeviceRun(wl.single_depthwise(16, 33, 576, 1, 1), api.GI_F16)
+    xs = [wl.make_input(run.spec)]
+    want = run.run(xs)
+    with profile(activities=[ProfilerActivity.CUDA], acc_events=True) as prof:
+        got = run.run(xs)
+    prof.export_chrome_trace(str(tmp_path / "trace.json"))
+    events = json.load(open(tmp_path / "trace.json"))["traceEvents"]
+    shared = [e["args"]["shared memory"] for e in events if "depthwise_f16_kernel<3, 2, false, true, true, 0>" in e.get("name", "")]
+    assert len(shared) == 1 and shared[0] // (4 * 1090 * 8 + 16) == buffers, shared
+    t = run.spec.outputs[0]
+    assert np.array_equal(want[t], got[t])
+    assert_close(got[t][:1], og.run(run.spec, [xs[0][:1]], storage="f16", fused=True)[t], api.GI_F16, str(cta_kb))
 
 
 # (graph, layout of its output, bytes between the start of the output and that of the input): one launch from the caller's input to
