@@ -480,9 +480,11 @@ static LaunchRec conv_rec(const gi_graph& g, const gi_exec* e, const ConvOps& c)
 }
 
 // Estimated time of the run's ops as launches of their own: 4 us each (what a launch adds to a chain of them) plus their bytes
-// at the rates the kernels reach inside MobileNetV2 - 6 TB/s, 3.2 for a stencil on planes without a straight-line form, 4 for
-// the stem - plus 4 ns (1.2 ns where eight warps share the sum) per input channel of a 1x1 convolution, its chain of matrix instructions.  Against the measured
-// times of the network's ops at batch 1, 21 and 256 it is within 15 %.
+// at the rates the kernels reach inside MobileNetV2 - 6 TB/s, for a stencil on planes without a straight-line form 4 (stride 1, 9 pixels
+// wide and more, up to 30 KB) or 3.2, 4 for the stem - plus 4 ns (1.2 ns where eight warps share the sum) per input channel of a 1x1 convolution, its chain of matrix instructions.  Against the measured
+// times of the network's ops at batch 1, 21 and 256 it is within 15 %; 318 random stencils of the 4 TB/s kind, above 10 MB, take 1.00 to
+// 1.13 times less in the median of each size, at 4.4 TB/s 0.96 to 1.10.  But with 4.4 MobileNetV2 at batch 28 to 45 gives up fused
+// blocks that are faster (294.4 us, 298.3), with 4 only slower ones (batch 229 at 185 pixels 936, 907; 123 at 205 688, 676).
 static double separate_us(const gi_graph& g, const gi_exec* e, const OpGroup& gr) {
   double us = 0.0;
   auto bytes = [&](int t) {
@@ -515,8 +517,9 @@ static double separate_us(const gi_graph& g, const gi_exec* e, const OpGroup& gr
       else us += (pointwise_mma_wanted(pw) ? 0.0012 : 0.004) * e->tensors[o.in0].c;
     }
     if (o.kind == GI_OP_DEPTHWISE_CONV2D) {
-      const int w = e->tensors[o.out].w;
-      if (w != 112 && w != 56 && w != 28 && w != 14 && w != 7) rate = 3.2e6;
+      const TensorDesc &t = e->tensors[o.out], &x = e->tensors[o.in0];
+      const bool small = t.w == x.w && t.h == x.h && t.w >= 9 && plane_pixels(t.h, t.w) * 8 <= 30 * 1024;
+      if (t.w != 112 && t.w != 56 && t.w != 28 && t.w != 14 && t.w != 7) rate = small ? 4.0e6 : 3.2e6;
     }
     us += 4.0 + b / rate;
   }

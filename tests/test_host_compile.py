@@ -791,6 +791,13 @@ def test_no_block_reads_an_image_of_the_callers_layout_beyond_32_bit_offsets(c, 
     assert names[0] == "pack", names
 
 
+# (batch, image, blocks that run as one launch): where launches of their own, at what the stencil on planes of odd sizes really takes,
+# are faster than the fused 12x12 and 13x13 blocks of a large batch, and where they are not
+@pytest.mark.parametrize("batch,size,blocks", [(229, 185, 7), (123, 205, 11), (28, 234, 13), (21, 205, 13)])
+def test_blocks_that_run_as_launches_of_their_own(batch, size, blocks):
+    assert _launch_names(wl.mobilenet_v2(batch, size=size)).count("block_mma") == blocks
+
+
 BIAS_SPLIT_MAIN = r"""
 #include <cstdio>
 #include <cstring>
