@@ -1345,6 +1345,8 @@ void each_config(const LaunchRec& r, int kind, F&& f) {
             // specialised warps: as many as fit one, two or three CTAs of an SM, or one less (a wide expansion's warps work in
             // pairs); wide ones, of which there are few tiles, any number.  Narrow ones stay in one CTA: their clusters are small
             // tiles for the older kernel.  Not with a bias of the expansion that has no parts (bias_split.h).
+            // More than four chunks of weights come through the ring: resident they take 0.96 to 0.99 times the time near the best
+            // choices where as many CTAs fit an SM, 1.1 to 1.3 times where one fewer does, which the estimate does not tell apart.
             int specialised = 0;  // cluster sizes with such a layout
             if (c.wk == 0 && c.first != kNone && r.split_bias && (c.ni == 1 || c.first == kExpWide)) {
               const int cap = max_warps(c.s, c.np, c.tr, true);
@@ -1353,14 +1355,11 @@ void each_config(const LaunchRec& r, int kind, F&& f) {
                 if (c.ks > 1 && units * c.ks > 148) break;
                 for (c.nw_min = cap; c.nw_min >= 2; --c.nw_min) {
                   if (c.first != kExpWide && cap / (cap / c.nw_min) != c.nw_min && cap / (cap / (c.nw_min + 1)) != c.nw_min + 1) continue;
-                  for (int rk = 0; rk < 2; ++rk) {
-                    c.resident_kb = rk ? 64 : 0;
-                    Layout l;
-                    if (!layout_of(r, c, &l) || (rk && !l.resident)) continue;
-                    specialised |= c.ks;
-                    if (c.ks == 1 || units <= cluster_slots(c.ks) * ctas_per_sm(c, l)) f(c, l, false);
-                    if (l.resident) break;
-                  }
+                  c.resident_kb = 0;
+                  Layout l;
+                  if (!layout_of(r, c, &l)) continue;
+                  specialised |= c.ks;
+                  if (c.ks == 1 || units <= cluster_slots(c.ks) * ctas_per_sm(c, l)) f(c, l, false);
                 }
               }
               c.ws = 0;
