@@ -1154,9 +1154,8 @@ def test_blocks_whose_input_ends_inside_a_step_of_channels(batch, hw, cin):
 
 
 # (batch, h, w, cin, hidden, cout, stride) of blocks whose expansion and depthwise operator run on warps of their own: the fewest
-# chunks of hidden channels it takes (four, the last one not full), more tiles than CTAs (two and more rounds of both hidden tiles),
-# rings and resident weights, one and two CTAs of an SM, tiles with and without pixels outside the image, clusters, several
-# images a tile, every width of the expansion and of the output
+# chunks of hidden channels it takes (four, the last one not full), one tile a CTA (56x56: two), one and two CTAs of an
+# SM, tiles with and without pixels outside the image, clusters, several images a tile, every width of the expansion
 WARP_ROLES_CASES = [(3, 129, 131, 16, 96, 24, 2), (40, 33, 35, 10, 50, 12, 1), (6, 131, 67, 16, 64, 40, 2), (8, 65, 67, 24, 144, 24, 1),
                     (24, 57, 55, 21, 100, 21, 2), (40, 56, 56, 24, 144, 24, 1), (16, 65, 63, 32, 192, 32, 1), (33, 29, 27, 30, 200, 64, 2),
                     (16, 33, 33, 64, 384, 64, 1), (21, 13, 13, 64, 384, 64, 1), (24, 13, 13, 96, 576, 96, 1), (24, 14, 14, 96, 576, 160, 2),
@@ -1166,8 +1165,8 @@ WARP_ROLES_CASES = [(3, 129, 131, 16, 96, 24, 2), (40, 33, 35, 10, 50, 12, 1), (
 @pytest.mark.parametrize("case", WARP_ROLES_CASES)
 @pytest.mark.parametrize("bias", [None, 7.0e4])
 def test_blocks_with_roles_for_warps(case, bias):
-    """Equal to the oracle (first and last image) and to one kernel per op (all) within the tolerance; the same bits again.  Biases of
-    the expansion beyond the range of fp16, and far below its smallest number, are as good as others."""
+    """Equal to the oracle (first and last image) and to one kernel per op (all) within the tolerance; the same bits again; biases of
+    the expansion beyond the range of fp16, and far below its smallest number, among them."""
     batch, h, w, cin, hidden, cout, stride = case
     spec = wl.inverted_residual_block(batch, h, w, cin, hidden, cout, stride)
     if bias is not None:
@@ -1183,6 +1182,44 @@ def test_blocks_with_roles_for_warps(case, bias):
     assert run.guard_intact()
     t = spec.outputs[0]
     sel = [0, batch - 1]
+    assert_close(outs[t][sel], og.run(spec, [xs[0][sel]], storage="f16", fused=True)[t], api.GI_F16, str(case))
+    assert_close(outs[t], DeviceRun(spec, api.GI_F16, cross_op=api.GI_XOP_OFF).run(xs)[t], api.GI_F16, "one kernel per op")
+    assert np.array_equal(outs[t], run.run(xs)[t])
+    assert api.gi_device_status() == 0
+
+
+# (batch, h, w, cin, hidden, cout, stride, width of the expansion: up to 16 / 24 / 32 / 160 channels, 16-channel blocks of the output, rows
+# a warp walks down): every instantiation of the kernel whose warps have roles, all but three with more tiles than fit the SMs at a
+# time (the next tile's input, both hidden tiles and the ring over a second and a third tile), clusters of two and four, one to four CTAs
+# an SM, weights of four chunks resident, whole images on tiles without a border, several a tile
+ROLES_FORMS = [(166, 21, 19, 16, 91, 12, 1, 1, 1, 2), (29, 64, 65, 8, 67, 8, 1, 1, 1, 4), (5, 13, 12, 4, 68, 30, 1, 1, 2, 1), (226, 20, 19, 4, 72, 24, 1, 1, 2, 2),
+               (25, 56, 57, 4, 69, 40, 1, 1, 4, 1), (286, 16, 17, 16, 64, 48, 1, 1, 4, 1), (304, 15, 15, 8, 97, 64, 1, 1, 4, 1), (177, 17, 18, 8, 125, 48, 1, 1, 4, 2),
+               (310, 13, 13, 20, 101, 8, 1, 2, 1, 2), (13, 95, 97, 20, 154, 8, 1, 2, 1, 4), (5, 11, 11, 24, 68, 32, 1, 2, 2, 1), (177, 18, 20, 20, 71, 24, 1, 2, 2, 2),
+               (247, 14, 15, 20, 87, 40, 1, 2, 4, 1), (21, 56, 57, 24, 185, 48, 1, 2, 4, 2), (196, 15, 14, 32, 75, 16, 1, 3, 1, 2),
+               (242, 18, 17, 30, 220, 8, 1, 3, 1, 4), (347, 13, 11, 32, 70, 30, 1, 3, 2, 1), (340, 12, 11, 32, 114, 24, 1, 3, 2, 2),
+               (166, 13, 15, 28, 142, 48, 1, 3, 4, 1), (218, 16, 18, 32, 65, 48, 1, 3, 4, 1), (38, 39, 38, 30, 211, 64, 1, 3, 4, 2), (1, 4, 4, 40, 549, 12, 1, 4, 2, 1),
+               (4, 7, 5, 64, 251, 32, 1, 4, 2, 1), (43, 28, 27, 40, 105, 30, 1, 4, 2, 1), (150, 9, 11, 80, 205, 16, 1, 4, 2, 2), (40, 33, 33, 64, 384, 64, 1, 4, 4, 1),
+               (303, 8, 10, 40, 228, 48, 1, 4, 4, 1), (600, 7, 7, 40, 160, 40, 1, 4, 4, 1), (349, 12, 10, 40, 341, 64, 1, 4, 4, 2),
+               (157, 12, 10, 48, 214, 96, 1, 4, 6, 1), (39, 5, 7, 80, 286, 120, 1, 4, 10, 1), (152, 18, 18, 4, 119, 24, 2, 1, 2, 2),
+               (297, 15, 13, 8, 121, 48, 2, 1, 4, 2), (167, 22, 21, 20, 161, 32, 2, 2, 2, 2), (339, 15, 13, 20, 127, 64, 2, 2, 4, 2),
+               (243, 16, 17, 28, 67, 16, 2, 3, 2, 2), (85, 31, 31, 32, 68, 64, 2, 3, 4, 2), (1, 4, 6, 40, 539, 8, 2, 4, 2, 2), (2, 4, 6, 112, 260, 24, 2, 4, 2, 2),
+               (80, 15, 16, 64, 144, 24, 2, 4, 2, 2), (149, 12, 10, 96, 128, 40, 2, 4, 4, 2), (152, 9, 9, 128, 97, 80, 2, 4, 6, 2),
+               (173, 10, 9, 40, 135, 120, 2, 4, 10, 2)]
+
+
+@pytest.mark.parametrize("case", ROLES_FORMS)
+def test_every_form_of_blocks_with_roles_for_warps(case):
+    """All images equal one kernel per op within the tolerance, the first and the last the oracle; the same bits again."""
+    batch, h, w, cin, hidden, cout, stride, first, np_, tr = case
+    spec = wl.inverted_residual_block(batch, h, w, cin, hidden, cout, stride)
+    xs = [wl.make_input(spec)]
+    run = DeviceRun(spec, api.GI_F16, guard_bytes=4096)
+    kernels = [k for k in device_kernels(run, xs) if k.startswith("block")]
+    assert kernels == [f"block_ws_kernel<{stride}, {first}, {np_}, {tr}>"], kernels
+    outs = run.run(xs)
+    assert run.guard_intact()
+    t = spec.outputs[0]
+    sel = sorted({0, batch - 1})
     assert_close(outs[t][sel], og.run(spec, [xs[0][sel]], storage="f16", fused=True)[t], api.GI_F16, str(case))
     assert_close(outs[t], DeviceRun(spec, api.GI_F16, cross_op=api.GI_XOP_OFF).run(xs)[t], api.GI_F16, "one kernel per op")
     assert np.array_equal(outs[t], run.run(xs)[t])
