@@ -984,21 +984,26 @@ __global__ void __launch_bounds__(32 * max_warps(S, NP, TR, true), 1) block_ws_k
             }
 #pragma unroll
             for (int i = 0; i < N; ++i) {
-              mma16816z(d[i][0], a[i], b0.x, b0.y);
-              mma16816z(d[i][1], a[i], b0.z, b0.w);
+              if (FIRST == kExp24) {
+                mma16816z(d[i][0], a[i], b0.x, b0.y);
+                mma16816z(d[i][1], a[i], b0.z, b0.w);
+              } else {  // the bias first: behind the products its sum is rounded once more (32 channels: 10 % more stored values differ)
+                mma1688z(d[i][0], ones, ones, one[0]);
+                mma1688z(d[i][1], ones, ones, one[1]);
+              }
+            }
+            if (FIRST != kExp24) {
+#pragma unroll
+              for (int i = 0; i < N; ++i) {
+                mma16816(d[i][0], a[i], b0.x, b0.y);
+                mma16816(d[i][1], a[i], b0.z, b0.w);
+              }
             }
             if (FIRST != kExp16) {
 #pragma unroll
               for (int i = 0; i < N; ++i) {
                 mma16816(d[i][0], a2[i], b1.x, b1.y);
                 mma16816(d[i][1], a2[i], b1.z, b1.w);
-              }
-            }
-            if (FIRST != kExp24) {
-#pragma unroll
-              for (int i = 0; i < N; ++i) {
-                mma1688(d[i][0], ones, ones, one[0]);
-                mma1688(d[i][1], ones, ones, one[1]);
               }
             }
 #pragma unroll

@@ -1280,6 +1280,23 @@ def test_small_tiles_whose_weights_stay_in_a_cluster(case):
     assert api.gi_device_status() == 0
 
 
+@pytest.mark.parametrize("case", [(3, 129, 131, 16, 96, 24, 2), (40, 61, 60, 16, 96, 40, 1), (16, 65, 63, 32, 192, 32, 1), (33, 57, 57, 30, 200, 64, 2)])
+def test_bias_products_and_sums_started_at_the_bias_are_the_same(case):
+    """A bias that has fp16 parts and one that has none, of a channel that is zero either way, choose the kernel: with warps of their
+    own for the expansion, whose bias is a product, and with sums that start at the bias.  Where the bias comes before the products (up to
+    16 and 25 to 32 channels, one CTA a tile) both round the same sums."""
+    batch, h, w, cin, hidden, cout, stride = case
+    outs, kernels = [], []
+    for bias in (-1.0e8, -1.0e9):
+        spec = wl.inverted_residual_block(batch, h, w, cin, hidden, cout, stride)
+        spec.ops[0].bias[1] = bias
+        run, xs = DeviceRun(spec, api.GI_F16), [wl.make_input(spec)]
+        kernels += [k.split("<")[0] for k in device_kernels(run, xs) if k.startswith("block")]
+        outs.append(run.run(xs)[spec.outputs[0]])
+    assert kernels == ["block_ws_kernel", "block_mma_kernel"], kernels
+    assert np.array_equal(*outs)
+
+
 def _twice_activated(kind, first, second):
     b = wl.GraphBuilder("twice_activated", 2, 32)
     if kind == "stem":
