@@ -37,8 +37,8 @@
 // MobileNetV2 batch 1 169 -> 160 us, 8 x 192 207 -> 186, segmentation batch 1 229 -> 211.
 //
 // What bounds it.  Small launches: that chain.  Large ones: block_ws_kernel.  Measured on one B200 against separate kernels, stem included
-// (stem_block.cu), MobileNetV2: batch 1 225 -> 155 us, 21 images of 205 pixels 340 -> 270, batch 256 1413 -> 1298;
-// segmentation network batch 1 289 -> 207, batch 16 961 -> 748.
+// (stem_block.cu), MobileNetV2: batch 1 225 -> 155 us, 21 images of 205 pixels 340 -> 270 (248 with specialised warps), batch 256
+// 1413 -> 1298 (1193); segmentation network batch 1 289 -> 207 (198), batch 16 961 -> 748 (684).
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
@@ -784,13 +784,13 @@ __global__ void __launch_bounds__(32 * max_warps(S, NP, TR), 1) block_mma_kernel
 // warps share, stay on the kernel above.
 //
 // What it is for: with both halves in one warp the projection's sums stay live through the expansion, the register file makes the
-// compiler move them, and a warp that waits for its shared memory has nobody to take its place.  Of 33.4 M warp instructions of 112x112
-// 16 -> 96 -> 24, stride 2, at batch 64 are left 24.8 M (3 M of them because a bias as a sum's start value costs four moves a
-// matrix instruction: the expansion's comes as a product with ones, the depthwise operator's as one two-wide addition behind the
-// sum).  Kernel above -> this one, us on one B200: that block 63.4 -> 52.3, 56x56 24 -> 144 -> 24 at batch 64 51.4 -> 43.7, 14x14
+// compiler move them, and a warp that waits for its shared memory has nobody to take its place.  Of 129 M warp instructions of 112x112
+// 16 -> 96 -> 24, stride 2, at batch 256 are left 98 M (some because a bias as a sum's start value costs four moves a matrix
+// instruction: the expansion's comes as a product with ones in front of the others, with 17 to 24 channels beside the last eight, the
+// depthwise operator's as one two-wide addition behind the sum).  Kernel above -> this one, us on one B200: that block 63.4 -> 52.3, 56x56 24 -> 144 -> 24 at batch 64 51.4 -> 43.7, 14x14
 // 64 -> 384 -> 64 at batch 64 22.2 -> 17.7, 33x33 64 -> 384 -> 64 at batch 16 29.9 -> 25.3.  MobileNetV2 at batch 256 1299 -> 1192, 21
-// images of 205 pixels 271 -> 250, segmentation at batch 16 748 -> 713.  What bounds it now: shared memory's pipe (62 % of its
-// wavefronts on the first of these) and the latency from ldmatrix to store with 12 to 16 warps; the matrix pipe is 27 % busy.
+// images of 205 pixels 271 -> 250, segmentation at batch 16 748 -> 713.  What bounds it now: shared memory's pipe (67 % of its
+// wavefronts on the first of these) and the latency from ldmatrix to store with 12 to 16 warps; the matrix pipe is 30 % busy.
 template <int S, int FIRST, int NP, int TR>
 __global__ void __launch_bounds__(32 * max_warps(S, NP, TR, true), 1) block_ws_kernel(const BlockParams p) {
   extern __shared__ __align__(128) unsigned char smem_raw[];

@@ -65,7 +65,7 @@ struct BlockCfg {
   int ks = 1;                   // CTAs (a cluster) that share a unit's hidden channels
   int wk = 0;                   // > 0: small tiles, sets of warps that share a chunk's channels, 16 each (`hc` is 1)
   int nw_min = 8;               // warps of a CTA, if the first operator has work for them; ws: exactly
-  int ws = 0;                   // narrow expansions: expansion and depthwise operator on warps of their own
+  int ws = 0;                   // expansion and depthwise operator on warps of their own
   int resident_kb = 0;          // weights of at most this size stay in shared memory
 };
 
